@@ -12,6 +12,8 @@ calibrates it; without it beta is 0.  ``kept`` = r keeps experts 0 .. r-1.
 """
 from __future__ import annotations
 
+import itertools
+
 import numpy as np
 import torch
 
@@ -183,3 +185,109 @@ def tolerance(case):
     if kind == "stack":
         return {"rel": 1e-2, "max": 0.085}   # bf16 states through several layers (seen: 2.7e-3, 0.021)
     return {"rel": 4e-3, "max": 0.032}       # bf16 outputs (seen: 8.4e-4, 0.0078 = one bf16 step)
+
+
+def _exact_weights(shape, seed):
+    s = SHAPES[shape]
+    return synth.make_layer_weights(s["h"], s["f"], s["E"], seed=seed, device=DEV)
+
+
+def _exact_logits(W, x, kept):
+    """Logits [T][E] over the first `kept` experts; the others cannot be chosen."""
+    logits = x.double() @ W.W_gate.double().T
+    logits[:, kept:] = -torch.inf
+    return logits
+
+
+def _exact_ranked(W, x, kept):
+    """The logits in descending order and their experts, ties to the lower index."""
+    return _exact_logits(W, x, kept).sort(dim=1, descending=True, stable=True)
+
+
+def _exact_expert(W, e, x):
+    x = x.double()
+    act = torch.nn.functional.silu(x @ W.W1[e].double().T) * (x @ W.W3[e].double().T)
+    return act @ W.W2[e].double().T
+
+
+def _exact_ratio_median(W, x, kept):
+    ranked, _ = _exact_ranked(W, x, kept)
+    ratio = torch.exp(ranked[:, 1] - ranked[:, 0]).sort().values
+    T = ratio.numel()
+    return float((ratio[(T - 1) // 2] + ratio[T // 2]) / 2)
+
+
+def _exact_mix(W, x, idx, wn):
+    """sum_m wn[:, m] E_idx[:, m](x); an expert of weight 0 is not run."""
+    z = torch.zeros(x.shape, dtype=torch.float64, device=x.device)
+    for e in range(W.E):
+        t, m = torch.nonzero((idx == e) & (wn > 0), as_tuple=True)
+        if t.numel():
+            z[t] += wn[t, m, None] * _exact_expert(W, e, x[t])   # a token has an expert once
+    return z
+
+
+def _exact_top2(W, x, kept, beta):
+    ranked, order = _exact_ranked(W, x, kept)
+    p = torch.exp(ranked[:, :2] - ranked[:, :1])
+    p[:, 1] *= ~(p[:, 1] < beta)
+    return order[:, :2], p / p.sum(1, keepdim=True)
+
+
+def _exact_topk(W, x, k, beta):
+    ranked, order = _exact_ranked(W, x, W.E)
+    p = torch.exp(ranked[:, :k] - ranked[:, :1])
+    tail = p.flip(1).cumsum(1).flip(1) - p                        # mass after rank m
+    n_active = (tail > beta * p.sum(1, keepdim=True)).sum(1) + 1   # the first i whose tail is small enough
+    p = p * (torch.arange(k, device=p.device)[None] < n_active[:, None])
+    return order[:, :k], p / p.sum(1, keepdim=True)
+
+
+def _exact_search(W, x, sizes):
+    logits = _exact_logits(W, x, W.E)
+    Y = torch.stack([_exact_expert(W, e, x) for e in range(W.E)], dim=1)
+    rows = torch.arange(x.shape[0], device=x.device)
+
+    def mixed(subset):
+        ranked, order = logits[:, subset].sort(dim=1, descending=True, stable=True)
+        p = torch.softmax(ranked[:, :2], dim=1)
+        order = torch.tensor(subset, device=x.device)[order]
+        return p[:, :1] * Y[rows, order[:, 0]] + p[:, 1:] * Y[rows, order[:, 1]]
+
+    full = mixed(list(range(W.E)))
+    return [np.array([float((mixed(list(c)) - full).norm()) for c in itertools.combinations(range(W.E), r)])
+            for r in sizes]
+
+
+def exact(case, seed):
+    """What ``run`` returns, computed in 64 bits from the same inputs without any intermediate rounding;
+    None for whole-number outputs."""
+    kind, T, base = case["kind"], case["tokens"], 1000 * seed
+    kept = case.get("kept", SHAPES[case["shape"]]["E"])
+    W = _exact_weights(case["shape"], base)
+    x = synth.make_tokens(T, W.h, seed=base + 500, device=DEV)
+
+    def beta(W, i=0):
+        if not case.get("skip"):
+            return 0.0
+        return _exact_ratio_median(W, synth.make_tokens(CAL_TOKENS, W.h, seed=base + 600 + i, device=DEV), kept)
+
+    if kind == "calibrate":
+        return _exact_ratio_median(W, x, kept)
+    if kind == "search":
+        return {"losses": _exact_search(W, x, [6, 4] if case["r4"] else [6]), "best": None}
+    if kind == "topk":
+        idx, wn = _exact_topk(W, x, case["k"], TOPK_BETA if case["skip"] else 0.0)
+        return {"y": _exact_mix(W, x, idx, wn), "idx": None, "wn": wn, "n_active": None}
+    if kind == "stack":
+        state = x.double()
+        for i in range(case["layers"]):
+            W = W if i == 0 else _exact_weights(case["shape"], base + i)
+            xn = state * torch.rsqrt(state.square().mean(1, keepdim=True) + 1e-5)
+            state = state + _exact_mix(W, xn, *_exact_top2(W, xn, kept, beta(W, i)))
+        return state
+    idx, wn = _exact_top2(W, x, kept, beta(W))
+    y = _exact_mix(W, x, idx, wn)
+    if case.get("record"):
+        return {"y": y, "idx": None, "wn": wn, "skipped": None, "count": None}
+    return y.cpu() if kind == "host" else y
