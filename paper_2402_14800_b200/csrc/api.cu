@@ -263,10 +263,11 @@ int check_status(moe_layer* L) {
   return MOE_OK;
 }
 
-// The two grouped GEMMs of the experts over a batch described by `meta`.
+// The two grouped GEMMs of the experts over a batch described by `meta`, of at most `pairs`
+// token-expert pairs.
 int run_expert_gemms(moe_layer* L, const Meta* meta, bool weights_m, const GemmMaps& m_gu,
                      const GemmMaps& m_dn, GemmArgs gu, GemmArgs dn, GemmOut dn_kind,
-                     const bf16* gu_A, const bf16* dn_A, int simt_rows, int T = 0) {
+                     const bf16* gu_A, const bf16* dn_A, int simt_rows, long long pairs, int T = 0) {
   gu.meta = meta; dn.meta = meta;
   gu.r = L->r; dn.r = L->r;
   gu.K = L->h; gu.n_w_rows = 2 * L->f;
@@ -284,6 +285,10 @@ int run_expert_gemms(moe_layer* L, const Meta* meta, bool weights_m, const GemmM
     CUDA_TRY(launch_gemm_tokens_d(true, m_gu, gu, (L->h + 63) / 64, L->stream));
     mark(L);
     CUDA_TRY(launch_gemm_tokens_d(false, m_dn, dn, down_kb_per_item(T), L->stream));
+  } else if (pairs <= (long long)kPairMaxRows * L->r) {
+    CUDA_TRY(launch_gemm_pair_n(true, kOutActBf16, m_gu, gu, L->stream));
+    mark(L);
+    CUDA_TRY(launch_gemm_pair_n(false, dn_kind, m_dn, dn, L->stream));
   } else {
     CUDA_TRY(launch_gemm_tokens_m(true, kOutActBf16, m_gu, gu, L->stream));
     mark(L);
@@ -388,7 +393,7 @@ int forward_impl(moe_layer* L, const void* x, int T, float beta, const void* res
   memcpy(m_gu.t, L->ws->tok_x, sizeof(m_gu.t));
   memcpy(m_dn.t, L->ws->tok_act, sizeof(m_dn.t));
   rc = run_expert_gemms(L, meta, wm, m_gu, m_dn, gu, dn, kOutF32, (const bf16*)L->ws->xperm.p,
-                        (const bf16*)L->ws->act.p, rows_cap, T);
+                        (const bf16*)L->ws->act.p, rows_cap, 2ll * T, T);
   if (rc) return rc;
   mark(L);
   if (dist)
@@ -640,7 +645,7 @@ int moe_forward_topk(moe_layer_t* L, const void* x, int T, int k, float beta, vo
   const bool prof_saved = L->prof;
   L->prof = false;
   rc = run_expert_gemms(L, meta, wm, m_gu, m_dn, gu, dn, kOutF32, (const bf16*)W.xperm.p,
-                        (const bf16*)W.act.p, rows_cap, T);
+                        (const bf16*)W.act.p, rows_cap, (long long)k * T, T);
   L->prof = prof_saved;
   if (rc) return rc;
   CUDA_TRY(launch_combine_topk((const float*)W.O.p, ksplit, split_stride, (int32_t*)W.k_pos.p,
@@ -865,7 +870,7 @@ static int search_impl(moe_layer_t* L, const void* x_calib, const float* F_ref, 
       dn.a_off_mul = 1; dn.out_off_mul = 1; dn.out_row_base = c * rows_chunk; dn.out_ld = h;
       dn.out = W.s_yall.p;
       if ((rc = run_expert_gemms(L, meta, false, m_gu, m_dn, gu, dn, kOutBf16, (const bf16*)W.s_xperm.p,
-                                 (const bf16*)W.s_act.p, rows_chunk))) {
+                                 (const bf16*)W.s_act.p, rows_chunk, (long long)K * rows))) {
         L->prof = prof_saved;
         return rc;
       }
@@ -911,7 +916,7 @@ static int search_impl(moe_layer_t* L, const void* x_calib, const float* F_ref, 
       dn.a_off_mul = 1; dn.out_row_base = t0; dn.out_off_mul = 0; dn.out_col_mul = h;
       dn.out_ld = (long long)E * h; dn.out = W.s_yall.p;
       if ((rc = run_expert_gemms(L, meta, false, m_gu, m_dn, gu, dn, kOutBf16, xa,
-                                 (const bf16*)W.s_act.p, rows))) {
+                                 (const bf16*)W.s_act.p, rows, (long long)E * rows))) {
         L->prof = prof_saved;
         return rc;
       }

@@ -20,6 +20,13 @@ constexpr int kInterleave = 16;           // W1/W3 rows are interleaved in group
 constexpr int kDecodeMaxT = 256;          // up to here the small-batch path (weights read once) is used
 constexpr int kTokensDPerExpert = 40;      // small batches with this many tokens per expert or more: token-major decode GEMM
 constexpr int kTokensDMaxKept = 6;         // ... on layers with at most this many kept experts
+// Large batches with at most this many pairs per kept expert run gemm_pair_n, the others
+// gemm_tokens_m.  Alternating 1.5 s runs at the power cap, Mixtral layer, 8 experts (gemm_tokens_m
+// vs gemm_pair_n, whole step): 1500 tokens 1.30 vs 1.17 ms, 2500 1.85 vs 1.70, 3500 2.40 vs 2.28,
+// 5000 3.23 vs 3.16; at 8192 (2048 a group) -1.5 .. +1.8 % depending on the board, and the search's
+// 6144 a group was up to 6 % slower on the pairs: with little padding to save, both are held by the
+// board's power and the pairs draw 1-3 % more energy per call.
+constexpr int kPairMaxRows = 1536;
 constexpr int kDecodeKbPerItem = 112;      // k-blocks (of 64) per split-K item, decode down-proj
 
 // Device-resident description of one permuted batch, written by the scan kernel
@@ -214,6 +221,9 @@ struct GemmMaps {
 // Token rows are the 128-row MMA operand, weights the 256-wide one (large T).
 cudaError_t launch_gemm_tokens_m(bool gate_up, GemmOut out_kind, const GemmMaps& maps,
                                  const GemmArgs& a, cudaStream_t st);
+// On CTA pairs: weight rows are the 256-row MMA operand, up to 256 tokens the other (large T).
+cudaError_t launch_gemm_pair_n(bool gate_up, GemmOut out_kind, const GemmMaps& maps,
+                               const GemmArgs& a, cudaStream_t st);
 // Weight rows are the 128-row MMA operand, tokens the narrow one (small T): weights stream once.
 cudaError_t launch_gemm_tokens_d(bool gate_up, const GemmMaps& maps, const GemmArgs& a, int kb_per_item,
                                  cudaStream_t st);

@@ -3,9 +3,11 @@
 //
 //   E_e(x) = W2_e ( silu(W1_e x) * (W3_e x) )      (Sec. 3.1; Mixtral's SwiGLU form)
 //
-// Three persistent, warp-specialised kernels share one pipeline skeleton:
-//   gemm_tokens_m   256 token rows x 256 weight rows per item on two accumulators; for large
+// Four persistent, warp-specialised kernels share one pipeline skeleton:
+//   gemm_tokens_m   256 token rows x 256 weight rows per item on two accumulators; for the largest
 //                   batches, where the work is a dense contraction bound by the tensor pipe.
+//   gemm_pair_n     512 weight rows x (32..256) tokens per item on a pair of CTAs; for batches
+//                   between the small and the largest, whose ragged groups it pads least.
 //   gemm_weights_m  128 weight rows x (16..128) tokens per item; for small batches, where
 //                   every weight byte is streamed from HBM exactly once.
 //   gemm_tokens_d   up to 128 token rows x 256 weight rows per item; small batches with many
@@ -220,17 +222,18 @@ struct Bars {
 };
 
 template <int NS>
-__device__ __forceinline__ void setup_barriers(Bars& b, uint32_t tmem_empty_arrivals = 4) {
+__device__ __forceinline__ void setup_barriers(Bars& b, uint32_t tmem_empty_arrivals = 4,
+                                               uint32_t mma_warps = 1) {
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(smem_u32(&b.full[s]), 1);
-      mbar_init(smem_u32(&b.empty[s]), 1);
+      mbar_init(smem_u32(&b.empty[s]), mma_warps);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&b.tmem_full[i]), 1);
       mbar_init(smem_u32(&b.tmem_empty[i]), tmem_empty_arrivals);
     }
-    mbar_init(smem_u32(&b.drain), 1);
+    mbar_init(smem_u32(&b.drain), mma_warps);
     b.abort_flag = 0;
     fence_barrier_init();
     fence_proxy_async();
@@ -564,6 +567,369 @@ gemm_tokens_m_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args)
   // whole run of this kernel costs issue slots and power
   pdl_launch_dependents();
   teardown<512>(bars, tmem_base, issued, ns, args.status);
+}
+
+// ------------------------------------------------------------------------- gemm_pair_n
+//
+// Batches between the small and the largest.  A pair of CTAs (cluster of two, cta_group::2)
+// computes 512 weight rows x up to 256 token rows per item.  The weights are the M operand (two
+// accumulators of M = 256: each CTA holds 128 rows of each), the tokens the N operand, half of
+// them staged by either CTA, so that
+//   - a ragged group is padded to the next 32 tokens, not to 128 (gemm_tokens_m multiplied 13-40 %
+//     of padding at 150-500 tokens a group), and an MMA of N columns takes N / 2 cycles;
+//   - a k-block brings 32 KB of weights + 64 B x N of tokens to an SM: 48 KB where gemm_tokens_m
+//     moves 64 KB for the same 1024 pipe cycles (13.1 instead of 17.4 GB from L2 for both launches
+//     of 3072 tokens on 4 experts).
+// What bounds it: HBM up to about 200 tokens a group, then the tensor pipe (84 % of its cycles busy
+// in the gate/up launch at 1536 tokens a group, of which 4 % is the partly filled last round) at
+// the clock that the board's power leaves.
+// Each accumulator has an issuing warp of its own: the pipe queues little beyond the MMA it executes,
+// so whatever one warp does between two MMAs (barrier wait, commit, loop) leaves it idle unless the
+// other's MMAs fill the gap.  One warp issuing for both took 5.04 ms at 8192 tokens, two take 4.8;
+// one warp that ran ahead on accumulator 0 by itself took 6.3.  With two warps that comes for free:
+// accumulator 0 is handed back as soon as the epilogue warps have it in registers, and its issuer goes
+// ahead through the ring while accumulator 1 is still being read.
+// Step, before (gemm_tokens_m) -> after, Mixtral layer, alternating runs: 512 tokens 719 -> 600 us,
+// 1024 1056 -> 901, 1500 1334 -> 1099, 2048 1658 -> 1442.
+//   full[s]        in the leader: one arrival (expect_tx of both CTAs' bytes) + the bytes
+//   empty[s]       in each CTA: the leader's two commits (one per accumulator) arrive on both
+//   tmem_full[a]   in each CTA: the leader's commit arrives on both
+//   tmem_empty[a]  in the leader: one arrival per epilogue warp of both CTAs
+
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// shared::cluster address of the same shared-memory offset in CTA `rank` of the pair
+__device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+__device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+}
+// loads of one CTA of a pair into its own shared memory, counted on a barrier of either CTA
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1,
+                                                 uint32_t bar_cluster) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3}], [%4];"
+      ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar_cluster)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1,
+                                                 int c2, uint32_t bar_cluster) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];"
+      ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(bar_cluster)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t smem_dst, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst),
+               "r"(ncols)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_relinquish_pair() {
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
+               : "memory");
+}
+__device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
+                                               uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n"
+      " .reg .pred p;\n"
+      " setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n"
+      "}\n"
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// arrives on the barrier at this shared-memory offset in both CTAs once the MMAs this thread
+// issued so far have completed
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+  const uint16_t both = 3;
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+      ::"r"(bar), "h"(both)
+      : "memory");
+}
+
+constexpr int PN_NS = 4;
+constexpr int PN_A_BYTES = 256 * 128;  // this CTA's 256 weight rows x 64 bf16
+constexpr int PN_B_BYTES = 128 * 128;  // this CTA's half of the token tile (16 .. 128 rows)
+constexpr int PN_STAGE = PN_A_BYTES + PN_B_BYTES;
+constexpr int PN_SMEM = PN_NS * PN_STAGE + 1024;
+constexpr int PN_W_ROWS = 512;         // weight rows of an item
+constexpr int PN_BAND = 16;            // at most so many token tiles sweep the weight tiles together
+constexpr int PN_EPI_WARPS = 16;
+constexpr int PN_THREADS = 96 + 32 * PN_EPI_WARPS;
+
+struct ItemN {
+  int c, nt;          // expert, weight tile
+  int tok0;           // first token of the tile inside the expert's group
+  int n, valid;       // columns of the MMA (a multiple of 32) and the tokens among them
+};
+
+// An expert's tokens are cut into as few tiles of at most 256 as hold them, of equal size up to
+// the grain of 32.
+__device__ __forceinline__ int token_tiles(int cnt) { return (cnt + 255) >> 8; }
+
+__device__ __forceinline__ void decode_item_n(const Meta& m, const GemmArgs& a, int item, int Nt, ItemN& t) {
+  int c = 0, first = 0, kt = token_tiles(m.count[0]);
+  while (c + 1 < a.r && item >= first + kt * Nt) {
+    first += kt * Nt;
+    kt = token_tiles(m.count[++c]);
+  }
+  const int local = item - first;
+  const int bands = (kt + PN_BAND - 1) / PN_BAND;
+  const int per_band = (kt + bands - 1) / bands;
+  const int band = local / (per_band * Nt);
+  const int rem = local - band * per_band * Nt;
+  const int band_tiles = min(per_band, kt - band * per_band);
+  t.c = c;
+  t.nt = rem / band_tiles;
+  const int i = band * per_band + rem - t.nt * band_tiles;
+  const int units = (m.count[c] + 31) >> 5;
+  const int q = units / kt, extra = units - q * kt;
+  t.tok0 = 32 * (i * q + min(i, extra));
+  t.n = 32 * (q + (i < extra ? 1 : 0));
+  t.valid = min(t.n, m.count[c] - t.tok0);
+}
+
+// 16 accumulator columns (tokens col0 .. col0 + 15 of the tile) of the 32 weight rows of a warp ->
+// output; `orow` = element offset of the tile's first token row, `wrow0` the first weight row.
+template <bool GATE_UP, int OUT>
+__device__ __forceinline__ void store_cols_n(const uint32_t* v, const GemmArgs& args, long long orow,
+                                             int wrow0, int col0, int valid, int lane) {
+  const int ld = (int)args.out_ld;
+  if (GATE_UP) {
+    // lanes 0-15 hold gate rows, lanes 16-31 the up rows of the same 16 features: of two tokens
+    // the lower half-warp takes the first, the upper half the second
+    const bool lo = lane < 16, odd = lane & 1;
+    const int tok = col0 + (lane >> 4) + 2 * (lane & 1);
+    bf16* out = reinterpret_cast<bf16*>(args.out) + orow + (wrow0 >> 1) + (lane & 14) + tok * ld;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float s[2];
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const uint32_t a = v[4 * q + 2 * p], b = v[4 * q + 2 * p + 1];
+        const uint32_t got = __shfl_xor_sync(0xffffffffu, lo ? b : a, 16);
+        s[p] = silu_mul(__uint_as_float(lo ? a : got), __uint_as_float(lo ? got : b));
+      }
+      // even lanes keep the first two tokens and the odd lanes the other two: two features each
+      const float got = __shfl_xor_sync(0xffffffffu, odd ? s[0] : s[1], 1);
+      const uint32_t packed = odd ? pack_bf16(got, s[1]) : pack_bf16(s[0], got);
+      if (tok + 4 * q < valid) *reinterpret_cast<uint32_t*>(out) = packed;
+      out += 4 * ld;
+    }
+  } else if (OUT == kOutF32) {
+    float* out = reinterpret_cast<float*>(args.out) + orow + wrow0 + lane + col0 * ld;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (col0 + i < valid) *out = __uint_as_float(v[i]);
+      out += ld;
+    }
+  } else {
+    const bool odd = lane & 1;
+    const int tok = col0 + (lane & 1);
+    bf16* out = reinterpret_cast<bf16*>(args.out) + orow + wrow0 + (lane & 30) + tok * ld;
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {
+      const float mine = __uint_as_float(odd ? v[i + 1] : v[i]);
+      const float got = __uint_as_float(__shfl_xor_sync(0xffffffffu, odd ? v[i] : v[i + 1], 1));
+      const uint32_t packed = odd ? pack_bf16(got, mine) : pack_bf16(mine, got);
+      if (tok + i < valid) *reinterpret_cast<uint32_t*>(out) = packed;
+      out += 2 * ld;
+    }
+  }
+}
+
+template <bool GATE_UP, int OUT>
+__global__ void __launch_bounds__(PN_THREADS, 1)
+gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ Bars bars;
+  __shared__ Meta s_meta;
+  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();  // 0 = leader of the pair
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+
+  setup_barriers<PN_NS>(bars, 2 * PN_EPI_WARPS, 2);
+  if (warp == 1) {
+    tmem_alloc_pair(smem_u32(&bars.tmem_base), 512);
+    tmem_relinquish_pair();
+  }
+  // everything above is independent of the preceding kernels; their results are read from here on
+  pdl_wait();
+  for (int i = threadIdx.x; i < (int)(sizeof(Meta) / 4); i += blockDim.x)
+    reinterpret_cast<int32_t*>(&s_meta)[i] = ld_l2(reinterpret_cast<const int32_t*>(args.meta) + i);
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();  // both CTAs' barriers exist before anything is signalled across the pair
+  tc_fence_after();
+  const uint32_t tmem_base = *(volatile uint32_t*)&bars.tmem_base;
+  volatile int* abort_flag = &bars.abort_flag;
+
+  const int KB = (args.K + BK - 1) / BK;
+  const int Nt = (args.n_w_rows + PN_W_ROWS - 1) / PN_W_ROWS;
+  int n_items = 0;
+  for (int c = 0; c < args.r; ++c) n_items += token_tiles(s_meta.count[c]) * Nt;
+  uint32_t issued = 0;
+
+  if (warp == 0) {
+    // ---- TMA producer of this CTA's 256 weight rows and its half of the tokens; the bytes of
+    // both CTAs are counted on the leader's barrier
+    uint32_t it = 0, s = 0, ph = 0;
+    bool ok = true;
+    for (int item = pair; item < n_items && ok; item += n_pairs) {
+      ItemN t;
+      decode_item_n(s_meta, args, item, Nt, t);
+      const int half = t.n >> 1;  // 16 .. 128 token rows, a multiple of 16
+      const int w_row = t.nt * PN_W_ROWS + 256 * (int)rank;
+      const int a_row = args.a_row_base + args.a_off_mul * s_meta.off[t.c] + t.tok0 + half * (int)rank;
+      const uint32_t bytes = 2u * (PN_A_BYTES + (uint32_t)half * 128u);
+      for (int kb = 0; kb < KB; ++kb, ++it) {
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.empty[s]), ph ^ 1u, abort_flag));
+        if (!ok) break;
+        if (lane == 0) {
+          const uint32_t full = map_to_cta(smem_u32(&bars.full[s]), 0);
+          const uint32_t sa = smem_base + s * PN_STAGE;
+          if (rank == 0) mbar_expect_tx(smem_u32(&bars.full[s]), bytes);
+          tma_load_3d_pair(sa, &maps.w, kb * BK, w_row, t.c, full);
+          if (half == 128) {
+            tma_load_2d_pair(sa + PN_A_BYTES, &maps.t[3], kb * BK, a_row, full);
+          } else {
+            int done = 0;
+#pragma unroll
+            for (int b = 2; b >= 0; --b)
+              if (half & (16 << b)) {
+                tma_load_2d_pair(sa + PN_A_BYTES + done * 128, &maps.t[b], kb * BK, a_row + done, full);
+                done += 16 << b;
+              }
+          }
+        }
+        if (++s == PN_NS) { s = 0; ph ^= 1u; }
+        __syncwarp();
+      }
+    }
+    issued = it;
+  } else if (warp <= 2) {
+    // ---- MMA issuers of the leader, one warp per accumulator (the other CTA's warp 1 owns that
+    // CTA's tensor memory)
+    if (rank == 0) {
+      const uint32_t acc = (uint32_t)warp - 1u;
+      const uint32_t d_tmem = tmem_base + 256u * acc;
+      const uint32_t tmem_full = smem_u32(&bars.tmem_full[acc]), tmem_empty = smem_u32(&bars.tmem_empty[acc]);
+      uint32_t s = 0, ph = 0, nu = 0;  // nu: items so far
+      bool ok = true;
+      for (int item = pair; item < n_items && ok; item += n_pairs, ++nu) {
+        ItemN t;
+        decode_item_n(s_meta, args, item, Nt, t);
+        const uint32_t idesc = idesc_bf16(256, t.n);
+        for (int kb = 0; kb < KB; ++kb) {
+          bool ready = mbar_wait(smem_u32(&bars.full[s]), ph, abort_flag);
+          if (kb == 0) ready = ready && mbar_wait(tmem_empty, (nu & 1u) ^ 1u, abort_flag);
+          ok = __all_sync(0xffffffffu, ready);
+          if (!ok) break;
+          tc_fence_after();
+          if (lane == 0) {
+            const uint32_t sa = smem_base + s * PN_STAGE;
+            const uint64_t adesc = smem_desc_k128(sa + acc * (128 * 128)), bdesc = smem_desc_k128(sa + PN_A_BYTES);
+            umma_bf16_pair(d_tmem, adesc, bdesc, idesc, kb > 0 ? 1u : 0u);
+            umma_bf16_pair(d_tmem, adesc + 2, bdesc + 2, idesc, 1u);
+            umma_bf16_pair(d_tmem, adesc + 4, bdesc + 4, idesc, 1u);
+            umma_bf16_pair(d_tmem, adesc + 6, bdesc + 6, idesc, 1u);
+            umma_commit_pair(smem_u32(&bars.empty[s]));
+            if (kb == KB - 1) umma_commit_pair(tmem_full);
+          }
+          if (++s == PN_NS) { s = 0; ph ^= 1u; }
+          __syncwarp();
+        }
+      }
+    }
+  } else {
+    // ---- epilogue of this CTA's 2 x 128 weight rows: warp w reads tensor-memory lanes
+    // 32 (w % 4) .. + 31, and of the column chunks of 16 tokens every fourth
+    const int wq = warp & 3, group = (warp - 3) >> 2;
+    const uint32_t empty0 = map_to_cta(smem_u32(&bars.tmem_empty[0]), 0);
+    const uint32_t empty1 = map_to_cta(smem_u32(&bars.tmem_empty[1]), 0);
+    uint32_t nu = 0;
+    bool ok = true;
+    for (int item = pair; item < n_items && ok; item += n_pairs, ++nu) {
+      ItemN t;
+      decode_item_n(s_meta, args, item, Nt, t);
+      const long long orow =
+          (long long)(args.out_row_base + args.out_off_mul * s_meta.off[t.c] + t.tok0) * args.out_ld +
+          (long long)t.c * args.out_col_mul;
+#pragma unroll 1
+      for (int acc = 0; acc < 2; ++acc) {
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.tmem_full[acc]), nu & 1u, abort_flag));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t taddr = tmem_base + ((uint32_t)(32 * wq) << 16) + 256 * acc;
+        const int wrow0 = t.nt * PN_W_ROWS + 256 * (int)rank + 128 * acc + 32 * wq;
+        const bool rows_ok = wrow0 < args.n_w_rows;
+        // get everything this warp wants of the accumulator into registers and hand it back before
+        // the long part (a SwiGLU per output, the stores)
+        uint32_t v[4][16];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tmem_ld16(taddr + 16 * (group + 4 * i), v[i]);
+        tmem_ld_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(acc ? empty1 : empty0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (rows_ok && 16 * (group + 4 * i) < t.valid)
+            store_cols_n<GATE_UP, OUT>(v[i], args, orow, wrow0, 16 * (group + 4 * i), t.valid, lane);
+      }
+    }
+  }
+
+  pdl_launch_dependents();
+  // ---- teardown: tell the partner if this CTA gave up, drain, and leave together (the leader's
+  // MMAs read the partner's shared memory, and tensor memory is released as a pair)
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag) st_cluster_u32(map_to_cta(smem_u32(&bars.abort_flag), rank ^ 1u), 1u);
+  cluster_sync_all();
+  if (*abort_flag) {
+    if (warp == 0 && lane == 0) {
+      int dummy = 0;
+      const uint32_t n = issued < (uint32_t)PN_NS ? issued : (uint32_t)PN_NS;
+      for (uint32_t i = 0; rank == 0 && i < n; ++i) {
+        const uint32_t it = issued - 1 - i;
+        mbar_wait(smem_u32(&bars.full[it % PN_NS]), (it / PN_NS) & 1u, &dummy, kDrainLimitNs);
+      }
+      if (args.status) atomicExch(args.status, 1);
+    }
+    if ((warp == 1 || warp == 2) && lane == 0 && rank == 0) {
+      int dummy = 0;
+      umma_commit_pair(smem_u32(&bars.drain));
+      mbar_wait(smem_u32(&bars.drain), 0, &dummy, kDrainLimitNs);
+    }
+    __syncwarp();
+    cluster_sync_all();
+  }
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem_base, 512);
+  }
 }
 
 // ----------------------------------------------------------------------- gemm_weights_m
@@ -1469,6 +1835,9 @@ cudaError_t gemm_set_attributes() {
   SET_ATTR((gemm_tokens_m_kernel<true, kOutActBf16>), TM_SMEM)
   SET_ATTR((gemm_tokens_m_kernel<false, kOutF32>), TM_SMEM)
   SET_ATTR((gemm_tokens_m_kernel<false, kOutBf16>), TM_SMEM)
+  SET_ATTR((gemm_pair_n_kernel<true, kOutActBf16>), PN_SMEM)
+  SET_ATTR((gemm_pair_n_kernel<false, kOutF32>), PN_SMEM)
+  SET_ATTR((gemm_pair_n_kernel<false, kOutBf16>), PN_SMEM)
   SET_ATTR((gemm_weights_m_kernel<true, 64>), WmCfg<64>::kSmem)
   SET_ATTR((gemm_weights_m_kernel<false, 64>), WmCfg<64>::kSmem)
   SET_ATTR((gemm_weights_m_kernel<true, 128>), WmCfg<128>::kSmem)
@@ -1525,6 +1894,31 @@ cudaError_t launch_gemm_tokens_m(bool gate_up, GemmOut out_kind, const GemmMaps&
   if (out_kind == kOutF32)
     return launch_plain(gemm_tokens_m_kernel<false, kOutF32>, dim3(grid), dim3(TmCfg<false>::kThreads), TM_SMEM, st, maps, a);
   return launch_plain(gemm_tokens_m_kernel<false, kOutBf16>, dim3(grid), dim3(TmCfg<false>::kThreads), TM_SMEM, st, maps, a);
+}
+
+// On CTA pairs (cluster of two), in plain stream order.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_pair(void (*kernel)(KArgs...), cudaStream_t st, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((g_num_sms > 0 ? g_num_sms : 148) & ~1);
+  cfg.blockDim = dim3(PN_THREADS);
+  cfg.dynamicSmemBytes = PN_SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+cudaError_t launch_gemm_pair_n(bool gate_up, GemmOut out_kind, const GemmMaps& maps, const GemmArgs& a,
+                               cudaStream_t st) {
+  if (gate_up) return launch_pair(gemm_pair_n_kernel<true, kOutActBf16>, st, maps, a);
+  if (out_kind == kOutF32) return launch_pair(gemm_pair_n_kernel<false, kOutF32>, st, maps, a);
+  return launch_pair(gemm_pair_n_kernel<false, kOutBf16>, st, maps, a);
 }
 
 cudaError_t launch_gemm_tokens_d(bool gate_up, const GemmMaps& maps, const GemmArgs& a, int kb_per_item,

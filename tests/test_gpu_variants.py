@@ -302,3 +302,27 @@ def test_plain_stream_order_gives_the_same_bits(weights, T):
         plain.close()
         layer_with_env(weights, MOE_NO_PDL=0).close()  # the switch is process-wide: back to the default
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("h,f,E,kept,T", [
+    # two kept experts and no skipping: both groups hold exactly T tokens, so T walks the edges of
+    # the token tiles (grain 32, at most 256 a tile) and, above 1536, the other large-batch kernel
+    (128, 448, 8, 0b00100100, 257), (128, 448, 8, 0b00100100, 287), (128, 448, 8, 0b00100100, 288),
+    (128, 448, 8, 0b00100100, 289), (128, 448, 8, 0b00100100, 512), (128, 448, 8, 0b00100100, 513),
+    (128, 448, 8, 0b00100100, 1536), (128, 448, 8, 0b00100100, 1537),
+    # many small ragged groups; one k-block; weight rows just above one item of 512
+    (128, 448, 8, 0xFF, 259), (64, 64, 16, 0xFFFF, 300), (64, 320, 3, 0b111, 333), (576, 64, 4, 0b1111, 700),
+])
+def test_large_batch_gemm_at_the_edges_of_its_tiles(h, f, E, kept, T):
+    build.build()
+    W = synth.make_layer_weights(h, f, E, seed=5, device=DEV)
+    w = (W.W_gate, W.W1, W.W3, W.W2)
+    x = synth.make_tokens(T, h, seed=6, device=DEV)
+    lay, dbg = binding.MoeLayer(*w, kept), layer_with_env(w, kept, MOE_DEBUG_SIMT=1)
+    y0, y1, y2 = dbg.forward(x), lay.forward(x), lay.forward(x)
+    torch.cuda.synchronize()
+    assert rel_l2(y1, y0) < 5e-3  # different summation orders, same rounding points
+    assert torch.equal(y1, y2)
+    assert lay.device_status() == 0
+    lay.close()
+    dbg.close()
