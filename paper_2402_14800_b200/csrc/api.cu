@@ -80,7 +80,7 @@ struct Workspace {
   Buf row_token, xperm, act, O, tail;
   CUtensorMap tok_x[4], tok_act[4];  // boxes of 16/32/64/128 rows over xperm and act
   // search scratch
-  Buf s_logits, s_yall, s_act, s_subsets, s_partial, s_loss_sq, s_losses, s_xpad, s_meta, s_xperm, s_rowtok;
+  Buf s_logits, s_yall, s_act, s_subsets, s_partial, s_loss_sq, s_losses, s_xpad, s_meta, s_xperm;
   // host staging and stack scratch
   Buf hx, hy, xn, cosel;
   // general top-k path
@@ -115,7 +115,7 @@ struct moe_layer {
   bool prof = false;
   std::vector<cudaEvent_t> prof_ev;  // MOE_PROFILE_STAGES + 1 marks per recorded call
   size_t prof_used = 0;
-  int* h_status = nullptr;  // pinned host copy of the device status word
+  int* h_words = nullptr;  // pinned host words (host_words)
 };
 
 namespace {
@@ -243,14 +243,20 @@ void mark(moe_layer* L) {
   cudaEventRecord(L->prof_ev[L->prof_used++], L->stream);
 }
 
-int check_status(moe_layer* L) {
-  // the status word is read into pinned memory: a copy to pageable memory is staged by the runtime
-  if (!L->h_status && cudaHostAlloc((void**)&L->h_status, sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+// Pinned host words of the handle that kernels and copies write results to ([0] status word,
+// [1..2] selected values); null if they cannot be had.  A copy to pageable memory would be staged
+// by the runtime.
+int* host_words(moe_layer* L) {
+  if (!L->h_words && cudaHostAlloc((void**)&L->h_words, 4 * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
     cudaGetLastError();
-    L->h_status = nullptr;
+    L->h_words = nullptr;
   }
+  return L->h_words;
+}
+
+int check_status(moe_layer* L) {
   int st_pageable = 0;
-  int* dst = L->h_status ? L->h_status : &st_pageable;
+  int* dst = host_words(L) ? L->h_words : &st_pageable;
   CUDA_TRY(cudaMemcpyAsync(dst, L->ws->status.p, 4, cudaMemcpyDeviceToHost, L->stream));
   CUDA_TRY(cudaStreamSynchronize(L->stream));
   const int st = *dst;
@@ -260,6 +266,27 @@ int check_status(moe_layer* L) {
     if (L->ws->tail.p) cudaMemsetAsync(L->ws->tail.p, 0, kTailHeaderBytes, L->stream);
     return fail(MOE_ERR_DEVICE_TIMEOUT, "a bounded wait inside a GEMM kernel expired");
   }
+  return MOE_OK;
+}
+
+// Which large-batch GEMM a batch of at most `pairs` token-expert pairs runs, and what its groups are
+// padded to.
+inline bool large_on_pairs(const moe_layer* L, long long pairs) { return pairs <= (long long)kPairMaxRows * L->r; }
+inline int group_pad(const moe_layer* L, long long pairs) { return large_on_pairs(L, pairs) ? kPairPad : kTileRows; }
+
+// Permutation of a top-k batch: idx [T][k], the first nact[t] slots of a token run.
+int permute_topk(moe_layer* L, const bf16* x, const int32_t* idx, const int32_t* nact, int T, int k, int pad,
+                 Meta* meta, int32_t* pair_pos, bf16* xperm) {
+  int32_t* base = nullptr;
+  if (T > kPermuteOwnT) {
+    base = (int32_t*)L->ws->blk_base.p;
+    const int nblk = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;
+    CUDA_TRY(launch_count_topk(idx, nact, T, k, (int32_t*)L->ws->blk_hist.p, L->stream));
+    CUDA_TRY(launch_scan((int32_t*)L->ws->blk_hist.p, nblk, L->r, pad, base, meta, nullptr, nullptr, nullptr,
+                         L->kept, L->E, L->stream));
+  }
+  CUDA_TRY(launch_permute(x, idx, nact, false, T, k, L->h, L->r, pad, base, meta, pair_pos, xperm, nullptr,
+                          nullptr, nullptr, L->kept, L->E, L->stream));
   return MOE_OK;
 }
 
@@ -285,7 +312,7 @@ int run_expert_gemms(moe_layer* L, const Meta* meta, bool weights_m, const GemmM
     CUDA_TRY(launch_gemm_tokens_d(true, m_gu, gu, (L->h + 63) / 64, L->stream));
     mark(L);
     CUDA_TRY(launch_gemm_tokens_d(false, m_dn, dn, down_kb_per_item(T), L->stream));
-  } else if (pairs <= (long long)kPairMaxRows * L->r) {
+  } else if (large_on_pairs(L, pairs)) {
     CUDA_TRY(launch_gemm_pair_n(true, kOutActBf16, m_gu, gu, L->stream));
     mark(L);
     CUDA_TRY(launch_gemm_pair_n(false, dn_kind, m_dn, dn, L->stream));
@@ -357,22 +384,16 @@ int forward_impl(moe_layer* L, const void* x, int T, float beta, const void* res
                                          (int32_t*)L->ws->pair_pos.p, (int32_t*)L->ws->row_token.p,
                                          (bf16*)L->ws->xperm.p, s_count, s_nsk, s_nt, L->kept, L->E, st));
   } else {
-    // the tensor-core router wins from about 64 tiles of 128 tokens on (T = 8192: routing stage
-    // 0.144 -> 0.115 ms, T = 32768: 0.52 -> 0.35 ms; T = 4096 equal, T = 2048 slower on its 16 CTAs)
-    if (L->debug_simt || T < 64 * kTileRows)
-      CUDA_TRY(launch_router((const bf16*)x, L->Wg, T, L->h, L->r, beta, L->kept, ro, st));
-    else
-      CUDA_TRY(launch_router_tc((const bf16*)x, L->Wg, T, L->h, L->r, beta, L->kept, ro,
-                                (int*)L->ws->status.p, st));
-    CUDA_TRY(launch_scan(ro.blk_hist, nblk, L->r, kTileRows, (int32_t*)L->ws->blk_base.p, meta,
-                         s_count, s_nsk, s_nt, L->kept, L->E, st));
-    CUDA_TRY(cudaMemsetAsync(L->ws->row_token.p, 0xff, (size_t)rows_cap * 4, st));
-    CUDA_TRY(launch_scatter(ro.idx, ro.skipped, (int32_t*)L->ws->blk_base.p, meta, T,
-                            (int32_t*)L->ws->pair_pos.p, (int32_t*)L->ws->row_token.p, st));
+    const bool own = T <= kPermuteOwnT;
+    if (own) ro.blk_hist = nullptr;
+    CUDA_TRY(launch_router((const bf16*)x, L->Wg, T, L->h, L->r, beta, L->kept, ro, st));
+    if (!own)
+      CUDA_TRY(launch_scan(ro.blk_hist, nblk, L->r, group_pad(L, 2ll * T), (int32_t*)L->ws->blk_base.p, meta,
+                           s_count, s_nsk, s_nt, L->kept, L->E, st));
+    CUDA_TRY(launch_permute((const bf16*)x, ro.idx, ro.skipped, true, T, 2, L->h, L->r, group_pad(L, 2ll * T),
+                            own ? nullptr : (int32_t*)L->ws->blk_base.p, meta, (int32_t*)L->ws->pair_pos.p,
+                            (bf16*)L->ws->xperm.p, s_count, s_nsk, s_nt, L->kept, L->E, st));
   }
-  if (!dec)
-    CUDA_TRY(launch_gather((const bf16*)x, (int32_t*)L->ws->row_token.p, meta, L->h, rows_cap,
-                           (bf16*)L->ws->xperm.p, st));
   mark(L);
 
   GemmArgs gu, dn;
@@ -478,7 +499,7 @@ moe_layer_t* moe_layer_create(const void* W_gate, const void* W1, const void* W3
   const char* dense = getenv("MOE_SEARCH_DENSE");
   L->search_dense = dense && dense[0] == '1';
 
-  // the router rows are padded with zero rows to kMaxE rows (the tensor-core router's operand)
+  // the router rows are stored padded with zero rows to kMaxE rows
   const size_t n_gate = (size_t)kMaxE * h * 2, n_13 = (size_t)L->r * 2 * f * h * 2,
                n_2 = (size_t)L->r * h * f * 2;
   size_t free_b = 0;
@@ -531,10 +552,10 @@ void moe_layer_destroy(moe_layer_t* L) {
   Buf* bufs[] = {&L->own.idx, &L->own.wn, &L->own.ratio, &L->own.skipped, &L->own.blk_hist, &L->own.blk_base, &L->own.pair_pos,
                  &L->own.meta, &L->own.status, &L->own.sel, &L->own.row_token, &L->own.xperm, &L->own.act, &L->own.O, &L->own.tail,
                  &L->own.s_logits, &L->own.s_yall, &L->own.s_act, &L->own.s_subsets, &L->own.s_partial, &L->own.s_loss_sq,
-                 &L->own.s_losses, &L->own.s_xpad, &L->own.s_meta, &L->own.s_xperm, &L->own.s_rowtok, &L->own.hx, &L->own.hy, &L->own.xn, &L->own.cosel, &L->own.k_idx, &L->own.k_wn, &L->own.k_pos, &L->own.k_nact};
+                 &L->own.s_losses, &L->own.s_xpad, &L->own.s_meta, &L->own.s_xperm, &L->own.hx, &L->own.hy, &L->own.xn, &L->own.cosel, &L->own.k_idx, &L->own.k_wn, &L->own.k_pos, &L->own.k_nact};
   for (Buf* b : bufs) release(L, *b);
   for (cudaEvent_t e : L->prof_ev) cudaEventDestroy(e);
-  if (L->h_status) cudaFreeHost(L->h_status);
+  if (L->h_words) cudaFreeHost(L->h_words);
   if (L->Wg) cudaFree(L->Wg);
   if (L->W13) cudaFree(L->W13);
   if (L->W2) cudaFree(L->W2);
@@ -610,21 +631,15 @@ int moe_forward_topk(moe_layer_t* L, const void* x, int T, int k, float beta, vo
   if ((rc = grow(L, W.k_nact, (size_t)T * 4))) return rc;
   cudaStream_t st = L->stream;
   const bool dec = decode_mode(T);
-  const int nblk = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;
   const int rows_cap = rows_for(L, T, k);
   Meta* meta = (Meta*)W.meta.p;
   int32_t* idx = (int32_t*)W.k_idx.p;
   int32_t* nact = (int32_t*)W.k_nact.p;
   CUDA_TRY(launch_router_topk((const bf16*)x, L->Wg, T, L->h, L->r, k, beta, L->kept, idx,
                               (float*)W.k_wn.p, nact, idx_out, wn_out, n_active_out, nullptr, st));
-  CUDA_TRY(launch_count_topk(idx, nact, T, k, (int32_t*)W.blk_hist.p, st));
-  CUDA_TRY(launch_scan((int32_t*)W.blk_hist.p, nblk, L->r, dec ? 16 : kTileRows, (int32_t*)W.blk_base.p,
-                       meta, nullptr, nullptr, nullptr, L->kept, L->E, st));
-  CUDA_TRY(cudaMemsetAsync(W.row_token.p, 0xff, (size_t)rows_cap * 4, st));
-  CUDA_TRY(launch_scatter_topk(idx, nact, (int32_t*)W.blk_base.p, meta, T, k, (int32_t*)W.k_pos.p,
-                               (int32_t*)W.row_token.p, st));
-  CUDA_TRY(launch_gather((const bf16*)x, (int32_t*)W.row_token.p, meta, L->h, rows_cap,
-                         (bf16*)W.xperm.p, st));
+  if ((rc = permute_topk(L, (const bf16*)x, idx, nact, T, k, dec ? 16 : group_pad(L, (long long)k * T), meta,
+                         (int32_t*)W.k_pos.p, (bf16*)W.xperm.p)))
+    return rc;
   GemmArgs gu, dn;
   memset(&gu, 0, sizeof(gu));
   memset(&dn, 0, sizeof(dn));
@@ -681,10 +696,14 @@ int moe_calibrate_beta(moe_layer_t* L, const void* x, int T, float* beta_out) {
   ro.idx = (int32_t*)L->ws->idx.p; ro.wn = (float*)L->ws->wn.p; ro.ratio = (float*)L->ws->ratio.p;
   ro.skipped = (uint8_t*)L->ws->skipped.p;
   CUDA_TRY(launch_router((const bf16*)x, L->Wg, T, L->h, L->r, 0.f, L->kept, ro, L->stream));
-  CUDA_TRY(launch_select2(ro.ratio, T, (T - 1) / 2, T / 2, (float*)L->ws->sel.p, L->stream));
+  // the two values go straight to mapped host memory where there is some
+  int* words = host_words(L);
+  float* sel = words ? (float*)(words + 1) : (float*)L->ws->sel.p;
+  CUDA_TRY(launch_select2(ro.ratio, T, (T - 1) / 2, T / 2, sel, L->stream));
   float v[2];
-  CUDA_TRY(cudaMemcpyAsync(v, L->ws->sel.p, 8, cudaMemcpyDeviceToHost, L->stream));
+  if (!words) CUDA_TRY(cudaMemcpyAsync(v, sel, 8, cudaMemcpyDeviceToHost, L->stream));
   CUDA_TRY(cudaStreamSynchronize(L->stream));
+  if (words) memcpy(v, sel, 8);
   *beta_out = (T & 1) ? v[0] : (float)(((double)v[0] + (double)v[1]) * 0.5);
   return MOE_OK;
 }
@@ -828,7 +847,6 @@ static int search_impl(moe_layer_t* L, const void* x_calib, const float* F_ref, 
     if ((rc = grow(L, W.s_yall, (size_t)nchunks * rows_chunk * h * 2))) return rc;
     if ((rc = grow(L, W.s_act, ((size_t)rows_chunk + kTileRows) * f * 2))) return rc;
     if ((rc = grow(L, W.s_xperm, ((size_t)rows_chunk + kTileRows) * h * 2))) return rc;
-    if ((rc = grow(L, W.s_rowtok, (size_t)rows_chunk * 4))) return rc;
     if ((rc = grow(L, W.k_idx, (size_t)T * K * 4))) return rc;
     if ((rc = grow(L, W.k_wn, (size_t)T * K * 4))) return rc;
     if ((rc = grow(L, W.k_pos, (size_t)T * K * 4))) return rc;
@@ -838,7 +856,6 @@ static int search_impl(moe_layer_t* L, const void* x_calib, const float* F_ref, 
     for (int c = 0; c < nchunks; ++c) {
       const int t0 = c * Tc;
       const int rows = (T - t0) < Tc ? (T - t0) : Tc;
-      const int nblk = (rows + kRouteTokPerBlock - 1) / kRouteTokPerBlock;
       const bf16* xc = (const bf16*)x_calib + (size_t)t0 * h;
       int32_t* idx = (int32_t*)W.k_idx.p + (size_t)t0 * K;
       int32_t* nact = (int32_t*)W.k_nact.p + t0;
@@ -848,19 +865,14 @@ static int search_impl(moe_layer_t* L, const void* x_calib, const float* F_ref, 
       cudaError_t e = launch_router_topk(xc, L->Wg, rows, h, E, K, -1.0f, L->kept, idx,
                                          (float*)W.k_wn.p + (size_t)t0 * K, nact, nullptr, nullptr,
                                          nullptr, (float*)W.s_logits.p + (size_t)t0 * E, st);
-      if (e == cudaSuccess) e = launch_count_topk(idx, nact, rows, K, (int32_t*)W.blk_hist.p, st);
-      if (e == cudaSuccess)
-        e = launch_scan((int32_t*)W.blk_hist.p, nblk, E, kTileRows, (int32_t*)W.blk_base.p, meta, nullptr,
-                        nullptr, nullptr, L->kept, E, st);
-      if (e == cudaSuccess) e = cudaMemsetAsync(W.s_rowtok.p, 0xff, (size_t)rows_chunk * 4, st);
-      if (e == cudaSuccess)
-        e = launch_scatter_topk(idx, nact, (int32_t*)W.blk_base.p, meta, rows, K, pos,
-                                (int32_t*)W.s_rowtok.p, st);
-      if (e == cudaSuccess)
-        e = launch_gather(xc, (int32_t*)W.s_rowtok.p, meta, h, rows_chunk, (bf16*)W.s_xperm.p, st);
-      if (e != cudaSuccess) {
+      if (e != cudaSuccess)
+        rc = fail(MOE_ERR_CUDA, "search routing: %s", cudaGetErrorString(e));
+      else
+        rc = permute_topk(L, xc, idx, nact, rows, K, group_pad(L, (long long)K * rows), meta, pos,
+                          (bf16*)W.s_xperm.p);
+      if (rc) {
         L->prof = prof_saved;
-        return fail(MOE_ERR_CUDA, "search permutation: %s", cudaGetErrorString(e));
+        return rc;
       }
       mark(L);
       GemmArgs gu, dn;

@@ -27,6 +27,10 @@ constexpr int kTokensDMaxKept = 6;         // ... on layers with at most this ma
 // 6144 a group was up to 6 % slower on the pairs: with little padding to save, both are held by the
 // board's power and the pairs draw 1-3 % more energy per call.
 constexpr int kPairMaxRows = 1536;
+constexpr int kPairPad = 32;        // grain of its token tiles
+// Up to here every block of the permutation counts the whole routing record itself (at 32 tokens a
+// thread, in bytes, 255 tokens a thread at most); beyond, the routers' histogram and the scan do.
+constexpr int kPermuteOwnT = 8192;
 constexpr int kDecodeKbPerItem = 112;      // k-blocks (of 64) per split-K item, decode down-proj
 
 // Device-resident description of one permuted batch, written by the scan kernel
@@ -128,12 +132,9 @@ struct RouteOut {
   uint8_t* s_skipped;
 };
 
+// w_const: Wg never changes (a handle's own rows) and may be read before the predecessor is done
 cudaError_t launch_router(const bf16* x, const bf16* Wg, int T, int h, int r, float beta,
-                          const KeptIds& kept, const RouteOut& out, cudaStream_t st);
-// Large batches (T > kDecodeMaxT): the logits on the tensor cores (gemm_sm100.cu), the decision as
-// in launch_router.  Wg16 = the kept router rows padded with zero rows to kMaxE rows.
-cudaError_t launch_router_tc(const bf16* x, const bf16* Wg16, int T, int h, int r, float beta,
-                             const KeptIds& kept, const RouteOut& out, int* status, cudaStream_t st);
+                          const KeptIds& kept, const RouteOut& out, cudaStream_t st, bool w_const = true);
 // T <= kDecodeMaxT: router with one block per token; permutation + gather with one block per token
 cudaError_t launch_router_small(const bf16* x, const bf16* Wg, int T, int h, int r, float beta,
                                 const KeptIds& kept, const RouteOut& out, cudaStream_t st);
@@ -149,11 +150,13 @@ cudaError_t launch_permute_gather_small(const bf16* x, const int32_t* idx, const
 cudaError_t launch_scan(const int32_t* blk_hist, int nblk, int r, int pad, int32_t* blk_base,
                         Meta* meta, int32_t* s_count, int32_t* s_nskipped, int32_t* s_ntouched,
                         const KeptIds& kept, int E, cudaStream_t st);
-cudaError_t launch_scatter(const int32_t* idx, const uint8_t* skipped, const int32_t* blk_base,
-                           const Meta* meta, int T, int32_t* pair_pos, int32_t* row_token,
-                           cudaStream_t st);
-cudaError_t launch_gather(const bf16* x, const int32_t* row_token, const Meta* meta, int h,
-                          int cap_rows, bf16* xperm, cudaStream_t st);
+// T > kDecodeMaxT.  blk_base: the scan's result, or null for at most kPermuteOwnT tokens (the kernel
+// then counts for itself and writes *meta and the record's counts).  active: skip flags (uint8,
+// top2) or the number of slots that run (int32).
+cudaError_t launch_permute(const bf16* x, const int32_t* idx, const void* active, bool top2, int T, int k, int h,
+                           int r, int pad, const int32_t* blk_base, Meta* meta, int32_t* pair_pos, bf16* xperm,
+                           int32_t* s_count, int32_t* s_nskipped, int32_t* s_ntouched, const KeptIds& kept,
+                           int E, cudaStream_t st);
 cudaError_t launch_combine(const float* O, int ksplit, size_t split_stride, const int32_t* pair_pos,
                            const float* wn, const bf16* residual, int T, int h, bf16* y,
                            cudaStream_t st);
@@ -164,9 +167,6 @@ cudaError_t launch_router_topk(const bf16* x, const bf16* Wg, int T, int h, int 
                                cudaStream_t st);
 cudaError_t launch_count_topk(const int32_t* idx, const int32_t* nact, int T, int k,
                               int32_t* blk_hist, cudaStream_t st);
-cudaError_t launch_scatter_topk(const int32_t* idx, const int32_t* nact, const int32_t* blk_base,
-                                const Meta* meta, int T, int k, int32_t* pair_pos,
-                                int32_t* row_token, cudaStream_t st);
 cudaError_t launch_combine_topk(const float* O, int ksplit, size_t split_stride,
                                 const int32_t* pair_pos, const float* wn, int k, int T, int h,
                                 bf16* y, cudaStream_t st);
@@ -177,7 +177,8 @@ cudaError_t launch_top2_distance(const float* O, int ksplit, size_t split_stride
 cudaError_t launch_rmsnorm(const bf16* x, int T, int h, float eps, bf16* out, cudaStream_t st);
 cudaError_t launch_set_dense_meta(Meta* meta, int E, int rows_per_expert, int off_stride,
                                   cudaStream_t st);
-// k-th smallest (0-based) of ratio[T] for k = k0 and k1, written to out[0], out[1]
+// k-th smallest (0-based) of ratio[T] for k = k0 and k1 (= k0 or k0 + 1), written to out[0], out[1]
+// (device memory or mapped host memory)
 cudaError_t launch_select2(const float* ratio, int T, int k0, int k1, float* out, cudaStream_t st);
 // W13[c][32q + s] = W1[id[c]][16q + s] (s < 16) | W3[id[c]][16q + s - 16] (s >= 16)
 cudaError_t launch_interleave(const bf16* W1, const bf16* W3, const KeptIds& kept, int r, int f,

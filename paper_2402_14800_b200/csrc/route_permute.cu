@@ -2,9 +2,9 @@
 //
 //   router_kernel   Sec. 3.1 (logits, softmax, top-2, Eq. 1), Sec. 3.2 (kept experts only),
 //                   Sec. 3.3 (skip test), App. A.2 (weight 1 after a skip); warp per token.
-//   scan / scatter  stable counting sort of the token-expert pairs that run, by expert;
-//                   no atomics, the order is a function of the routing alone.
-//   gather          copies the routed rows of x into expert-contiguous order.
+//   scan / permute  stable counting sort of the token-expert pairs that run, by expert (no atomics,
+//                   the order is a function of the routing alone), and the copy of the routed rows
+//                   of x into that order.
 //   combine         Eq. 2: y = bf16(residual + w~_e0 o_e0 + w~_e1 o_e1), slot 0 first.
 //
 // Every kernel here that is launched as a programmatic dependent reads what earlier kernels of
@@ -237,83 +237,215 @@ permute_gather_small_kernel(const bf16* x, const int32_t* idx, const uint8_t* sk
   }
 }
 
-// Large batches: one warp per token, kRouteTokPerBlock tokens per block (whose pair counts go
-// to the block's histogram row).  A lane first fetches its whole share of the token's row (the
-// loads that come from DRAM, all independent), then walks it against the router rows, which
-// sit in L1 after the block's first pass.
+// Batches of more than kDecodeMaxT tokens: a warp takes the logits of TB tokens.  A lane walks the
+// same 8-element slices of the TB rows and of the router rows, so a slice of a router row is read
+// and unpacked once for TB tokens; the products of two tokens go through one fma.rn.f32x2.  A logit
+// is one chain of fused multiply-adds per lane (slices, then elements, in order) and a butterfly over
+// the lanes, whatever the batch and the tokens beside it.
+//   - The router rows are copied to shared memory once per block, before the wait for the
+//     predecessor (they never change), where they fit beside the ring: read through L1 they cost a
+//     chain of L2 round trips per slice, 62 us for 611 tokens.
+//   - The token rows come through a ring of kRouteStages slices per warp, filled with cp.async.cg
+//     (which reads at L2, as the rule beside launch_pdl asks): a lane copies exactly the bytes it
+//     will use itself, so no barrier is needed, and the loads in flight cost no registers.
+// Bound by the issue slots of the fp32 work and, beside them, the shared-memory port; 134 MB of token
+// rows at 16384 tokens take 20 us to stream.  Router launch, before (one warp per token, router rows
+// through L1; a tensor-core kernel from 8192 tokens on: 33 us at 8192) -> after: 611 tokens 19.4 ->
+// 10.3 us, 4000 26.7 -> 14.9, 16384 88.9 -> 40.2; top-k, 8192 tokens, 8 experts 73.9 -> 25.3 us.
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ void fma_f32x2(uint64_t& acc, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ void split_f32x2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ void cp_async16(void* dst_shared, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+               ::"r"((uint32_t)__cvta_generic_to_shared(dst_shared)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
-template <int R>
-__global__ void __launch_bounds__(32 * kRouteTokPerBlock)
-router_kernel(const bf16* x, const bf16* __restrict__ Wg, int T, int h, int r,
-              float beta, KeptIds kept, RouteOut o) {
-  pdl_launch_dependents();
-  pdl_wait();
-  __shared__ int s_e[kRouteTokPerBlock][2];
-  __shared__ int s_skip[kRouteTokPerBlock];
-  constexpr int kRouteXVec = R > 8 ? 8 : 16;  // 16-byte vectors of the row a lane holds at a time
-  const int tl = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = blockIdx.x * kRouteTokPerBlock + tl;
+// Sums N values (a power of two up to 32) over the 32 lanes, halving the values a lane carries at
+// every exchange; lane l returns the total of value l / (32 / N).
+template <int N, int OFF = 16>
+__device__ __forceinline__ float reduce_scatter(const float (&v)[N], int lane) {
+  if constexpr (OFF == 0) {
+    return v[0];
+  } else if constexpr (N == 1) {
+    const float one[1] = {v[0] + __shfl_xor_sync(0xffffffffu, v[0], OFF)};
+    return reduce_scatter<1, OFF / 2>(one, lane);
+  } else {
+    const bool up = lane & OFF;
+    float half[N / 2];
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+      const float got = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + N / 2], OFF);
+      half[i] = (up ? v[i + N / 2] : v[i]) + got;
+    }
+    return reduce_scatter<N / 2, OFF / 2>(half, lane);
+  }
+}
+
+// R = experts computed (>= r), RP = R rounded up to a power of two, TB = tokens per warp.  A team of
+// kTeamWarps warps takes the kRouteTokPerBlock tokens of one row of the permutation's histogram;
+// a block of 16 warps is several teams, and the blocks go round until the tokens are done.
+constexpr int kRouteStages = 4;
+constexpr int kRouteWarps = 16;
+template <int R> struct RouteCfg {
+  static constexpr int kRP = R <= 2 ? 2 : (R <= 4 ? 4 : (R <= 8 ? 8 : 16));
+  static constexpr int kTB = R <= 8 ? 4 : 2;
+  static constexpr int kN = kRP * kTB;
+  static constexpr int kTeamWarps = kRouteTokPerBlock / kTB;
+  static constexpr int kTeams = kRouteWarps / kTeamWarps;
+  static constexpr size_t kRingBytes = (size_t)kRouteWarps * kRouteStages * kTB * 32 * 16;
+};
+constexpr size_t kRouteSmemMax = 227 * 1024 - 8 * 1024;  // dynamic part; the records are static
+
+// Copies the r router rows behind the ring.  Every thread of the block calls it, then a barrier.
+__device__ __forceinline__ void stage_router_rows(uint4* s_w, const bf16* __restrict__ Wg, int n) {
+  const uint4* src = reinterpret_cast<const uint4*>(Wg);
+  for (int i = threadIdx.x; i < n; i += 32 * kRouteWarps) cp_async16(s_w + i, src + i);
+  cp_async_commit();
+  cp_async_wait<0>();
+}
+
+// Logits of this warp's tokens t0 .. t0 + TB - 1 (tokens past the end repeat the last): lane l
+// returns the one of token q / RP and expert q % RP, q = l / (32 / N); experts beyond r repeat the
+// last.  WS: w = the rows in shared memory, else in global memory.
+template <int R, bool WS>
+__device__ __forceinline__ float warp_logits(const bf16* x, const uint4* __restrict__ w, int t0, int T, int h,
+                                             int r, uint4* ring) {
+  constexpr int RP = RouteCfg<R>::kRP, TB = RouteCfg<R>::kTB, N = RouteCfg<R>::kN;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nvec = h >> 3;
-
-  float acc[R];
+  uint64_t acc[TB / 2][R];  // two tokens each
 #pragma unroll
-  for (int c = 0; c < R; ++c) acc[c] = 0.f;
-  // a token past the end reads the last token's row; its result is dropped below
-  const uint4* xr = reinterpret_cast<const uint4*>(x + (size_t)min(t, T - 1) * h);
-  for (int v0 = lane; v0 < nvec; v0 += 32 * kRouteXVec) {
-    uint4 xv[kRouteXVec];
+  for (int i = 0; i < TB / 2; ++i)
 #pragma unroll
-    for (int i = 0; i < kRouteXVec; ++i)
-      xv[i] = (v0 + 32 * i < nvec) ? ld_l2(xr + v0 + 32 * i) : make_uint4(0u, 0u, 0u, 0u);
+    for (int c = 0; c < R; ++c) acc[i][c] = 0ull;
+  const uint4* xr[TB];
 #pragma unroll
-    for (int i = 0; i < kRouteXVec; ++i) {
-      const int v = v0 + 32 * i;
-      if (v < nvec) {
-        uint4 wv[R];
+  for (int i = 0; i < TB; ++i) xr[i] = reinterpret_cast<const uint4*>(x + (size_t)min(t0 + i, T - 1) * h) + lane;
+  uint4* mine = ring + warp * (kRouteStages * TB * 32) + lane;  // [stage][token][lane]
+  auto fetch = [&](int v, int s) {  // slice v / 32 into stage s
+    if (v + lane < nvec) {
 #pragma unroll
-        for (int c = 0; c < R; ++c)
-          if (c < r) wv[c] = __ldg(reinterpret_cast<const uint4*>(Wg + (size_t)c * h) + v);
-        float xf[8];
-        unpack8(xv[i], xf);
+      for (int i = 0; i < TB; ++i) cp_async16(mine + (s * TB + i) * 32, xr[i] + v);
+    }
+    cp_async_commit();
+  };
 #pragma unroll
-        for (int c = 0; c < R; ++c) {
-          if (c < r) {
+  for (int s = 0; s < kRouteStages - 1; ++s) fetch(32 * s, s);
+  int s = 0;
+#pragma unroll 1
+  for (int v = 0; v < nvec; v += 32) {
+    cp_async_wait<kRouteStages - 2>();
+    uint64_t xf[TB / 2][8];
+#pragma unroll
+    for (int i = 0; i < TB / 2; ++i) {
+      float lo[8], hi[8];
+      unpack8(mine[(s * TB + 2 * i) * 32], lo);
+      unpack8(mine[(s * TB + 2 * i + 1) * 32], hi);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) xf[i][e] = pack_f32x2(lo[e], hi[e]);
+    }
+    fetch(v + 32 * (kRouteStages - 1), s == 0 ? kRouteStages - 1 : s - 1);
+    if (v + lane < nvec) {
+      constexpr int kBatch = WS ? 2 : (R < 4 ? R : 4);  // router slices in flight
+#pragma unroll
+      for (int c0 = 0; c0 < R; c0 += kBatch) {
+        uint4 wv[kBatch];
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+          const uint4* row = w + (size_t)min(c0 + b, r - 1) * nvec + v + lane;
+          wv[b] = WS ? *row : __ldg(row);
+        }
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+          if (c0 + b < R) {
             float wf[8];
-            unpack8(wv[c], wf);
+            unpack8(wv[b], wf);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) acc[c] = fmaf(xf[k], wf[k], acc[c]);
+            for (int e = 0; e < 8; ++e)
+#pragma unroll
+              for (int i = 0; i < TB / 2; ++i)
+                fma_f32x2(acc[i][c0 + b < R ? c0 + b : 0], xf[i][e], pack_f32x2(wf[e], wf[e]));
           }
         }
       }
     }
+    if (++s == kRouteStages) s = 0;
   }
+  float val[N];
 #pragma unroll
-  for (int c = 0; c < R; ++c) {
+  for (int q = 0; q < N; ++q) val[q] = 0.f;
 #pragma unroll
-    for (int s = 16; s > 0; s >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], s);
-  }
-  if (lane == 0) {
-    if (t >= T) {
-      s_e[tl][0] = -1; s_e[tl][1] = -1; s_skip[tl] = 0;
-    } else {
-      int e0, e1;
-      bool skip;
-      route_decide<R>(acc, r, beta, t, kept, o, e0, e1, skip);
-      s_e[tl][0] = e0;
-      s_e[tl][1] = skip ? -1 : e1;
-      s_skip[tl] = skip ? 1 : 0;
+  for (int i = 0; i < TB / 2; ++i)
+#pragma unroll
+    for (int c = 0; c < R; ++c) split_f32x2(acc[i][c], val[2 * i * RP + c], val[(2 * i + 1) * RP + c]);
+  return reduce_scatter<N>(val, lane);
+}
+
+// Top-2 routing.
+template <int R, bool WS>
+__global__ void __launch_bounds__(32 * kRouteWarps, 1)
+router_kernel(const bf16* x, const bf16* __restrict__ Wg, int T, int h, int r, float beta, KeptIds kept,
+              RouteOut o, bool w_const) {
+  pdl_launch_dependents();
+  using Cfg = RouteCfg<R>;
+  constexpr int RP = Cfg::kRP, TB = Cfg::kTB, N = Cfg::kN;
+  extern __shared__ uint4 ring[];
+  __shared__ float s_l[kRouteWarps][N];
+  __shared__ int s_e[Cfg::kTeams][kRouteTokPerBlock][2];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int team = warp / Cfg::kTeamWarps, tw = warp % Cfg::kTeamWarps;
+  uint4* s_w = ring + Cfg::kRingBytes / 16;
+  if (WS && w_const) stage_router_rows(s_w, Wg, r * (h >> 3));
+  pdl_wait();
+  if (WS && !w_const) stage_router_rows(s_w, Wg, r * (h >> 3));
+  if (WS) __syncthreads();
+  const int units = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;
+  for (int u = blockIdx.x + gridDim.x * team; u < units; u += gridDim.x * Cfg::kTeams) {
+    const int t0 = u * kRouteTokPerBlock;
+    const float mine = warp_logits<R, WS>(x, WS ? s_w : reinterpret_cast<const uint4*>(Wg), t0 + tw * TB, T, h, r, ring);
+    if (lane % (32 / N) == 0) s_l[warp][lane / (32 / N)] = mine;
+    __syncwarp();
+    const int i = tw * TB + lane, t = t0 + i;
+    int e0 = -1, e1 = -1;
+    bool skip = false;
+    if (lane < TB && t < T) {
+      float l[R];
+#pragma unroll
+      for (int c = 0; c < R; ++c) l[c] = s_l[warp][lane * RP + c];
+      route_decide<R>(l, r, beta, t, kept, o, e0, e1, skip);
+      if (skip) e1 = -1;
     }
-  }
-  __syncthreads();
-  if (o.blk_hist && threadIdx.x < kHistCols) {
-    int n = 0;
-    if (threadIdx.x == 2 * kMaxE) {
-      for (int i = 0; i < kRouteTokPerBlock; ++i) n += s_skip[i];
-    } else {
-      const int c = threadIdx.x >> 1, slot = threadIdx.x & 1;
-      for (int i = 0; i < kRouteTokPerBlock; ++i) n += (s_e[i][slot] == c);
+    __syncwarp();
+    if (!o.blk_hist) continue;
+    // pair counts of the unit, by the team's threads
+    if (lane < TB) { s_e[team][i][0] = e0; s_e[team][i][1] = e1; }
+    constexpr int kTeamThreads = 32 * Cfg::kTeamWarps;
+    asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kTeamThreads) : "memory");
+    const int col = threadIdx.x - team * kTeamThreads;
+    if (col < kHistCols) {
+      const int n_tok = min(kRouteTokPerBlock, T - t0);
+      int n = 0;
+      if (col == 2 * kMaxE) {
+        for (int q = 0; q < n_tok; ++q) n += s_e[team][q][1] < 0;
+      } else {
+        const int c = col >> 1, slot = col & 1;
+        for (int q = 0; q < n_tok; ++q) n += (s_e[team][q][slot] == c);
+      }
+      o.blk_hist[(size_t)u * kHistCols + col] = n;
     }
-    o.blk_hist[(size_t)blockIdx.x * kHistCols + threadIdx.x] = n;
+    asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kTeamThreads) : "memory");
   }
 }
 
@@ -397,56 +529,164 @@ scan_kernel(const int32_t* blk_hist, int nblk, int r, int pad,
   }
 }
 
-// ------------------------------------------------------------------------------- scatter
+// ------------------------------------------------------------------------------- permute
 
-// Position of pair (t, slot) = start of its expert's group + pairs of that expert in earlier
-// blocks + pairs of that expert among the earlier tokens of this block.
-__global__ void __launch_bounds__(2 * kRouteTokPerBlock)
-scatter_kernel(const int32_t* idx, const uint8_t* skipped, const int32_t* blk_base, const Meta* meta, int T,
-               int32_t* __restrict__ pair_pos, int32_t* __restrict__ row_token) {
-  pdl_launch_dependents();
-  pdl_wait();
-  __shared__ int s_e[kRouteTokPerBlock][2];
-  const int tl = threadIdx.x >> 1, slot = threadIdx.x & 1;
-  const int t = blockIdx.x * kRouteTokPerBlock + tl;
-  int c = -1;
-  if (t < T) {
-    c = ld_l2(idx + 2 * t + slot);
-    if (slot == 1 && ld_l2(skipped + t)) c = -1;
-  }
-  s_e[tl][slot] = c;
-  __syncthreads();
-  if (t >= T) return;
-  int pos = -1;
-  if (c >= 0) {
-    int rank = 0;
-    for (int i = 0; i < tl; ++i) rank += (s_e[i][0] == c) + (s_e[i][1] == c);
-    pos = ld_l2(&meta->off[c]) + ld_l2(blk_base + (size_t)blockIdx.x * kMaxE + c) + rank;
-    row_token[pos] = t;
-  }
-  pair_pos[2 * t + slot] = pos;
+// Permutation and gather of batches beyond kDecodeMaxT tokens: block (b, y) places the pairs of the
+// kRouteTokPerBlock tokens of unit b and copies column share y of their rows to the places.
+// TOP2: two slots per token, the second off where `active` (the skip flag) is set; otherwise k slots,
+// the first `active` of them on.
+// Position of a pair = start of its expert's group + pairs of that expert in earlier units + pairs of
+// that expert among the earlier tokens of the unit.  blk_base == null (at most kPermuteOwnT tokens):
+// every block counts the pairs of the whole routing record and of the units before its own itself,
+// which costs a block a few microseconds and saves the launches of a histogram and a scan; block
+// (0, 0) publishes the batch description.  Else both come from the scan.
+// The rows between a group's end and its padded end are zeroed (the tensor cores draw less power on
+// zeros than on stale rows).
+// Bound by the copy (x once, its k places once); before, as memset + count + scan + scatter + gather
+// with x read once per slot: 611 tokens, two slots 21 -> 10.8 us of kernel time and three launches
+// less; 8192 tokens, six slots 172 -> 135 us.
+__device__ __forceinline__ void count_pair(uint64_t (&n)[2], int e) {  // one byte per expert
+  const uint64_t one = 1ull << (8 * (e & 7));
+  if (e < 8) n[0] += one;
+  else n[1] += one;
 }
 
-// -------------------------------------------------------------------------------- gather
-
+template <bool TOP2>
 __global__ void __launch_bounds__(256)
-gather_kernel(const bf16* x, const int32_t* row_token, const Meta* meta, int h,
-              bf16* __restrict__ xperm) {
+permute_kernel(const bf16* x, const int32_t* idx, const void* active, int T, int k, int h, int r, int pad,
+               const int32_t* blk_base, Meta* meta, int32_t* __restrict__ pair_pos, bf16* __restrict__ xperm,
+               int32_t* s_count, int32_t* s_nskipped, int32_t* s_ntouched, KeptIds kept, int E) {
   pdl_launch_dependents();
   pdl_wait();
-  const int rows = ld_l2(&meta->rows_total);
-  const int lane = threadIdx.x & 31;
-  const int nvec = h >> 3;
-  for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < rows; row += gridDim.x * 8) {
-    const int t = ld_l2(row_token + row);
-    uint4* dst = reinterpret_cast<uint4*>(xperm + (size_t)row * h);
-    if (t >= 0) {
-      const uint4* src = reinterpret_cast<const uint4*>(x + (size_t)t * h);
-      for (int v = lane; v < nvec; v += 32) dst[v] = ld_l2(src + v);
-    } else {
-      for (int v = lane; v < nvec; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
+  __shared__ int s_part[3][8][kMaxE];  // slot-0 pairs, other pairs, pairs of earlier units; per warp
+  __shared__ int s_off[kMaxE], s_cnt[kMaxE], s_end[kMaxE], s_base[kMaxE];
+  __shared__ int s_e[kRouteTokPerBlock][kMaxE];
+  __shared__ int s_pos[kRouteTokPerBlock][kMaxE];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int t0 = blockIdx.x * kRouteTokPerBlock;
+  auto n_active = [&](int t) {
+    if (TOP2) return ld_l2(reinterpret_cast<const uint8_t*>(active) + t) ? 1 : 2;
+    return ld_l2(reinterpret_cast<const int32_t*>(active) + t);
+  };
+  if (blk_base == nullptr) {
+    uint64_t n0[2] = {0, 0}, n1[2] = {0, 0}, nb[2] = {0, 0};
+    for (int t = tid; t < T; t += 256) {
+      const int n = n_active(t);
+      const int32_t* e = idx + (size_t)t * k;
+      const int first = ld_l2(e);
+      count_pair(n0, first);
+      if (t < t0) count_pair(nb, first);
+      for (int m = 1; m < n; ++m) {
+        const int em = ld_l2(e + m);
+        count_pair(n1, em);
+        if (t < t0) count_pair(nb, em);
+      }
+    }
+    for (int c = 0; c < r; ++c) {
+      const int q = c >> 3, s = 8 * (c & 7);
+      const unsigned v0 = __reduce_add_sync(0xffffffffu, (unsigned)((q ? n0[1] : n0[0]) >> s) & 255u);
+      const unsigned v1 = __reduce_add_sync(0xffffffffu, (unsigned)((q ? n1[1] : n1[0]) >> s) & 255u);
+      const unsigned vb = __reduce_add_sync(0xffffffffu, (unsigned)((q ? nb[1] : nb[0]) >> s) & 255u);
+      if (lane == 0) { s_part[0][warp][c] = (int)v0; s_part[1][warp][c] = (int)v1; s_part[2][warp][c] = (int)vb; }
     }
   }
+  // the unit's own pairs
+  if (tid < kRouteTokPerBlock * kMaxE) {
+    const int tl = tid / kMaxE, m = tid % kMaxE, t = t0 + tl;
+    s_e[tl][m] = (m < k && t < T && m < n_active(t)) ? ld_l2(idx + (size_t)t * k + m) : -1;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const bool on = lane < r;
+    int off, cnt, padded, base;
+    if (blk_base == nullptr) {
+      int c0 = 0, c1 = 0, before = 0;
+      for (int w = 0; on && w < 8; ++w) {
+        c0 += s_part[0][w][lane];
+        c1 += s_part[1][w][lane];
+        before += s_part[2][w][lane];
+      }
+      cnt = c0 + c1;
+      padded = (cnt + pad - 1) / pad * pad;
+      const int mine_tiles = (cnt + kTileRows - 1) / kTileRows;
+      int end = padded, tiles = mine_tiles;  // inclusive sums over the experts
+#pragma unroll
+      for (int s = 1; s < kMaxE; s <<= 1) {
+        const int a = __shfl_up_sync(0xffffffffu, end, s), b = __shfl_up_sync(0xffffffffu, tiles, s);
+        if (lane >= s) { end += a; tiles += b; }
+      }
+      off = end - padded;
+      base = off + before;
+      if (blockIdx.x == 0 && blockIdx.y == 0) {
+        const int pairs = __reduce_add_sync(0xffffffffu, cnt);
+        const int touched = __popc(__ballot_sync(0xffffffffu, cnt > 0));
+        if (lane < kMaxE) {
+          meta->count[lane] = cnt;
+          meta->count_slot[lane][0] = TOP2 ? c0 : cnt;
+          meta->count_slot[lane][1] = TOP2 ? c1 : 0;
+          meta->off[lane + 1] = end;
+          meta->tile_prefix[lane + 1] = tiles;
+          if (s_count && lane < E) { s_count[2 * lane] = 0; s_count[2 * lane + 1] = 0; }
+        }
+        __syncwarp();
+        if (s_count && on) { s_count[2 * kept.id[lane]] = c0; s_count[2 * kept.id[lane] + 1] = c1; }
+        if (lane == kMaxE - 1) {
+          meta->off[0] = 0;
+          meta->tile_prefix[0] = 0;
+          meta->rows_total = end;
+          meta->n_skipped = T * k - pairs;
+          meta->n_touched = touched;
+          meta->reserved = 0;
+          if (s_count) { *s_nskipped = T * k - pairs; *s_ntouched = touched; }
+        }
+      }
+    } else {
+      off = on ? ld_l2(&meta->off[lane]) : 0;
+      cnt = on ? ld_l2(&meta->count[lane]) : 0;
+      padded = on ? ld_l2(&meta->off[lane + 1]) - off : 0;
+      base = on ? off + ld_l2(blk_base + (size_t)blockIdx.x * kMaxE + lane) : 0;
+    }
+    if (on) { s_off[lane] = off; s_cnt[lane] = cnt; s_end[lane] = off + padded; s_base[lane] = base; }
+  }
+  __syncthreads();
+  if (tid < kRouteTokPerBlock * kMaxE) {
+    const int tl = tid / kMaxE, m = tid % kMaxE, c = s_e[tl][m];
+    int pos = -1;
+    if (c >= 0) {
+      int rank = 0;
+      for (int i = 0; i < tl; ++i)
+        for (int q = 0; q < k; ++q) rank += (s_e[i][q] == c);
+      pos = s_base[c] + rank;
+    }
+    s_pos[tl][m] = pos;
+    if (blockIdx.y == 0 && m < k && t0 + tl < T) pair_pos[(size_t)(t0 + tl) * k + m] = pos;
+  }
+  __syncthreads();
+  const int nvec = h >> 3;
+  const int share = (nvec + gridDim.y - 1) / gridDim.y;
+  const int v0 = blockIdx.y * share, v1 = min(nvec, v0 + share);
+  uint4* rows = reinterpret_cast<uint4*>(xperm);
+  for (int tl = warp; tl < kRouteTokPerBlock && t0 + tl < T; tl += 8) {
+    const uint4* src = reinterpret_cast<const uint4*>(x + (size_t)(t0 + tl) * h);
+    constexpr int kAhead = 8;  // loads in flight per lane
+    for (int v = v0 + lane; v < v1; v += 32 * kAhead) {
+      uint4 val[kAhead];
+#pragma unroll
+      for (int a = 0; a < kAhead; ++a)
+        if (v + 32 * a < v1) val[a] = ld_l2(src + v + 32 * a);
+      for (int m = 0; m < k; ++m) {
+        const int pos = s_pos[tl][m];
+        if (pos < 0) continue;
+        uint4* dst = rows + (size_t)pos * nvec;
+#pragma unroll
+        for (int a = 0; a < kAhead; ++a)
+          if (v + 32 * a < v1) dst[v + 32 * a] = val[a];
+      }
+    }
+  }
+  for (int c = blockIdx.x; c < r; c += gridDim.x)
+    for (int row = s_off[c] + s_cnt[c] + warp; row < s_end[c]; row += 8)
+      for (int v = v0 + lane; v < v1; v += 32) rows[(size_t)row * nvec + v] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // ------------------------------------------------------------------------------- combine
@@ -496,91 +736,73 @@ combine_kernel(const float* O, int ksplit, size_t split_stride, const int32_t* p
 
 // ------------------------------------------------------------------ general top-k path
 
-// Top-k routing with the generalised skipping rule of App. A.2, one block per token:
+// Top-k routing with the generalised skipping rule of App. A.2:
 //   e_0..e_{k-1} = kept experts with the k largest logits (ties to the lower index),
 //   p_m = exp(l_em - l_e0);  keep the top i* = min i : sum_{m>i} p_m <= beta * sum_{m<=k} p_m;
 //   weights p_m / sum_{m<=i*} p_m.  The fp32 summation orders are fixed: total ascending in m,
 //   tails from the smallest upwards, kept mass ascending in m.
-__global__ void __launch_bounds__(256)
-router_topk_kernel(const bf16* __restrict__ x, const bf16* __restrict__ Wg, int T, int h, int r,
-                   int k, float beta, KeptIds kept, int32_t* __restrict__ idx,
-                   float* __restrict__ wn, int32_t* __restrict__ nact, int32_t* u_idx, float* u_wn,
-                   int32_t* u_nact, float* logits) {
-  __shared__ float s_part[8][kMaxE];
-  const int t = blockIdx.x;
+// Ranking by counting, one lane per (token, kept expert): the rank of expert c is the number of kept
+// experts that beat it (larger logit, or equal logit and lower index), so the expert of rank m is
+// the m-th choice; the three sums are one lane's per token (k <= 16 values).
+template <int R, bool WS>
+__global__ void __launch_bounds__(32 * kRouteWarps, 1)
+router_topk_kernel(const bf16* x, const bf16* __restrict__ Wg, int T, int h, int r, int k, float beta,
+                   KeptIds kept, int32_t* __restrict__ idx, float* __restrict__ wn, int32_t* __restrict__ nact,
+                   int32_t* u_idx, float* u_wn, int32_t* u_nact, float* logits) {
+  pdl_launch_dependents();
+  using Cfg = RouteCfg<R>;
+  constexpr int RP = Cfg::kRP, TB = Cfg::kTB, N = Cfg::kN;
+  constexpr int kLanes = 32 / N;  // lanes that hold the same logit
+  extern __shared__ uint4 ring[];
+  __shared__ float s_p[kRouteWarps][TB][RP];
+  __shared__ int s_sel[kRouteWarps][TB][RP];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nvec = h >> 3;
-  float acc[kMaxE];
-#pragma unroll
-  for (int c = 0; c < kMaxE; ++c) acc[c] = 0.f;
-  const uint4* xr = reinterpret_cast<const uint4*>(x + (size_t)t * h);
-  for (int v = threadIdx.x; v < nvec; v += 256) {
-    float xf[8];
-    unpack8(ld_l2(xr + v), xf);
-#pragma unroll
-    for (int c = 0; c < kMaxE; ++c) {
-      if (c < r) {
-        float wf[8];
-        unpack8(__ldg(reinterpret_cast<const uint4*>(Wg + (size_t)c * h) + v), wf);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) acc[c] = fmaf(xf[q], wf[q], acc[c]);
-      }
+  uint4* s_w = ring + Cfg::kRingBytes / 16;
+  if (WS) stage_router_rows(s_w, Wg, r * (h >> 3));
+  pdl_wait();
+  if (WS) __syncthreads();
+  const int groups = (T + TB - 1) / TB;
+  for (int g = blockIdx.x + gridDim.x * warp; g < groups; g += gridDim.x * kRouteWarps) {
+  const int t0 = g * TB;
+  const float mine = warp_logits<R, WS>(x, WS ? s_w : reinterpret_cast<const uint4*>(Wg), t0, T, h, r, ring);
+  const int i = lane / kLanes / RP, c = lane / kLanes % RP;
+  int rank = 0;
+  float top = -INFINITY;
+  for (int d = 0; d < r; ++d) {
+    const float o = __shfl_sync(0xffffffffu, mine, (i * RP + d) * kLanes);
+    rank += (o > mine) || (o == mine && d < c);
+    top = d == 0 || o > top ? o : top;
+  }
+  if (lane % kLanes == 0) {  // logits that compare with nothing (NaN) leave ranks unclaimed: name some expert
+    s_sel[warp][i][c] = min(c, r - 1);
+    s_p[warp][i][c] = 0.f;
+  }
+  __syncwarp();
+  if (c < r && lane % kLanes == 0) {
+    if (logits && t0 + i < T) logits[(size_t)(t0 + i) * r + c] = mine;
+    if (rank < k) {
+      s_sel[warp][i][rank] = c;
+      s_p[warp][i][rank] = expf(mine - top);
     }
   }
-#pragma unroll
-  for (int c = 0; c < kMaxE; ++c) {
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], s);
-    if (lane == 0) s_part[warp][c] = acc[c];
-  }
-  __syncthreads();
-  // Ranking by counting, one thread per kept expert: the rank of expert c is the number of kept
-  // experts that beat it (larger logit, or equal logit and lower index), so the expert of rank m
-  // is the m-th choice.  The k chosen experts' softmax numerators relative to the largest,
-  // p_m = exp(l_m - l_0), then go through the three fixed-order sums of the rule, which one
-  // thread evaluates (k <= 8 values).
-  __shared__ float s_l[kMaxE];
-  __shared__ float s_p[kMaxE];
-  __shared__ int s_sel[kMaxE];
-  const int c = threadIdx.x;
-  if (c < r) {
-    float v = 0.f;
-    for (int w = 0; w < 8; ++w) v += s_part[w][c];
-    s_l[c] = v;
-    if (logits) logits[(size_t)t * r + c] = v;
-  }
-  __syncthreads();
-  if (c < r) {
-    const float mine = s_l[c];
-    int rank = 0;
-    for (int d = 0; d < r; ++d) {
-      const float o = s_l[d];
-      rank += (o > mine) || (o == mine && d < c);
-    }
-    if (rank < k) s_sel[rank] = c;
-  }
-  __syncthreads();
-  if (c < k) s_p[c] = expf(s_l[s_sel[c]] - s_l[s_sel[0]]);
-  __syncthreads();
-  if (c != 0) return;
+  __syncwarp();
+  const int t = t0 + lane;
+  if (lane < TB && t < T) {
+  const float* p = s_p[warp][lane];
+  const int* sel = s_sel[warp][lane];
   // i* = the smallest i in 1..k whose dropped mass p_i + .. + p_{k-1} (added from the smallest
   // value upwards) is at most beta times the whole mass p_0 + .. + p_{k-1} (added in rank order)
   float whole = 0.f;
-  for (int m = 0; m < k; ++m) whole += s_p[m];
+  for (int m = 0; m < k; ++m) whole += p[m];
   const float bound = beta * whole;
-  int istar = 1;
-  {
-    float dropped = 0.f;   // mass beyond rank i - 1, for i = k, k - 1, ..: walk down while it fits
-    int i = k;
-    while (i > 1 && dropped + s_p[i - 1] <= bound) { dropped += s_p[i - 1]; --i; }
-    // dropped = p_i + .. + p_{k-1} fits; p_{i-1} + dropped does not (or i = 1)
-    istar = i;
-  }
+  float dropped = 0.f;  // mass beyond rank istar - 1, for istar = k, k - 1, ..: walk down while it fits
+  int istar = k;
+  while (istar > 1 && dropped + p[istar - 1] <= bound) { dropped += p[istar - 1]; --istar; }
   float kept_mass = 0.f;
-  for (int m = 0; m < istar; ++m) kept_mass += s_p[m];
+  for (int m = 0; m < istar; ++m) kept_mass += p[m];
   for (int m = 0; m < k; ++m) {
-    const float w = m < istar ? s_p[m] / kept_mass : 0.f;
-    const int e = s_sel[m];
+    const float w = m < istar ? p[m] / kept_mass : 0.f;
+    const int e = sel[m];
     idx[(size_t)t * k + m] = e;
     wn[(size_t)t * k + m] = w;
     if (u_idx) u_idx[(size_t)t * k + m] = kept.id[e];
@@ -588,6 +810,9 @@ router_topk_kernel(const bf16* __restrict__ x, const bf16* __restrict__ Wg, int 
   }
   nact[t] = istar;
   if (u_nact) u_nact[t] = istar;
+  }
+  __syncwarp();
+  }
 }
 
 // Per block of kRouteTokPerBlock tokens: active pairs per expert, in the column layout scan_kernel reads
@@ -610,57 +835,50 @@ count_topk_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ n
   blk_hist[(size_t)blockIdx.x * kHistCols + col] = n;
 }
 
-// Position of pair (t, m): start of the expert's group + pairs of that expert in earlier
-// blocks + pairs of that expert among the earlier tokens of this block.
-__global__ void __launch_bounds__(kRouteTokPerBlock)
-scatter_topk_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ nact,
-                    const int32_t* __restrict__ blk_base, const Meta* __restrict__ meta, int T,
-                    int k, int32_t* __restrict__ pair_pos, int32_t* __restrict__ row_token) {
-  __shared__ int s_e[kRouteTokPerBlock][kMaxE];
-  const int tl = threadIdx.x;
-  const int t = blockIdx.x * kRouteTokPerBlock + tl;
-  for (int m = 0; m < k; ++m) s_e[tl][m] = (t < T && m < nact[t]) ? idx[(size_t)t * k + m] : -1;
-  __syncthreads();
-  if (t >= T) return;
-  for (int m = 0; m < k; ++m) {
-    const int c = s_e[tl][m];
-    int pos = -1;
-    if (c >= 0) {
-      int rank = 0;
-      for (int i = 0; i < tl; ++i)
-        for (int q = 0; q < k; ++q) rank += (s_e[i][q] == c);
-      pos = meta->off[c] + blk_base[(size_t)blockIdx.x * kMaxE + c] + rank;
-      row_token[pos] = t;
-    }
-    pair_pos[(size_t)t * k + m] = pos;
-  }
-}
-
 __global__ void __launch_bounds__(128)
-combine_topk_kernel(const float* __restrict__ O, int ksplit, size_t split_stride,
-                    const int32_t* __restrict__ pair_pos, const float* __restrict__ wn, int k,
-                    int T, int h, bf16* y) {
+combine_topk_kernel(const float* O, int ksplit, size_t split_stride, const int32_t* pair_pos, const float* wn,
+                    int k, int T, int h, bf16* y) {
+  pdl_launch_dependents();
+  pdl_wait();
+  constexpr int kAhead = 4;  // slots whose loads are in flight together
+  __shared__ int s_p[kMaxE];
+  __shared__ float s_w[kMaxE];
   const int t = blockIdx.x;
   const int nvec = h >> 3;
+  if (threadIdx.x < kMaxE) {
+    const bool on = (int)threadIdx.x < k;
+    s_p[threadIdx.x] = on ? ld_l2(pair_pos + (size_t)t * k + threadIdx.x) : -1;
+    s_w[threadIdx.x] = on ? ld_l2(wn + (size_t)t * k + threadIdx.x) : 0.f;
+  }
+  __syncthreads();
   for (int v = blockIdx.y * blockDim.x + threadIdx.x; v < nvec; v += gridDim.y * blockDim.x) {
     float z[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) z[q] = 0.f;
-    for (int m = 0; m < k; ++m) {
-      const int p = pair_pos[(size_t)t * k + m];
-      if (p < 0) continue;
-      const float w = wn[(size_t)t * k + m];
-      float a[8];
+    for (int m0 = 0; m0 < k; m0 += kAhead) {
+      float4 q0[kAhead], q1[kAhead];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) a[q] = 0.f;
-      for (int s = 0; s < ksplit; ++s) {
-        const float4* o = reinterpret_cast<const float4*>(O + s * split_stride + (size_t)p * h) + 2 * v;
-        const float4 q0 = o[0], q1 = o[1];
-        a[0] += q0.x; a[1] += q0.y; a[2] += q0.z; a[3] += q0.w;
-        a[4] += q1.x; a[5] += q1.y; a[6] += q1.z; a[7] += q1.w;
+      for (int m = 0; m < kAhead; ++m) {
+        q0[m] = q1[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (s_p[m0 + m] >= 0) {
+          const float4* o = reinterpret_cast<const float4*>(O + (size_t)s_p[m0 + m] * h) + 2 * v;
+          q0[m] = ld_l2(o);
+          q1[m] = ld_l2(o + 1);
+        }
       }
 #pragma unroll
-      for (int q = 0; q < 8; ++q) z[q] = fmaf(w, a[q], z[q]);
+      for (int m = 0; m < kAhead; ++m) {
+        if (s_p[m0 + m] < 0) continue;
+        float a[8] = {q0[m].x, q0[m].y, q0[m].z, q0[m].w, q1[m].x, q1[m].y, q1[m].z, q1[m].w};
+        for (int s = 1; s < ksplit; ++s) {
+          const float4* o = reinterpret_cast<const float4*>(O + s * split_stride + (size_t)s_p[m0 + m] * h) + 2 * v;
+          const float4 r0 = ld_l2(o), r1 = ld_l2(o + 1);
+          a[0] += r0.x; a[1] += r0.y; a[2] += r0.z; a[3] += r0.w;
+          a[4] += r1.x; a[5] += r1.y; a[6] += r1.z; a[7] += r1.w;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) z[q] = fmaf(s_w[m0 + m], a[q], z[q]);
+      }
     }
     uint4 outv;
     outv.x = pack2(z[0], z[1]); outv.y = pack2(z[2], z[3]);
@@ -788,40 +1006,86 @@ __device__ __forceinline__ float key_float(uint32_t k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
-// Exact k-th smallest by radix selection on the ordered bit patterns, 8 bits per pass.
-__global__ void __launch_bounds__(1024)
-select2_kernel(const float* __restrict__ v, int n, int k0, int k1, float* out) {
-  __shared__ unsigned hist[256];
-  __shared__ unsigned s_prefix;
-  __shared__ int s_k;
-  for (int which = 0; which < 2; ++which) {
-    if (threadIdx.x == 0) { s_prefix = 0; s_k = which ? k1 : k0; }
-    unsigned mask = 0;
-    for (int pass = 3; pass >= 0; --pass) {
-      const int shift = pass * 8;
-      if (threadIdx.x < 256) hist[threadIdx.x] = 0;
-      __syncthreads();
-      const unsigned prefix = s_prefix;
-      for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const unsigned key = float_key(v[i]);
-        if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        int k = s_k;
-        unsigned bin = 0;
-        for (; bin < 255; ++bin) {
-          if (k < (int)hist[bin]) break;
-          k -= (int)hist[bin];
-        }
-        s_k = k;
-        s_prefix = prefix | (bin << shift);
-      }
-      mask |= 0xffu << shift;
-      __syncthreads();
+// Exact k0-th and k1-th smallest (0-based, k1 = k0 or k0 + 1) by radix selection on the ordered bit
+// patterns: digits of 11, 11 and 10 bits, the counts of a digit in shared memory, then one more
+// pass for the smallest key above the k0-th.  NV > 0: up to NV keys per thread stay in registers
+// (NV * 1024 values); NV = 0: every pass reads the values again.  One block: bound by the shared-
+// memory additions of the first digit (few exponents, so few bins).  16384 values 36.8 -> 12.9 us
+// against four 8-bit passes per rank over memory.
+constexpr int kSelThreads = 1024;
+template <int NV>
+__global__ void __launch_bounds__(kSelThreads)
+select2_kernel(const float* v, int n, int k0, int k1, float* out) {
+  pdl_wait();
+  __shared__ unsigned hist[2048];
+  __shared__ unsigned s_warp[32];
+  __shared__ unsigned s_prefix, s_rank, s_count;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint32_t keys[NV > 0 ? NV : 1];
+  if (NV > 0) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int p = tid + i * kSelThreads;
+      keys[i] = p < n ? float_key(ld_l2(v + p)) : 0u;
     }
-    if (threadIdx.x == 0) out[which] = key_float(s_prefix);
+  }
+  auto each = [&](auto&& f) {
+    if (NV > 0) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i)
+        if (tid + i * kSelThreads < n) f(keys[i]);
+    } else {
+      for (int p = tid; p < n; p += kSelThreads) f(float_key(ld_l2(v + p)));
+    }
+  };
+  uint32_t prefix = 0, mask = 0;
+  unsigned rank = (unsigned)k0, count = 0;
+#pragma unroll
+  for (int pass = 0; pass < 3; ++pass) {
+    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
+    const uint32_t digit = pass == 2 ? 1023u : 2047u;
+    hist[2 * tid] = 0u;
+    hist[2 * tid + 1] = 0u;
     __syncthreads();
+    each([&](uint32_t key) {
+      if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & digit], 1u);
+    });
+    __syncthreads();
+    // exclusive sums over the bins, two bins a thread; the thread whose bin holds the rank says so
+    const unsigned h0 = hist[2 * tid], h1 = hist[2 * tid + 1];
+    unsigned inc = h0 + h1;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const unsigned up = __shfl_up_sync(0xffffffffu, inc, s);
+      if (lane >= s) inc += up;
+    }
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    const unsigned before = __reduce_add_sync(0xffffffffu, lane < warp ? s_warp[lane] : 0u) + inc - h0 - h1;
+    if (rank >= before && rank < before + h0 + h1) {
+      const bool second = rank >= before + h0;
+      s_prefix = prefix | ((uint32_t)(2 * tid + (second ? 1 : 0)) << shift);
+      s_rank = rank - before - (second ? h0 : 0u);
+      s_count = second ? h1 : h0;
+    }
+    __syncthreads();
+    prefix = s_prefix;
+    rank = s_rank;
+    count = s_count;
+    mask |= digit << shift;
+  }
+  uint32_t next = prefix;
+  if (k1 > k0 && rank + 1 >= count) {  // the k0-th is the last of its value
+    uint32_t best = 0xffffffffu;
+    each([&](uint32_t key) { if (key > prefix) best = min(best, key); });
+    best = __reduce_min_sync(0xffffffffu, best);
+    if (lane == 0) s_warp[warp] = best;
+    __syncthreads();
+    next = __reduce_min_sync(0xffffffffu, s_warp[lane]);
+  }
+  if (tid == 0) {
+    out[0] = key_float(prefix);
+    out[1] = key_float(next);
   }
 }
 
@@ -851,17 +1115,35 @@ interleave_kernel(const bf16* __restrict__ W1, const bf16* __restrict__ W3, Kept
 
 // ------------------------------------------------------------------------------ launchers
 
-cudaError_t launch_router(const bf16* x, const bf16* Wg, int T, int h, int r, float beta,
-                          const KeptIds& kept, const RouteOut& out, cudaStream_t st) {
-  const int nblk = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;
-  switch (r) {
-    case 2: return launch_pdl(router_kernel<2>, dim3(nblk), dim3(32 * kRouteTokPerBlock), 0, st, x, Wg, T, h, r, beta, kept, out);
-    case 3: case 4: return launch_pdl(router_kernel<4>, dim3(nblk), dim3(32 * kRouteTokPerBlock), 0, st, x, Wg, T, h, r, beta, kept, out);
-    case 5: case 6: return launch_pdl(router_kernel<6>, dim3(nblk), dim3(32 * kRouteTokPerBlock), 0, st, x, Wg, T, h, r, beta, kept, out);
-    case 7: case 8: return launch_pdl(router_kernel<8>, dim3(nblk), dim3(32 * kRouteTokPerBlock), 0, st, x, Wg, T, h, r, beta, kept, out);
-    default: return launch_pdl(router_kernel<kMaxE>, dim3(nblk), dim3(32 * kRouteTokPerBlock), 0, st, x, Wg, T, h, r, beta, kept, out);
+// One block per SM at most; `work` blocks have something to do.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_route(void (*kernel)(KArgs...), int work, size_t smem, cudaStream_t st, Args&&... args) {
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRouteSmemMax);
+    if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return launch_pdl(kernel, dim3(work < 148 ? work : 148), dim3(32 * kRouteWarps), smem, st, args...);
+}
+
+cudaError_t launch_router(const bf16* x, const bf16* Wg, int T, int h, int r, float beta,
+                          const KeptIds& kept, const RouteOut& out, cudaStream_t st, bool w_const) {
+  const size_t w_bytes = (size_t)r * h * 2;
+#define MOE_ROUTER(R)                                                                                          \
+  {                                                                                                            \
+    const bool ws = RouteCfg<R>::kRingBytes + w_bytes <= kRouteSmemMax;                                        \
+    const size_t smem = RouteCfg<R>::kRingBytes + (ws ? w_bytes : 0);                                          \
+    const int units = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;                                         \
+    return launch_route(ws ? router_kernel<R, true> : router_kernel<R, false>, units, smem, st, x, Wg, T, h, r, \
+                        beta, kept, out, w_const);                                                             \
+  }
+  switch (r) {
+    case 2: MOE_ROUTER(2)
+    case 3: case 4: MOE_ROUTER(4)
+    case 5: case 6: MOE_ROUTER(6)
+    case 7: case 8: MOE_ROUTER(8)
+    default: MOE_ROUTER(kMaxE)
+  }
+#undef MOE_ROUTER
 }
 
 cudaError_t launch_router_small(const bf16* x, const bf16* Wg, int T, int h, int r, float beta,
@@ -909,20 +1191,18 @@ cudaError_t launch_scan(const int32_t* blk_hist, int nblk, int r, int pad, int32
                     s_count, s_nskipped, s_ntouched, kept, E);
 }
 
-cudaError_t launch_scatter(const int32_t* idx, const uint8_t* skipped, const int32_t* blk_base,
-                           const Meta* meta, int T, int32_t* pair_pos, int32_t* row_token,
-                           cudaStream_t st) {
-  const int nblk = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;
-  return launch_pdl(scatter_kernel, dim3(nblk), dim3(2 * kRouteTokPerBlock), 0, st, idx, skipped,
-                    blk_base, meta, T, pair_pos, row_token);
-}
-
-cudaError_t launch_gather(const bf16* x, const int32_t* row_token, const Meta* meta, int h,
-                          int cap_rows, bf16* xperm, cudaStream_t st) {
-  int blocks = (cap_rows + 7) / 8;
-  if (blocks > 148 * 16) blocks = 148 * 16;
-  if (blocks < 1) blocks = 1;
-  return launch_pdl(gather_kernel, dim3(blocks), dim3(256), 0, st, x, row_token, meta, h, xperm);
+cudaError_t launch_permute(const bf16* x, const int32_t* idx, const void* active, bool top2, int T, int k, int h,
+                           int r, int pad, const int32_t* blk_base, Meta* meta, int32_t* pair_pos, bf16* xperm,
+                           int32_t* s_count, int32_t* s_nskipped, int32_t* s_ntouched, const KeptIds& kept,
+                           int E, cudaStream_t st) {
+  const int units = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;
+  // column shares: enough blocks to keep every SM copying, at least 64 vectors each
+  int ny = 148 * 4 / units, most = (h >> 3) / 64;
+  if (ny > most) ny = most;
+  if (ny < 1) ny = 1;
+  return launch_pdl(top2 ? permute_kernel<true> : permute_kernel<false>, dim3(units, ny), dim3(256), 0, st, x, idx,
+                    active, T, k, h, r, pad, blk_base, meta, pair_pos, xperm, s_count, s_nskipped, s_ntouched,
+                    kept, E);
 }
 
 cudaError_t launch_combine(const float* O, int ksplit, size_t split_stride, const int32_t* pair_pos,
@@ -938,9 +1218,23 @@ cudaError_t launch_router_topk(const bf16* x, const bf16* Wg, int T, int h, int 
                                const KeptIds& kept, int32_t* idx, float* wn, int32_t* nact,
                                int32_t* u_idx, float* u_wn, int32_t* u_nact, float* logits,
                                cudaStream_t st) {
-  router_topk_kernel<<<T, 256, 0, st>>>(x, Wg, T, h, r, k, beta, kept, idx, wn, nact, u_idx, u_wn, u_nact,
-                                        logits);
-  return cudaGetLastError();
+  const size_t w_bytes = (size_t)r * h * 2;
+#define MOE_ROUTER_TOPK(R)                                                                                   \
+  {                                                                                                          \
+    const bool ws = RouteCfg<R>::kRingBytes + w_bytes <= kRouteSmemMax;                                      \
+    const size_t smem = RouteCfg<R>::kRingBytes + (ws ? w_bytes : 0);                                        \
+    const int groups = (T + RouteCfg<R>::kTB - 1) / RouteCfg<R>::kTB;                                        \
+    return launch_route(ws ? router_topk_kernel<R, true> : router_topk_kernel<R, false>, groups, smem, st, x, Wg, \
+                        T, h, r, k, beta, kept, idx, wn, nact, u_idx, u_wn, u_nact, logits);                 \
+  }
+  switch (r) {
+    case 2: MOE_ROUTER_TOPK(2)
+    case 3: case 4: MOE_ROUTER_TOPK(4)
+    case 5: case 6: MOE_ROUTER_TOPK(6)
+    case 7: case 8: MOE_ROUTER_TOPK(8)
+    default: MOE_ROUTER_TOPK(kMaxE)
+  }
+#undef MOE_ROUTER_TOPK
 }
 
 cudaError_t launch_count_topk(const int32_t* idx, const int32_t* nact, int T, int k,
@@ -950,22 +1244,13 @@ cudaError_t launch_count_topk(const int32_t* idx, const int32_t* nact, int T, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_topk(const int32_t* idx, const int32_t* nact, const int32_t* blk_base,
-                                const Meta* meta, int T, int k, int32_t* pair_pos,
-                                int32_t* row_token, cudaStream_t st) {
-  const int nblk = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;
-  scatter_topk_kernel<<<nblk, kRouteTokPerBlock, 0, st>>>(idx, nact, blk_base, meta, T, k, pair_pos,
-                                                          row_token);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_combine_topk(const float* O, int ksplit, size_t split_stride,
                                 const int32_t* pair_pos, const float* wn, int k, int T, int h,
                                 bf16* y, cudaStream_t st) {
   int ychunks = ((h >> 3) + 127) / 128;
   if (T > 4096) ychunks = 1;
-  combine_topk_kernel<<<dim3(T, ychunks), 128, 0, st>>>(O, ksplit, split_stride, pair_pos, wn, k, T, h, y);
-  return cudaGetLastError();
+  return launch_pdl(combine_topk_kernel, dim3(T, ychunks), dim3(128), 0, st, O, ksplit, split_stride, pair_pos,
+                    wn, k, T, h, y);
 }
 
 cudaError_t launch_coselection(const int32_t* idx, int T, int E, const KeptIds& kept, int32_t* counts,
@@ -993,8 +1278,10 @@ cudaError_t launch_set_dense_meta(Meta* meta, int E, int rows_per_expert, int of
 }
 
 cudaError_t launch_select2(const float* ratio, int T, int k0, int k1, float* out, cudaStream_t st) {
-  select2_kernel<<<1, 1024, 0, st>>>(ratio, T, k0, k1, out);
-  return cudaGetLastError();
+  if (T <= 8 * kSelThreads) return launch_pdl(select2_kernel<8>, dim3(1), dim3(kSelThreads), 0, st, ratio, T, k0, k1, out);
+  if (T <= 16 * kSelThreads) return launch_pdl(select2_kernel<16>, dim3(1), dim3(kSelThreads), 0, st, ratio, T, k0, k1, out);
+  if (T <= 32 * kSelThreads) return launch_pdl(select2_kernel<32>, dim3(1), dim3(kSelThreads), 0, st, ratio, T, k0, k1, out);
+  return launch_pdl(select2_kernel<0>, dim3(1), dim3(kSelThreads), 0, st, ratio, T, k0, k1, out);
 }
 
 cudaError_t launch_interleave(const bf16* W1, const bf16* W3, const KeptIds& kept, int r, int f,

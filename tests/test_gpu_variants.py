@@ -326,3 +326,67 @@ def test_large_batch_gemm_at_the_edges_of_its_tiles(h, f, E, kept, T):
     assert lay.device_status() == 0
     lay.close()
     dbg.close()
+
+
+@pytest.mark.parametrize("h,f,E,kept,T,k", [
+    # expert counts between the instantiations, slices of a row that do not fill a warp, router rows
+    # beyond the shared memory (8192 x 13), a last unit of one token, batches beyond the permutation
+    # that counts for itself
+    (64, 64, 3, 0b111, 257, 2), (576, 64, 5, 0b11111, 300, 3), (128, 64, 16, 0xFFFF, 513, 5),
+    (8192, 64, 13, 0x1FFF, 300, 4), (128, 64, 13, 0x1FFF, 8193, 3), (128, 64, 2, 0b11, 9001, 2),
+    (320, 64, 12, 0b111111111111, 8192, 8),
+])
+def test_routing_and_permutation_of_large_batches_equal_small_ones(h, f, E, kept, T, k):
+    # the same tokens through the small-batch sequences, at most 256 at a time
+    build.build()
+    W = synth.make_layer_weights(h, f, E, seed=8, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2, kept)
+    x = synth.make_tokens(T, h, seed=9, device=DEV)
+    stats = binding.RoutingStats(T, E, DEV)
+    y = layer.forward(x, 0.5, stats=stats)
+    yk, idx, wn, n_active = layer.forward_topk(x, k, 0.2, record=True)
+    torch.cuda.synchronize()
+    counts = torch.zeros_like(stats.count)
+    logits = (x.double() @ W.W_gate.double().T).sort(dim=1, descending=True)
+    clear = (logits.values[:, :-1] - logits.values[:, 1:]).min(dim=1).values > 1e-4 if E > 1 else None
+    p = torch.exp(logits.values - logits.values[:, :1])
+    far = (p[:, 1] - 0.5).abs() > 1e-4
+    assert torch.equal(stats.idx[clear].long(), logits.indices[clear, :2])
+    assert torch.equal(stats.skipped[clear & far].bool(), p[clear & far, 1] < 0.5)
+    assert torch.equal(idx[clear].long(), logits.indices[clear, :k])
+    assert torch.allclose(stats.ratio.double(), p[:, 1], atol=1e-4)
+    for slot in (0, 1):
+        on = stats.idx[:, slot][(stats.skipped == 0) | (slot == 0)]
+        counts[:, slot] = torch.bincount(on.long(), minlength=E).to(counts.dtype)
+    assert torch.equal(stats.count, counts)
+    assert int(stats.n_skipped) == int(stats.skipped.sum())
+    assert int(stats.n_experts_touched) == int((counts.sum(1) > 0).sum())
+    starts = [0, (T // 512) * 256, T - min(T, 200)]
+    for t0 in starts:
+        xs = x[t0:t0 + 200].contiguous()
+        s = binding.RoutingStats(xs.shape[0], E, DEV)
+        ys = layer.forward(xs, 0.5, stats=s)
+        yks, idxs, _, nas = layer.forward_topk(xs, k, 0.2, record=True)
+        torch.cuda.synchronize()
+        same = (s.idx == stats.idx[t0:t0 + 200]).all(1) & (s.skipped == stats.skipped[t0:t0 + 200])
+        assert same.float().mean() > 0.95 and rel_l2(ys[same], y[t0:t0 + 200][same]) < 5e-3
+        same = (idxs == idx[t0:t0 + 200]).all(1) & (nas == n_active[t0:t0 + 200])
+        assert same.float().mean() > 0.95 and rel_l2(yks[same], yk[t0:t0 + 200][same]) < 5e-3
+    assert layer.device_status() == 0
+    layer.close()
+
+
+@pytest.mark.parametrize("T,distinct", [(1, 1), (2, 2), (257, 257), (8192, 8192), (8193, 8193), (16385, 16385),
+                                        (32769, 32769), (5000, 3), (5001, 1), (40000, 2)])
+def test_calibrated_beta_is_the_exact_median_of_the_ratios(weights, T, distinct):
+    # repeated tokens make the middle values equal, or put both sides of the middle on two values
+    layer = binding.MoeLayer(*weights)
+    x = synth.make_tokens(distinct, H, seed=11, device=DEV).repeat((T + distinct - 1) // distinct, 1)[:T].contiguous()
+    got = layer.calibrate_beta(x)
+    stats = binding.RoutingStats(T, E, DEV)
+    layer.forward(x, 0.0, stats=stats)
+    r = stats.ratio.double().sort().values
+    want = float(((r[(T - 1) // 2] + r[T // 2]) / 2).float())
+    # up to 256 tokens forward adds its logits in another order: a few units in the last place
+    assert abs(got - want) <= (2e-6 if T <= 256 else 0.0)
+    layer.close()
