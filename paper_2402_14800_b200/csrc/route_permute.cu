@@ -136,7 +136,8 @@ route_single_kernel(const bf16* x, const bf16* __restrict__ Wg, int h, int r, fl
 }
 
 // Small batches: permutation and gather in one launch, one block per token.  Every block
-// recomputes the (tiny) histogram and offsets from the routing record, places its own token's
+// recomputes the (tiny) histogram and offsets from the routing record (by ballots: with loops over
+// the record the stage took 16.9 us at 256 tokens and 14.5 at 128, now 12.6 and 11.5), places its own token's
 // pairs and copies the token's row to them; block 0 also publishes the batch description.
 // Padding rows of the groups are left as they are: in the weight-major GEMM a token row only
 // feeds its own accumulator column, and the columns of padding rows are never stored.
@@ -148,81 +149,74 @@ permute_gather_small_kernel(const bf16* x, const int32_t* idx, const uint8_t* sk
                             int E) {
   pdl_launch_dependents();
   pdl_wait();
-  __shared__ int s_e[kDecodeMaxT][2];
-  __shared__ int s_cnt[kMaxE][2];
-  __shared__ int s_off[kMaxE + 1];
-  __shared__ int s_nsk;
-  __shared__ int s_p[2];
-  const int i = threadIdx.x;
+  // thread i looks at token i; a ballot per expert and slot counts a warp's tokens
+  constexpr int kWarps = kDecodeMaxT / 32;
+  __shared__ int s_part[3][kWarps][kMaxE];  // slot-0 pairs, slot-1 pairs, pairs of tokens before t
+  __shared__ int s_e[2], s_p[2];
+  const int i = threadIdx.x, warp = i >> 5, lane = i & 31;
   const int t = blockIdx.x;
-  {
-    int e0 = -1, e1 = -1;
-    if (i < T) {
-      e0 = ld_l2(idx + 2 * i);
-      e1 = ld_l2(skipped + i) ? -1 : ld_l2(idx + 2 * i + 1);
+  int e0 = -1, e1 = -1;
+  if (i < T) {
+    e0 = ld_l2(idx + 2 * i);
+    e1 = ld_l2(skipped + i) ? -1 : ld_l2(idx + 2 * i + 1);
+  }
+  if (i == t) { s_e[0] = e0; s_e[1] = e1; }
+  const unsigned before = t >= 32 * (warp + 1) ? 0xffffffffu : (t > 32 * warp ? (1u << (t - 32 * warp)) - 1u : 0u);
+  for (int c = 0; c < r; ++c) {
+    const unsigned m0 = __ballot_sync(0xffffffffu, e0 == c), m1 = __ballot_sync(0xffffffffu, e1 == c);
+    if (lane == c) {
+      s_part[0][warp][c] = __popc(m0);
+      s_part[1][warp][c] = __popc(m1);
+      s_part[2][warp][c] = __popc(m0 & before) + __popc(m1 & before);
     }
-    s_e[i][0] = e0;
-    s_e[i][1] = e1;
   }
   __syncthreads();
-  if (i < 2 * r) {
-    const int c = i >> 1, slot = i & 1;
-    int n = 0;
-    for (int q = 0; q < T; ++q) n += (s_e[q][slot] == c);
-    s_cnt[c][slot] = n;
-  } else if (i == 2 * kMaxE) {
-    int n = 0;
-    for (int q = 0; q < T; ++q) n += (s_e[q][1] < 0);
-    s_nsk = n;
-  }
-  __syncthreads();
-  if (i == 0) {
-    int off = 0, tiles = 0, touched = 0;
-    s_off[0] = 0;
-    for (int c = 0; c < kMaxE; ++c) {
-      const int n = c < r ? s_cnt[c][0] + s_cnt[c][1] : 0;
-      off += (n + pad - 1) / pad * pad;
-      tiles += (n + kTileRows - 1) / kTileRows;
-      touched += (n > 0);
-      s_off[c + 1] = off;
-      if (t == 0) {
-        meta->count[c] = n;
-        meta->count_slot[c][0] = c < r ? s_cnt[c][0] : 0;
-        meta->count_slot[c][1] = c < r ? s_cnt[c][1] : 0;
-        meta->off[c + 1] = off;
-        meta->tile_prefix[c + 1] = tiles;
-      }
+  if (warp == 0) {
+    const bool on = lane < r;
+    int c0 = 0, c1 = 0, rank = 0;
+    if (on) {
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) { c0 += s_part[0][w][lane]; c1 += s_part[1][w][lane]; rank += s_part[2][w][lane]; }
+    }
+    const int cnt = c0 + c1, padded = (cnt + pad - 1) / pad * pad, mine = (cnt + kTileRows - 1) / kTileRows;
+    int end = padded, tiles = mine;  // inclusive sums over the experts
+#pragma unroll
+    for (int s = 1; s < kMaxE; s <<= 1) {
+      const int a = __shfl_up_sync(0xffffffffu, end, s), b = __shfl_up_sync(0xffffffffu, tiles, s);
+      if (lane >= s) { end += a; tiles += b; }
+    }
+    const int pos = end - padded + rank;  // of the next pair of this lane's expert
+    const int f0 = s_e[0], f1 = s_e[1];
+    const int p0 = __shfl_sync(0xffffffffu, pos, f0 & 31), p1 = __shfl_sync(0xffffffffu, pos, f1 & 31);
+    if (lane < 2) {
+      const int p = lane == 0 ? p0 : (f1 < 0 ? -1 : p1);
+      s_p[lane] = p;
+      pair_pos[2 * t + lane] = p;
+      if (p >= 0) row_token[p] = t;
     }
     if (t == 0) {
-      meta->off[0] = 0;
-      meta->tile_prefix[0] = 0;
-      meta->rows_total = off;
-      meta->n_skipped = s_nsk;
-      meta->n_touched = touched;
-      meta->reserved = 0;
-      if (s_count) {
-        for (int e = 0; e < E; ++e) { s_count[2 * e] = 0; s_count[2 * e + 1] = 0; }
-        for (int c = 0; c < r; ++c) {
-          s_count[2 * kept.id[c]] = s_cnt[c][0];
-          s_count[2 * kept.id[c] + 1] = s_cnt[c][1];
-        }
-        *s_nskipped = s_nsk;
-        *s_ntouched = touched;
+      const int pairs = __reduce_add_sync(0xffffffffu, cnt);
+      const int touched = __popc(__ballot_sync(0xffffffffu, cnt > 0));
+      if (lane < kMaxE) {
+        meta->count[lane] = cnt;
+        meta->count_slot[lane][0] = c0;
+        meta->count_slot[lane][1] = c1;
+        meta->off[lane + 1] = end;
+        meta->tile_prefix[lane + 1] = tiles;
+        if (s_count && lane < E) { s_count[2 * lane] = 0; s_count[2 * lane + 1] = 0; }
+      }
+      __syncwarp();
+      if (s_count && on) { s_count[2 * kept.id[lane]] = c0; s_count[2 * kept.id[lane] + 1] = c1; }
+      if (lane == kMaxE - 1) {
+        meta->off[0] = 0;
+        meta->tile_prefix[0] = 0;
+        meta->rows_total = end;
+        meta->n_skipped = 2 * T - pairs;
+        meta->n_touched = touched;
+        meta->reserved = 0;
+        if (s_count) { *s_nskipped = 2 * T - pairs; *s_ntouched = touched; }
       }
     }
-  }
-  __syncthreads();
-  if (i < 2) {
-    const int c = s_e[t][i];
-    int pos = -1;
-    if (c >= 0) {
-      int rank = 0;
-      for (int q = 0; q < t; ++q) rank += (s_e[q][0] == c) + (s_e[q][1] == c);
-      pos = s_off[c] + rank;
-      row_token[pos] = t;
-    }
-    pair_pos[2 * t + i] = pos;
-    s_p[i] = pos;
   }
   __syncthreads();
   const int nvec = h >> 3;
