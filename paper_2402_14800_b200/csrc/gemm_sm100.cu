@@ -579,9 +579,10 @@ gemm_tokens_m_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args)
 //   - a k-block brings 32 KB of weights + 64 B x N of tokens to an SM: 48 KB where gemm_tokens_m
 //     moves 64 KB for the same 1024 pipe cycles (13.1 instead of 17.4 GB from L2 for both launches
 //     of 3072 tokens on 4 experts).
-// What bounds it: HBM up to about 200 tokens a group, then the tensor pipe (84 % of its cycles busy
-// in the gate/up launch at 1536 tokens a group, of which 4 % is the partly filled last round) at
-// the clock that the board's power leaves.
+// What bounds it: HBM and the traffic from L2 (about 9.5 TB/s) up to about 200 tokens a group, then
+// L2 until the tiles are full, then the tensor pipe (84 % of its cycles busy in the gate/up launch at
+// 1536 tokens a group, of which 4 % is the partly filled last round) at the clock that the board's
+// power leaves.
 // Each accumulator has an issuing warp of its own: the pipe queues little beyond the MMA it executes,
 // so whatever one warp does between two MMAs (barrier wait, commit, loop) leaves it idle unless the
 // other's MMAs fill the gap.  One warp issuing for both took 5.04 ms at 8192 tokens, two take 4.8;
@@ -666,11 +667,10 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
       : "memory");
 }
 
-constexpr int PN_NS = 4;
-constexpr int PN_A_BYTES = 256 * 128;  // this CTA's 256 weight rows x 64 bf16
-constexpr int PN_B_BYTES = 128 * 128;  // this CTA's half of the token tile (16 .. 128 rows)
-constexpr int PN_STAGE = PN_A_BYTES + PN_B_BYTES;
-constexpr int PN_SMEM = PN_NS * PN_STAGE + 1024;
+constexpr int PN_NS = 5;                // stages at most
+constexpr int PN_A_BYTES = 256 * 128;   // this CTA's 256 weight rows x 64 bf16
+constexpr int PN_B_UNIT = 16 * 128;     // this CTA's half of 32 tokens
+constexpr int PN_SMEM = 5 * (PN_A_BYTES + 6 * PN_B_UNIT) + 1024;  // 5 stages of up to 192 tokens, 4 of more
 constexpr int PN_W_ROWS = 512;         // weight rows of an item
 constexpr int PN_BAND = 16;            // at most so many token tiles sweep the weight tiles together
 constexpr int PN_EPI_WARPS = 16;
@@ -682,15 +682,47 @@ struct ItemN {
   int n, valid;       // columns of the MMA (a multiple of 32) and the tokens among them
 };
 
-// An expert's tokens are cut into as few tiles of at most 256 as hold them, of equal size up to
+// An expert's tokens are cut into as few tiles of at most 32 * cap as hold them, of equal size up to
 // the grain of 32.
-__device__ __forceinline__ int token_tiles(int cnt) { return (cnt + 255) >> 8; }
+__device__ __forceinline__ int token_tiles(int cnt, int cap) { return (((cnt + 31) >> 5) + cap - 1) / cap; }
 
-__device__ __forceinline__ void decode_item_n(const Meta& m, const GemmArgs& a, int item, int Nt, ItemN& t) {
-  int c = 0, first = 0, kt = token_tiles(m.count[0]);
+// The largest tile of a launch, in units of 32 tokens: smaller ones than need be where they fill the last
+// round better.  The model, per item of n tokens: what bounds a k-block is the traffic from L2 (64 KB of
+// weights + 128 B x n for the pair; the machine draws about 9.5 TB/s of it, so an item of 64 tokens takes
+// 0.75 of the time of one of 256, not a quarter), or HBM, 64 KB of weights for the kt tiles that share them;
+// to the rounds of items the epilogue of the last one is added.  Units: the time of 128 bytes from L2.
+// Largest tile 256 -> chosen (Mixtral layer): down launch of 1000 tokens 287 -> 259 us, of 700 tokens on 4
+// experts 170 -> 130; gate/up of 1500 tokens 594 -> 574.  The results are the same bits for every size.
+// Warp-collective: lane l tries size l % 8 + 1 for the experts l / 8, l / 8 + 4, ..; all lanes return the best.
+__device__ __forceinline__ int choose_tile_cap(const Meta& m, const GemmArgs& a, int KB, int Nt, int n_pairs) {
+  const int lane = threadIdx.x & 31, cap = (lane & 7) + 1;
+  int items = 0, work = 0;  // of one weight tile; work per k-block
+  for (int c = lane >> 3; c < a.r; c += 4) {
+    const int kt = token_tiles(m.count[c], cap);
+    if (kt == 0) continue;
+    items += kt;
+    work += max(512 * kt + m.count[c], 743);  // kt items
+  }
+#pragma unroll
+  for (int s = 8; s < 32; s <<= 1) {
+    items += __shfl_xor_sync(0xffffffffu, items, s);
+    work += __shfl_xor_sync(0xffffffffu, work, s);
+  }
+  if (items == 0) items = 1;
+  const int rounds = (items * Nt + n_pairs - 1) / n_pairs;
+  const float cost = __fdividef((float)rounds * (float)work, (float)items) * (float)KB + 20.f * 32.f * (float)cap;
+  // positive floats order like their bits; on (nearly) equal costs the larger tile
+  const unsigned best = __reduce_min_sync(0xffffffffu, (__float_as_uint(cost) & ~7u) | (unsigned)(8 - cap));
+  return 8 - (int)(best & 7u);
+}
+
+// tiles[c] = token tiles of expert c
+__device__ __forceinline__ void decode_item_n(const Meta& m, const GemmArgs& a, int item, int Nt, const int* tiles,
+                                              ItemN& t) {
+  int c = 0, first = 0, kt = tiles[0];
   while (c + 1 < a.r && item >= first + kt * Nt) {
     first += kt * Nt;
-    kt = token_tiles(m.count[++c]);
+    kt = tiles[++c];
   }
   const int local = item - first;
   const int bands = (kt + PN_BAND - 1) / PN_BAND;
@@ -763,6 +795,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ Bars bars;
   __shared__ Meta s_meta;
+  __shared__ int s_tiles[kMaxE];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();  // 0 = leader of the pair
@@ -777,17 +810,21 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
   pdl_wait();
   for (int i = threadIdx.x; i < (int)(sizeof(Meta) / 4); i += blockDim.x)
     reinterpret_cast<int32_t*>(&s_meta)[i] = ld_l2(reinterpret_cast<const int32_t*>(args.meta) + i);
-  tc_fence_before();
   __syncthreads();
+  const int KB = (args.K + BK - 1) / BK;
+  const int Nt = (args.n_w_rows + PN_W_ROWS - 1) / PN_W_ROWS;
+  const int cap = choose_tile_cap(s_meta, args, KB, Nt, n_pairs);
+  if (threadIdx.x < kMaxE) s_tiles[threadIdx.x] = token_tiles(s_meta.count[threadIdx.x], cap);
+  tc_fence_before();
   cluster_sync_all();  // both CTAs' barriers exist before anything is signalled across the pair
   tc_fence_after();
   const uint32_t tmem_base = *(volatile uint32_t*)&bars.tmem_base;
   volatile int* abort_flag = &bars.abort_flag;
 
-  const int KB = (args.K + BK - 1) / BK;
-  const int Nt = (args.n_w_rows + PN_W_ROWS - 1) / PN_W_ROWS;
+  const uint32_t stage_bytes = (uint32_t)(PN_A_BYTES + cap * PN_B_UNIT);
+  const uint32_t ns = cap <= 6 ? 5u : 4u;
   int n_items = 0;
-  for (int c = 0; c < args.r; ++c) n_items += token_tiles(s_meta.count[c]) * Nt;
+  for (int c = 0; c < args.r; ++c) n_items += s_tiles[c] * Nt;
   uint32_t issued = 0;
 
   if (warp == 0) {
@@ -797,7 +834,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
     bool ok = true;
     for (int item = pair; item < n_items && ok; item += n_pairs) {
       ItemN t;
-      decode_item_n(s_meta, args, item, Nt, t);
+      decode_item_n(s_meta, args, item, Nt, s_tiles, t);
       const int half = t.n >> 1;  // 16 .. 128 token rows, a multiple of 16
       const int w_row = t.nt * PN_W_ROWS + 256 * (int)rank;
       const int a_row = args.a_row_base + args.a_off_mul * s_meta.off[t.c] + t.tok0 + half * (int)rank;
@@ -807,7 +844,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
         if (!ok) break;
         if (lane == 0) {
           const uint32_t full = map_to_cta(smem_u32(&bars.full[s]), 0);
-          const uint32_t sa = smem_base + s * PN_STAGE;
+          const uint32_t sa = smem_base + s * stage_bytes;
           if (rank == 0) mbar_expect_tx(smem_u32(&bars.full[s]), bytes);
           tma_load_3d_pair(sa, &maps.w, kb * BK, w_row, t.c, full);
           if (half == 128) {
@@ -822,7 +859,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
               }
           }
         }
-        if (++s == PN_NS) { s = 0; ph ^= 1u; }
+        if (++s == ns) { s = 0; ph ^= 1u; }
         __syncwarp();
       }
     }
@@ -838,7 +875,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
       bool ok = true;
       for (int item = pair; item < n_items && ok; item += n_pairs, ++nu) {
         ItemN t;
-        decode_item_n(s_meta, args, item, Nt, t);
+        decode_item_n(s_meta, args, item, Nt, s_tiles, t);
         const uint32_t idesc = idesc_bf16(256, t.n);
         for (int kb = 0; kb < KB; ++kb) {
           bool ready = mbar_wait(smem_u32(&bars.full[s]), ph, abort_flag);
@@ -847,7 +884,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
           if (!ok) break;
           tc_fence_after();
           if (lane == 0) {
-            const uint32_t sa = smem_base + s * PN_STAGE;
+            const uint32_t sa = smem_base + s * stage_bytes;
             const uint64_t adesc = smem_desc_k128(sa + acc * (128 * 128)), bdesc = smem_desc_k128(sa + PN_A_BYTES);
             umma_bf16_pair(d_tmem, adesc, bdesc, idesc, kb > 0 ? 1u : 0u);
             umma_bf16_pair(d_tmem, adesc + 2, bdesc + 2, idesc, 1u);
@@ -856,7 +893,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
             umma_commit_pair(smem_u32(&bars.empty[s]));
             if (kb == KB - 1) umma_commit_pair(tmem_full);
           }
-          if (++s == PN_NS) { s = 0; ph ^= 1u; }
+          if (++s == ns) { s = 0; ph ^= 1u; }
           __syncwarp();
         }
       }
@@ -871,7 +908,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
     bool ok = true;
     for (int item = pair; item < n_items && ok; item += n_pairs, ++nu) {
       ItemN t;
-      decode_item_n(s_meta, args, item, Nt, t);
+      decode_item_n(s_meta, args, item, Nt, s_tiles, t);
       const long long orow =
           (long long)(args.out_row_base + args.out_off_mul * s_meta.off[t.c] + t.tok0) * args.out_ld +
           (long long)t.c * args.out_col_mul;
@@ -910,10 +947,10 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
   if (*abort_flag) {
     if (warp == 0 && lane == 0) {
       int dummy = 0;
-      const uint32_t n = issued < (uint32_t)PN_NS ? issued : (uint32_t)PN_NS;
+      const uint32_t n = issued < ns ? issued : ns;
       for (uint32_t i = 0; rank == 0 && i < n; ++i) {
         const uint32_t it = issued - 1 - i;
-        mbar_wait(smem_u32(&bars.full[it % PN_NS]), (it / PN_NS) & 1u, &dummy, kDrainLimitNs);
+        mbar_wait(smem_u32(&bars.full[it % ns]), (it / ns) & 1u, &dummy, kDrainLimitNs);
       }
       if (args.status) atomicExch(args.status, 1);
     }
