@@ -204,9 +204,9 @@ class MoeLayer:
             y = torch.empty_like(x)
         idx = wn = na = None
         if record:
-            idx = torch.zeros((T, max(k, 1)), dtype=torch.int32, device=x.device)
-            wn = torch.zeros((T, max(k, 1)), dtype=torch.float32, device=x.device)
-            na = torch.zeros((T,), dtype=torch.int32, device=x.device)
+            idx = torch.empty((T, max(k, 1)), dtype=torch.int32, device=x.device)
+            wn = torch.empty((T, max(k, 1)), dtype=torch.float32, device=x.device)
+            na = torch.empty((T,), dtype=torch.int32, device=x.device)
         _check(load_library().moe_forward_topk(
             self._h, x.data_ptr(), T, k, beta, y.data_ptr(),
             idx.data_ptr() if record else None, wn.data_ptr() if record else None,

@@ -244,10 +244,12 @@ void mark(moe_layer* L) {
 }
 
 // Pinned host words of the handle that kernels and copies write results to ([0] status word,
-// [1..2] selected values); null if they cannot be had.  A copy to pageable memory would be staged
-// by the runtime.
+// [1..2] selected values, [kHostLosses..] losses of a search); null if they cannot be had.  A copy to
+// pageable memory would be staged by the runtime, with a wait of its own.
+constexpr int kHostLosses = 4, kMaxHostLosses = 1020;
 int* host_words(moe_layer* L) {
-  if (!L->h_words && cudaHostAlloc((void**)&L->h_words, 4 * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+  if (!L->h_words && cudaHostAlloc((void**)&L->h_words, (kHostLosses + kMaxHostLosses) * sizeof(int),
+                                   cudaHostAllocDefault) != cudaSuccess) {
     cudaGetLastError();
     L->h_words = nullptr;
   }
@@ -630,14 +632,16 @@ int moe_forward_topk(moe_layer_t* L, const void* x, int T, int k, float beta, vo
   if ((rc = grow(L, W.k_pos, (size_t)T * k * 4))) return rc;
   if ((rc = grow(L, W.k_nact, (size_t)T * 4))) return rc;
   cudaStream_t st = L->stream;
-  const bool dec = decode_mode(T);
+  // few rows per expert: the small-batch GEMMs (not where their split-K planes would need scratch that
+  // a large batch does not have)
+  const bool few = decode_mode(T) || ((long long)k * T <= (long long)kFewRows * L->r && ksplit_for(L, T) == 1);
   const int rows_cap = rows_for(L, T, k);
   Meta* meta = (Meta*)W.meta.p;
   int32_t* idx = (int32_t*)W.k_idx.p;
   int32_t* nact = (int32_t*)W.k_nact.p;
   CUDA_TRY(launch_router_topk((const bf16*)x, L->Wg, T, L->h, L->r, k, beta, L->kept, idx,
                               (float*)W.k_wn.p, nact, idx_out, wn_out, n_active_out, nullptr, st));
-  if ((rc = permute_topk(L, (const bf16*)x, idx, nact, T, k, dec ? 16 : group_pad(L, (long long)k * T), meta,
+  if ((rc = permute_topk(L, (const bf16*)x, idx, nact, T, k, few ? 16 : group_pad(L, (long long)k * T), meta,
                          (int32_t*)W.k_pos.p, (bf16*)W.xperm.p)))
     return rc;
   GemmArgs gu, dn;
@@ -645,7 +649,7 @@ int moe_forward_topk(moe_layer_t* L, const void* x, int T, int k, float beta, vo
   memset(&dn, 0, sizeof(dn));
   gu.a_off_mul = 1; gu.out_off_mul = 1; gu.out_ld = L->f; gu.out = W.act.p;
   dn.a_off_mul = 1; dn.out_off_mul = 1; dn.out_ld = L->h; dn.out = W.O.p;
-  const bool wm = dec && !L->debug_simt;
+  const bool wm = few && !L->debug_simt;
   if (wm) {
     gu.tail = (float*)W.tail.p; dn.tail = (float*)W.tail.p;
   }
@@ -945,7 +949,7 @@ static int search_impl(moe_layer_t* L, const void* x_calib, const float* F_ref, 
   // the same operations in the same order as in a pass of its own size.
   std::vector<std::vector<uint32_t>> masks(n_r);
   for (int i = 0; i < n_r; ++i) masks[i] = subset_masks(E, rs[i]);
-  size_t o = 0;
+  size_t o = 0, mapped = 0;
   for (int i0 = 0; i0 < n_r;) {
     // sizes i0 .. i1 - 1 go through one pass (as many as the per-warp loss table has room for)
     std::vector<uint32_t> batch = masks[i0];
@@ -956,10 +960,14 @@ static int search_impl(moe_layer_t* L, const void* x_calib, const float* F_ref, 
     }
     const size_t n = batch.size();
     CUDA_TRY(cudaMemcpyAsync(W.s_subsets.p, batch.data(), n * 4, cudaMemcpyHostToDevice, st));
+    // a single short pass leaves its losses in mapped host memory, read after the one wait below
+    float* direct = i0 == 0 && i1 == n_r && n <= (size_t)kMaxHostLosses && host_words(L)
+                        ? (float*)(L->h_words + kHostLosses) : nullptr;
     CUDA_TRY(launch_enumerate((const float*)W.s_logits.p, (const bf16*)W.s_yall.p, T, E, r, h,
                               (const uint32_t*)W.s_subsets.p, (int)n, (float*)W.s_partial.p,
-                              (double*)W.s_loss_sq.p, (float*)W.s_losses.p, F_ref, src, st));
-    CUDA_TRY(cudaMemcpyAsync(losses + o, L->ws->s_losses.p, n * 4, cudaMemcpyDeviceToHost, st));
+                              (double*)W.s_loss_sq.p, direct ? direct : (float*)W.s_losses.p, F_ref, src, st));
+    if (direct) mapped = n;
+    else CUDA_TRY(cudaMemcpyAsync(losses + o, L->ws->s_losses.p, n * 4, cudaMemcpyDeviceToHost, st));
     // the host list is reused for the next pass: the copy above must have left it
     if (i1 < n_r) CUDA_TRY(cudaStreamSynchronize(st));
     o += n;
@@ -967,6 +975,7 @@ static int search_impl(moe_layer_t* L, const void* x_calib, const float* F_ref, 
   }
   mark(L);
   if ((rc = check_status(L))) return rc;
+  if (mapped) memcpy(losses, L->h_words + kHostLosses, mapped * 4);
   o = 0;
   for (int i = 0; i < n_r; ++i) {
     const size_t n = masks[i].size();

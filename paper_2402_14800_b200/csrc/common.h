@@ -27,6 +27,12 @@ constexpr int kTokensDMaxKept = 6;         // ... on layers with at most this ma
 // 6144 a group was up to 6 % slower on the pairs: with little padding to save, both are held by the
 // board's power and the pairs draw 1-3 % more energy per call.
 constexpr int kPairMaxRows = 1536;
+// Top-k calls of more than kDecodeMaxT tokens with at most this many pairs per kept expert, two thirds
+// of the weight-major kernel's token tile, run that kernel: it cuts the last round into K-slices, and hardly
+// any group needs a second tile yet.  Layer of 16 experts (h 2048, f 4096), gemm_pair_n vs weight-major,
+// whole call: 32 pairs per expert 189 vs 169 us, 62 190 vs 180, 75 201 vs 194, 83 201 vs 196; 112 217
+// vs 250, 125 216 vs 252.
+constexpr int kFewRows = 85;
 constexpr int kPairPad = 32;        // grain of its token tiles
 // Up to here every block of the permutation counts the whole routing record itself (at 32 tokens a
 // thread, in bytes, 255 tokens a thread at most); beyond, the routers' histogram and the scan do.

@@ -1722,7 +1722,9 @@ cudaError_t launch_gemm_tokens_m(bool gate_up, GemmOut out_kind, const GemmMaps&
   return launch_plain(gemm_tokens_m_kernel<false, kOutBf16>, dim3(grid), dim3(TmCfg<false>::kThreads), TM_SMEM, st, maps, a);
 }
 
-// On CTA pairs (cluster of two), in plain stream order.
+// On CTA pairs (cluster of two), as programmatic dependents: set-up, tensor-memory allocation and the
+// fetch of the tensor maps overlap the predecessor (search on the tiny layer 88 -> 78 us, tiny layer at
+// 2000 tokens 48.4 -> 43.5; equal where the launches are long).
 template <typename... KArgs, typename... Args>
 static cudaError_t launch_pair(void (*kernel)(KArgs...), cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -1730,13 +1732,15 @@ static cudaError_t launch_pair(void (*kernel)(KArgs...), cudaStream_t st, Args&&
   cfg.blockDim = dim3(PN_THREADS);
   cfg.dynamicSmemBytes = PN_SMEM;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = g_pdl_enabled ? 1 : 0;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 

@@ -15,7 +15,7 @@ namespace moe {
 
 namespace {
 
-constexpr int kTokPerWarp = 2;
+constexpr int kTokPerWarp = 1;  // a token is a chain of latencies: blocks before tokens per warp
 constexpr int kMaxBlocks = 148 * 16;
 
 __device__ __forceinline__ void unpack8f(const uint4& v, float* f) {
