@@ -390,10 +390,10 @@ def launches_per_forward(T):
     # T = 1: routing + gate/up matrix-vector kernel, down kernel with the weighted sum
     #   (with the GEMM path forced: routing, gate/up GEMM, down GEMM, combine);
     # T <= 256: router, permute+gather, gate/up GEMM, down GEMM, combine;
-    # larger T: router, scan, scatter, gather, gate/up GEMM, down GEMM, combine
+    # larger T: the same, with a scan before the permutation beyond 8192 tokens
     if T == 1:
         return 2 if single_token_gemv() else 4
-    return 5 if T <= 256 else 7
+    return 5 if T <= 8192 else 6
 
 
 def forward_case(layer, x, y, beta, workload, wname, steps, warmup, stream, dev, rank, local, world, peaks,
@@ -449,9 +449,10 @@ def forward_case(layer, x, y, beta, workload, wname, steps, warmup, stream, dev,
         dn_flop = pairs * 2 * H * F
         ach = gu_flop / (gu_ms * 1e-3) / 1e12
         step_tf = (gu_flop + dn_flop) / (ms_step * 1e-3) / 1e12
-        roofline = {"bound": "tensor", "kernel": "gemm_tokens_m_kernel<gate_up>", "achieved": ach,
+        kernel = "gemm_pair_n_kernel<gate_up>" if 2 * T <= 1536 * r_kept else "gemm_tokens_m_kernel<gate_up>"
+        roofline = {"bound": "tensor", "kernel": kernel, "achieved": ach,
                     "peak": peaks["tf_sust"], "unit": "TFLOP/s", "frac": ach / peaks["tf_sust"],
-                    "traffic": recorded_traffic(wname, "gemm_tokens_m_kernel<gate_up>"),
+                    "traffic": recorded_traffic(wname, kernel),
                     "peak_source": peaks["source"] + " (sustained bf16; these runs sit at the power cap)",
                     "frac_of_burst": ach / peaks["tf_burst"],
                     "frac_of_nominal_dense_bf16": ach / NOMINAL_BF16_TFLOPS,
@@ -510,9 +511,9 @@ def search_case(layer, x, steps, warmup, stream, dev, rank, local, world, peaks,
                 "whole_step_frac_of_burst": step_tf / peaks["tf_burst"]}
     stages = {"route_permute_ms": stage_ms[0] / n_search, "gate_up_ms": gu_ms, "down_ms": dn_ms,
               "enumerate_ms": en_ms, "searches": n_search}
-    # per chunk: route, count, scan, scatter, gather, 2 GEMMs; then enumerate + reduce per size
+    # per chunk of at most 8192 tokens: route, permute, 2 GEMMs; then one enumeration + reduction
     return dict(T=T, timing=timing, clocks=clocks, stages=stages, roofline=roofline, ms_step=ms_step,
-                launches_per_step=chunks * 7 + 2 * 2)
+                launches_per_step=chunks * 4 + 2)
 
 
 def matrix_rows(W, xcal, layers, stream, dev, rank, local, world, peaks, head, rows):
@@ -986,7 +987,7 @@ def run_stack(a):
                     "frac_of_nominal_dense_bf16": ach / NOMINAL_BF16_TFLOPS,
                     "peak_source": peaks["source"] + " (sustained bf16)"}
     if rank == 0:
-        per_layer = ((2 if single_token_gemv() else 4) if T == 1 else (5 if T <= 256 else 7)) + 1   # the layer's kernels + its RMSNorm
+        per_layer = ((2 if single_token_gemv() else 4) if T == 1 else (5 if T <= 8192 else 6)) + 1   # the layer's kernels + its RMSNorm
         line = {
             "metric": "MoE-stack tokens/s on 1 B200 (32 layers, RMSNorm + residual, attention omitted)",
             "value": value, "unit": "tokens/s", "n_gpus": world, "steps": a.steps,
