@@ -757,55 +757,55 @@ router_topk_kernel(const bf16* x, const bf16* __restrict__ Wg, int T, int h, int
   if (WS) __syncthreads();
   const int groups = (T + TB - 1) / TB;
   for (int g = blockIdx.x + gridDim.x * warp; g < groups; g += gridDim.x * kRouteWarps) {
-  const int t0 = g * TB;
-  const float mine = warp_logits<R, WS>(x, WS ? s_w : reinterpret_cast<const uint4*>(Wg), t0, T, h, r, ring);
-  const int i = lane / kLanes / RP, c = lane / kLanes % RP;
-  int rank = 0;
-  float top = -INFINITY;
-  for (int d = 0; d < r; ++d) {
-    const float o = __shfl_sync(0xffffffffu, mine, (i * RP + d) * kLanes);
-    rank += (o > mine) || (o == mine && d < c);
-    top = d == 0 || o > top ? o : top;
-  }
-  if (lane % kLanes == 0) {  // logits that compare with nothing (NaN) leave ranks unclaimed: name some expert
-    s_sel[warp][i][c] = min(c, r - 1);
-    s_p[warp][i][c] = 0.f;
-  }
-  __syncwarp();
-  if (c < r && lane % kLanes == 0) {
-    if (logits && t0 + i < T) logits[(size_t)(t0 + i) * r + c] = mine;
-    if (rank < k) {
-      s_sel[warp][i][rank] = c;
-      s_p[warp][i][rank] = expf(mine - top);
+    const int t0 = g * TB;
+    const float mine = warp_logits<R, WS>(x, WS ? s_w : reinterpret_cast<const uint4*>(Wg), t0, T, h, r, ring);
+    const int i = lane / kLanes / RP, c = lane / kLanes % RP;
+    int rank = 0;
+    float top = -INFINITY;
+    for (int d = 0; d < r; ++d) {
+      const float o = __shfl_sync(0xffffffffu, mine, (i * RP + d) * kLanes);
+      rank += (o > mine) || (o == mine && d < c);
+      top = d == 0 || o > top ? o : top;
     }
-  }
-  __syncwarp();
-  const int t = t0 + lane;
-  if (lane < TB && t < T) {
-  const float* p = s_p[warp][lane];
-  const int* sel = s_sel[warp][lane];
-  // i* = the smallest i in 1..k whose dropped mass p_i + .. + p_{k-1} (added from the smallest
-  // value upwards) is at most beta times the whole mass p_0 + .. + p_{k-1} (added in rank order)
-  float whole = 0.f;
-  for (int m = 0; m < k; ++m) whole += p[m];
-  const float bound = beta * whole;
-  float dropped = 0.f;  // mass beyond rank istar - 1, for istar = k, k - 1, ..: walk down while it fits
-  int istar = k;
-  while (istar > 1 && dropped + p[istar - 1] <= bound) { dropped += p[istar - 1]; --istar; }
-  float kept_mass = 0.f;
-  for (int m = 0; m < istar; ++m) kept_mass += p[m];
-  for (int m = 0; m < k; ++m) {
-    const float w = m < istar ? p[m] / kept_mass : 0.f;
-    const int e = sel[m];
-    idx[(size_t)t * k + m] = e;
-    wn[(size_t)t * k + m] = w;
-    if (u_idx) u_idx[(size_t)t * k + m] = kept.id[e];
-    if (u_wn) u_wn[(size_t)t * k + m] = w;
-  }
-  nact[t] = istar;
-  if (u_nact) u_nact[t] = istar;
-  }
-  __syncwarp();
+    if (lane % kLanes == 0) {  // logits that compare with nothing (NaN) leave ranks unclaimed: name some expert
+      s_sel[warp][i][c] = min(c, r - 1);
+      s_p[warp][i][c] = 0.f;
+    }
+    __syncwarp();
+    if (c < r && lane % kLanes == 0) {
+      if (logits && t0 + i < T) logits[(size_t)(t0 + i) * r + c] = mine;
+      if (rank < k) {
+        s_sel[warp][i][rank] = c;
+        s_p[warp][i][rank] = expf(mine - top);
+      }
+    }
+    __syncwarp();
+    const int t = t0 + lane;
+    if (lane < TB && t < T) {
+      const float* p = s_p[warp][lane];
+      const int* sel = s_sel[warp][lane];
+      // i* = the smallest i in 1..k whose dropped mass p_i + .. + p_{k-1} (added from the smallest
+      // value upwards) is at most beta times the whole mass p_0 + .. + p_{k-1} (added in rank order)
+      float whole = 0.f;
+      for (int m = 0; m < k; ++m) whole += p[m];
+      const float bound = beta * whole;
+      float dropped = 0.f;  // mass beyond rank istar - 1, for istar = k, k - 1, ..: walk down while it fits
+      int istar = k;
+      while (istar > 1 && dropped + p[istar - 1] <= bound) { dropped += p[istar - 1]; --istar; }
+      float kept_mass = 0.f;
+      for (int m = 0; m < istar; ++m) kept_mass += p[m];
+      for (int m = 0; m < k; ++m) {
+        const float w = m < istar ? p[m] / kept_mass : 0.f;
+        const int e = sel[m];
+        idx[(size_t)t * k + m] = e;
+        wn[(size_t)t * k + m] = w;
+        if (u_idx) u_idx[(size_t)t * k + m] = kept.id[e];
+        if (u_wn) u_wn[(size_t)t * k + m] = w;
+      }
+      nact[t] = istar;
+      if (u_nact) u_nact[t] = istar;
+    }
+    __syncwarp();
   }
 }
 
