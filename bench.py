@@ -8,8 +8,10 @@ One step = one pass of the whole hot path (router, permutation, both grouped GEM
 or the pruning search) over one batch of seeded synthetic tokens at the Mixtral-8x7B layer
 shape.  Prints ONE JSON line.  The timed region is R blocks of exactly --steps steps (median
 block reported, best beside it).  The default run (decode, T = 128, all experts, beta = 0, one
-GPU) also measures the other configured workloads afterwards and reports them under "matrix":
-decode at other batch sizes and on pruned layers, prefill with skipping off and on, the search.  With N > 1 (launched by torch.distributed.run) every rank runs
+GPU) also measures the other configured workloads afterwards (decode at other batch sizes and on
+pruned layers, prefill with skipping off and on, the search) and prints them to standard error,
+one JSON object per line, so that the line on standard output stays short enough to be read back
+by tools that keep only the end of it; --matrix-out FILE writes them to a file as well.  With N > 1 (launched by torch.distributed.run) every rank runs
 an independent replica on its own GPU: the path has no exchange step, so no collective sits
 on the data path; timing is the max over ranks.
 """
@@ -679,6 +681,16 @@ def stack_matrix_rows(stream, dev, rank, local, world, peaks, n_layers=32, T=16,
     return rows
 
 
+def report_matrix(rows, path):
+    """The rows of the other workloads: one JSON object per line on standard error, and in a file."""
+    text = "".join(json.dumps(r) + "\n" for r in rows)
+    sys.stderr.write(text)
+    sys.stderr.flush()
+    if path:
+        with open(path, "w") as f:
+            f.write(text)
+
+
 def run_ours(a):
     from paper_2402_14800_b200 import binding, build
     rank, world, local = dist_env()
@@ -817,8 +829,9 @@ def run_ours(a):
         if baselines:
             line["pruning_baselines"] = baselines
         if matrix is not None:
-            line["matrix"] = matrix
-            line["matrix_wall_s"] = matrix_s
+            line["matrix_rows"] = len(matrix)
+            line["matrix_wall_s"] = round(matrix_s, 1)
+            report_matrix(matrix, a.matrix_out)
         print(json.dumps(line), flush=True)
     layer.close()
     if world > 1:
@@ -1039,6 +1052,7 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-matrix", dest="matrix", action="store_false",
                     help="headline workload only (the default decode run also measures the other configured workloads)")
+    ap.add_argument("--matrix-out", default=None, help="also write the rows of the other workloads to this file")
     ap.add_argument("--min-repeats", type=int, default=30,
                     help="blocks of --steps steps in the timed region at least (1 with --target-seconds 0 for a profiler)")
     ap.add_argument("--no-stack-rows", dest="stack_rows", action="store_false",

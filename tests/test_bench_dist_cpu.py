@@ -64,3 +64,15 @@ def test_reference_arm_non_zero_rank_exits_without_work():
     r = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference", "--gpus", "2"],
                        capture_output=True, text=True, env=env, timeout=120)
     assert r.returncode == 0 and r.stdout.strip() == ""
+
+
+def test_rows_of_the_other_workloads_stay_out_of_the_headline_line(tmp_path, capsys):
+    # standard output carries one short line; the rows go to standard error and to --matrix-out
+    import json
+    import bench
+    rows = [{"workload": "w%d" % i, "ms_per_step": 0.5 * i} for i in range(3)]
+    bench.report_matrix(rows, str(tmp_path / "rows"))
+    said = capsys.readouterr()
+    assert said.out == ""
+    assert [json.loads(l) for l in said.err.splitlines()] == rows
+    assert [json.loads(l) for l in open(tmp_path / "rows")] == rows
