@@ -238,7 +238,13 @@ permute_gather_small_kernel(const bf16* x, const int32_t* idx, const uint8_t* sk
 // the lanes, whatever the batch and the tokens beside it.
 //   - The router rows are copied to shared memory once per block, before the wait for the
 //     predecessor (they never change), where they fit beside the ring: read through L1 they cost a
-//     chain of L2 round trips per slice, 62 us for 611 tokens.
+//     chain of L2 round trips per slice, 62 us for 611 tokens.  Longer rows (from h = 5824 on with 8
+//     experts) pass through the same memory in two halves of as many columns as fit: while the warps
+//     of the block work on one, all threads fetch the next into the other, with the token slices'
+//     groups.  The block then walks its tokens in step, a barrier per part; the sums are the same.
+//     (Read through L1 instead: layer of 16 experts, h 6144, f 512, whole forward of 300 tokens 138 us
+//     against 121, of 16384 tokens 1324 against 1282; and rows that a caller has just written may not be
+//     read that way at all, see the rule beside launch_pdl.)
 //   - The token rows come through a ring of kRouteStages slices per warp, filled with cp.async.cg
 //     (which reads at L2, as the rule beside launch_pdl asks): a lane copies exactly the bytes it
 //     will use itself, so no barrier is needed, and the loads in flight cost no registers.
@@ -302,20 +308,38 @@ template <int R> struct RouteCfg {
 };
 constexpr size_t kRouteSmemMax = 227 * 1024 - 8 * 1024;  // dynamic part; the records are static
 
-// Copies the r router rows behind the ring.  Every thread of the block calls it, then a barrier.
-__device__ __forceinline__ void stage_router_rows(uint4* s_w, const bf16* __restrict__ Wg, int n) {
-  const uint4* src = reinterpret_cast<const uint4*>(Wg);
-  for (int i = threadIdx.x; i < n; i += 32 * kRouteWarps) cp_async16(s_w + i, src + i);
-  cp_async_commit();
-  cp_async_wait<0>();
+// 16-byte vectors of a router row that shared memory holds at a time: the whole row, or a part of it (a
+// whole number of slices; at least 9 for every R) of which two fit.
+template <int R> inline int route_part(int h, int r) {
+  const size_t room = kRouteSmemMax - RouteCfg<R>::kRingBytes;
+  if ((size_t)r * h * 2 <= room) return h >> 3;
+  return (int)(room / 2 / ((size_t)r * 512)) * 32;
+}
+
+// Starts the copy of vectors v0 .. of the r router rows, at most `part` of each, to dst[row][part]
+// (WHOLE: of the whole rows, which lie one after the other).  Every thread of the block calls it.
+template <bool WHOLE>
+__device__ __forceinline__ void fetch_router_part(uint4* dst, const bf16* Wg, int v0, int part, int nvec, int r) {
+  const uint4* src = reinterpret_cast<const uint4*>(Wg) + v0;
+  if (WHOLE) {
+    for (int i = threadIdx.x; i < r * nvec; i += 32 * kRouteWarps) cp_async16(dst + i, src + i);
+    return;
+  }
+  const int len = min(part, nvec - v0);
+  for (int c = 0; c < r; ++c)
+    for (int i = threadIdx.x; i < len; i += 32 * kRouteWarps) cp_async16(dst + c * part + i, src + (size_t)c * nvec + i);
 }
 
 // Logits of this warp's tokens t0 .. t0 + TB - 1 (tokens past the end repeat the last): lane l
 // returns the one of token q / RP and expert q % RP, q = l / (32 / N); experts beyond r repeat the
-// last.  WS: w = the rows in shared memory, else in global memory.
-template <int R, bool WS>
-__device__ __forceinline__ float warp_logits(const bf16* x, const uint4* __restrict__ w, int t0, int T, int h,
-                                             int r, uint4* ring) {
+// last.  WHOLE: s_w holds the router rows [r][nvec].  Otherwise it holds two parts [2][r][part], the
+// first of which is in `half` or on its way there, and all warps of the block call this together, those
+// that have no tokens (t0 >= T) to fetch their shares of the parts; the first part comes round again
+// behind the last one, for the next call.
+template <int R, bool WHOLE>
+__device__ __forceinline__ float warp_logits(const bf16* x, uint4* s_w, const bf16* Wg, int part, int& half,
+                                             int t0, int T, int h, int r, uint4* ring) {
+  const bool on = WHOLE || t0 < T;
   constexpr int RP = RouteCfg<R>::kRP, TB = RouteCfg<R>::kTB, N = RouteCfg<R>::kN;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nvec = h >> 3;
@@ -329,7 +353,7 @@ __device__ __forceinline__ float warp_logits(const bf16* x, const uint4* __restr
   for (int i = 0; i < TB; ++i) xr[i] = reinterpret_cast<const uint4*>(x + (size_t)min(t0 + i, T - 1) * h) + lane;
   uint4* mine = ring + warp * (kRouteStages * TB * 32) + lane;  // [stage][token][lane]
   auto fetch = [&](int v, int s) {  // slice v / 32 into stage s
-    if (v + lane < nvec) {
+    if (on && v + lane < nvec) {
 #pragma unroll
       for (int i = 0; i < TB; ++i) cp_async16(mine + (s * TB + i) * 32, xr[i] + v);
     }
@@ -337,10 +361,24 @@ __device__ __forceinline__ float warp_logits(const bf16* x, const uint4* __restr
   };
 #pragma unroll
   for (int s = 0; s < kRouteStages - 1; ++s) fetch(32 * s, s);
-  int s = 0;
+  int s = 0, left = 0;  // vectors of the present part still to come
+  const uint4* w = s_w + lane;
 #pragma unroll 1
-  for (int v = 0; v < nvec; v += 32) {
+  for (int v = 0; v < nvec; v += 32, left -= 32) {
     cp_async_wait<kRouteStages - 2>();
+    if (!WHOLE && left <= 0) {
+      // this part was fetched with or before a token slice that has arrived; no warp reads the other half now
+      __syncthreads();
+      w = s_w + half * r * part + lane - v;
+      half ^= 1;
+      left = part;
+      const int next = v + part < nvec ? v + part : 0;
+      fetch_router_part<WHOLE>(s_w + half * r * part, Wg, next, part, nvec, r);  // committed with the slice below
+    }
+    if (!on) {
+      cp_async_commit();
+      continue;
+    }
     uint64_t xf[TB / 2][8];
 #pragma unroll
     for (int i = 0; i < TB / 2; ++i) {
@@ -352,15 +390,12 @@ __device__ __forceinline__ float warp_logits(const bf16* x, const uint4* __restr
     }
     fetch(v + 32 * (kRouteStages - 1), s == 0 ? kRouteStages - 1 : s - 1);
     if (v + lane < nvec) {
-      constexpr int kBatch = WS ? 2 : (R < 4 ? R : 4);  // router slices in flight
+      constexpr int kBatch = 2;  // router slices in flight
 #pragma unroll
       for (int c0 = 0; c0 < R; c0 += kBatch) {
         uint4 wv[kBatch];
 #pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-          const uint4* row = w + (size_t)min(c0 + b, r - 1) * nvec + v + lane;
-          wv[b] = WS ? *row : __ldg(row);
-        }
+        for (int b = 0; b < kBatch; ++b) wv[b] = w[(size_t)min(c0 + b, r - 1) * (WHOLE ? nvec : part) + v];
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
           if (c0 + b < R) {
@@ -388,9 +423,9 @@ __device__ __forceinline__ float warp_logits(const bf16* x, const uint4* __restr
 }
 
 // Top-2 routing.
-template <int R, bool WS>
+template <int R, bool WHOLE>
 __global__ void __launch_bounds__(32 * kRouteWarps, 1)
-router_kernel(const bf16* x, const bf16* __restrict__ Wg, int T, int h, int r, float beta, KeptIds kept,
+router_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part, float beta, KeptIds kept,
               RouteOut o, bool w_const) {
   pdl_launch_dependents();
   using Cfg = RouteCfg<R>;
@@ -401,14 +436,21 @@ router_kernel(const bf16* x, const bf16* __restrict__ Wg, int T, int h, int r, f
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int team = warp / Cfg::kTeamWarps, tw = warp % Cfg::kTeamWarps;
   uint4* s_w = ring + Cfg::kRingBytes / 16;
-  if (WS && w_const) stage_router_rows(s_w, Wg, r * (h >> 3));
+  if (w_const) fetch_router_part<WHOLE>(s_w, Wg, 0, part, h >> 3, r);
   pdl_wait();
-  if (WS && !w_const) stage_router_rows(s_w, Wg, r * (h >> 3));
-  if (WS) __syncthreads();
+  if (!w_const) fetch_router_part<WHOLE>(s_w, Wg, 0, part, h >> 3, r);
+  cp_async_commit();
+  if (WHOLE) {
+    cp_async_wait<0>();
+    __syncthreads();
+  }
   const int units = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;
-  for (int u = blockIdx.x + gridDim.x * team; u < units; u += gridDim.x * Cfg::kTeams) {
+  int half = 0;
+  // with the rows in parts all warps of the block stay in step: a team goes on while the first has a unit
+  for (int u = blockIdx.x + gridDim.x * team; u - (WHOLE ? 0 : (int)gridDim.x * team) < units; u += gridDim.x * Cfg::kTeams) {
     const int t0 = u * kRouteTokPerBlock;
-    const float mine = warp_logits<R, WS>(x, WS ? s_w : reinterpret_cast<const uint4*>(Wg), t0 + tw * TB, T, h, r, ring);
+    const float mine = warp_logits<R, WHOLE>(x, s_w, Wg, part, half, t0 + tw * TB, T, h, r, ring);
+    if (!WHOLE && u >= units) continue;
     if (lane % (32 / N) == 0) s_l[warp][lane / (32 / N)] = mine;
     __syncwarp();
     const int i = tw * TB + lane, t = t0 + i;
@@ -441,6 +483,7 @@ router_kernel(const bf16* x, const bf16* __restrict__ Wg, int T, int h, int r, f
     }
     asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kTeamThreads) : "memory");
   }
+  if (!WHOLE) cp_async_wait<0>();  // the first part, fetched once more behind the last
 }
 
 // ---------------------------------------------------------------------------------- scan
@@ -738,10 +781,10 @@ combine_kernel(const float* O, int ksplit, size_t split_stride, const int32_t* p
 // Ranking by counting, one lane per (token, kept expert): the rank of expert c is the number of kept
 // experts that beat it (larger logit, or equal logit and lower index), so the expert of rank m is
 // the m-th choice; the three sums are one lane's per token (k <= 16 values).
-template <int R, bool WS>
+template <int R, bool WHOLE>
 __global__ void __launch_bounds__(32 * kRouteWarps, 1)
-router_topk_kernel(const bf16* x, const bf16* __restrict__ Wg, int T, int h, int r, int k, float beta,
-                   KeptIds kept, int32_t* __restrict__ idx, float* __restrict__ wn, int32_t* __restrict__ nact,
+router_topk_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part, int k, float beta, KeptIds kept,
+                   int32_t* __restrict__ idx, float* __restrict__ wn, int32_t* __restrict__ nact,
                    int32_t* u_idx, float* u_wn, int32_t* u_nact, float* logits) {
   pdl_launch_dependents();
   using Cfg = RouteCfg<R>;
@@ -752,13 +795,19 @@ router_topk_kernel(const bf16* x, const bf16* __restrict__ Wg, int T, int h, int
   __shared__ int s_sel[kRouteWarps][TB][RP];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint4* s_w = ring + Cfg::kRingBytes / 16;
-  if (WS) stage_router_rows(s_w, Wg, r * (h >> 3));
+  fetch_router_part<WHOLE>(s_w, Wg, 0, part, h >> 3, r);
+  cp_async_commit();
   pdl_wait();
-  if (WS) __syncthreads();
+  if (WHOLE) {
+    cp_async_wait<0>();
+    __syncthreads();
+  }
   const int groups = (T + TB - 1) / TB;
-  for (int g = blockIdx.x + gridDim.x * warp; g < groups; g += gridDim.x * kRouteWarps) {
+  int half = 0;
+  for (int g = blockIdx.x + gridDim.x * warp; g - (WHOLE ? 0 : (int)gridDim.x * warp) < groups; g += gridDim.x * kRouteWarps) {
     const int t0 = g * TB;
-    const float mine = warp_logits<R, WS>(x, WS ? s_w : reinterpret_cast<const uint4*>(Wg), t0, T, h, r, ring);
+    const float mine = warp_logits<R, WHOLE>(x, s_w, Wg, part, half, t0, T, h, r, ring);
+    if (!WHOLE && g >= groups) continue;
     const int i = lane / kLanes / RP, c = lane / kLanes % RP;
     int rank = 0;
     float top = -INFINITY;
@@ -807,6 +856,7 @@ router_topk_kernel(const bf16* x, const bf16* __restrict__ Wg, int T, int h, int
     }
     __syncwarp();
   }
+  if (!WHOLE) cp_async_wait<0>();  // the first part, fetched once more behind the last
 }
 
 // Per block of kRouteTokPerBlock tokens: active pairs per expert, in the column layout scan_kernel reads
@@ -1121,14 +1171,14 @@ static cudaError_t launch_route(void (*kernel)(KArgs...), int work, size_t smem,
 
 cudaError_t launch_router(const bf16* x, const bf16* Wg, int T, int h, int r, float beta,
                           const KeptIds& kept, const RouteOut& out, cudaStream_t st, bool w_const) {
-  const size_t w_bytes = (size_t)r * h * 2;
 #define MOE_ROUTER(R)                                                                                          \
   {                                                                                                            \
-    const bool ws = RouteCfg<R>::kRingBytes + w_bytes <= kRouteSmemMax;                                        \
-    const size_t smem = RouteCfg<R>::kRingBytes + (ws ? w_bytes : 0);                                          \
+    const int part = route_part<R>(h, r);                                                                      \
+    const bool whole = part == (h >> 3);                                                                       \
+    const size_t smem = RouteCfg<R>::kRingBytes + (size_t)(whole ? 1 : 2) * r * part * 16;                     \
     const int units = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;                                         \
-    return launch_route(ws ? router_kernel<R, true> : router_kernel<R, false>, units, smem, st, x, Wg, T, h, r, \
-                        beta, kept, out, w_const);                                                             \
+    return launch_route(whole ? router_kernel<R, true> : router_kernel<R, false>, units, smem, st, x, Wg, T, h, \
+                        r, part, beta, kept, out, w_const);                                                    \
   }
   switch (r) {
     case 2: MOE_ROUTER(2)
@@ -1212,14 +1262,14 @@ cudaError_t launch_router_topk(const bf16* x, const bf16* Wg, int T, int h, int 
                                const KeptIds& kept, int32_t* idx, float* wn, int32_t* nact,
                                int32_t* u_idx, float* u_wn, int32_t* u_nact, float* logits,
                                cudaStream_t st) {
-  const size_t w_bytes = (size_t)r * h * 2;
 #define MOE_ROUTER_TOPK(R)                                                                                   \
   {                                                                                                          \
-    const bool ws = RouteCfg<R>::kRingBytes + w_bytes <= kRouteSmemMax;                                      \
-    const size_t smem = RouteCfg<R>::kRingBytes + (ws ? w_bytes : 0);                                        \
+    const int part = route_part<R>(h, r);                                                                    \
+    const bool whole = part == (h >> 3);                                                                     \
+    const size_t smem = RouteCfg<R>::kRingBytes + (size_t)(whole ? 1 : 2) * r * part * 16;                   \
     const int groups = (T + RouteCfg<R>::kTB - 1) / RouteCfg<R>::kTB;                                        \
-    return launch_route(ws ? router_topk_kernel<R, true> : router_topk_kernel<R, false>, groups, smem, st, x, Wg, \
-                        T, h, r, k, beta, kept, idx, wn, nact, u_idx, u_wn, u_nact, logits);                 \
+    return launch_route(whole ? router_topk_kernel<R, true> : router_topk_kernel<R, false>, groups, smem, st, x, \
+                        Wg, T, h, r, part, k, beta, kept, idx, wn, nact, u_idx, u_wn, u_nact, logits);       \
   }
   switch (r) {
     case 2: MOE_ROUTER_TOPK(2)

@@ -392,3 +392,65 @@ def test_calibrated_beta_is_the_exact_median_of_the_ratios(weights, T, distinct)
     # up to 256 tokens forward adds its logits in another order: a few units in the last place
     assert abs(got - want) <= (2e-6 if T <= 256 else 0.0)
     layer.close()
+
+
+def wide_router_layer(h, offset, narrow, f=64):
+    """A layer of width h whose router rows are zero but for `narrow`'s columns, from column `offset` on."""
+    E, hn = narrow.shape
+    W = synth.make_layer_weights(h, f, E, seed=21, device=DEV)
+    Wg = torch.zeros_like(W.W_gate)
+    Wg[:, offset:offset + hn] = narrow
+    return binding.MoeLayer(Wg, W.W1, W.W3, W.W2), Wg
+
+
+@pytest.mark.parametrize("E", [3, 5, 8, 16])
+@pytest.mark.parametrize("T", [5, 300, 10000])
+def test_router_rows_longer_than_shared_memory(E, T):
+    # rows of 16384 columns (2 to 8 parts) that are zero but for 1024 columns: a lane's chain of
+    # multiply-adds is that of a layer of 1024 columns with zeros added before and behind, so the
+    # weights are the same bits wherever the columns lie (first part, across parts, last part).
+    # 10000 tokens are several rounds of a block, whose first part then comes round again.
+    build.build()
+    hn, h, k = 1024, 16384, 3 if T <= 300 else 2
+    Wn = synth.make_layer_weights(hn, 64, E, seed=20, device=DEV)
+    ref = binding.MoeLayer(Wn.W_gate, Wn.W1, Wn.W3, Wn.W2)
+    xn = synth.make_tokens(T, hn, seed=22, device=DEV)
+    want = ref.forward_topk(xn, k, 0.1, record=True)[1:]
+    beta = ref.calibrate_beta(xn)
+    x = torch.ones((T, h), dtype=torch.bfloat16, device=DEV)
+    for offset in (0, 2304, 8192 - 512, h - hn):
+        layer, Wg = wide_router_layer(h, offset, Wn.W_gate)
+        x[:, offset:offset + hn] = xn
+        got = layer.forward_topk(x, k, 0.1, record=True)[1:]
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
+        if T == 300:
+            s, sn = binding.RoutingStats(T, E, DEV), binding.RoutingStats(T, E, DEV)
+            layer.forward(x, 0.5, stats=s)
+            ref.forward(xn, 0.5, stats=sn)
+            for name in ("idx", "wn", "ratio", "skipped", "count"):
+                assert torch.equal(getattr(s, name), getattr(sn, name))
+        assert layer.calibrate_beta(x) == beta
+        assert binding.calibrate_beta_noalloc(Wg, x) == beta
+        x[:, offset:offset + hn] = 1.0
+        assert layer.device_status() == 0
+        layer.close()
+    ref.close()
+
+
+def test_allocation_free_calibration_reads_rows_written_just_before(weights):
+    # the router rows are the caller's: here a kernel of the stream, which lets its dependents start
+    # early, writes other ones before every call; widths on both sides of the shared memory
+    for h in (4096, 8192):
+        x = synth.make_tokens(500, h, seed=30, device=DEV)
+        rows = torch.empty((8, h), dtype=torch.bfloat16, device=DEV)
+        src = [synth.make_layer_weights(h, 64, 8, seed=31 + i, device=DEV).W_gate for i in range(6)]
+        want = []
+        for w in src:
+            binding.rmsnorm(w, out=rows)
+            torch.cuda.synchronize()
+            want.append(binding.calibrate_beta_noalloc(rows, x))
+        assert len(set(want)) == len(want)
+        for i in list(range(6)) * 4:
+            binding.rmsnorm(src[i], out=rows)
+            assert binding.calibrate_beta_noalloc(rows, x) == want[i]
