@@ -388,7 +388,11 @@ int forward_impl(moe_layer* L, const void* x, int T, float beta, const void* res
   } else {
     const bool own = T <= kPermuteOwnT;
     if (own) ro.blk_hist = nullptr;
-    CUDA_TRY(launch_router((const bf16*)x, L->Wg, T, L->h, L->r, beta, L->kept, ro, st));
+    if (L->debug_simt || T < kRouterTcT || L->h < kRouterTcH)
+      CUDA_TRY(launch_router((const bf16*)x, L->Wg, T, L->h, L->r, beta, L->kept, ro, st));
+    else
+      CUDA_TRY(launch_router_tc((const bf16*)x, L->Wg, T, L->h, L->r, beta, L->kept, ro,
+                                (int*)L->ws->status.p, st));
     if (!own)
       CUDA_TRY(launch_scan(ro.blk_hist, nblk, L->r, group_pad(L, 2ll * T), (int32_t*)L->ws->blk_base.p, meta,
                            s_count, s_nsk, s_nt, L->kept, L->E, st));
@@ -501,7 +505,7 @@ moe_layer_t* moe_layer_create(const void* W_gate, const void* W1, const void* W3
   const char* dense = getenv("MOE_SEARCH_DENSE");
   L->search_dense = dense && dense[0] == '1';
 
-  // the router rows are stored padded with zero rows to kMaxE rows
+  // the router rows are padded with zero rows to kMaxE rows (the tensor-core router's operand)
   const size_t n_gate = (size_t)kMaxE * h * 2, n_13 = (size_t)L->r * 2 * f * h * 2,
                n_2 = (size_t)L->r * h * f * 2;
   size_t free_b = 0;

@@ -1,7 +1,8 @@
 // Router, token permutation, combine and the small element-wise kernels.
 //
 //   router_kernel   Sec. 3.1 (logits, softmax, top-2, Eq. 1), Sec. 3.2 (kept experts only),
-//                   Sec. 3.3 (skip test), App. A.2 (weight 1 after a skip); warp per token.
+//                   Sec. 3.3 (skip test), App. A.2 (weight 1 after a skip); several tokens per warp
+//                   (large forward batches: router_tc_kernel, on the tensor cores).
 //   scan / permute  stable counting sort of the token-expert pairs that run, by expert (no atomics,
 //                   the order is a function of the routing alone), and the copy of the routed rows
 //                   of x into that order.

@@ -454,3 +454,33 @@ def test_allocation_free_calibration_reads_rows_written_just_before(weights):
         for i in list(range(6)) * 4:
             binding.rmsnorm(src[i], out=rows)
             assert binding.calibrate_beta_noalloc(rows, x) == want[i]
+
+
+@pytest.mark.parametrize("h", [4096, 8192])
+@pytest.mark.parametrize("call", ["forward_8192"])
+def test_routing_weights_against_64_bits(h, call):
+    # A logit of 2 to 4 rounded to fp32 is off by up to 1.2e-7, and what else the weights lose depends on
+    # how long the chains of the sum are: 1.2e-7 to 1.4e-7 (2-norm over the batch) with chains of up to 32
+    # products, 1.5e-7 and 2.0e-7 with one chain of h / 32 per lane.
+    build.build()
+    got_err = []
+    for seed in range(3):
+        W = synth.make_layer_weights(h, 64, 8, seed=50 + seed, device=DEV)
+        layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
+        T = 8192 if call == "forward_8192" else 333
+        x = synth.make_tokens(T, h, seed=90 + seed, device=DEV)
+        ranked = (x.double() @ W.W_gate.double().T).sort(dim=1, descending=True)
+        if call == "forward_8192":
+            k, stats = 2, binding.RoutingStats(T, 8, DEV)
+            layer.forward(x, 0.0, stats=stats)
+            idx, wn = stats.idx, stats.wn
+        else:
+            k = 4
+            _, idx, wn, _ = layer.forward_topk(x, k, 0.0, record=True)
+        same = (idx.long() == ranked.indices[:, :k]).all(1)
+        assert same.float().mean() > 0.99
+        p = torch.softmax(ranked.values[same, :k], 1)
+        got_err.append(float((wn[same].double() - p).norm() / p.norm()))
+        assert layer.device_status() == 0
+        layer.close()
+    assert np.mean(got_err) < 1.45e-7, got_err
