@@ -236,10 +236,10 @@ permute_gather_small_kernel(const bf16* x, const int32_t* idx, const uint8_t* sk
 // same 8-element slices of the TB rows and of the router rows, so a slice of a router row is read
 // and unpacked once for TB tokens; the products of two tokens go through one fma.rn.f32x2.  A logit
 // is one chain of fused multiply-adds per lane (slices, then elements, in order) and a butterfly over
-// the lanes, whatever the batch and the tokens beside it.
+// the lanes (top-k: shorter chains, see FOLD), whatever the batch and the tokens beside it.
 //   - The router rows are copied to shared memory once per block, before the wait for the
 //     predecessor (they never change), where they fit beside the ring: read through L1 they cost a
-//     chain of L2 round trips per slice, 62 us for 611 tokens.  Longer rows (from h = 5824 on with 8
+//     chain of L2 round trips per slice, 62 us for 611 tokens.  Longer rows (beyond h = 5824 with 8
 //     experts) pass through the same memory in two halves of as many columns as fit: while the warps
 //     of the block work on one, all threads fetch the next into the other, with the token slices'
 //     groups.  The block then walks its tokens in step, a barrier per part; the sums are the same.
@@ -252,7 +252,7 @@ permute_gather_small_kernel(const bf16* x, const int32_t* idx, const uint8_t* sk
 // Bound by the issue slots of the fp32 work and, beside them, the shared-memory port; 134 MB of token
 // rows at 16384 tokens take 20 us to stream.  Router launch, before (one warp per token, router rows
 // through L1; a tensor-core kernel from 8192 tokens on: 33 us at 8192) -> after: 611 tokens 19.4 ->
-// 10.3 us, 4000 26.7 -> 14.9, 16384 88.9 -> 40.2; top-k, 8192 tokens, 8 experts 73.9 -> 25.3 us.
+// 10.3 us, 4000 26.7 -> 14.9, 16384 88.9 -> 40.2.
 __device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
   uint64_t d;
   asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
@@ -260,6 +260,9 @@ __device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
 }
 __device__ __forceinline__ void fma_f32x2(uint64_t& acc, uint64_t a, uint64_t b) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ void add_f32x2(uint64_t& acc, uint64_t a) {
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc) : "l"(a));
 }
 __device__ __forceinline__ void split_f32x2(uint64_t v, float& lo, float& hi) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
@@ -299,9 +302,9 @@ __device__ __forceinline__ float reduce_scatter(const float (&v)[N], int lane) {
 // a block of 16 warps is several teams, and the blocks go round until the tokens are done.
 constexpr int kRouteStages = 4;
 constexpr int kRouteWarps = 16;
-template <int R> struct RouteCfg {
+template <int R, bool FOLD> struct RouteCfg {
   static constexpr int kRP = R <= 2 ? 2 : (R <= 4 ? 4 : (R <= 8 ? 8 : 16));
-  static constexpr int kTB = R <= 8 ? 4 : 2;
+  static constexpr int kTB = R <= 8 && !FOLD ? 4 : 2;
   static constexpr int kN = kRP * kTB;
   static constexpr int kTeamWarps = kRouteTokPerBlock / kTB;
   static constexpr int kTeams = kRouteWarps / kTeamWarps;
@@ -311,8 +314,8 @@ constexpr size_t kRouteSmemMax = 227 * 1024 - 8 * 1024;  // dynamic part; the re
 
 // 16-byte vectors of a router row that shared memory holds at a time: the whole row, or a part of it (a
 // whole number of slices; at least 9 for every R) of which two fit.
-template <int R> inline int route_part(int h, int r) {
-  const size_t room = kRouteSmemMax - RouteCfg<R>::kRingBytes;
+template <int R, bool FOLD> inline int route_part(int h, int r) {
+  const size_t room = kRouteSmemMax - RouteCfg<R, FOLD>::kRingBytes;
   if ((size_t)r * h * 2 <= room) return h >> 3;
   return (int)(room / 2 / ((size_t)r * 512)) * 32;
 }
@@ -337,11 +340,17 @@ __device__ __forceinline__ void fetch_router_part(uint4* dst, const bf16* Wg, in
 // first of which is in `half` or on its way there, and all warps of the block call this together, those
 // that have no tokens (t0 >= T) to fetch their shares of the parts; the first part comes round again
 // behind the last one, for the next call.
-template <int R, bool WHOLE>
+// FOLD: shorter chains.  The sum of every kRouteFold slices is closed and added to a second one, and that
+// is closed over the lanes every kRouteSpan vectors: no chain is longer than 16 products, 8 sums or
+// h / 4096 totals.  Error of the weights of 4 experts against 64 bits (2-norm, 2000 tokens) without / with it
+// (h 2048, 16 experts) 1.49e-7 / 1.31e-7, (h 4096, 8 experts) 1.54e-7 / 1.23e-7; 2 tokens per warp instead of 4
+// make room for the second sums (with 4: call of 8 tokens, h 6144, 80 -> 86 us; with 2, 75).
+constexpr int kRouteFold = 2, kRouteSpan = 512;
+template <int R, bool WHOLE, bool FOLD>
 __device__ __forceinline__ float warp_logits(const bf16* x, uint4* s_w, const bf16* Wg, int part, int& half,
                                              int t0, int T, int h, int r, uint4* ring) {
   const bool on = WHOLE || t0 < T;
-  constexpr int RP = RouteCfg<R>::kRP, TB = RouteCfg<R>::kTB, N = RouteCfg<R>::kN;
+  constexpr int RP = RouteCfg<R, FOLD>::kRP, TB = RouteCfg<R, FOLD>::kTB, N = RouteCfg<R, FOLD>::kN;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nvec = h >> 3;
   uint64_t acc[TB / 2][R];  // two tokens each
@@ -349,6 +358,18 @@ __device__ __forceinline__ float warp_logits(const bf16* x, uint4* s_w, const bf
   for (int i = 0; i < TB / 2; ++i)
 #pragma unroll
     for (int c = 0; c < R; ++c) acc[i][c] = 0ull;
+  uint64_t tot[FOLD ? TB / 2 : 1][FOLD ? R : 1];
+  int open = 0;  // slices in acc
+  auto fold = [&]() {
+#pragma unroll
+    for (int i = 0; i < TB / 2; ++i)
+#pragma unroll
+      for (int c = 0; c < R; ++c) {
+        add_f32x2(tot[FOLD ? i : 0][FOLD ? c : 0], acc[i][c]);
+        acc[i][c] = 0ull;
+      }
+    open = 0;
+  };
   const uint4* xr[TB];
 #pragma unroll
   for (int i = 0; i < TB; ++i) xr[i] = reinterpret_cast<const uint4*>(x + (size_t)min(t0 + i, T - 1) * h) + lane;
@@ -364,63 +385,79 @@ __device__ __forceinline__ float warp_logits(const bf16* x, uint4* s_w, const bf
   for (int s = 0; s < kRouteStages - 1; ++s) fetch(32 * s, s);
   int s = 0, left = 0;  // vectors of the present part still to come
   const uint4* w = s_w + lane;
+  float sum = 0.f;
 #pragma unroll 1
-  for (int v = 0; v < nvec; v += 32, left -= 32) {
-    cp_async_wait<kRouteStages - 2>();
-    if (!WHOLE && left <= 0) {
-      // this part was fetched with or before a token slice that has arrived; no warp reads the other half now
-      __syncthreads();
-      w = s_w + half * r * part + lane - v;
-      half ^= 1;
-      left = part;
-      const int next = v + part < nvec ? v + part : 0;
-      fetch_router_part<WHOLE>(s_w + half * r * part, Wg, next, part, nvec, r);  // committed with the slice below
+  for (int v1 = 0; v1 < nvec; v1 += FOLD ? kRouteSpan : nvec) {
+    const int v2 = FOLD ? min(nvec, v1 + kRouteSpan) : nvec;
+    if (FOLD) {
+#pragma unroll
+      for (int i = 0; i < TB / 2; ++i)
+#pragma unroll
+        for (int c = 0; c < R; ++c) tot[FOLD ? i : 0][FOLD ? c : 0] = 0ull;
     }
-    if (!on) {
-      cp_async_commit();
-      continue;
-    }
-    uint64_t xf[TB / 2][8];
+#pragma unroll 1
+    for (int v = v1; v < v2; v += 32, left -= 32) {
+      cp_async_wait<kRouteStages - 2>();
+      if (!WHOLE && left <= 0) {
+        // this part was fetched with or before a token slice that has arrived; no warp reads the other half now
+        __syncthreads();
+        w = s_w + half * r * part + lane - v;
+        half ^= 1;
+        left = part;
+        const int next = v + part < nvec ? v + part : 0;
+        fetch_router_part<WHOLE>(s_w + half * r * part, Wg, next, part, nvec, r);  // committed with the slice below
+      }
+      if (!on) {
+        cp_async_commit();
+        continue;
+      }
+      uint64_t xf[TB / 2][8];
 #pragma unroll
-    for (int i = 0; i < TB / 2; ++i) {
-      float lo[8], hi[8];
-      unpack8(mine[(s * TB + 2 * i) * 32], lo);
-      unpack8(mine[(s * TB + 2 * i + 1) * 32], hi);
+      for (int i = 0; i < TB / 2; ++i) {
+        float lo[8], hi[8];
+        unpack8(mine[(s * TB + 2 * i) * 32], lo);
+        unpack8(mine[(s * TB + 2 * i + 1) * 32], hi);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) xf[i][e] = pack_f32x2(lo[e], hi[e]);
-    }
-    fetch(v + 32 * (kRouteStages - 1), s == 0 ? kRouteStages - 1 : s - 1);
-    if (v + lane < nvec) {
-      constexpr int kBatch = 2;  // router slices in flight
+        for (int e = 0; e < 8; ++e) xf[i][e] = pack_f32x2(lo[e], hi[e]);
+      }
+      fetch(v + 32 * (kRouteStages - 1), s == 0 ? kRouteStages - 1 : s - 1);
+      if (v + lane < nvec) {
+        constexpr int kBatch = 2;  // router slices in flight
 #pragma unroll
-      for (int c0 = 0; c0 < R; c0 += kBatch) {
-        uint4 wv[kBatch];
+        for (int c0 = 0; c0 < R; c0 += kBatch) {
+          uint4 wv[kBatch];
 #pragma unroll
-        for (int b = 0; b < kBatch; ++b) wv[b] = w[(size_t)min(c0 + b, r - 1) * (WHOLE ? nvec : part) + v];
+          for (int b = 0; b < kBatch; ++b) wv[b] = w[(size_t)min(c0 + b, r - 1) * (WHOLE ? nvec : part) + v];
 #pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-          if (c0 + b < R) {
-            float wf[8];
-            unpack8(wv[b], wf);
+          for (int b = 0; b < kBatch; ++b) {
+            if (c0 + b < R) {
+              float wf[8];
+              unpack8(wv[b], wf);
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
+              for (int e = 0; e < 8; ++e)
 #pragma unroll
-              for (int i = 0; i < TB / 2; ++i)
-                fma_f32x2(acc[i][c0 + b < R ? c0 + b : 0], xf[i][e], pack_f32x2(wf[e], wf[e]));
+                for (int i = 0; i < TB / 2; ++i)
+                  fma_f32x2(acc[i][c0 + b < R ? c0 + b : 0], xf[i][e], pack_f32x2(wf[e], wf[e]));
+            }
           }
         }
       }
+      if (FOLD && ++open == kRouteFold) fold();
+      if (++s == kRouteStages) s = 0;
     }
-    if (++s == kRouteStages) s = 0;
+    if (FOLD) fold();
+    float val[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) val[q] = 0.f;
+#pragma unroll
+    for (int i = 0; i < TB / 2; ++i)
+#pragma unroll
+      for (int c = 0; c < R; ++c)
+        split_f32x2(FOLD ? tot[FOLD ? i : 0][FOLD ? c : 0] : acc[i][c], val[2 * i * RP + c], val[(2 * i + 1) * RP + c]);
+    const float got = reduce_scatter<N>(val, lane);
+    sum = v1 == 0 ? got : sum + got;
   }
-  float val[N];
-#pragma unroll
-  for (int q = 0; q < N; ++q) val[q] = 0.f;
-#pragma unroll
-  for (int i = 0; i < TB / 2; ++i)
-#pragma unroll
-    for (int c = 0; c < R; ++c) split_f32x2(acc[i][c], val[2 * i * RP + c], val[(2 * i + 1) * RP + c]);
-  return reduce_scatter<N>(val, lane);
+  return sum;
 }
 
 // Top-2 routing.
@@ -429,7 +466,7 @@ __global__ void __launch_bounds__(32 * kRouteWarps, 1)
 router_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part, float beta, KeptIds kept,
               RouteOut o, bool w_const) {
   pdl_launch_dependents();
-  using Cfg = RouteCfg<R>;
+  using Cfg = RouteCfg<R, false>;
   constexpr int RP = Cfg::kRP, TB = Cfg::kTB, N = Cfg::kN;
   extern __shared__ uint4 ring[];
   __shared__ float s_l[kRouteWarps][N];
@@ -450,7 +487,7 @@ router_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part, floa
   // with the rows in parts all warps of the block stay in step: a team goes on while the first has a unit
   for (int u = blockIdx.x + gridDim.x * team; u - (WHOLE ? 0 : (int)gridDim.x * team) < units; u += gridDim.x * Cfg::kTeams) {
     const int t0 = u * kRouteTokPerBlock;
-    const float mine = warp_logits<R, WHOLE>(x, s_w, Wg, part, half, t0 + tw * TB, T, h, r, ring);
+    const float mine = warp_logits<R, WHOLE, false>(x, s_w, Wg, part, half, t0 + tw * TB, T, h, r, ring);
     if (!WHOLE && u >= units) continue;
     if (lane % (32 / N) == 0) s_l[warp][lane / (32 / N)] = mine;
     __syncwarp();
@@ -788,7 +825,7 @@ router_topk_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part,
                    int32_t* __restrict__ idx, float* __restrict__ wn, int32_t* __restrict__ nact,
                    int32_t* u_idx, float* u_wn, int32_t* u_nact, float* logits) {
   pdl_launch_dependents();
-  using Cfg = RouteCfg<R>;
+  using Cfg = RouteCfg<R, true>;
   constexpr int RP = Cfg::kRP, TB = Cfg::kTB, N = Cfg::kN;
   constexpr int kLanes = 32 / N;  // lanes that hold the same logit
   extern __shared__ uint4 ring[];
@@ -807,7 +844,7 @@ router_topk_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part,
   int half = 0;
   for (int g = blockIdx.x + gridDim.x * warp; g - (WHOLE ? 0 : (int)gridDim.x * warp) < groups; g += gridDim.x * kRouteWarps) {
     const int t0 = g * TB;
-    const float mine = warp_logits<R, WHOLE>(x, s_w, Wg, part, half, t0, T, h, r, ring);
+    const float mine = warp_logits<R, WHOLE, true>(x, s_w, Wg, part, half, t0, T, h, r, ring);
     if (!WHOLE && g >= groups) continue;
     const int i = lane / kLanes / RP, c = lane / kLanes % RP;
     int rank = 0;
@@ -1174,9 +1211,9 @@ cudaError_t launch_router(const bf16* x, const bf16* Wg, int T, int h, int r, fl
                           const KeptIds& kept, const RouteOut& out, cudaStream_t st, bool w_const) {
 #define MOE_ROUTER(R)                                                                                          \
   {                                                                                                            \
-    const int part = route_part<R>(h, r);                                                                      \
+    const int part = route_part<R, false>(h, r);                                                                      \
     const bool whole = part == (h >> 3);                                                                       \
-    const size_t smem = RouteCfg<R>::kRingBytes + (size_t)(whole ? 1 : 2) * r * part * 16;                     \
+    const size_t smem = RouteCfg<R, false>::kRingBytes + (size_t)(whole ? 1 : 2) * r * part * 16;                     \
     const int units = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;                                         \
     return launch_route(whole ? router_kernel<R, true> : router_kernel<R, false>, units, smem, st, x, Wg, T, h, \
                         r, part, beta, kept, out, w_const);                                                    \
@@ -1265,10 +1302,10 @@ cudaError_t launch_router_topk(const bf16* x, const bf16* Wg, int T, int h, int 
                                cudaStream_t st) {
 #define MOE_ROUTER_TOPK(R)                                                                                   \
   {                                                                                                          \
-    const int part = route_part<R>(h, r);                                                                    \
+    const int part = route_part<R, true>(h, r);                                                                    \
     const bool whole = part == (h >> 3);                                                                     \
-    const size_t smem = RouteCfg<R>::kRingBytes + (size_t)(whole ? 1 : 2) * r * part * 16;                   \
-    const int groups = (T + RouteCfg<R>::kTB - 1) / RouteCfg<R>::kTB;                                        \
+    const size_t smem = RouteCfg<R, true>::kRingBytes + (size_t)(whole ? 1 : 2) * r * part * 16;                   \
+    const int groups = (T + RouteCfg<R, true>::kTB - 1) / RouteCfg<R, true>::kTB;                                        \
     return launch_route(whole ? router_topk_kernel<R, true> : router_topk_kernel<R, false>, groups, smem, st, x, \
                         Wg, T, h, r, part, k, beta, kept, idx, wn, nact, u_idx, u_wn, u_nact, logits);       \
   }

@@ -408,7 +408,10 @@ def wide_router_layer(h, offset, narrow, f=64):
 def test_router_rows_longer_than_shared_memory(E, T):
     # rows of 16384 columns (2 to 8 parts) that are zero but for 1024 columns: a lane's chain of
     # multiply-adds is that of a layer of 1024 columns with zeros added before and behind, so the
-    # weights are the same bits wherever the columns lie (first part, across parts, last part).
+    # weights are the same bits wherever the columns lie (first part, across parts, last part), as long
+    # as they lie at a multiple of the 512 columns after which the top-k router closes a chain.  The
+    # first part ends at column 7680 with 3 experts, 4608 with 5, 2816 with 8 and 2304 with 16 (top-k
+    # router: whole rows, 7936, 4864 and 2304).
     # 10000 tokens are several rounds of a block, whose first part then comes round again.
     build.build()
     hn, h, k = 1024, 16384, 3 if T <= 300 else 2
@@ -418,7 +421,7 @@ def test_router_rows_longer_than_shared_memory(E, T):
     want = ref.forward_topk(xn, k, 0.1, record=True)[1:]
     beta = ref.calibrate_beta(xn)
     x = torch.ones((T, h), dtype=torch.bfloat16, device=DEV)
-    for offset in (0, 2304, 8192 - 512, h - hn):
+    for offset in (0, 2048, 4096, 7168, h - hn):
         layer, Wg = wide_router_layer(h, offset, Wn.W_gate)
         x[:, offset:offset + hn] = xn
         got = layer.forward_topk(x, k, 0.1, record=True)[1:]
@@ -457,7 +460,7 @@ def test_allocation_free_calibration_reads_rows_written_just_before(weights):
 
 
 @pytest.mark.parametrize("h", [4096, 8192])
-@pytest.mark.parametrize("call", ["forward_8192"])
+@pytest.mark.parametrize("call", ["forward_8192", "topk_333"])
 def test_routing_weights_against_64_bits(h, call):
     # A logit of 2 to 4 rounded to fp32 is off by up to 1.2e-7, and what else the weights lose depends on
     # how long the chains of the sum are: 1.2e-7 to 1.4e-7 (2-norm over the batch) with chains of up to 32
