@@ -9,13 +9,14 @@
 //   loss(C) = sqrt( sum_t || F'(x_t, C) - F(x_t) ||^2 )
 // Reduction order is fixed: tokens of a warp in order (fp32), warps of a block in order,
 // blocks in order (fp64); no atomics.
+#include <algorithm>
+
 #include "common.h"
 
 namespace moe {
 
 namespace {
 
-constexpr int kTokPerWarp = 1;  // a token is a chain of latencies: blocks before tokens per warp
 constexpr int kMaxBlocks = 148 * 16;
 
 __device__ __forceinline__ void unpack8f(const uint4& v, float* f) {
@@ -266,15 +267,28 @@ reduce_partials_kernel(const float* __restrict__ partial, int nblk, int nC,
 }
 
 int warps_for(int nC) { return nC <= 2048 ? 4 : 1; }
+size_t enumerate_smem(int nC) {
+  const size_t nw = warps_for(nC);
+  return (nw * nC + nw * kMaxE * kMaxE + 3 * nw * kMaxE) * 4;
+}
 
 }  // namespace
 
+// A token is a chain of latencies, so a warp starts with one of them.  In a long enumeration (more than 2048
+// subsets, one warp per block) a block's own work, clearing its accumulators and writing them out, is about
+// 0.3 of a token's, and shared memory lets few blocks run at once: there two tokens per warp are taken
+// where that saves enough rounds of blocks.  Whole search, 16 experts, h 128, one token vs two:
+// 12870 subsets, 256 tokens 1242 vs 1513 us, 1024 tokens 1550 vs 1468, 2048 2198 vs 2060, 4096 2999 vs 3187;
+// 8008 subsets, 1024 tokens 934 vs 890, 2048 1138 vs 1222, 3000 1291 vs 1238; 4368 subsets, 1024 tokens 429 vs
+// 497, 2048 542 vs 500.
 int enumerate_num_blocks(int T, int nC) {
-  const int per_block = warps_for(nC) * kTokPerWarp;
-  int n = (T + per_block - 1) / per_block;
-  if (n > kMaxBlocks) n = kMaxBlocks;
-  if (n < 1) n = 1;
-  return n;
+  const int nw = warps_for(nC);
+  auto blocks = [&](int tokens) { return std::min((T + nw * tokens - 1) / (nw * tokens), kMaxBlocks); };
+  const int one = blocks(1), two = blocks(2);
+  if (nw > 1) return one;
+  const int at_once = 148 * (int)(227 * 1024 / (enumerate_smem(nC) + 1024));
+  auto cost = [&](int n) { return (n + at_once - 1) / at_once * (3 + 10 * ((T + n - 1) / n)); };
+  return cost(two) < cost(one) ? two : one;
 }
 
 cudaError_t launch_enumerate(const float* logits, const bf16* Yall, int T, int E, int r, int h,
@@ -283,7 +297,7 @@ cudaError_t launch_enumerate(const float* logits, const bf16* Yall, int T, int E
                              cudaStream_t st) {
   const int nw = warps_for(nC);
   const int nblk = enumerate_num_blocks(T, nC);
-  const size_t smem = ((size_t)nw * nC + (size_t)nw * kMaxE * kMaxE + 3 * (size_t)nw * kMaxE) * 4;
+  const size_t smem = enumerate_smem(nC);
   if (smem > 96 * 1024) return cudaErrorInvalidValue;
   const int K = E - r + 2;
   void (*kernel)(const float*, const bf16*, int, int, int, int, const uint32_t*, int, float*, const float*,

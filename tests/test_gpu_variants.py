@@ -487,3 +487,15 @@ def test_routing_weights_against_64_bits(h, call):
         assert layer.device_status() == 0
         layer.close()
     assert np.mean(got_err) < 1.45e-7, got_err
+
+
+def test_long_enumerations_with_one_and_two_tokens_per_warp():
+    # 12870 subsets: 512 tokens go one to a warp, 1024 two; the squared losses of the halves add up
+    # (fp32 sums of squares of at most two tokens, then fp64: 2e-7 relative)
+    build.build()
+    W = synth.make_layer_weights(64, 64, 16, seed=41, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
+    x = synth.make_tokens(1024, 64, seed=42, device=DEV)
+    whole, a, b = (np.array(layer.prune_search(t.contiguous(), 8)[0], np.float64) for t in (x, x[:512], x[512:]))
+    np.testing.assert_allclose(whole ** 2, a ** 2 + b ** 2, rtol=2e-6)
+    layer.close()
