@@ -27,12 +27,18 @@ constexpr int kTokensDMaxKept = 6;         // ... on layers with at most this ma
 // 6144 a group was up to 6 % slower on the pairs: with little padding to save, both are held by the
 // board's power and the pairs draw 1-3 % more energy per call.
 constexpr int kPairMaxRows = 1536;
-// Top-k calls of more than kDecodeMaxT tokens with at most this many pairs per kept expert, two thirds
-// of the weight-major kernel's token tile, run that kernel: it cuts the last round into K-slices, and hardly
-// any group needs a second tile yet.  Layer of 16 experts (h 2048, f 4096), gemm_pair_n vs weight-major,
-// whole call: 32 pairs per expert 189 vs 169 us, 62 190 vs 180, 75 201 vs 194, 83 201 vs 196; 112 217
-// vs 250, 125 216 vs 252.
-constexpr int kFewRows = 85;
+// Top-k calls of more than kDecodeMaxT tokens with at most this many pairs per kept expert, half of the
+// weight-major kernel's token tile, run that kernel: it cuts the last round into K-slices, and hardly any
+// group needs a second tile.  Whole call in us, gemm_pair_n vs weight-major, layers of 16 experts (h, f):
+//   pairs per expert   44          65          80-85 (four / one or two experts per token)
+//   768, 512           46 vs 37    45 vs 37    52 vs 44    48 vs 43
+//   1024, 2048         77 vs 70    83 vs 81    87 vs 73    87 vs 92-99
+//   1536, 3072         118 vs 108  126 vs 120  130 vs 152  130 vs 143
+//   2048, 4096         183 vs 170  188 vs 193  194 vs 191  200 vs 225
+//   4096, 4096         312 vs 308  338 vs 341  347 vs 369  352 vs 389
+//   6144, 512          123 vs 105  129 vs 110  133 vs 113  136 vs 123
+// From 95 on the pairs won by up to a quarter except on the smallest weights.
+constexpr int kFewRows = 64;
 constexpr int kPairPad = 32;        // grain of its token tiles
 // Up to here every block of the permutation counts the whole routing record itself (at 32 tokens a
 // thread, in bytes, 255 tokens a thread at most); beyond, the routers' histogram and the scan do.

@@ -499,3 +499,34 @@ def test_long_enumerations_with_one_and_two_tokens_per_warp():
     whole, a, b = (np.array(layer.prune_search(t.contiguous(), 8)[0], np.float64) for t in (x, x[:512], x[512:]))
     np.testing.assert_allclose(whole ** 2, a ** 2 + b ** 2, rtol=2e-6)
     layer.close()
+
+
+@pytest.mark.parametrize("h,f,E,T,k,skew", [
+    # up to 64 pairs per expert beyond 256 tokens: the weight-major GEMM, at the line and just beyond it,
+    # K-sliced (contraction of 1024) and not, on few experts, and with every token on one expert (three tiles)
+    (64, 64, 6, 384, 1, False), (64, 64, 6, 385, 1, False), (128, 448, 5, 257, 1, False), (128, 64, 16, 257, 3, False),
+    (1024, 256, 16, 270, 3, False), (128, 448, 6, 384, 1, True), (1024, 1024, 6, 300, 1, True),
+])
+def test_topk_calls_with_few_pairs_per_expert(h, f, E, T, k, skew):
+    build.build()
+    W = synth.make_layer_weights(h, f, E, seed=13, device=DEV)
+    x = synth.make_tokens(T, h, seed=14, device=DEV)
+    if skew:
+        W.W_gate[:, 0] = 0
+        W.W_gate[2, 0] = 1.0
+        x[:, 0] = 64.0
+    layers = [binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2),
+              layer_with_env((W.W_gate, W.W1, W.W3, W.W2), (1 << E) - 1, MOE_DECODE_KERNEL="td"),
+              layer_with_env((W.W_gate, W.W1, W.W3, W.W2), (1 << E) - 1, MOE_DEBUG_SIMT=1)]
+    got = [l.forward_topk(x, k, 0.2, record=True) for l in layers]
+    again = layers[0].forward_topk(x, k, 0.2)
+    torch.cuda.synchronize()
+    if skew:
+        assert int((got[0][1] == 2).sum()) == T
+    assert torch.equal(got[0][0], again)
+    for l, g in zip(layers, got):
+        for a, b in zip(g[1:], got[0][1:]):
+            assert torch.equal(a, b)
+        assert rel_l2(got[0][0], g[0]) < 5e-3  # different summation orders, same rounding points
+        assert l.device_status() == 0
+        l.close()
