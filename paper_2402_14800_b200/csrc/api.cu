@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 #include <vector>
 
 #include "common.h"
@@ -245,16 +246,55 @@ void mark(moe_layer* L) {
 }
 
 // Pinned host words of the handle that kernels and copies write results to ([0] status word,
-// [1..2] selected values, [kHostLosses..] losses of a search); null if they cannot be had.  A copy to
-// pageable memory would be staged by the runtime, with a wait of its own.
-constexpr int kHostLosses = 4, kMaxHostLosses = 1020;
-int* host_words(moe_layer* L) {
-  if (!L->h_words && cudaHostAlloc((void**)&L->h_words, (kHostLosses + kMaxHostLosses) * sizeof(int),
-                                   cudaHostAllocDefault) != cudaSuccess) {
-    cudaGetLastError();
-    L->h_words = nullptr;
+// [1..2] selected values, [kHostLosses..] losses of a search); null if there are none.  A copy to
+// pageable memory would be staged by the runtime, with a wait of its own.  Pinning takes 1-3 ms, far
+// longer than the calls that use the words, so no call does it: the first handle of a process pins
+// kWordSlots slots (256 KB, kept until the process ends: a program that makes and destroys one handle
+// after the other would pin them again for each), and a handle has a slot from its first use to its end.
+// Only the calls of handles beyond them that need words (`pin`) pin some of their own.
+constexpr int kHostLosses = 4, kMaxHostLosses = 1020, kSlotInts = kHostLosses + kMaxHostLosses, kWordSlots = 64;
+struct WordPool {
+  std::mutex mu;
+  int* base = nullptr;
+  bool tried = false;
+  uint64_t used = 0;  // slots given out
+};
+WordPool g_words;
+
+int* pin_ints(int n) {
+  int* p = nullptr;
+  if (cudaHostAlloc((void**)&p, (size_t)n * sizeof(int), cudaHostAllocPortable) == cudaSuccess) return p;
+  cudaGetLastError();
+  return nullptr;
+}
+
+void pin_word_slots() {
+  std::lock_guard<std::mutex> lock(g_words.mu);
+  if (!g_words.tried) g_words.base = pin_ints(kWordSlots * kSlotInts);
+  g_words.tried = true;
+}
+
+int* host_words(moe_layer* L, bool pin = true) {
+  if (L->h_words) return L->h_words;
+  std::lock_guard<std::mutex> lock(g_words.mu);
+  if (g_words.base && ~g_words.used) {
+    const int slot = __builtin_ctzll(~g_words.used);
+    g_words.used |= 1ull << slot;
+    L->h_words = g_words.base + slot * kSlotInts;
+  } else if (pin) {
+    L->h_words = pin_ints(kSlotInts);
   }
   return L->h_words;
+}
+
+void release_words(moe_layer* L) {
+  if (!L->h_words) return;
+  std::lock_guard<std::mutex> lock(g_words.mu);
+  if (g_words.base && L->h_words >= g_words.base && L->h_words < g_words.base + kWordSlots * kSlotInts)
+    g_words.used &= ~(1ull << ((L->h_words - g_words.base) / kSlotInts));
+  else
+    cudaFreeHost(L->h_words);
+  L->h_words = nullptr;
 }
 
 int check_status(moe_layer* L) {
@@ -488,6 +528,7 @@ moe_layer_t* moe_layer_create(const void* W_gate, const void* W1, const void* W3
   if (e == cudaSuccess) e = gemv_single_setup();
   if (e != cudaSuccess) { fail(MOE_ERR_CUDA, "kernel attributes: %s", cudaGetErrorString(e)); return nullptr; }
 
+  pin_word_slots();
   moe_layer* L = new (std::nothrow) moe_layer();
   if (!L) { fail(MOE_ERR_OOM, "host allocation failed"); return nullptr; }
   L->h = h; L->f = f; L->E = E; L->kept_mask = kept_mask; L->r = popc(kept_mask);
@@ -562,7 +603,7 @@ void moe_layer_destroy(moe_layer_t* L) {
                  &L->own.s_losses, &L->own.s_xpad, &L->own.s_meta, &L->own.s_xperm, &L->own.hx, &L->own.hy, &L->own.xn, &L->own.cosel, &L->own.k_idx, &L->own.k_wn, &L->own.k_pos, &L->own.k_nact};
   for (Buf* b : bufs) release(L, *b);
   for (cudaEvent_t e : L->prof_ev) cudaEventDestroy(e);
-  if (L->h_words) cudaFreeHost(L->h_words);
+  release_words(L);
   if (L->Wg) cudaFree(L->Wg);
   if (L->W13) cudaFree(L->W13);
   if (L->W2) cudaFree(L->W2);
@@ -705,8 +746,8 @@ int moe_calibrate_beta(moe_layer_t* L, const void* x, int T, float* beta_out) {
   ro.idx = (int32_t*)L->ws->idx.p; ro.wn = (float*)L->ws->wn.p; ro.ratio = (float*)L->ws->ratio.p;
   ro.skipped = (uint8_t*)L->ws->skipped.p;
   CUDA_TRY(launch_router((const bf16*)x, L->Wg, T, L->h, L->r, 0.f, L->kept, ro, L->stream));
-  // the two values go straight to mapped host memory where there is some
-  int* words = host_words(L);
+  // the two values go straight to mapped host memory where the handle has some
+  int* words = host_words(L, false);
   float* sel = words ? (float*)(words + 1) : (float*)L->ws->sel.p;
   CUDA_TRY(launch_select2(ro.ratio, T, (T - 1) / 2, T / 2, sel, L->stream));
   float v[2];

@@ -530,3 +530,37 @@ def test_topk_calls_with_few_pairs_per_expert(h, f, E, T, k, skew):
         assert rel_l2(got[0][0], g[0]) < 5e-3  # different summation orders, same rounding points
         assert l.device_status() == 0
         l.close()
+
+
+def test_results_in_pinned_words_with_many_handles_and_threads(weights):
+    # more handles than the process' pinned words have slots for, then handles that come and go in threads
+    import threading
+    x = synth.make_tokens(300, H, seed=51, device=DEV)
+    layers = [binding.MoeLayer(*weights) for _ in range(70)]
+    want, found = layers[0].calibrate_beta(x), layers[0].prune_search_multi(x, [6, 4])
+    for l in layers + layers[60:]:
+        assert l.calibrate_beta(x) == want
+    for l in layers[::3] + layers[60:]:
+        assert l.prune_search_multi(x, [6, 4]) == found
+        assert l.calibrate_beta(x) == want and l.device_status() == 0
+    for l in layers:
+        l.close()
+    wrong = []
+
+    def work(seed):
+        stream = torch.cuda.Stream(DEV)
+        with torch.cuda.stream(stream):
+            for i in range(8):
+                l = binding.MoeLayer(*weights)
+                l.set_stream(stream)
+                if any(l.calibrate_beta(x) != want for _ in range(3)) or (i % 3 == seed % 3 and l.prune_search_multi(x, [6, 4]) != found):
+                    wrong.append((seed, i))
+                l.close()
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
