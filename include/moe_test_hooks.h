@@ -31,6 +31,15 @@ extern "C" {
 int moe_test_wait_expiry(moe_layer_t* layer, unsigned limit_us, int poison_tail);
 
 /*
+ * The same for the CTA-pair GEMM: one pair of CTAs sets up its barrier block and
+ * its tensor memory; CTA `cta` (0 = the leader, 1) waits on a barrier nobody
+ * arrives on until `limit_us` run out, the other one has nothing to wait for and
+ * learns of the abort from its partner.  Both take the kernel's own teardown.
+ * Errors: MOE_ERR_INVALID_ARG, MOE_ERR_OOM, MOE_ERR_CUDA.
+ */
+int moe_test_wait_expiry_pair(moe_layer_t* layer, unsigned limit_us, int cta);
+
+/*
  * Host side only.  Make every later scratch or weight allocation of this process
  * see at most `bytes` of free device memory (the library compares its request
  * with cudaMemGetInfo before it calls cudaMalloc), so that MOE_ERR_OOM can be

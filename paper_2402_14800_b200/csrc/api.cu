@@ -643,6 +643,16 @@ int moe_test_wait_expiry(moe_layer_t* L, unsigned limit_us, int poison_tail) {
   return MOE_OK;
 }
 
+int moe_test_wait_expiry_pair(moe_layer_t* L, unsigned limit_us, int cta) {
+  if (!L) return fail(MOE_ERR_INVALID_ARG, "layer is NULL");
+  if (limit_us < 1 || limit_us > 100000) return fail(MOE_ERR_INVALID_ARG, "limit_us = %u outside 1..100000", limit_us);
+  if (cta != 0 && cta != 1) return fail(MOE_ERR_INVALID_ARG, "cta = %d is not 0 or 1", cta);
+  int rc;
+  if ((rc = ensure_route(L, 1))) return rc;
+  CUDA_TRY(launch_wait_expiry_pair((int*)L->ws->status.p, (unsigned long long)limit_us * 1000ull, cta, L->stream));
+  return MOE_OK;
+}
+
 size_t moe_layer_weight_bytes(const moe_layer_t* L) { return L ? L->weight_bytes : 0; }
 size_t moe_layer_scratch_bytes(const moe_layer_t* L) { return L ? L->own.scratch_bytes : 0; }
 

@@ -275,6 +275,7 @@ cudaError_t gemm_set_attributes();
 // Test hook: one CTA runs the GEMMs' bounded wait on a barrier nobody arrives on, then their
 // abort path (see moe_test_hooks.h).
 cudaError_t launch_wait_expiry(int* status, unsigned long long limit_ns, cudaStream_t st);
+cudaError_t launch_wait_expiry_pair(int* status, unsigned long long limit_ns, int cta, cudaStream_t st);
 
 // ---- search (search.cu) ---------------------------------------------------------------
 // Where the enumeration finds the expert outputs.  Dense (topk_idx == null): Yall[T][E][h].

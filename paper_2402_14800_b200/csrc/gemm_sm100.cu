@@ -668,6 +668,41 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
       : "memory");
 }
 
+// End of a pair: tell the partner if this CTA gave up, drain (bounded), and leave together (the leader's
+// MMAs read the partner's shared memory, and tensor memory is released as a pair).
+__device__ __forceinline__ void teardown_pair(Bars& b, uint32_t tmem_base, uint32_t tmem_cols, uint32_t issued,
+                                              uint32_t ns, uint32_t rank, int* status) {
+  volatile int* abort_flag = &b.abort_flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag) st_cluster_u32(map_to_cta(smem_u32(&b.abort_flag), rank ^ 1u), 1u);
+  __syncwarp();  // the cluster barrier is an aligned instruction
+  cluster_sync_all();
+  if (*abort_flag) {
+    if (warp == 0 && lane == 0) {
+      int dummy = 0;
+      const uint32_t n = issued < ns ? issued : ns;
+      for (uint32_t i = 0; rank == 0 && i < n; ++i) {
+        const uint32_t it = issued - 1 - i;
+        mbar_wait(smem_u32(&b.full[it % ns]), (it / ns) & 1u, &dummy, kDrainLimitNs);
+      }
+      if (status) atomicExch(status, 1);
+    }
+    if ((warp == 1 || warp == 2) && lane == 0) {
+      int dummy = 0;
+      if (rank == 0) umma_commit_pair(smem_u32(&b.drain));
+      mbar_wait(smem_u32(&b.drain), 0, &dummy, kDrainLimitNs);  // either CTA its own arrivals
+    }
+    __syncwarp();
+    cluster_sync_all();
+  }
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem_base, tmem_cols);
+  }
+}
+
 constexpr int PN_NS = 5;                // stages at most
 constexpr int PN_A_BYTES = 256 * 128;   // this CTA's 256 weight rows x 64 bf16
 constexpr int PN_B_UNIT = 16 * 128;     // this CTA's half of 32 tokens
@@ -816,6 +851,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
   const int Nt = (args.n_w_rows + PN_W_ROWS - 1) / PN_W_ROWS;
   const int cap = choose_tile_cap(s_meta, args, KB, Nt, n_pairs);
   if (threadIdx.x < kMaxE) s_tiles[threadIdx.x] = token_tiles(s_meta.count[threadIdx.x], cap);
+  __syncwarp();
   tc_fence_before();
   cluster_sync_all();  // both CTAs' barriers exist before anything is signalled across the pair
   tc_fence_after();
@@ -939,34 +975,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
   }
 
   pdl_launch_dependents();
-  // ---- teardown: tell the partner if this CTA gave up, drain, and leave together (the leader's
-  // MMAs read the partner's shared memory, and tensor memory is released as a pair)
-  tc_fence_before();
-  __syncthreads();
-  if (threadIdx.x == 0 && *abort_flag) st_cluster_u32(map_to_cta(smem_u32(&bars.abort_flag), rank ^ 1u), 1u);
-  cluster_sync_all();
-  if (*abort_flag) {
-    if (warp == 0 && lane == 0) {
-      int dummy = 0;
-      const uint32_t n = issued < ns ? issued : ns;
-      for (uint32_t i = 0; rank == 0 && i < n; ++i) {
-        const uint32_t it = issued - 1 - i;
-        mbar_wait(smem_u32(&bars.full[it % ns]), (it / ns) & 1u, &dummy, kDrainLimitNs);
-      }
-      if (args.status) atomicExch(args.status, 1);
-    }
-    if ((warp == 1 || warp == 2) && lane == 0 && rank == 0) {
-      int dummy = 0;
-      umma_commit_pair(smem_u32(&bars.drain));
-      mbar_wait(smem_u32(&bars.drain), 0, &dummy, kDrainLimitNs);
-    }
-    __syncwarp();
-    cluster_sync_all();
-  }
-  if (warp == 1) {
-    tc_fence_after();
-    tmem_dealloc_pair(tmem_base, 512);
-  }
+  teardown_pair(bars, tmem_base, 512, issued, ns, rank, args.status);
 }
 
 // ----------------------------------------------------------------------- gemm_weights_m
@@ -1734,6 +1743,30 @@ wait_expiry_kernel(int* status, unsigned long long limit_ns) {
   teardown<32>(bars, tmem_base, 0u, 1u, status);
 }
 
+// The same for a pair of CTAs: CTA `cta` waits in vain, its partner has nothing to wait for.
+__global__ void __launch_bounds__(kThreads, 1)
+wait_expiry_pair_kernel(int* status, unsigned long long limit_ns, uint32_t cta) {
+  __shared__ Bars bars;
+  const int warp = threadIdx.x >> 5;
+  const uint32_t rank = cluster_ctarank();
+  setup_barriers<1>(bars, 1, 2);
+  if (warp == 1) {
+    tmem_alloc_pair(smem_u32(&bars.tmem_base), 32);
+    tmem_relinquish_pair();
+  }
+  __syncthreads();
+  tc_fence_before();
+  cluster_sync_all();
+  tc_fence_after();
+  const uint32_t tmem_base = *(volatile uint32_t*)&bars.tmem_base;
+  volatile int* abort_flag = &bars.abort_flag;
+  if (rank == cta) {
+    const uint32_t bar = warp == 0 ? smem_u32(&bars.full[0]) : smem_u32(&bars.tmem_full[0]);
+    (void)__all_sync(0xffffffffu, mbar_wait(bar, 0u, abort_flag, warp == 0 ? limit_ns : 2 * limit_ns));
+  }
+  teardown_pair(bars, tmem_base, 32, 0u, 1u, rank, status);
+}
+
 // ------------------------------------------------------------ CUDA-core debug kernels
 
 __device__ __forceinline__ float dot8(const uint4& a, const uint4& b, float acc) {
@@ -1912,15 +1945,16 @@ cudaError_t launch_gemm_tokens_m(bool gate_up, GemmOut out_kind, const GemmMaps&
   return launch_plain(gemm_tokens_m_kernel<false, kOutBf16>, dim3(grid), dim3(TmCfg<false>::kThreads), TM_SMEM, st, maps, a);
 }
 
-// On CTA pairs (cluster of two), as programmatic dependents: set-up, tensor-memory allocation and the
-// fetch of the tensor maps overlap the predecessor (search on the tiny layer 88 -> 78 us, tiny layer at
-// 2000 tokens 48.4 -> 43.5; equal where the launches are long).
+// On CTA pairs (cluster of two).  The GEMM is a programmatic dependent: set-up and tensor-memory allocation
+// overlap the predecessor (search on the tiny layer 88 -> 78 us, tiny layer at 2000 tokens 48.4 -> 43.5;
+// equal where the launches are long).
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_pair(void (*kernel)(KArgs...), cudaStream_t st, Args&&... args) {
+static cudaError_t launch_pair(void (*kernel)(KArgs...), int grid, int threads, int smem, bool pdl, cudaStream_t st,
+                               Args&&... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((g_num_sms > 0 ? g_num_sms : 148) & ~1);
-  cfg.blockDim = dim3(PN_THREADS);
-  cfg.dynamicSmemBytes = PN_SMEM;
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1928,7 +1962,7 @@ static cudaError_t launch_pair(void (*kernel)(KArgs...), cudaStream_t st, Args&&
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = g_pdl_enabled ? 1 : 0;
+  attr[1].val.programmaticStreamSerializationAllowed = pdl && g_pdl_enabled ? 1 : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
@@ -1936,9 +1970,15 @@ static cudaError_t launch_pair(void (*kernel)(KArgs...), cudaStream_t st, Args&&
 
 cudaError_t launch_gemm_pair_n(bool gate_up, GemmOut out_kind, const GemmMaps& maps, const GemmArgs& a,
                                cudaStream_t st) {
-  if (gate_up) return launch_pair(gemm_pair_n_kernel<true, kOutActBf16>, st, maps, a);
-  if (out_kind == kOutF32) return launch_pair(gemm_pair_n_kernel<false, kOutF32>, st, maps, a);
-  return launch_pair(gemm_pair_n_kernel<false, kOutBf16>, st, maps, a);
+  const int grid = (g_num_sms > 0 ? g_num_sms : 148) & ~1;
+  if (gate_up) return launch_pair(gemm_pair_n_kernel<true, kOutActBf16>, grid, PN_THREADS, PN_SMEM, true, st, maps, a);
+  if (out_kind == kOutF32)
+    return launch_pair(gemm_pair_n_kernel<false, kOutF32>, grid, PN_THREADS, PN_SMEM, true, st, maps, a);
+  return launch_pair(gemm_pair_n_kernel<false, kOutBf16>, grid, PN_THREADS, PN_SMEM, true, st, maps, a);
+}
+
+cudaError_t launch_wait_expiry_pair(int* status, unsigned long long limit_ns, int cta, cudaStream_t st) {
+  return launch_pair(wait_expiry_pair_kernel, 2, kThreads, 0, false, st, status, limit_ns, (uint32_t)cta);
 }
 
 cudaError_t launch_gemm_tokens_d(bool gate_up, const GemmMaps& maps, const GemmArgs& a, int kb_per_item,

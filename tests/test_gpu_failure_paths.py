@@ -111,3 +111,19 @@ def test_scratch_that_does_not_fit_is_an_error_and_the_handle_stays_usable(tiny)
         check_against_oracle(layer, host, T, 0xFF, 0.3, seed=6 + T)
     assert layer.device_status() == 0
     layer.close()
+
+
+@pytest.mark.parametrize("cta", [0, 1])
+def test_an_expired_wait_in_one_cta_of_a_pair_ends_both(tiny, cta):
+    # the leader's wait runs out, or its partner's: the other CTA learns of it in the teardown they share
+    host, dev = tiny
+    lib = binding.load_library()
+    layer = binding.MoeLayer(*dev)
+    check_against_oracle(layer, host, 700, 0xFF, 0.3, seed=7)
+    for _ in range(3):
+        assert lib.moe_test_wait_expiry_pair(layer._h, 1000, cta) == 0
+        assert layer.device_status() == MOE_ERR_DEVICE_TIMEOUT
+        assert layer.device_status() == 0
+        check_against_oracle(layer, host, 700, 0xFF, 0.3, seed=8)   # on the CTA pairs
+    assert lib.moe_test_wait_expiry_pair(layer._h, 1000, 2) == -1 and lib.moe_test_wait_expiry_pair(layer._h, 0, 0) == -1
+    layer.close()
