@@ -40,6 +40,15 @@ int moe_test_wait_expiry(moe_layer_t* layer, unsigned limit_us, int poison_tail)
 int moe_test_wait_expiry_pair(moe_layer_t* layer, unsigned limit_us, int cta);
 
 /*
+ * Later calls on this handle run their batches of the large-batch sequence on the
+ * given grouped GEMM: 0 = the library's choice, 1 = the CTA-pair kernel, 2 = the
+ * token-major kernel; tile_cap = largest token tile of the pair kernel in units of
+ * 32 tokens (1 .. 8; 0 = the kernel's choice).
+ * Errors: MOE_ERR_INVALID_ARG.
+ */
+int moe_test_large_batch(moe_layer_t* layer, int kernel, int tile_cap);
+
+/*
  * Host side only.  Make every later scratch or weight allocation of this process
  * see at most `bytes` of free device memory (the library compares its request
  * with cudaMemGetInfo before it calls cudaMalloc), so that MOE_ERR_OOM can be

@@ -117,6 +117,7 @@ struct moe_layer {
   std::vector<cudaEvent_t> prof_ev;  // MOE_PROFILE_STAGES + 1 marks per recorded call
   size_t prof_used = 0;
   int* h_words = nullptr;  // pinned host words (host_words)
+  int large_kernel = 0, tile_cap = 0;  // moe_test_large_batch
 };
 
 namespace {
@@ -314,7 +315,9 @@ int check_status(moe_layer* L) {
 
 // Which large-batch GEMM a batch of at most `pairs` token-expert pairs runs, and what its groups are
 // padded to.
-inline bool large_on_pairs(const moe_layer* L, long long pairs) { return pairs <= (long long)kPairMaxRows * L->r; }
+inline bool large_on_pairs(const moe_layer* L, long long pairs) {
+  return L->large_kernel == 1 || (L->large_kernel == 0 && pairs <= (long long)kPairMaxRows * L->r);
+}
 inline int group_pad(const moe_layer* L, long long pairs) { return large_on_pairs(L, pairs) ? kPairPad : kTileRows; }
 
 // Permutation of a top-k batch: idx [T][k], the first nact[t] slots of a token run.
@@ -343,6 +346,7 @@ int run_expert_gemms(moe_layer* L, const Meta* meta, bool weights_m, const GemmM
   gu.K = L->h; gu.n_w_rows = 2 * L->f;
   dn.K = L->f; dn.n_w_rows = L->h;
   gu.status = (int*)L->ws->status.p; dn.status = (int*)L->ws->status.p;
+  gu.tile_cap = L->tile_cap; dn.tile_cap = L->tile_cap;
   if (L->debug_simt) {
     CUDA_TRY(launch_simt_gate_up(gu_A, L->W13, gu, simt_rows, L->stream));
     mark(L);
@@ -650,6 +654,15 @@ int moe_test_wait_expiry_pair(moe_layer_t* L, unsigned limit_us, int cta) {
   int rc;
   if ((rc = ensure_route(L, 1))) return rc;
   CUDA_TRY(launch_wait_expiry_pair((int*)L->ws->status.p, (unsigned long long)limit_us * 1000ull, cta, L->stream));
+  return MOE_OK;
+}
+
+int moe_test_large_batch(moe_layer_t* L, int kernel, int tile_cap) {
+  if (!L) return fail(MOE_ERR_INVALID_ARG, "layer is NULL");
+  if (kernel < 0 || kernel > 2 || tile_cap < 0 || tile_cap > 8)
+    return fail(MOE_ERR_INVALID_ARG, "kernel = %d outside 0..2 or tile_cap = %d outside 0..8", kernel, tile_cap);
+  L->large_kernel = kernel;
+  L->tile_cap = tile_cap;
   return MOE_OK;
 }
 

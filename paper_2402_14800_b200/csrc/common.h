@@ -227,6 +227,7 @@ struct GemmArgs {
   // weight-major kernel: arrival counters (kTailHeaderBytes, zero between launches) followed by
   // the partial tiles of the K-sliced tail items; null = no slicing
   float* tail;
+  int tile_cap;  // pair kernel: largest token tile / 32, 0 = chosen by the kernel (tests set it)
 };
 
 constexpr size_t kTailHeaderBytes = 4096;  // four arrival counters per tail item

@@ -849,7 +849,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
   __syncthreads();
   const int KB = (args.K + BK - 1) / BK;
   const int Nt = (args.n_w_rows + PN_W_ROWS - 1) / PN_W_ROWS;
-  const int cap = choose_tile_cap(s_meta, args, KB, Nt, n_pairs);
+  const int cap = args.tile_cap ? args.tile_cap : choose_tile_cap(s_meta, args, KB, Nt, n_pairs);
   if (threadIdx.x < kMaxE) s_tiles[threadIdx.x] = token_tiles(s_meta.count[threadIdx.x], cap);
   __syncwarp();
   tc_fence_before();

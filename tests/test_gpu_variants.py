@@ -564,3 +564,73 @@ def test_results_in_pinned_words_with_many_handles_and_threads(weights):
     for t in threads:
         t.join()
     assert not wrong
+
+
+def forced(layer, kernel, cap=0):
+    assert binding.load_library().moe_test_large_batch(layer._h, kernel, cap) == 0
+    return layer
+
+
+@pytest.mark.parametrize("cap", [0, 1, 2, 3, 4, 5, 6, 7, 8])
+@pytest.mark.parametrize("h,f", [(128, 448), (576, 320), (1024, 64)])
+def test_pair_gemm_equals_the_token_major_one_for_every_token_tile(cap, h, f):
+    # Both add up a contraction in the same order, so the bits are the same whatever the tile.  Two kept
+    # experts and no skipping: two groups of T tokens, at n tiles of 32 cap tokens, one less and one more
+    # (and in between, where the tiles are uneven); weight rows that end inside an item of 512.
+    build.build()
+    W = synth.make_layer_weights(h, f, 3, seed=61, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2, 0b101)
+    step = 32 * (cap or 8)
+    n = -(-257 // step)
+    sizes = sorted({T for m in (n, n + 1) for T in (m * step - 1, m * step, m * step + 1, m * step + 17) if T > 256})
+    x = synth.make_tokens(sizes[-1], h, seed=62, device=DEV)
+    for T in sizes:
+        xs = x[:T].contiguous()
+        want = forced(layer, 2).forward(xs)
+        got = forced(layer, 1, cap).forward(xs)
+        assert torch.equal(got, want), T
+        assert torch.equal(forced(layer, 1, cap).top2_distance(xs), forced(layer, 2).top2_distance(xs))
+    assert layer.device_status() == 0
+    layer.close()
+    # bf16 outputs (the search), ragged groups of all experts
+    full = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
+    for T in (257, 300, 777):
+        xs = x[:T].contiguous()
+        for r in (2, 3):  # r = 2 evaluates every expert on every token, r = 3 two experts of a token
+            assert forced(full, 1, cap).prune_search(xs, r) == forced(full, 2).prune_search(xs, r)
+    full.close()
+
+
+@pytest.mark.parametrize("cap", [0, 1, 5, 8])
+@pytest.mark.parametrize("beta", [0.0, 2.0])
+def test_pair_gemm_on_skewed_groups(cap, beta):
+    # every token on the same two experts of eight (beta = 2: on the first of them alone): groups of 6000
+    # tokens beside empty ones, more token tiles than sweep the weight tiles together
+    build.build()
+    h, f, E, T = 192, 640, 8, 6000
+    W = synth.make_layer_weights(h, f, E, seed=63, device=DEV)
+    x = synth.make_tokens(T, h, seed=64, device=DEV)
+    W.W_gate[:, 0] = 0
+    W.W_gate[2, 0], W.W_gate[5, 0] = 2.0, 1.0
+    x[:, 0] = 128.0
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
+    stats = binding.RoutingStats(T, E, DEV)
+    got = forced(layer, 1, cap).forward(x, beta, stats=stats)
+    torch.cuda.synchronize()
+    assert int(stats.count[2, 0]) == T and int(stats.count[5, 1]) == (T if beta == 0 else 0)
+    assert torch.equal(got, forced(layer, 2).forward(x, beta))
+    dbg = layer_with_env((W.W_gate, W.W1, W.W3, W.W2), MOE_DEBUG_SIMT=1)
+    assert rel_l2(got, dbg.forward(x, beta)) < 5e-3
+    assert torch.equal(forced(layer, 0).forward(x, beta), got)
+    assert layer.device_status() == 0
+    layer.close()
+    dbg.close()
+
+
+def test_large_batch_hook_rejects_what_it_does_not_know(weights):
+    layer = binding.MoeLayer(*weights)
+    lib = binding.load_library()
+    for kernel, cap in ((-1, 0), (3, 0), (1, -1), (1, 9)):
+        assert lib.moe_test_large_batch(layer._h, kernel, cap) == -1
+    assert lib.moe_test_large_batch(None, 0, 0) == -1
+    layer.close()
