@@ -379,13 +379,10 @@ def timing_record(blocks, steps, clocks):
     return rec
 
 
-def decode_kernel_name(T, r_kept):
-    forced = os.environ.get("MOE_DECODE_KERNEL", "")
-    if T == 1 and single_token_gemv():
-        return "gemv_route_gate_up_kernel"
-    # the library's crossover: many tokens per expert -> token-major decode kernel
-    token_major = forced == "td" or (forced != "wm" and 2 * T >= 40 * r_kept and r_kept <= 6)
-    return "gemm_tokens_d_kernel<gate_up>" if token_major else "gemm_weights_m_kernel<gate_up>"
+def gate_up_kernel(layer, T):
+    """The dominant kernel as the profiles name it, from the library's own choice."""
+    name = layer.forward_kernel(T)
+    return name if name.startswith("gemv") else name + "<gate_up>"
 
 
 def launches_per_forward(T):
@@ -432,12 +429,11 @@ def forward_case(layer, x, y, beta, workload, wname, steps, warmup, stream, dev,
     gu_ms, dn_ms = stage_ms[1] / ncalls, stage_ms[2] / ncalls
     stages = {"route_permute_ms": stage_ms[0] / ncalls, "gate_up_ms": gu_ms, "down_ms": dn_ms,
               "combine_ms": stage_ms[3] / ncalls, "steps": ncalls}
-    r_kept = bin(kept).count("1")
     if workload == "decode":
         gu_bytes = touched * 2 * F * H * 2 + pairs * H * 2 + pairs * F * 2
         dn_bytes = touched * H * F * 2 + pairs * F * 2 + 2 * pairs * H * 4
         ach = gu_bytes / (gu_ms * 1e-3) / 1e9
-        kernel = decode_kernel_name(T, r_kept)
+        kernel = gate_up_kernel(layer, T)
         roofline = {"bound": "hbm", "kernel": kernel, "achieved": ach,
                     "peak": peaks["hbm"], "unit": "GB/s", "frac": ach / peaks["hbm"],
                     "traffic": recorded_traffic(wname, kernel),
@@ -451,7 +447,7 @@ def forward_case(layer, x, y, beta, workload, wname, steps, warmup, stream, dev,
         dn_flop = pairs * 2 * H * F
         ach = gu_flop / (gu_ms * 1e-3) / 1e12
         step_tf = (gu_flop + dn_flop) / (ms_step * 1e-3) / 1e12
-        kernel = "gemm_pair_n_kernel<gate_up>" if 2 * T <= 1536 * r_kept else "gemm_tokens_m_kernel<gate_up>"
+        kernel = gate_up_kernel(layer, T)
         roofline = {"bound": "tensor", "kernel": kernel, "achieved": ach,
                     "peak": peaks["tf_sust"], "unit": "TFLOP/s", "frac": ach / peaks["tf_sust"],
                     "traffic": recorded_traffic(wname, kernel),

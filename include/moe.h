@@ -90,6 +90,10 @@ size_t moe_layer_weight_bytes(const moe_layer_t* layer);
 /* Bytes of device memory the handle currently holds as scratch. */
 size_t moe_layer_scratch_bytes(const moe_layer_t* layer);
 
+/* Name of the kernel that does the gate/up products of a forward call of T tokens
+ * (for reports; a static string, empty for a NULL layer or T < 1). */
+const char* moe_layer_forward_kernel(const moe_layer_t* layer, int T);
+
 /*
  * Layer forward for T tokens (Sec. 3.1 Eq. 1-2, Sec. 3.2, Sec. 3.3, App. A.2):
  *   l = W_gate x over the kept experts, w = Softmax(l), e0/e1 = top-2 (ties to

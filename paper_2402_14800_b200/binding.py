@@ -51,6 +51,8 @@ def load_library(path: str | None = None):
     lib.moe_layer_weight_bytes.argtypes = [vp]
     lib.moe_layer_scratch_bytes.restype = ctypes.c_size_t
     lib.moe_layer_scratch_bytes.argtypes = [vp]
+    lib.moe_layer_forward_kernel.restype = ctypes.c_char_p
+    lib.moe_layer_forward_kernel.argtypes = [vp, ci]
     lib.moe_forward.argtypes = [vp, vp, ci, cf, vp, vp]
     lib.moe_forward_residual.argtypes = [vp, vp, ci, cf, vp, vp, vp]
     lib.moe_forward_host.argtypes = [vp, vp, ci, cf, vp]
@@ -180,6 +182,10 @@ class MoeLayer:
     @property
     def scratch_bytes(self) -> int:
         return int(load_library().moe_layer_scratch_bytes(self._h))
+
+    def forward_kernel(self, T: int) -> str:
+        """Name of the kernel that does the gate/up products of a forward call of T tokens."""
+        return load_library().moe_layer_forward_kernel(self._h, T).decode()
 
     def forward(self, x, beta: float = 0.0, y=None, stats: RoutingStats | None = None, residual=None):
         """``moe_forward`` / ``moe_forward_residual``; returns y."""

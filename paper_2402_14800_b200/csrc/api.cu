@@ -78,7 +78,7 @@ struct Workspace {
   // GEMM scratch (capacity in permuted rows)
   int cap_rows = 0;
   int map_h = 0, map_f = 0;
-  Buf row_token, xperm, act, O, tail;
+  Buf xperm, act, O, tail;
   CUtensorMap tok_x[4], tok_act[4];  // boxes of 16/32/64/128 rows over xperm and act
   // search scratch
   Buf s_logits, s_yall, s_act, s_subsets, s_partial, s_loss_sq, s_losses, s_xpad, s_meta, s_xperm;
@@ -169,8 +169,10 @@ int ensure_route(moe_layer* L, int T) {
   if ((rc = grow(L, L->ws->ratio, (size_t)T * 4))) return rc;
   if ((rc = grow(L, L->ws->skipped, align_up((size_t)T, 16)))) return rc;
   if ((rc = grow(L, L->ws->pair_pos, (size_t)T * 8))) return rc;
-  if ((rc = grow(L, L->ws->blk_hist, nblk * kHistCols * 4))) return rc;
-  if ((rc = grow(L, L->ws->blk_base, nblk * kMaxE * 4))) return rc;
+  if (T > kPermuteOwnT) {  // the others count for themselves
+    if ((rc = grow(L, L->ws->blk_hist, nblk * kHistCols * 4))) return rc;
+    if ((rc = grow(L, L->ws->blk_base, nblk * kMaxE * 4))) return rc;
+  }
   L->ws->cap_route_T = T;
   return MOE_OK;
 }
@@ -215,7 +217,6 @@ int ensure_gemm(moe_layer* L, int T, int k = 2) {
   if (need < L->ws->cap_rows) need = L->ws->cap_rows;
   int rc;
   L->ws->cap_rows = 0;  // void until every buffer has grown and the tensor maps are rebuilt
-  if ((rc = grow(L, L->ws->row_token, (size_t)need * 4))) return rc;
   if ((rc = grow(L, L->ws->xperm, (size_t)need * L->h * 2))) return rc;
   if ((rc = grow(L, L->ws->act, (size_t)need * L->f * 2))) return rc;
   if ((rc = grow(L, L->ws->O, need_O * 4))) return rc;
@@ -412,7 +413,7 @@ int forward_impl(moe_layer* L, const void* x, int T, float beta, const void* res
     // one token: routing inside the gate/up matrix-vector kernel; the second kernel also forms
     // the weighted sum and writes y
     CUDA_TRY(launch_gemv_route_gate_up((const bf16*)x, L->Wg, L->W13, L->r, L->h, L->f, beta, L->kept, ro,
-                                       meta, (int32_t*)L->ws->pair_pos.p, (int32_t*)L->ws->row_token.p,
+                                       meta, (int32_t*)L->ws->pair_pos.p,
                                        s_count, s_nsk, s_nt, L->E, (bf16*)L->ws->act.p, st));
     mark(L);
     CUDA_TRY(launch_gemv_down_combine((const bf16*)L->ws->act.p, L->W2, ro.idx, ro.skipped, ro.wn,
@@ -423,12 +424,12 @@ int forward_impl(moe_layer* L, const void* x, int T, float beta, const void* res
   }
   if (T == 1) {
     CUDA_TRY(launch_route_single((const bf16*)x, L->Wg, L->h, L->r, beta, L->kept, ro, 16, meta,
-                                 (int32_t*)L->ws->pair_pos.p, (int32_t*)L->ws->row_token.p,
+                                 (int32_t*)L->ws->pair_pos.p,
                                  (bf16*)L->ws->xperm.p, s_count, s_nsk, s_nt, L->E, st));
   } else if (dec) {
     CUDA_TRY(launch_router_small((const bf16*)x, L->Wg, T, L->h, L->r, beta, L->kept, ro, st));
     CUDA_TRY(launch_permute_gather_small((const bf16*)x, ro.idx, ro.skipped, T, L->h, L->r, 16, meta,
-                                         (int32_t*)L->ws->pair_pos.p, (int32_t*)L->ws->row_token.p,
+                                         (int32_t*)L->ws->pair_pos.p,
                                          (bf16*)L->ws->xperm.p, s_count, s_nsk, s_nt, L->kept, L->E, st));
   } else {
     const bool own = T <= kPermuteOwnT;
@@ -602,7 +603,7 @@ void moe_layer_destroy(moe_layer_t* L) {
   if (!L) return;
   cudaStreamSynchronize(L->stream);
   Buf* bufs[] = {&L->own.idx, &L->own.wn, &L->own.ratio, &L->own.skipped, &L->own.blk_hist, &L->own.blk_base, &L->own.pair_pos,
-                 &L->own.meta, &L->own.status, &L->own.sel, &L->own.row_token, &L->own.xperm, &L->own.act, &L->own.O, &L->own.tail,
+                 &L->own.meta, &L->own.status, &L->own.sel, &L->own.xperm, &L->own.act, &L->own.O, &L->own.tail,
                  &L->own.s_logits, &L->own.s_yall, &L->own.s_act, &L->own.s_subsets, &L->own.s_partial, &L->own.s_loss_sq,
                  &L->own.s_losses, &L->own.s_xpad, &L->own.s_meta, &L->own.s_xperm, &L->own.hx, &L->own.hy, &L->own.xn, &L->own.cosel, &L->own.k_idx, &L->own.k_wn, &L->own.k_pos, &L->own.k_nact};
   for (Buf* b : bufs) release(L, *b);
@@ -664,6 +665,14 @@ int moe_test_large_batch(moe_layer_t* L, int kernel, int tile_cap) {
   L->large_kernel = kernel;
   L->tile_cap = tile_cap;
   return MOE_OK;
+}
+
+const char* moe_layer_forward_kernel(const moe_layer_t* L, int T) {
+  if (!L || T < 1) return "";
+  if (L->debug_simt) return "simt_gate_up_kernel";
+  if (T == 1 && L->single_gemv) return "gemv_route_gate_up_kernel";
+  if (decode_mode(T)) return decode_weights_m(L, T) ? "gemm_weights_m_kernel" : "gemm_tokens_d_kernel";
+  return large_on_pairs(L, 2ll * T) ? "gemm_pair_n_kernel" : "gemm_tokens_m_kernel";
 }
 
 size_t moe_layer_weight_bytes(const moe_layer_t* L) { return L ? L->weight_bytes : 0; }

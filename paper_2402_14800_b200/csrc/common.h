@@ -14,14 +14,14 @@ typedef __nv_bfloat16 bf16;
 
 constexpr int kMaxE = MOE_MAX_EXPERTS;
 constexpr int kTileRows = 128;            // token rows per row tile of the grouped GEMMs
-constexpr int kRouteTokPerBlock = 16;     // tokens routed by one block (one warp per token)
+constexpr int kRouteTokPerBlock = 16;     // tokens of a unit: a row of the routers' histogram, a block of the permutation
 constexpr int kHistCols = 2 * kMaxE + 1;  // per (expert, slot) pair counts + skipped count
 constexpr int kInterleave = 16;           // W1/W3 rows are interleaved in groups of 16
 constexpr int kDecodeMaxT = 256;          // up to here the small-batch path (weights read once) is used
 constexpr int kTokensDPerExpert = 40;      // small batches with this many tokens per expert or more: token-major decode GEMM
 constexpr int kTokensDMaxKept = 6;         // ... on layers with at most this many kept experts
-// Large batches with at most this many pairs per kept expert run gemm_pair_n, the others
-// gemm_tokens_m.  Alternating 1.5 s runs at the power cap, Mixtral layer, 8 experts (gemm_tokens_m
+// Large batches with at most this many pairs per kept expert (a forward call counts two per token, skipped
+// or not) run gemm_pair_n, the others gemm_tokens_m.  Alternating 1.5 s runs at the power cap, Mixtral layer, 8 experts (gemm_tokens_m
 // vs gemm_pair_n, whole step): 1500 tokens 1.30 vs 1.17 ms, 2500 1.85 vs 1.70, 3500 2.40 vs 2.28,
 // 5000 3.23 vs 3.16; at 8192 (2048 a group) -1.5 .. +1.8 % depending on the board, and the search's
 // 6144 a group was up to 6 % slower on the pairs: with little padding to save, both are held by the
@@ -52,14 +52,13 @@ constexpr int kRouterTcT = 64 * 128;
 constexpr int kRouterTcH = 2048;
 constexpr int kDecodeKbPerItem = 112;      // k-blocks (of 64) per split-K item, decode down-proj
 
-// Device-resident description of one permuted batch, written by the scan kernel
-// (or by set_dense_meta for the search) and read by every later kernel.
+// Device-resident description of one permuted batch, written by the permutation (beyond kPermuteOwnT
+// tokens by the scan, for the dense search by set_dense_meta) and read by every later kernel.
 struct Meta {
   int32_t count[kMaxE];            // token-expert pairs that run, per kept expert (compact index)
   int32_t count_slot[kMaxE][2];    // the same, split by top-2 slot
   int32_t off[kMaxE + 1];          // first permuted row of each expert's group (padded groups)
   int32_t tile_prefix[kMaxE + 1];  // cumulative number of 128-row tiles
-  int32_t rows_total;              // off[r]
   int32_t n_skipped;
   int32_t n_touched;
   int32_t reserved;
@@ -163,11 +162,11 @@ cudaError_t launch_router_small(const bf16* x, const bf16* Wg, int T, int h, int
                                 const KeptIds& kept, const RouteOut& out, cudaStream_t st);
 cudaError_t launch_route_single(const bf16* x, const bf16* Wg, int h, int r, float beta,
                                 const KeptIds& kept, const RouteOut& out, int pad, Meta* meta,
-                                int32_t* pair_pos, int32_t* row_token, bf16* xperm, int32_t* s_count,
+                                int32_t* pair_pos, bf16* xperm, int32_t* s_count,
                                 int32_t* s_nskipped, int32_t* s_ntouched, int E, cudaStream_t st);
 cudaError_t launch_permute_gather_small(const bf16* x, const int32_t* idx, const uint8_t* skipped, int T,
                                         int h, int r, int pad, Meta* meta, int32_t* pair_pos,
-                                        int32_t* row_token, bf16* xperm, int32_t* s_count,
+                                        bf16* xperm, int32_t* s_count,
                                         int32_t* s_nskipped, int32_t* s_ntouched, const KeptIds& kept,
                                         int E, cudaStream_t st);
 cudaError_t launch_scan(const int32_t* blk_hist, int nblk, int r, int pad, int32_t* blk_base,
@@ -260,7 +259,7 @@ cudaError_t gemv_single_setup();
 bool gemv_single_fits(int h, int f);
 cudaError_t launch_gemv_route_gate_up(const bf16* x, const bf16* Wg, const bf16* W13, int r, int h, int f,
                                       float beta, const KeptIds& kept, const RouteOut& ro, Meta* meta,
-                                      int32_t* pair_pos, int32_t* row_token, int32_t* s_count,
+                                      int32_t* pair_pos, int32_t* s_count,
                                       int32_t* s_nskipped, int32_t* s_ntouched, int E, bf16* act,
                                       cudaStream_t st);
 cudaError_t launch_gemv_down_combine(const bf16* act, const bf16* W2, const int32_t* idx,

@@ -3,7 +3,8 @@
 //
 //   E_e(x) = W2_e ( silu(W1_e x) * (W3_e x) )      (Sec. 3.1; Mixtral's SwiGLU form)
 //
-// Four persistent, warp-specialised kernels share one pipeline skeleton:
+// Four persistent, warp-specialised kernels share one pipeline skeleton (and so does router_tc, the router
+// of the largest batches):
 //   gemm_tokens_m   256 token rows x 256 weight rows per item on two accumulators; for the largest
 //                   batches, where the work is a dense contraction bound by the tensor pipe.
 //   gemm_pair_n     512 weight rows x (32..256) tokens per item on a pair of CTAs; for batches
@@ -1020,7 +1021,10 @@ struct SchedW {
 
 constexpr int kMinSliceKb = 4;                     // a slice covers at least this many k-blocks
 // Contractions of fewer k-blocks are never sliced: leaving, counting and folding the partial tiles takes
-// longer than the whole sum (tiny layer, 7 k-blocks, 256 tokens: down stage 22.4 -> 11.5 us).
+// longer than the whole sum (tiny layer, 7 k-blocks, 256 tokens: down stage 22.4 -> 11.5 us).  Whole call with
+// the rule and the changes made together with it, 24 and 256 tokens: h 704, f 832 (11 and 13 k-blocks) 29.0 ->
+// 22.9 us and 48.1 -> 30.2, h 960, f 960 (15) 30.3 -> 24.9 and 49.9 -> 31.8; h 1024, f 2048 (16 and 32, sliced
+// before and after) 48.2 -> 47.2 and 76.8 -> 68.5.
 constexpr int kMinSlicedKb = 16;
 constexpr int kSliceFixedKb = 6;                   // modelled fixed cost of a slice, in k-blocks
 constexpr int kFoldLoads = 512;                    // tokens x slices one thread adds up at most

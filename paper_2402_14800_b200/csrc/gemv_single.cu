@@ -55,7 +55,7 @@ constexpr int kDnThreads = 896;  // one block per SM (148 x 28 warps cover 4096 
 struct SingleOut {
   RouteOut ro;
   Meta* meta;
-  int32_t *pair_pos, *row_token, *s_count, *s_nskipped, *s_ntouched;
+  int32_t *pair_pos, *s_count, *s_nskipped, *s_ntouched;
   int E;
 };
 
@@ -107,7 +107,7 @@ gemv_route_gate_up_kernel(const bf16* __restrict__ x, const bf16* __restrict__ W
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     route_decide<R>(l, r, beta, 0, kept, out.ro, e0, e1, skip);
     int p0, p1;
-    publish_single(e0, skip ? -1 : e1, 16, kept, out.meta, out.pair_pos, out.row_token, out.s_count,
+    publish_single(e0, skip ? -1 : e1, 16, kept, out.meta, out.pair_pos, out.s_count,
                    out.s_nskipped, out.s_ntouched, out.E, p0, p1);
   } else {
     float w0, w1, p1;
@@ -215,12 +215,12 @@ bool gemv_single_fits(int h, int f) { return (size_t)h * 2 <= 48 * 1024 && (size
 
 cudaError_t launch_gemv_route_gate_up(const bf16* x, const bf16* Wg, const bf16* W13, int r, int h, int f,
                                       float beta, const KeptIds& kept, const RouteOut& ro, Meta* meta,
-                                      int32_t* pair_pos, int32_t* row_token, int32_t* s_count,
+                                      int32_t* pair_pos, int32_t* s_count,
                                       int32_t* s_nskipped, int32_t* s_ntouched, int E, bf16* act,
                                       cudaStream_t st) {
   const int sms = g_sms > 0 ? g_sms : 148;
   SingleOut out;
-  out.ro = ro; out.meta = meta; out.pair_pos = pair_pos; out.row_token = row_token;
+  out.ro = ro; out.meta = meta; out.pair_pos = pair_pos;
   out.s_count = s_count; out.s_nskipped = s_nskipped; out.s_ntouched = s_ntouched; out.E = E;
 #define MOE_GEMV_ROUTE(R)                                                                            \
   return launch_pdl(gemv_route_gate_up_kernel<R>, dim3(2 * sms), dim3(kGuThreads), (size_t)h * 2, st, x, \

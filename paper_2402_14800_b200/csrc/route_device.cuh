@@ -73,7 +73,7 @@ __device__ __forceinline__ void route_decide(const float (&acc)[R], int r, float
 // Batch description of a single token (one thread): one permuted row for e0, one for e1 unless
 // it was skipped (e1 < 0); p0 / p1 return those rows (p1 = -1 after a skip).
 __device__ __forceinline__ void publish_single(int e0, int e1, int pad, const KeptIds& kept, Meta* meta,
-                                               int32_t* pair_pos, int32_t* row_token, int32_t* s_count,
+                                               int32_t* pair_pos, int32_t* s_count,
                                                int32_t* s_nskipped, int32_t* s_ntouched, int E, int& p0,
                                                int& p1) {
   const bool skip = e1 < 0;
@@ -95,14 +95,11 @@ __device__ __forceinline__ void publish_single(int e0, int e1, int pad, const Ke
     meta->off[c + 1] = off;
     meta->tile_prefix[c + 1] = tiles;
   }
-  meta->rows_total = off;
   meta->n_skipped = skip ? 1 : 0;
   meta->n_touched = skip ? 1 : 2;
   meta->reserved = 0;
   pair_pos[0] = p0;
   pair_pos[1] = p1;
-  row_token[p0] = 0;
-  if (!skip) row_token[p1] = 0;
   if (s_count) {
     for (int e = 0; e < E; ++e) { s_count[2 * e] = 0; s_count[2 * e + 1] = 0; }
     s_count[2 * kept.id[e0]] = 1;

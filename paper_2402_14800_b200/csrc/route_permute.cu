@@ -77,7 +77,7 @@ template <int R>
 __global__ void __launch_bounds__(256)
 route_single_kernel(const bf16* x, const bf16* __restrict__ Wg, int h, int r, float beta,
                     KeptIds kept, RouteOut o, int pad, Meta* meta, int32_t* __restrict__ pair_pos,
-                    int32_t* __restrict__ row_token, bf16* __restrict__ xperm, int32_t* s_count,
+                    bf16* __restrict__ xperm, int32_t* s_count,
                     int32_t* s_nskipped, int32_t* s_ntouched, int E) {
   pdl_launch_dependents();
   pdl_wait();
@@ -122,7 +122,7 @@ route_single_kernel(const bf16* x, const bf16* __restrict__ Wg, int h, int r, fl
     bool skip;
     route_decide<R>(l, r, beta, 0, kept, o, e0, e1, skip);
     if (skip) e1 = -1;
-    publish_single(e0, e1, pad, kept, meta, pair_pos, row_token, s_count, s_nskipped, s_ntouched, E,
+    publish_single(e0, e1, pad, kept, meta, pair_pos, s_count, s_nskipped, s_ntouched, E,
                    s_p[0], s_p[1]);
   }
   __syncthreads();
@@ -145,7 +145,7 @@ route_single_kernel(const bf16* x, const bf16* __restrict__ Wg, int h, int r, fl
 __global__ void __launch_bounds__(kDecodeMaxT)
 permute_gather_small_kernel(const bf16* x, const int32_t* idx, const uint8_t* skipped, int T, int h, int r, int pad,
                             Meta* meta, int32_t* __restrict__ pair_pos,
-                            int32_t* __restrict__ row_token, bf16* __restrict__ xperm,
+                            bf16* __restrict__ xperm,
                             int32_t* s_count, int32_t* s_nskipped, int32_t* s_ntouched, KeptIds kept,
                             int E) {
   pdl_launch_dependents();
@@ -193,7 +193,6 @@ permute_gather_small_kernel(const bf16* x, const int32_t* idx, const uint8_t* sk
       const int p = lane == 0 ? p0 : (f1 < 0 ? -1 : p1);
       s_p[lane] = p;
       pair_pos[2 * t + lane] = p;
-      if (p >= 0) row_token[p] = t;
     }
     if (t == 0) {
       const int pairs = __reduce_add_sync(0xffffffffu, cnt);
@@ -211,7 +210,6 @@ permute_gather_small_kernel(const bf16* x, const int32_t* idx, const uint8_t* sk
       if (lane == kMaxE - 1) {
         meta->off[0] = 0;
         meta->tile_prefix[0] = 0;
-        meta->rows_total = end;
         meta->n_skipped = 2 * T - pairs;
         meta->n_touched = touched;
         meta->reserved = 0;
@@ -306,7 +304,7 @@ template <int R, bool FOLD> struct RouteCfg {
   static constexpr int kRP = R <= 2 ? 2 : (R <= 4 ? 4 : (R <= 8 ? 8 : 16));
   static constexpr int kTB = R <= 8 && !FOLD ? 4 : 2;
   static constexpr int kN = kRP * kTB;
-  static constexpr int kTeamWarps = kRouteTokPerBlock / kTB;
+  static constexpr int kTeamWarps = kRouteTokPerBlock / kTB;  // (teams: router_kernel only)
   static constexpr int kTeams = kRouteWarps / kTeamWarps;
   static constexpr size_t kRingBytes = (size_t)kRouteWarps * kRouteStages * kTB * 32 * 16;
 };
@@ -588,7 +586,6 @@ scan_kernel(const int32_t* blk_hist, int nblk, int r, int pad,
       meta->off[c + 1] = off;
       meta->tile_prefix[c + 1] = tiles;
     }
-    meta->rows_total = off;
     meta->n_skipped = s_skipped;
     meta->n_touched = touched;
     meta->reserved = 0;
@@ -708,8 +705,7 @@ permute_kernel(const bf16* x, const int32_t* idx, const void* active, int T, int
         if (lane == kMaxE - 1) {
           meta->off[0] = 0;
           meta->tile_prefix[0] = 0;
-          meta->rows_total = end;
-          meta->n_skipped = T * k - pairs;
+            meta->n_skipped = T * k - pairs;
           meta->n_touched = touched;
           meta->reserved = 0;
           if (s_count) { *s_nskipped = T * k - pairs; *s_ntouched = touched; }
@@ -1072,7 +1068,6 @@ __global__ void set_dense_meta_kernel(Meta* meta, int E, int rows, int off_strid
       meta->count_slot[c][1] = 0;
     }
   }
-  meta->rows_total = E * off_stride;
   meta->n_skipped = 0;
   meta->n_touched = E;
   meta->reserved = 0;
@@ -1242,11 +1237,11 @@ cudaError_t launch_router_small(const bf16* x, const bf16* Wg, int T, int h, int
 
 cudaError_t launch_route_single(const bf16* x, const bf16* Wg, int h, int r, float beta,
                                 const KeptIds& kept, const RouteOut& out, int pad, Meta* meta,
-                                int32_t* pair_pos, int32_t* row_token, bf16* xperm, int32_t* s_count,
+                                int32_t* pair_pos, bf16* xperm, int32_t* s_count,
                                 int32_t* s_nskipped, int32_t* s_ntouched, int E, cudaStream_t st) {
 #define MOE_ROUTE_SINGLE(R)                                                                        \
   return launch_pdl(route_single_kernel<R>, dim3(1), dim3(256), 0, st, x, Wg, h, r, beta, kept, out, \
-                    pad, meta, pair_pos, row_token, xperm, s_count, s_nskipped, s_ntouched, E)
+                    pad, meta, pair_pos, xperm, s_count, s_nskipped, s_ntouched, E)
   switch (r) {
     case 2: MOE_ROUTE_SINGLE(2);
     case 3: case 4: MOE_ROUTE_SINGLE(4);
@@ -1259,11 +1254,11 @@ cudaError_t launch_route_single(const bf16* x, const bf16* Wg, int h, int r, flo
 
 cudaError_t launch_permute_gather_small(const bf16* x, const int32_t* idx, const uint8_t* skipped, int T,
                                         int h, int r, int pad, Meta* meta, int32_t* pair_pos,
-                                        int32_t* row_token, bf16* xperm, int32_t* s_count,
+                                        bf16* xperm, int32_t* s_count,
                                         int32_t* s_nskipped, int32_t* s_ntouched, const KeptIds& kept,
                                         int E, cudaStream_t st) {
   return launch_pdl(permute_gather_small_kernel, dim3(T), dim3(kDecodeMaxT), 0, st, x, idx, skipped, T, h,
-                    r, pad, meta, pair_pos, row_token, xperm, s_count, s_nskipped, s_ntouched, kept, E);
+                    r, pad, meta, pair_pos, xperm, s_count, s_nskipped, s_ntouched, kept, E);
 }
 
 cudaError_t launch_scan(const int32_t* blk_hist, int nblk, int r, int pad, int32_t* blk_base,

@@ -634,3 +634,14 @@ def test_large_batch_hook_rejects_what_it_does_not_know(weights):
         assert lib.moe_test_large_batch(layer._h, kernel, cap) == -1
     assert lib.moe_test_large_batch(None, 0, 0) == -1
     layer.close()
+
+
+def test_forward_kernel_names_the_kernel_that_runs(weights):
+    eight, four = binding.MoeLayer(*weights), binding.MoeLayer(*weights, 0x0F)
+    names = [(eight, 1, "gemv_route_gate_up_kernel"), (eight, 2, "gemm_weights_m_kernel"), (eight, 256, "gemm_weights_m_kernel"),
+             (four, 79, "gemm_weights_m_kernel"), (four, 80, "gemm_tokens_d_kernel"), (four, 257, "gemm_pair_n_kernel"),
+             (eight, 6144, "gemm_pair_n_kernel"), (eight, 6145, "gemm_tokens_m_kernel"), (eight, 0, "")]
+    for layer, T, name in names:
+        assert layer.forward_kernel(T) == name, T
+    eight.close()
+    four.close()
