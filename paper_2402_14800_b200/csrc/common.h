@@ -21,11 +21,11 @@ constexpr int kDecodeMaxT = 256;          // up to here the small-batch path (we
 constexpr int kTokensDPerExpert = 40;      // small batches with this many tokens per expert or more: token-major decode GEMM
 constexpr int kTokensDMaxKept = 6;         // ... on layers with at most this many kept experts
 // Large batches with at most this many pairs per kept expert (a forward call counts two per token, skipped
-// or not) run gemm_pair_n, the others gemm_tokens_m.  Alternating 1.5 s runs at the power cap, Mixtral layer, 8 experts (gemm_tokens_m
-// vs gemm_pair_n, whole step): 1500 tokens 1.30 vs 1.17 ms, 2500 1.85 vs 1.70, 3500 2.40 vs 2.28,
-// 5000 3.23 vs 3.16; at 8192 (2048 a group) -1.5 .. +1.8 % depending on the board, and the search's
-// 6144 a group was up to 6 % slower on the pairs: with little padding to save, both are held by the
-// board's power and the pairs draw 1-3 % more energy per call.
+// or not) run gemm_pair_n, the others gemm_tokens_m.  Alternating 1.5 s runs at the power cap, Mixtral
+// layer, 8 experts (gemm_tokens_m vs gemm_pair_n, whole step): 1500 tokens 1.30 vs 1.17 ms, 2500 1.85 vs
+// 1.70, 3500 2.40 vs 2.28, 5000 3.23 vs 3.16; at 8192 (2048 a group) -1.5 .. +1.8 % depending on the board,
+// and the search's 6144 a group was up to 6 % slower on the pairs: with little padding to save, both are
+// held by the board's power and the pairs draw 1-3 % more energy per call.
 constexpr int kPairMaxRows = 1536;
 // Top-k calls of more than kDecodeMaxT tokens with at most this many pairs per kept expert, half of the
 // weight-major kernel's token tile, run that kernel: it cuts the last round into K-slices, and hardly any

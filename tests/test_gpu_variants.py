@@ -335,7 +335,7 @@ def test_large_batch_gemm_at_the_edges_of_its_tiles(h, f, E, kept, T):
     (64, 64, 3, 0b111, 257, 2), (576, 64, 5, 0b11111, 300, 3), (128, 64, 16, 0xFFFF, 513, 5),
     (8192, 64, 13, 0x1FFF, 300, 4), (128, 64, 13, 0x1FFF, 8193, 3), (128, 64, 2, 0b11, 9001, 2),
     (320, 64, 12, 0b111111111111, 8192, 8),
-    # top-k calls with few pairs per expert (weight-major GEMM beyond 256 tokens), K-sliced and not
+    # top-k calls just above the 64 pairs per expert up to which the weight-major GEMM runs beyond 256 tokens
     (128, 64, 16, 0xFFFF, 300, 4), (1024, 256, 16, 0xFFFF, 270, 4),
 ])
 def test_routing_and_permutation_of_large_batches_equal_small_ones(h, f, E, kept, T, k):
