@@ -3,6 +3,8 @@
 //   router_kernel   Sec. 3.1 (logits, softmax, top-2, Eq. 1), Sec. 3.2 (kept experts only),
 //                   Sec. 3.3 (skip test), App. A.2 (weight 1 after a skip); several tokens per warp
 //                   (large forward batches: router_tc_kernel, on the tensor cores).
+//   ratio_kernel    Sec. 3.3: w_e1 / w_e0 for calibration, on warp-level tensor-core instructions, as
+//                   router_topk_kernel (App. A.2).
 //   scan / permute  stable counting sort of the token-expert pairs that run, by expert (no atomics,
 //                   the order is a function of the routing alone), and the copy of the routed rows
 //                   of x into that order.
@@ -230,11 +232,12 @@ permute_gather_small_kernel(const bf16* x, const int32_t* idx, const uint8_t* sk
   }
 }
 
-// Batches of more than kDecodeMaxT tokens: a warp takes the logits of TB tokens.  A lane walks the
+// Forward batches of more than kDecodeMaxT tokens (up to kRouterTcT on wide rows), and calibration on narrow rows: a
+// warp takes the logits of TB tokens.  A lane walks the
 // same 8-element slices of the TB rows and of the router rows, so a slice of a router row is read
 // and unpacked once for TB tokens; the products of two tokens go through one fma.rn.f32x2.  A logit
 // is one chain of fused multiply-adds per lane (slices, then elements, in order) and a butterfly over
-// the lanes (top-k: shorter chains, see FOLD), whatever the batch and the tokens beside it.
+// the lanes, whatever the batch and the tokens beside it.
 //   - The router rows are copied to shared memory once per block, before the wait for the
 //     predecessor (they never change), where they fit beside the ring: read through L1 they cost a
 //     chain of L2 round trips per slice, 62 us for 611 tokens.  Longer rows (beyond h = 5824 with 8
@@ -258,9 +261,6 @@ __device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
 }
 __device__ __forceinline__ void fma_f32x2(uint64_t& acc, uint64_t a, uint64_t b) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ void add_f32x2(uint64_t& acc, uint64_t a) {
-  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc) : "l"(a));
 }
 __device__ __forceinline__ void split_f32x2(uint64_t v, float& lo, float& hi) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
@@ -300,11 +300,11 @@ __device__ __forceinline__ float reduce_scatter(const float (&v)[N], int lane) {
 // a block of 16 warps is several teams, and the blocks go round until the tokens are done.
 constexpr int kRouteStages = 4;
 constexpr int kRouteWarps = 16;
-template <int R, bool FOLD> struct RouteCfg {
+template <int R> struct RouteCfg {
   static constexpr int kRP = R <= 2 ? 2 : (R <= 4 ? 4 : (R <= 8 ? 8 : 16));
-  static constexpr int kTB = R <= 8 && !FOLD ? 4 : 2;
+  static constexpr int kTB = R <= 8 ? 4 : 2;
   static constexpr int kN = kRP * kTB;
-  static constexpr int kTeamWarps = kRouteTokPerBlock / kTB;  // (teams: router_kernel only)
+  static constexpr int kTeamWarps = kRouteTokPerBlock / kTB;
   static constexpr int kTeams = kRouteWarps / kTeamWarps;
   static constexpr size_t kRingBytes = (size_t)kRouteWarps * kRouteStages * kTB * 32 * 16;
 };
@@ -312,8 +312,8 @@ constexpr size_t kRouteSmemMax = 227 * 1024 - 8 * 1024;  // dynamic part; the re
 
 // 16-byte vectors of a router row that shared memory holds at a time: the whole row, or a part of it (a
 // whole number of slices; at least 9 for every R) of which two fit.
-template <int R, bool FOLD> inline int route_part(int h, int r) {
-  const size_t room = kRouteSmemMax - RouteCfg<R, FOLD>::kRingBytes;
+template <int R> inline int route_part(int h, int r) {
+  const size_t room = kRouteSmemMax - RouteCfg<R>::kRingBytes;
   if ((size_t)r * h * 2 <= room) return h >> 3;
   return (int)(room / 2 / ((size_t)r * 512)) * 32;
 }
@@ -338,17 +338,11 @@ __device__ __forceinline__ void fetch_router_part(uint4* dst, const bf16* Wg, in
 // first of which is in `half` or on its way there, and all warps of the block call this together, those
 // that have no tokens (t0 >= T) to fetch their shares of the parts; the first part comes round again
 // behind the last one, for the next call.
-// FOLD: shorter chains.  The sum of every kRouteFold slices is closed and added to a second one, and that
-// is closed over the lanes every kRouteSpan vectors: no chain is longer than 16 products, 8 sums or
-// h / 4096 totals.  Error of the weights of 4 experts against 64 bits (2-norm, 2000 tokens) without / with it
-// (h 2048, 16 experts) 1.49e-7 / 1.31e-7, (h 4096, 8 experts) 1.54e-7 / 1.23e-7; 2 tokens per warp instead of 4
-// make room for the second sums (with 4: call of 8 tokens, h 6144, 80 -> 86 us; with 2, 75).
-constexpr int kRouteFold = 2, kRouteSpan = 512;
-template <int R, bool WHOLE, bool FOLD>
+template <int R, bool WHOLE>
 __device__ __forceinline__ float warp_logits(const bf16* x, uint4* s_w, const bf16* Wg, int part, int& half,
                                              int t0, int T, int h, int r, uint4* ring) {
   const bool on = WHOLE || t0 < T;
-  constexpr int RP = RouteCfg<R, FOLD>::kRP, TB = RouteCfg<R, FOLD>::kTB, N = RouteCfg<R, FOLD>::kN;
+  constexpr int RP = RouteCfg<R>::kRP, TB = RouteCfg<R>::kTB, N = RouteCfg<R>::kN;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nvec = h >> 3;
   uint64_t acc[TB / 2][R];  // two tokens each
@@ -356,18 +350,6 @@ __device__ __forceinline__ float warp_logits(const bf16* x, uint4* s_w, const bf
   for (int i = 0; i < TB / 2; ++i)
 #pragma unroll
     for (int c = 0; c < R; ++c) acc[i][c] = 0ull;
-  uint64_t tot[FOLD ? TB / 2 : 1][FOLD ? R : 1];
-  int open = 0;  // slices in acc
-  auto fold = [&]() {
-#pragma unroll
-    for (int i = 0; i < TB / 2; ++i)
-#pragma unroll
-      for (int c = 0; c < R; ++c) {
-        add_f32x2(tot[FOLD ? i : 0][FOLD ? c : 0], acc[i][c]);
-        acc[i][c] = 0ull;
-      }
-    open = 0;
-  };
   const uint4* xr[TB];
 #pragma unroll
   for (int i = 0; i < TB; ++i) xr[i] = reinterpret_cast<const uint4*>(x + (size_t)min(t0 + i, T - 1) * h) + lane;
@@ -383,79 +365,63 @@ __device__ __forceinline__ float warp_logits(const bf16* x, uint4* s_w, const bf
   for (int s = 0; s < kRouteStages - 1; ++s) fetch(32 * s, s);
   int s = 0, left = 0;  // vectors of the present part still to come
   const uint4* w = s_w + lane;
-  float sum = 0.f;
 #pragma unroll 1
-  for (int v1 = 0; v1 < nvec; v1 += FOLD ? kRouteSpan : nvec) {
-    const int v2 = FOLD ? min(nvec, v1 + kRouteSpan) : nvec;
-    if (FOLD) {
-#pragma unroll
-      for (int i = 0; i < TB / 2; ++i)
-#pragma unroll
-        for (int c = 0; c < R; ++c) tot[FOLD ? i : 0][FOLD ? c : 0] = 0ull;
+  for (int v = 0; v < nvec; v += 32, left -= 32) {
+    cp_async_wait<kRouteStages - 2>();
+    if (!WHOLE && left <= 0) {
+      // this part was fetched with or before a token slice that has arrived; no warp reads the other half now
+      __syncthreads();
+      w = s_w + half * r * part + lane - v;
+      half ^= 1;
+      left = part;
+      const int next = v + part < nvec ? v + part : 0;
+      fetch_router_part<WHOLE>(s_w + half * r * part, Wg, next, part, nvec, r);  // committed with the slice below
     }
-#pragma unroll 1
-    for (int v = v1; v < v2; v += 32, left -= 32) {
-      cp_async_wait<kRouteStages - 2>();
-      if (!WHOLE && left <= 0) {
-        // this part was fetched with or before a token slice that has arrived; no warp reads the other half now
-        __syncthreads();
-        w = s_w + half * r * part + lane - v;
-        half ^= 1;
-        left = part;
-        const int next = v + part < nvec ? v + part : 0;
-        fetch_router_part<WHOLE>(s_w + half * r * part, Wg, next, part, nvec, r);  // committed with the slice below
-      }
-      if (!on) {
-        cp_async_commit();
-        continue;
-      }
-      uint64_t xf[TB / 2][8];
+    if (!on) {
+      cp_async_commit();
+      continue;
+    }
+    uint64_t xf[TB / 2][8];
 #pragma unroll
-      for (int i = 0; i < TB / 2; ++i) {
-        float lo[8], hi[8];
-        unpack8(mine[(s * TB + 2 * i) * 32], lo);
-        unpack8(mine[(s * TB + 2 * i + 1) * 32], hi);
+    for (int i = 0; i < TB / 2; ++i) {
+      float lo[8], hi[8];
+      unpack8(mine[(s * TB + 2 * i) * 32], lo);
+      unpack8(mine[(s * TB + 2 * i + 1) * 32], hi);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) xf[i][e] = pack_f32x2(lo[e], hi[e]);
-      }
-      fetch(v + 32 * (kRouteStages - 1), s == 0 ? kRouteStages - 1 : s - 1);
-      if (v + lane < nvec) {
-        constexpr int kBatch = 2;  // router slices in flight
+      for (int e = 0; e < 8; ++e) xf[i][e] = pack_f32x2(lo[e], hi[e]);
+    }
+    fetch(v + 32 * (kRouteStages - 1), s == 0 ? kRouteStages - 1 : s - 1);
+    if (v + lane < nvec) {
+      constexpr int kBatch = 2;  // router slices in flight
 #pragma unroll
-        for (int c0 = 0; c0 < R; c0 += kBatch) {
-          uint4 wv[kBatch];
+      for (int c0 = 0; c0 < R; c0 += kBatch) {
+        uint4 wv[kBatch];
 #pragma unroll
-          for (int b = 0; b < kBatch; ++b) wv[b] = w[(size_t)min(c0 + b, r - 1) * (WHOLE ? nvec : part) + v];
+        for (int b = 0; b < kBatch; ++b) wv[b] = w[(size_t)min(c0 + b, r - 1) * (WHOLE ? nvec : part) + v];
 #pragma unroll
-          for (int b = 0; b < kBatch; ++b) {
-            if (c0 + b < R) {
-              float wf[8];
-              unpack8(wv[b], wf);
+        for (int b = 0; b < kBatch; ++b) {
+          if (c0 + b < R) {
+            float wf[8];
+            unpack8(wv[b], wf);
 #pragma unroll
-              for (int e = 0; e < 8; ++e)
+            for (int e = 0; e < 8; ++e)
 #pragma unroll
-                for (int i = 0; i < TB / 2; ++i)
-                  fma_f32x2(acc[i][c0 + b < R ? c0 + b : 0], xf[i][e], pack_f32x2(wf[e], wf[e]));
-            }
+              for (int i = 0; i < TB / 2; ++i)
+                fma_f32x2(acc[i][c0 + b < R ? c0 + b : 0], xf[i][e], pack_f32x2(wf[e], wf[e]));
           }
         }
       }
-      if (FOLD && ++open == kRouteFold) fold();
-      if (++s == kRouteStages) s = 0;
     }
-    if (FOLD) fold();
-    float val[N];
-#pragma unroll
-    for (int q = 0; q < N; ++q) val[q] = 0.f;
-#pragma unroll
-    for (int i = 0; i < TB / 2; ++i)
-#pragma unroll
-      for (int c = 0; c < R; ++c)
-        split_f32x2(FOLD ? tot[FOLD ? i : 0][FOLD ? c : 0] : acc[i][c], val[2 * i * RP + c], val[(2 * i + 1) * RP + c]);
-    const float got = reduce_scatter<N>(val, lane);
-    sum = v1 == 0 ? got : sum + got;
+    if (++s == kRouteStages) s = 0;
   }
-  return sum;
+  float val[N];
+#pragma unroll
+  for (int q = 0; q < N; ++q) val[q] = 0.f;
+#pragma unroll
+  for (int i = 0; i < TB / 2; ++i)
+#pragma unroll
+    for (int c = 0; c < R; ++c) split_f32x2(acc[i][c], val[2 * i * RP + c], val[(2 * i + 1) * RP + c]);
+  return reduce_scatter<N>(val, lane);
 }
 
 // Top-2 routing.
@@ -464,7 +430,7 @@ __global__ void __launch_bounds__(32 * kRouteWarps, 1)
 router_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part, float beta, KeptIds kept,
               RouteOut o, bool w_const) {
   pdl_launch_dependents();
-  using Cfg = RouteCfg<R, false>;
+  using Cfg = RouteCfg<R>;
   constexpr int RP = Cfg::kRP, TB = Cfg::kTB, N = Cfg::kN;
   extern __shared__ uint4 ring[];
   __shared__ float s_l[kRouteWarps][N];
@@ -485,7 +451,7 @@ router_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part, floa
   // with the rows in parts all warps of the block stay in step: a team goes on while the first has a unit
   for (int u = blockIdx.x + gridDim.x * team; u - (WHOLE ? 0 : (int)gridDim.x * team) < units; u += gridDim.x * Cfg::kTeams) {
     const int t0 = u * kRouteTokPerBlock;
-    const float mine = warp_logits<R, WHOLE, false>(x, s_w, Wg, part, half, t0 + tw * TB, T, h, r, ring);
+    const float mine = warp_logits<R, WHOLE>(x, s_w, Wg, part, half, t0 + tw * TB, T, h, r, ring);
     if (!WHOLE && u >= units) continue;
     if (lane % (32 / N) == 0) s_l[warp][lane / (32 / N)] = mine;
     __syncwarp();
@@ -520,6 +486,248 @@ router_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part, floa
     asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kTeamThreads) : "memory");
   }
   if (!WHOLE) cp_async_wait<0>();  // the first part, fetched once more behind the last
+}
+
+// Calibration on rows of kRatioMinH columns and more, the top-k and the search router: a team of TW warps takes
+// tiles of 8 NT tokens in turn, its warps sharing the columns of a row (blocks of 64 columns); a block of
+// kRouteWarps warps is one team or several.  The products of 16 columns of up to 16 tokens with 8 router rows are
+// one mma.sync.m16n8k16: a [T x h] x [h x 16] contraction is bound by reading the token rows, which a handful of
+// warp-level instructions keeps up with, and tokens go from global memory to the instruction's registers without
+// passing through shared or tensor memory (the order of the columns inside a block is free, so the 16 bytes of a
+// row that a lane reads are its operands of two instructions).  Whole calibration call, before (router_kernel) ->
+// after, us: h 4096, 8 experts, 300 tokens 23.5 -> 19.5, 8192 36 -> 28.5, 16384 56.5 -> 50.5 (3.9 TB/s from DRAM);
+// h 2048, 16 experts, 16384 tokens 60 -> 39.  With 4 experts router_kernel, which then has half the arithmetic, stays
+// ahead on batches that L2 does not hold (16384 tokens of h 4096 46.5 -> 50.5).  What is slower: one warp that decides
+// while the others wait (67 us at 16384 tokens), 8 tokens as the narrow operand (twice the instructions, 61), a column
+// phase of its own per block and deeper prefetch to L2 (no gain, and 58-60).
+//   - A logit: sums of 64 products by the tensor core, added up by each warp in column order and then over the
+//     warps, both as compensated fp32 sums (the tensor core drops bits that an IEEE addition would round, which
+//     costs little over 64 products and too much over a row).
+//   - The router rows wait in shared memory in operand order, fetched before the wait for the predecessor where
+//     they never change; rows too long for it (h beyond 10880 with 8 experts, 4416 with 16) are read at L2.
+//   - Up to 8 NT loads of 16 bytes per lane are in flight; a slot is refilled, from the next tile if need be, as
+//     soon as it is used.
+//   - After a tile's one barrier every warp of the team adds up and decides its share of the tokens.
+
+// d += A (16 tokens x 16 columns) B (16 columns x 8 router rows)
+__device__ __forceinline__ void mma_16x8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                         uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// Compensated sum: `lost` collects exactly what each addition drops (Knuth's two-sum), the sum is acc + lost.
+// Adding zero changes neither.
+__device__ __forceinline__ void add_compensated(float& acc, float& lost, float v) {
+  const float sum = __fadd_rn(acc, v), part = __fsub_rn(sum, acc);
+  lost = __fadd_rn(lost, __fadd_rn(__fsub_rn(acc, __fsub_rn(sum, part)), __fsub_rn(v, part)));
+  acc = sum;
+}
+// (an infinite sum has lost NaN)
+__device__ __forceinline__ float closed_sum(float acc, float lost) { return lost == lost ? acc + lost : acc; }
+
+constexpr int kRouteSlots = 4;  // blocks of 64 columns that a warp has in flight
+constexpr size_t kTileSmemMax = 227 * 1024 - 9 * 1024;  // dynamic part; the records are static
+// R = experts computed (>= r; 8 or 16), NT = groups of 8 tokens in a tile, TW = warps of a team
+template <int R, int NT, int TW> struct TileCfg {
+  static constexpr int kTeams = kRouteWarps / TW;
+  static constexpr int kPlanes = R > 8 ? 2 : 1;         // 8 router rows each
+  static constexpr int kTokens = 8 * NT;
+  static constexpr int kStride = R > 8 ? 20 : 12;       // floats per token: spreads the tokens over the banks
+  static constexpr int kPart = kTokens * kStride;       // floats a warp leaves, twice (sums, what they lost)
+  static constexpr size_t kPartBytes = (size_t)4 * kRouteWarps * kPart * 4;
+  static size_t w_bytes(int h) { return (size_t)((h + 63) / 64) * kPlanes * 1024; }
+  // a tile's decision: kRP lanes per token, kTPP tokens per pass, kLanes lanes with the same logit
+  static constexpr int kRP = R;
+  static constexpr int kTPW = kTokens > TW ? kTokens / TW : 1;  // tokens of a warp
+  static constexpr int kTPP = kTPW * kRP > 32 ? 32 / kRP : kTPW;
+  static constexpr int kLanes = 32 / (kTPP * kRP);
+};
+
+// 16 bytes of a token row, read at L2 (the rule beside launch_pdl); their 256 bytes are fetched to L2 along with them.
+// `once`: a batch that L2 does not hold; the lines in flight are not allocated in L1 either, which holds few of
+// them beside the shared memory (16384 / 32768 tokens of h 4096 from DRAM 53.5 / 87 -> 50.1 / 82.6 us; 8192 tokens,
+// from L2, 27.9 -> 30.9).
+__device__ __forceinline__ uint4 ld_row(const uint4* p, bool once) {
+  uint4 v;
+  if (once)
+    asm volatile("ld.relaxed.gpu.global.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  else
+    asm volatile("ld.global.cg.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+constexpr size_t kRouteOnceBytes = (size_t)96 << 20;
+template <int N> __device__ __forceinline__ void named_sync(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(N) : "memory");
+}
+// Calls decide(t0, n, mine) for all tokens, up to kTPP of them at a time (t0 .. t0 + n - 1; none if n <= 0), by a
+// converged warp: a lane brings the logit of token t0 + lane / kLanes / kRP and expert lane / kLanes % kRP (beyond
+// n and r: anything).
+// WHOLE: the router rows pass through shared memory.
+template <int R, int NT, int TW, bool WHOLE, class Decide>
+__device__ __forceinline__ void route_tiles(const bf16* x, const bf16* Wg, int T, int h, int r, bool w_const,
+                                            Decide&& decide) {
+  using Cfg = TileCfg<R, NT, TW>;
+  constexpr int PL = Cfg::kPlanes, S = Cfg::kStride, U = kRouteSlots;
+  constexpr int kMembers = 32 * TW;
+  extern __shared__ uint4 s_dyn[];
+  uint4* s_w = s_dyn + Cfg::kPartBytes / 16;        // [block of 64 columns][plane][half][lane]
+  const int team = threadIdx.x / kMembers, warp = threadIdx.x / 32 % TW;
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  float* s_part = reinterpret_cast<float*>(s_dyn) + team * 4 * TW * Cfg::kPart;  // [2][warp][sum, lost][token][S]
+  const int nvec = h >> 3, blocks = (h + 63) >> 6;
+  auto fetch_w = [&]() {
+    if (!WHOLE) return;
+    for (int i = threadIdx.x; i < blocks * PL * 64; i += 32 * kRouteWarps) {
+      const int row = (i >> 2 & 7) + 8 * (i / 64 % PL), v = 8 * (i / (64 * PL)) + 4 * (i >> 5 & 1) + (i & 3);
+      if (row >= r) continue;  // whatever lies there only reaches the sums of experts that do not exist
+      if (v < nvec) cp_async16(s_w + i, reinterpret_cast<const uint4*>(Wg) + (size_t)row * nvec + v);
+      else s_w[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  if (w_const) fetch_w();
+  pdl_wait();
+  if (!w_const) fetch_w();
+
+  const int tiles = (T + Cfg::kTokens - 1) / Cfg::kTokens, stride = (int)gridDim.x * Cfg::kTeams;
+  const int rounds = (blocks + U * TW - 1) / (U * TW);
+  const bool once = (size_t)T * h * 2 > kRouteOnceBytes;
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  uint4 slot[U][NT][2];  // [block][8 tokens][half]
+  const uint4* row[NT];
+  // one team for the whole block: neighbouring warps, neighbouring blocks; small teams: a warp reads 512 bytes
+  // of a row at a time
+  constexpr bool kDeal = TW == kRouteWarps;
+  auto block_of = [&](int b, int u) { return kDeal ? (b * U + u) * TW + warp : (b * TW + warp) * U + u; };
+  auto set_rows = [&](int tile) {
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+      row[n] = reinterpret_cast<const uint4*>(x) + (size_t)min(tile * Cfg::kTokens + 8 * n + g, T - 1) * nvec + q;
+  };
+  auto fill = [&](int c, uint4 (&dst)[NT][2]) {
+    if (8 * c + 8 <= nvec) {
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int o = 0; o < 2; ++o) dst[n][o] = ld_row(row[n] + 8 * c + 4 * o, once);
+    } else if (8 * c < nvec) {  // the last, partly filled block
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int o = 0; o < 2; ++o) dst[n][o] = 8 * c + 4 * o + q < nvec ? ld_row(row[n] + 8 * c + 4 * o, once) : zero;
+    }
+  };
+  auto take = [&](int tile, int b) {  // this warp's tokens
+    constexpr int RP = Cfg::kRP, TPP = Cfg::kTPP, kLanes = Cfg::kLanes;
+    const int used = min(TW, kDeal ? blocks : (blocks + U - 1) / U);  // warps that have columns
+    const int i = lane / kLanes / RP, c = min(lane / kLanes % RP, R - 1);
+    if (warp * Cfg::kTPW >= Cfg::kTokens) return;
+#pragma unroll
+    for (int p = 0; p < Cfg::kTPW / TPP; ++p) {
+      const int first = warp * Cfg::kTPW + p * TPP;
+      const float* from = s_part + b * TW * 2 * Cfg::kPart + (first + i) * S + c;
+      float sum = 0.f, drop = 0.f;
+      for (int w = lane % kLanes; w < used; w += kLanes) {
+        add_compensated(sum, drop, from[w * 2 * Cfg::kPart]);
+        drop += from[w * 2 * Cfg::kPart + Cfg::kPart];
+      }
+#pragma unroll
+      for (int o = 1; o < kLanes; o <<= 1) {  // lower lane first on both sides: the same bits
+        const float s1 = __shfl_xor_sync(0xffffffffu, sum, o), d1 = __shfl_xor_sync(0xffffffffu, drop, o);
+        const bool up = lane & o;
+        float acc = up ? s1 : sum;
+        drop = up ? d1 + drop : drop + d1;
+        add_compensated(acc, drop, up ? sum : s1);
+        sum = acc;
+      }
+      decide(tile * Cfg::kTokens + first, min(TPP, T - tile * Cfg::kTokens - first), closed_sum(sum, drop));
+    }
+  };
+  int tile = blockIdx.x + gridDim.x * team;
+  if (tile < tiles) {
+    set_rows(tile);
+#pragma unroll
+    for (int u = 0; u < U; ++u) fill(block_of(0, u), slot[u]);
+  }
+  if (WHOLE) {
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+  }
+  int it = 0;
+  for (; tile < tiles; tile += stride, ++it) {
+    float acc[PL][4], lost[PL][4];
+#pragma unroll
+    for (int p = 0; p < PL; ++p)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[p][i] = lost[p][i] = 0.f;
+#pragma unroll 1
+    for (int b = 0; b < rounds; ++b) {
+      const bool last = b + 1 == rounds, more = !last || tile + stride < tiles;
+      if (last && more) set_rows(tile + stride);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int c = block_of(b, u);
+        if (c < blocks) {
+#pragma unroll
+          for (int p = 0; p < PL; ++p) {
+            float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int o = 0; o < 2; ++o) {
+              uint4 w;
+              if (WHOLE) w = s_w[((c * PL + p) * 2 + o) * 32 + lane];
+              else w = 8 * c + 4 * o + q < nvec
+                           ? ld_l2(reinterpret_cast<const uint4*>(Wg) + (size_t)min(g + 8 * p, r - 1) * nvec + 8 * c + 4 * o + q)
+                           : zero;
+              const uint4 lo = slot[u][0][o], hi = NT > 1 ? slot[u][NT - 1][o] : zero;
+              mma_16x8(sum, lo.x, hi.x, lo.y, hi.y, w.x, w.y);
+              mma_16x8(sum, lo.z, hi.z, lo.w, hi.w, w.z, w.w);
+            }
+#pragma unroll
+            for (int i = 0; i < 2 * NT; ++i) add_compensated(acc[p][i], lost[p][i], sum[i]);
+          }
+        }
+        if (more) fill(block_of(last ? 0 : b + 1, u), slot[u]);
+      }
+    }
+    const int b = it & 1;
+    float* mine = s_part + (b * TW + warp) * 2 * Cfg::kPart;
+#pragma unroll
+    for (int p = 0; p < PL; ++p)
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        float* at = mine + (8 * n + g) * S + 8 * p + 2 * q;
+        *reinterpret_cast<float2*>(at) = make_float2(acc[p][2 * n], acc[p][2 * n + 1]);
+        *reinterpret_cast<float2*>(at + Cfg::kPart) = make_float2(lost[p][2 * n], lost[p][2 * n + 1]);
+      }
+    __syncwarp();
+    named_sync<kMembers>(1 + team);
+    take(tile, b);
+  }
+}
+
+// Calibration: w_e1 / w_e0 of every token.
+template <int R, int NT, int TW, bool WHOLE>
+__global__ void __launch_bounds__(32 * kRouteWarps, 1)
+ratio_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, float* __restrict__ ratio, bool w_const) {
+  pdl_launch_dependents();
+  using Cfg = TileCfg<R, NT, TW>;
+  const int lane = threadIdx.x & 31;
+  route_tiles<R, NT, TW, WHOLE>(x, Wg, T, h, r, w_const, [&](int t0, int n, float mine) {
+    constexpr int kPer = Cfg::kRP * Cfg::kLanes;  // lanes of a token
+    const int i = lane / kPer;
+    float l[R], w0, w1, p1;
+#pragma unroll
+    for (int c = 0; c < R; ++c) l[c] = __shfl_sync(0xffffffffu, mine, i * kPer + c * Cfg::kLanes);
+    if (lane % kPer || i >= n) return;
+    int e0, e1;
+    bool skip;
+    route_choose<R>(l, r, 0.f, e0, e1, skip, w0, w1, p1);
+    ratio[t0 + i] = p1;
+  });
 }
 
 // ---------------------------------------------------------------------------------- scan
@@ -815,33 +1023,18 @@ combine_kernel(const float* O, int ksplit, size_t split_stride, const int32_t* p
 // Ranking by counting, one lane per (token, kept expert): the rank of expert c is the number of kept
 // experts that beat it (larger logit, or equal logit and lower index), so the expert of rank m is
 // the m-th choice; the three sums are one lane's per token (k <= 16 values).
-template <int R, bool WHOLE>
+template <int R, int NT, int TW, bool WHOLE>
 __global__ void __launch_bounds__(32 * kRouteWarps, 1)
-router_topk_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part, int k, float beta, KeptIds kept,
+router_topk_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int k, float beta, KeptIds kept,
                    int32_t* __restrict__ idx, float* __restrict__ wn, int32_t* __restrict__ nact,
                    int32_t* u_idx, float* u_wn, int32_t* u_nact, float* logits) {
   pdl_launch_dependents();
-  using Cfg = RouteCfg<R, true>;
-  constexpr int RP = Cfg::kRP, TB = Cfg::kTB, N = Cfg::kN;
-  constexpr int kLanes = 32 / N;  // lanes that hold the same logit
-  extern __shared__ uint4 ring[];
-  __shared__ float s_p[kRouteWarps][TB][RP];
-  __shared__ int s_sel[kRouteWarps][TB][RP];
+  using Cfg = TileCfg<R, NT, TW>;
+  constexpr int RP = Cfg::kRP, TPP = Cfg::kTPP, kLanes = Cfg::kLanes;
+  __shared__ float s_p[kRouteWarps][TPP][RP];
+  __shared__ int s_sel[kRouteWarps][TPP][RP];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint4* s_w = ring + Cfg::kRingBytes / 16;
-  fetch_router_part<WHOLE>(s_w, Wg, 0, part, h >> 3, r);
-  cp_async_commit();
-  pdl_wait();
-  if (WHOLE) {
-    cp_async_wait<0>();
-    __syncthreads();
-  }
-  const int groups = (T + TB - 1) / TB;
-  int half = 0;
-  for (int g = blockIdx.x + gridDim.x * warp; g - (WHOLE ? 0 : (int)gridDim.x * warp) < groups; g += gridDim.x * kRouteWarps) {
-    const int t0 = g * TB;
-    const float mine = warp_logits<R, WHOLE, true>(x, s_w, Wg, part, half, t0, T, h, r, ring);
-    if (!WHOLE && g >= groups) continue;
+  route_tiles<R, NT, TW, WHOLE>(x, Wg, T, h, r, true, [&](int t0, int n, float mine) {
     const int i = lane / kLanes / RP, c = lane / kLanes % RP;
     int rank = 0;
     float top = -INFINITY;
@@ -856,7 +1049,7 @@ router_topk_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part,
     }
     __syncwarp();
     if (c < r && lane % kLanes == 0) {
-      if (logits && t0 + i < T) logits[(size_t)(t0 + i) * r + c] = mine;
+      if (logits && i < n) logits[(size_t)(t0 + i) * r + c] = mine;
       if (rank < k) {
         s_sel[warp][i][rank] = c;
         s_p[warp][i][rank] = expf(mine - top);
@@ -864,7 +1057,7 @@ router_topk_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part,
     }
     __syncwarp();
     const int t = t0 + lane;
-    if (lane < TB && t < T) {
+    if (lane < n) {
       const float* p = s_p[warp][lane];
       const int* sel = s_sel[warp][lane];
       // i* = the smallest i in 1..k whose dropped mass p_i + .. + p_{k-1} (added from the smallest
@@ -889,8 +1082,7 @@ router_topk_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part,
       if (u_nact) u_nact[t] = istar;
     }
     __syncwarp();
-  }
-  if (!WHOLE) cp_async_wait<0>();  // the first part, fetched once more behind the last
+  });
 }
 
 // Per block of kRouteTokPerBlock tokens: active pairs per expert, in the column layout scan_kernel reads
@@ -1206,9 +1398,9 @@ cudaError_t launch_router(const bf16* x, const bf16* Wg, int T, int h, int r, fl
                           const KeptIds& kept, const RouteOut& out, cudaStream_t st, bool w_const) {
 #define MOE_ROUTER(R)                                                                                          \
   {                                                                                                            \
-    const int part = route_part<R, false>(h, r);                                                                      \
+    const int part = route_part<R>(h, r);                                                                             \
     const bool whole = part == (h >> 3);                                                                       \
-    const size_t smem = RouteCfg<R, false>::kRingBytes + (size_t)(whole ? 1 : 2) * r * part * 16;                     \
+    const size_t smem = RouteCfg<R>::kRingBytes + (size_t)(whole ? 1 : 2) * r * part * 16;                     \
     const int units = (T + kRouteTokPerBlock - 1) / kRouteTokPerBlock;                                         \
     return launch_route(whole ? router_kernel<R, true> : router_kernel<R, false>, units, smem, st, x, Wg, T, h, \
                         r, part, beta, kept, out, w_const);                                                    \
@@ -1221,6 +1413,47 @@ cudaError_t launch_router(const bf16* x, const bf16* Wg, int T, int h, int r, fl
     default: MOE_ROUTER(kMaxE)
   }
 #undef MOE_ROUTER
+}
+
+// One block per SM at most.  Up to 8 tokens per SM: a tile of 8 for the whole block, the shortest way to one
+// tile's end.  Then, up to two tiles of 16 per block, the whole block again; beyond, and for narrow rows that
+// leave 16 warps little to share, four teams, which run out of step and so keep more loads in flight.  Router
+// rows that do not fit shared memory are read once per tile and warp: the whole block shares them.  Calibration
+// in us, one team / four teams, 2000, 4096, 8192, 16384 tokens: h 4096 21.6 / 22.9, 25.1 / 25.6, 31.8 / 28.0,
+// 54.8 / 53.4; h 1024, 8192 tokens 26.0 / 21.2; h 128, 8192 tokens 23.7 / 19.6; h 8192, 16 experts (not in
+// shared memory), 4096 tokens 35 / 49.
+constexpr int kRouteShort = 148 * 8;
+inline bool route_in_teams(int T, int h, bool whole) { return whole && (h < 2048 || T > 2 * 148 * 16); }
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_tiles(void (*kernel)(KArgs...), int tiles, size_t smem, cudaStream_t st, Args&&... args) {
+  if (smem > 32 * 1024) {  // with the records (static) possibly more than the default limit of 48 KB
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemMax);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_pdl(kernel, dim3(tiles < 148 ? tiles : 148), dim3(32 * kRouteWarps), smem, st, args...);
+}
+
+#define MOE_TILES_LAUNCH(kernel, R, NT, TW, whole, ...)                                                       \
+  return launch_tiles(kernel<R, NT, TW, whole>, (T + 8 * NT - 1) / (8 * NT),                                  \
+                      TileCfg<R, NT, TW>::kPartBytes + (whole ? TileCfg<R, NT, TW>::w_bytes(h) : 0), st, x, Wg, T, h, r, \
+                      __VA_ARGS__)
+#define MOE_TILES_R(kernel, R, ...)                                                                           \
+  {                                                                                                           \
+    const bool whole = TileCfg<R, 2, 4>::kPartBytes + TileCfg<R, 2, 4>::w_bytes(h) <= kTileSmemMax;         \
+    if (route_in_teams(T, h, whole) && T > kRouteShort) MOE_TILES_LAUNCH(kernel, R, 2, 4, true, __VA_ARGS__); \
+    if (T > kRouteShort && whole) MOE_TILES_LAUNCH(kernel, R, 2, kRouteWarps, true, __VA_ARGS__);             \
+    if (T > kRouteShort) MOE_TILES_LAUNCH(kernel, R, 2, kRouteWarps, false, __VA_ARGS__);                     \
+    if (whole) MOE_TILES_LAUNCH(kernel, R, 1, kRouteWarps, true, __VA_ARGS__);                                \
+    MOE_TILES_LAUNCH(kernel, R, 1, kRouteWarps, false, __VA_ARGS__);                                          \
+  }
+// (with fewer than 8 experts the tensor core computes 8 columns all the same)
+#define MOE_TILES_SWITCH(kernel, ...)                                                                         \
+  if (r <= 8) MOE_TILES_R(kernel, 8, __VA_ARGS__)                                                             \
+  MOE_TILES_R(kernel, kMaxE, __VA_ARGS__)
+
+cudaError_t launch_ratios(const bf16* x, const bf16* Wg, int T, int h, int r, float* ratio, cudaStream_t st,
+                          bool w_const) {
+  MOE_TILES_SWITCH(ratio_kernel, ratio, w_const)
 }
 
 cudaError_t launch_router_small(const bf16* x, const bf16* Wg, int T, int h, int r, float beta,
@@ -1295,23 +1528,7 @@ cudaError_t launch_router_topk(const bf16* x, const bf16* Wg, int T, int h, int 
                                const KeptIds& kept, int32_t* idx, float* wn, int32_t* nact,
                                int32_t* u_idx, float* u_wn, int32_t* u_nact, float* logits,
                                cudaStream_t st) {
-#define MOE_ROUTER_TOPK(R)                                                                                   \
-  {                                                                                                          \
-    const int part = route_part<R, true>(h, r);                                                                    \
-    const bool whole = part == (h >> 3);                                                                     \
-    const size_t smem = RouteCfg<R, true>::kRingBytes + (size_t)(whole ? 1 : 2) * r * part * 16;                   \
-    const int groups = (T + RouteCfg<R, true>::kTB - 1) / RouteCfg<R, true>::kTB;                                        \
-    return launch_route(whole ? router_topk_kernel<R, true> : router_topk_kernel<R, false>, groups, smem, st, x, \
-                        Wg, T, h, r, part, k, beta, kept, idx, wn, nact, u_idx, u_wn, u_nact, logits);       \
-  }
-  switch (r) {
-    case 2: MOE_ROUTER_TOPK(2)
-    case 3: case 4: MOE_ROUTER_TOPK(4)
-    case 5: case 6: MOE_ROUTER_TOPK(6)
-    case 7: case 8: MOE_ROUTER_TOPK(8)
-    default: MOE_ROUTER_TOPK(kMaxE)
-  }
-#undef MOE_ROUTER_TOPK
+  MOE_TILES_SWITCH(router_topk_kernel, k, beta, kept, idx, wn, nact, u_idx, u_wn, u_nact, logits)
 }
 
 cudaError_t launch_count_topk(const int32_t* idx, const int32_t* nact, int T, int k,

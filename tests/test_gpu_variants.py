@@ -645,3 +645,53 @@ def test_forward_kernel_names_the_kernel_that_runs(weights):
         assert layer.forward_kernel(T) == name, T
     eight.close()
     four.close()
+
+
+@pytest.mark.parametrize("h,E,T", [
+    # one team per block with tiles of 8 and of 16 tokens, four teams: the lines between them (1184 tokens, 4736, rows
+    # of 2048 columns), tiles that end inside a warp's tokens; rows of one block of 64 columns, of fewer blocks than
+    # warps, of one more than a round of them; router rows just within shared memory and just beyond it
+    (64, 2, 300), (64, 3, 1185), (320, 16, 8200), (1984, 5, 1184), (1984, 7, 1193), (2048, 8, 4736), (2048, 8, 4737),
+    (4160, 6, 9473), (4416, 16, 1185), (4480, 16, 1199), (4480, 16, 300), (10944, 4, 1201),
+])
+def test_router_at_the_edges_of_its_tiles_against_64_bits(h, E, T):
+    # A logit of 2 to 4 rounded to fp32 is off by up to 1.2e-7, which is most of what the weights lose; sums of 64
+    # products by the tensor core add little to it (0.7e-7 to 1.1e-7 seen, 2-norm over the batch).
+    build.build()
+    W = synth.make_layer_weights(h, 64, E, seed=70, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
+    x = synth.make_tokens(T, h, seed=71, device=DEV)
+    x[T // 2, 5] = 3e38  # an infinite logit leads alone
+    ranked = (x.double() @ W.W_gate.double().T).sort(dim=1, descending=True)
+    k = min(E, 4)
+    _, idx, wn, n_active = layer.forward_topk(x, k, 0.0, record=True)
+    finite = torch.arange(T, device=DEV) != T // 2
+    same = (idx.long() == ranked.indices[:, :k]).all(1) & finite
+    assert same[finite].float().mean() > 0.99 and torch.isfinite(wn[finite]).all() and int(n_active.min()) >= 1
+    want = torch.softmax(ranked.values[same, :k], 1)
+    assert float((wn[same].double() - want).norm() / want.norm()) < 1.45e-7
+    # the median of the ratios: two logits of up to 8 in magnitude, whose last bit is 4.8e-7; the infinite one has
+    # a ratio of 0
+    ratio = torch.exp(ranked.values[:, 1] - ranked.values[:, 0])
+    ratio[T // 2] = 0.0
+    s = ratio.sort().values
+    want = float((s[(T - 1) // 2] + s[T // 2]) / 2)
+    assert abs(layer.calibrate_beta(x) - want) <= 2e-6 * want
+    assert layer.device_status() == 0
+    layer.close()
+
+
+@pytest.mark.parametrize("h,r,T", [(8, 2, 300), (72, 5, 1300), (1032, 8, 5000), (4456, 16, 1201)])
+def test_allocation_free_calibration_of_ragged_rows_against_64_bits(h, r, T):
+    # rows that end inside a block of 64 columns; an infinite logit has a ratio of 0
+    Wg = synth.make_layer_weights(max(64, -(-h // 64) * 64), 64, 16, seed=72, device=DEV).W_gate[:r, :h].contiguous()
+    x = synth.make_tokens(T, h, seed=73, device=DEV)
+    x[7, 0] = 3e38
+    top = (x.double() @ Wg.double().T).sort(dim=1, descending=True).values
+    ratio = torch.exp(top[:, 1] - top[:, 0])
+    ratio[7] = 0.0
+    s = ratio.sort().values
+    want = float((s[(T - 1) // 2] + s[T // 2]) / 2)
+    got = binding.calibrate_beta_noalloc(Wg, x)
+    # of logits of up to 8 in magnitude, whose last bit is 4.8e-7
+    assert abs(got - want) <= 2e-6 * want
