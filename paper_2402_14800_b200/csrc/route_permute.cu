@@ -1275,20 +1275,29 @@ __device__ __forceinline__ float key_float(uint32_t k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
-// Exact k0-th and k1-th smallest (0-based, k1 = k0 or k0 + 1) by radix selection on the ordered bit
-// patterns: digits of 11, 11 and 10 bits, the counts of a digit in shared memory, then one more
-// pass for the smallest key above the k0-th.  NV > 0: up to NV keys per thread stay in registers
-// (NV * 1024 values); NV = 0: every pass reads the values again.  One block: bound by the shared-
-// memory additions of the first digit (few exponents, so few bins).  16384 values 36.8 -> 12.9 us
-// against four 8-bit passes per rank over memory.
+// Exact k0-th and k1-th smallest (0-based, k1 = k0 or k0 + 1).  The ratios lie in 0 .. 1, so one histogram
+// of 2048 even bins leaves a handful of candidates around rank k0, which are ranked by counting.  Where more
+// than kSelCand values share the bin (equal ratios, values outside 0 .. 1) the bit patterns are selected by
+// radix: digits of 11, 11 and 10 bits, the counts of a digit in shared memory.  Then one more pass for the
+// smallest key above the k0-th, if it is wanted and not among the candidates.  NV > 0: up to NV keys per thread
+// stay in registers (NV * 1024 values); NV = 0: every pass reads the values again.  One block: bound by the
+// latency of its passes (the first radix digit alone, few exponents and so few bins, serialised its additions).
 constexpr int kSelThreads = 1024;
+constexpr int kSelCand = 1024;
+// monotone in the key
+__device__ __forceinline__ int even_bin(uint32_t key) {
+  if (key <= 0x80000000u) return 0;     // +0 and below
+  if (key >= 0xbf800000u) return 2047;  // 1 and above
+  return (int)(key_float(key) * 2048.f);
+}
 template <int NV>
 __global__ void __launch_bounds__(kSelThreads)
 select2_kernel(const float* v, int n, int k0, int k1, float* out) {
   pdl_wait();
   __shared__ unsigned hist[2048];
   __shared__ unsigned s_warp[32];
-  __shared__ unsigned s_prefix, s_rank, s_count;
+  __shared__ unsigned s_prefix, s_rank, s_count, s_next;
+  __shared__ uint32_t s_cand[kSelCand];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   uint32_t keys[NV > 0 ? NV : 1];
   if (NV > 0) {
@@ -1307,19 +1316,8 @@ select2_kernel(const float* v, int n, int k0, int k1, float* out) {
       for (int p = tid; p < n; p += kSelThreads) f(float_key(ld_l2(v + p)));
     }
   };
-  uint32_t prefix = 0, mask = 0;
-  unsigned rank = (unsigned)k0, count = 0;
-#pragma unroll
-  for (int pass = 0; pass < 3; ++pass) {
-    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-    const uint32_t digit = pass == 2 ? 1023u : 2047u;
-    hist[2 * tid] = 0u;
-    hist[2 * tid + 1] = 0u;
-    __syncthreads();
-    each([&](uint32_t key) {
-      if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & digit], 1u);
-    });
-    __syncthreads();
+  // counts in hist[] -> s_prefix = bin that holds rank `rank`, s_rank = rank inside it, s_count = values in it
+  auto find_bin = [&](unsigned rank) {
     // exclusive sums over the bins, two bins a thread; the thread whose bin holds the rank says so
     const unsigned h0 = hist[2 * tid], h1 = hist[2 * tid + 1];
     unsigned inc = h0 + h1;
@@ -1333,18 +1331,70 @@ select2_kernel(const float* v, int n, int k0, int k1, float* out) {
     const unsigned before = __reduce_add_sync(0xffffffffu, lane < warp ? s_warp[lane] : 0u) + inc - h0 - h1;
     if (rank >= before && rank < before + h0 + h1) {
       const bool second = rank >= before + h0;
-      s_prefix = prefix | ((uint32_t)(2 * tid + (second ? 1 : 0)) << shift);
+      s_prefix = (uint32_t)(2 * tid + (second ? 1 : 0));
       s_rank = rank - before - (second ? h0 : 0u);
       s_count = second ? h1 : h0;
     }
     __syncthreads();
+  };
+  auto clear_bins = [&]() {
+    hist[2 * tid] = 0u;
+    hist[2 * tid + 1] = 0u;
+    __syncthreads();
+  };
+  clear_bins();
+  each([&](uint32_t key) { atomicAdd(&hist[even_bin(key)], 1u); });
+  __syncthreads();
+  find_bin((unsigned)k0);
+  const int bin = (int)s_prefix;
+  unsigned rank = s_rank, count = s_count;
+  uint32_t prefix = 0, next = 0;
+  bool have_next = false;
+  if (count <= kSelCand) {
+    __syncthreads();  // everyone has read what find_bin left
+    if (tid == 0) s_count = 0u;
+    __syncthreads();
+    each([&](uint32_t key) { if (even_bin(key) == bin) s_cand[atomicAdd(&s_count, 1u)] = key; });
+    __syncthreads();
+    if (tid < (int)count) {
+      const uint32_t mine = s_cand[tid];
+      unsigned less = 0, same = 0;
+      for (unsigned i = 0; i < count; ++i) {
+        less += s_cand[i] < mine;
+        same += s_cand[i] == mine;
+      }
+      // equal keys write equal values
+      if (less <= rank && rank < less + same) s_prefix = mine;
+      if (less <= rank + 1 && rank + 1 < less + same) s_next = mine;
+    }
+    __syncthreads();
     prefix = s_prefix;
-    rank = s_rank;
-    count = s_count;
-    mask |= digit << shift;
+    have_next = rank + 1 < count;
+    next = s_next;
+  } else {
+    uint32_t mask = 0;
+    rank = (unsigned)k0;
+#pragma unroll
+    for (int pass = 0; pass < 3; ++pass) {
+      const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
+      const uint32_t digit = pass == 2 ? 1023u : 2047u;
+      clear_bins();
+      each([&](uint32_t key) {
+        if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & digit], 1u);
+      });
+      __syncthreads();
+      find_bin(rank);
+      prefix |= s_prefix << shift;
+      rank = s_rank;
+      count = s_count;
+      mask |= digit << shift;
+    }
+    have_next = rank + 1 < count;
+    next = prefix;
   }
-  uint32_t next = prefix;
-  if (k1 > k0 && rank + 1 >= count) {  // the k0-th is the last of its value
+  if (k1 == k0) {
+    next = prefix;
+  } else if (!have_next) {  // the k0-th is the last of its value, or of its bin
     uint32_t best = 0xffffffffu;
     each([&](uint32_t key) { if (key > prefix) best = min(best, key); });
     best = __reduce_min_sync(0xffffffffu, best);

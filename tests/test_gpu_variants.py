@@ -695,3 +695,20 @@ def test_allocation_free_calibration_of_ragged_rows_against_64_bits(h, r, T):
     got = binding.calibrate_beta_noalloc(Wg, x)
     # of logits of up to 8 in magnitude, whose last bit is 4.8e-7
     assert abs(got - want) <= 2e-6 * want
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -6, 2.0 ** -16, 0.0])
+@pytest.mark.parametrize("T", [2, 1000, 8193, 20000])
+def test_median_of_crowded_ratios(weights, T, scale):
+    # the smaller the router's weights the nearer to 1 the ratios: a few candidates per bin, thousands of different
+    # values in one bin, one value
+    Wg = weights[0] * scale
+    layer = binding.MoeLayer(Wg, *weights[1:])
+    x = synth.make_tokens(T, H, seed=74, device=DEV)
+    stats = binding.RoutingStats(max(T, 300), E, DEV)
+    if T < 300:  # the forward call that uses the same router
+        x = torch.cat([x, synth.make_tokens(300 - T, H, seed=75, device=DEV)])
+    layer.forward(x, 0.0, stats=stats)
+    r = stats.ratio[:T].double().sort().values
+    assert layer.calibrate_beta(x[:T].contiguous()) == float(((r[(T - 1) // 2] + r[T // 2]) / 2).float())
+    layer.close()
