@@ -570,6 +570,19 @@ gemm_tokens_m_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args)
   teardown<512>(bars, tmem_base, issued, ns, args.status);
 }
 
+// Hand-over from the gate/up launch to the down launch that follows it (pair and small-batch kernels).  The
+// gate/up CTAs let the down grid launch as soon as they have passed their own wait; its CTAs need the whole
+// shared memory of an SM, so they move in one by one as gate/up CTAs leave.  What they may touch before the last
+// of those has left: the batch description (written before the gate/up launch passed its wait) and the
+// weights, so they read the work list, set up and fetch the weights of their first stages; every role waits
+// before it touches anything else.  Before, launch latency, set-up and the first trip to HBM lay between the two.
+template <bool GATE_UP> __device__ __forceinline__ void handover_wait() {
+  if (GATE_UP) {
+    pdl_wait();
+    pdl_launch_dependents();
+  }
+}
+
 // ------------------------------------------------------------------------- gemm_pair_n
 //
 // Batches between the small and the largest.  A pair of CTAs (cluster of two, cta_group::2)
@@ -843,8 +856,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
     tmem_alloc_pair(smem_u32(&bars.tmem_base), 512);
     tmem_relinquish_pair();
   }
-  // everything above is independent of the preceding kernels; their results are read from here on
-  pdl_wait();
+  handover_wait<GATE_UP>();
   for (int i = threadIdx.x; i < (int)(sizeof(Meta) / 4); i += blockDim.x)
     reinterpret_cast<int32_t*>(&s_meta)[i] = ld_l2(reinterpret_cast<const int32_t*>(args.meta) + i);
   __syncthreads();
@@ -868,8 +880,24 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
   if (warp == 0) {
     // ---- TMA producer of this CTA's 256 weight rows and its half of the tokens; the bytes of
     // both CTAs are counted on the leader's barrier
-    uint32_t it = 0, s = 0, ph = 0;
+    int it = 0;
+    uint32_t s = 0, ph = 0;
     bool ok = true;
+    // a down launch starts with the weights of its first ring of stages (see handover_wait)
+    const int ahead = !GATE_UP && pair < n_items ? min((int)ns, KB) : 0;
+    if constexpr (!GATE_UP) {
+      if (ahead && lane == 0) {
+        ItemN t;
+        decode_item_n(s_meta, args, pair, Nt, s_tiles, t);
+        for (int kb = 0; kb < ahead; ++kb) {
+          if (rank == 0) mbar_expect_tx(smem_u32(&bars.full[kb]), 2u * (PN_A_BYTES + (uint32_t)(t.n >> 1) * 128u));
+          tma_load_3d_pair(smem_base + kb * stage_bytes, &maps.w, kb * BK, t.nt * PN_W_ROWS + 256 * (int)rank, t.c,
+                           map_to_cta(smem_u32(&bars.full[kb]), 0));
+        }
+      }
+      __syncwarp();
+      pdl_wait();
+    }
     for (int item = pair; item < n_items && ok; item += n_pairs) {
       ItemN t;
       decode_item_n(s_meta, args, item, Nt, s_tiles, t);
@@ -883,8 +911,10 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
         if (lane == 0) {
           const uint32_t full = map_to_cta(smem_u32(&bars.full[s]), 0);
           const uint32_t sa = smem_base + s * stage_bytes;
-          if (rank == 0) mbar_expect_tx(smem_u32(&bars.full[s]), bytes);
-          tma_load_3d_pair(sa, &maps.w, kb * BK, w_row, t.c, full);
+          if (GATE_UP || it >= ahead) {
+            if (rank == 0) mbar_expect_tx(smem_u32(&bars.full[s]), bytes);
+            tma_load_3d_pair(sa, &maps.w, kb * BK, w_row, t.c, full);
+          }
           if (half == 128) {
             tma_load_2d_pair(sa + PN_A_BYTES, &maps.t[3], kb * BK, a_row, full);
           } else {
@@ -901,7 +931,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
         __syncwarp();
       }
     }
-    issued = it;
+    issued = (uint32_t)max(it, ahead);
   } else if (warp <= 2) {
     // ---- MMA issuers of the leader, one warp per accumulator (the other CTA's warp 1 owns that
     // CTA's tensor memory)
@@ -939,6 +969,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
   } else {
     // ---- epilogue of this CTA's 2 x 128 weight rows: warp w reads tensor-memory lanes
     // 32 (w % 4) .. + 31, and of the column chunks of 16 tokens every fourth
+    pdl_wait();
     const int wq = warp & 3, group = (warp - 3) >> 2;
     const uint32_t empty0 = map_to_cta(smem_u32(&bars.tmem_empty[0]), 0);
     const uint32_t empty1 = map_to_cta(smem_u32(&bars.tmem_empty[1]), 0);
@@ -975,7 +1006,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
     }
   }
 
-  pdl_launch_dependents();
+  if (!GATE_UP) pdl_launch_dependents();
   teardown_pair(bars, tmem_base, 512, issued, ns, rank, args.status);
 }
 
@@ -1167,8 +1198,7 @@ gemm_weights_m_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args
     tmem_alloc(smem_u32(&bars.tmem_base), 256);
     tmem_relinquish();
   }
-  // everything above is independent of the preceding kernels; their results are read from here on
-  pdl_wait();
+  handover_wait<GATE_UP>();
   for (int i = threadIdx.x; i < (int)(sizeof(Meta) / 4); i += blockDim.x)
     reinterpret_cast<int32_t*>(&s_meta)[i] = ld_l2(reinterpret_cast<const int32_t*>(args.meta) + i);
   tc_fence_before();
@@ -1182,34 +1212,47 @@ gemm_weights_m_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args
   uint32_t issued = 0;
 
   if (warp == 0) {
-    uint32_t it = 0;
+    int it = 0, ahead = 0;
     bool ok = true;
     const uint64_t evict_first = l2_policy_evict_first();
+    // every weight byte is read exactly once: do not let it push the token rows, the activations and
+    // the partial sums out of L2
+    auto fetch_weights = [&](const ItemW& w, int kb, int nk, int s) {
+      mbar_expect_tx(smem_u32(&bars.full[s]), (WM_A_BYTES + (16u << w.bucket) * 128u) * nk);
+      for (int j = 0; j < nk; ++j)
+        tma_load_3d_hint(smem_base + s * WM_STAGE + j * WM_A_BYTES, &maps.w, (kb + j) * BK, w.mt * 128, w.c,
+                         smem_u32(&bars.full[s]), evict_first);
+    };
+    if constexpr (!GATE_UP) {  // the weights of the first ring of stages (see handover_wait)
+      for (int item = blockIdx.x; item < n_items && ahead < WM_NS; item += gridDim.x) {
+        ItemW w;
+        decode_item_w(s_meta, args, sched, item, w);
+        for (int kb = w.kb0; kb < w.kb1 && ahead < WM_NS; kb += 2, ++ahead)
+          if (lane == 0) fetch_weights(w, kb, min(2, w.kb1 - kb), ahead);
+      }
+      __syncwarp();
+      pdl_wait();
+    }
     for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
       ItemW w;
       decode_item_w(s_meta, args, sched, item, w);
       if (w.kb0 >= w.kb1) continue;
-      const uint32_t bytes = WM_A_BYTES + (16u << w.bucket) * 128u;  // of one k-block
       for (int kb = w.kb0; kb < w.kb1; kb += 2, ++it) {
-        const uint32_t s = it % WM_NS, ph = (it / WM_NS) & 1u;
+        const int s = it % WM_NS;
+        const uint32_t ph = (it / WM_NS) & 1u;
         const int nk = min(2, w.kb1 - kb);
         ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.empty[s]), ph ^ 1u, abort_flag));
         if (!ok) break;
         if (lane == 0) {
-          const uint32_t full = smem_u32(&bars.full[s]);
-          const uint32_t sa = smem_base + s * WM_STAGE;
-          mbar_expect_tx(full, bytes * nk);
-          for (int j = 0; j < nk; ++j) {
-            // every weight byte is read exactly once: do not let it push the token rows, the
-            // activations and the partial sums out of L2
-            tma_load_3d_hint(sa + j * WM_A_BYTES, &maps.w, (kb + j) * BK, w.mt * 128, w.c, full, evict_first);
-            tma_load_2d(sa + 2 * WM_A_BYTES + j * WM_TOK_BYTES, &maps.t[w.bucket], (kb + j) * BK, w.tok_row, full);
-          }
+          if (GATE_UP || it >= ahead) fetch_weights(w, kb, nk, s);
+          for (int j = 0; j < nk; ++j)
+            tma_load_2d(smem_base + s * WM_STAGE + 2 * WM_A_BYTES + j * WM_TOK_BYTES, &maps.t[w.bucket], (kb + j) * BK,
+                        w.tok_row, smem_u32(&bars.full[s]));
         }
         __syncwarp();
       }
     }
-    issued = it;
+    issued = (uint32_t)max(it, ahead);
   } else if (warp == 1) {
     uint32_t it = 0, tile_it = 0;
     bool ok = true;
@@ -1246,6 +1289,7 @@ gemm_weights_m_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args
       ++tile_it;
     }
   } else {
+    pdl_wait();
     const int wq = warp & 3;
     uint32_t tile_it = 0;
     bool ok = true;
@@ -1318,7 +1362,7 @@ gemm_weights_m_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args
       ++tile_it;
     }
   }
-  pdl_launch_dependents();
+  if (!GATE_UP) pdl_launch_dependents();
   teardown<256>(bars, tmem_base, issued, WM_NS, args.status);
 }
 
@@ -1384,7 +1428,7 @@ gemm_tokens_d_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args,
         reinterpret_cast<uint4*>(gen + s * TD_STAGE)[i] = make_uint4(0u, 0u, 0u, 0u);
     fence_proxy_async();
   }
-  pdl_wait();
+  handover_wait<GATE_UP>();
   for (int i = threadIdx.x; i < (int)(sizeof(Meta) / 4); i += blockDim.x)
     reinterpret_cast<int32_t*>(&s_meta)[i] = ld_l2(reinterpret_cast<const int32_t*>(args.meta) + i);
   tc_fence_before();
@@ -1398,29 +1442,41 @@ gemm_tokens_d_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args,
   uint32_t issued = 0;
 
   if (warp == 0) {
-    uint32_t it = 0;
+    int it = 0, ahead = 0;
     bool ok = true;
     const uint64_t evict_first = l2_policy_evict_first();
+    auto fetch_weights = [&](const ItemW& w, int kb, int s) {
+      mbar_expect_tx(smem_u32(&bars.full[s]), TD_B_BYTES + (16u << w.bucket) * 128u);
+      tma_load_3d_hint(smem_base + s * TD_STAGE + TD_A_BYTES, &maps.w, kb * BK, w.mt * TD_BN, w.c,
+                       smem_u32(&bars.full[s]), evict_first);
+    };
+    if constexpr (!GATE_UP) {  // the weights of the first ring of stages (see handover_wait)
+      for (int item = blockIdx.x; item < n_items && ahead < TD_NS; item += gridDim.x) {
+        ItemW w;
+        decode_item_w(s_meta, args, sched, item, w);
+        for (int kb = w.kb0; kb < w.kb1 && ahead < TD_NS; ++kb, ++ahead)
+          if (lane == 0) fetch_weights(w, kb, ahead);
+      }
+      __syncwarp();
+      pdl_wait();
+    }
     for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
       ItemW w;
       decode_item_w(s_meta, args, sched, item, w);
       if (w.kb0 >= w.kb1) continue;
-      const uint32_t bytes = TD_B_BYTES + (16u << w.bucket) * 128u;
       for (int kb = w.kb0; kb < w.kb1; ++kb, ++it) {
-        const uint32_t s = it % TD_NS, ph = (it / TD_NS) & 1u;
+        const int s = it % TD_NS;
+        const uint32_t ph = (it / TD_NS) & 1u;
         ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.empty[s]), ph ^ 1u, abort_flag));
         if (!ok) break;
         if (lane == 0) {
-          const uint32_t full = smem_u32(&bars.full[s]);
-          const uint32_t sa = smem_base + s * TD_STAGE;
-          mbar_expect_tx(full, bytes);
-          tma_load_3d_hint(sa + TD_A_BYTES, &maps.w, kb * BK, w.mt * TD_BN, w.c, full, evict_first);
-          tma_load_2d(sa, &maps.t[w.bucket], kb * BK, w.tok_row, full);
+          if (GATE_UP || it >= ahead) fetch_weights(w, kb, s);
+          tma_load_2d(smem_base + s * TD_STAGE, &maps.t[w.bucket], kb * BK, w.tok_row, smem_u32(&bars.full[s]));
         }
         __syncwarp();
       }
     }
-    issued = it;
+    issued = (uint32_t)max(it, ahead);
   } else if (warp == 1) {
     uint32_t it = 0, tile_it = 0;
     bool ok = true;
@@ -1457,6 +1513,7 @@ gemm_tokens_d_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args,
   } else {
     // epilogue warp wq reads tensor-memory lanes 32 wq .. 32 wq + 31.  M = 128: lane l of the
     // tile is token row l.  M = 64: rows 16 q .. 16 q + 15 sit in lanes 32 q .. 32 q + 15.
+    pdl_wait();
     const int wq = warp & 3;
     uint32_t tile_it = 0;
     bool ok = true;
@@ -1547,7 +1604,7 @@ gemm_tokens_d_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args,
       if (lane == 0) *counter = 0;  // ready for the next launch
     }
   }
-  pdl_launch_dependents();
+  if (!GATE_UP) pdl_launch_dependents();
   teardown<512>(bars, tmem_base, issued, TD_NS, args.status);
 }
 
