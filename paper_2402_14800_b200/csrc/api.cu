@@ -299,10 +299,11 @@ void release_words(moe_layer* L) {
   L->h_words = nullptr;
 }
 
-int check_status(moe_layer* L) {
+// `sent`: a kernel of the stream already copies the status word to h_words[0].
+int check_status(moe_layer* L, bool sent = false) {
   int st_pageable = 0;
   int* dst = host_words(L) ? L->h_words : &st_pageable;
-  CUDA_TRY(cudaMemcpyAsync(dst, L->ws->status.p, 4, cudaMemcpyDeviceToHost, L->stream));
+  if (!sent) CUDA_TRY(cudaMemcpyAsync(dst, L->ws->status.p, 4, cudaMemcpyDeviceToHost, L->stream));
   CUDA_TRY(cudaStreamSynchronize(L->stream));
   const int st = *dst;
   if (st != 0) {
@@ -1038,13 +1039,15 @@ static int search_impl(moe_layer_t* L, const void* x_calib, const float* F_ref, 
       ++i1;
     }
     const size_t n = batch.size();
-    CUDA_TRY(cudaMemcpyAsync(W.s_subsets.p, batch.data(), n * 4, cudaMemcpyHostToDevice, st));
+    if (!enumerate_takes_list((int)n))
+      CUDA_TRY(cudaMemcpyAsync(W.s_subsets.p, batch.data(), n * 4, cudaMemcpyHostToDevice, st));
     // a single short pass leaves its losses in mapped host memory, read after the one wait below
     float* direct = i0 == 0 && i1 == n_r && n <= (size_t)kMaxHostLosses && host_words(L)
                         ? (float*)(L->h_words + kHostLosses) : nullptr;
     CUDA_TRY(launch_enumerate((const float*)W.s_logits.p, (const bf16*)W.s_yall.p, T, E, r, h,
-                              (const uint32_t*)W.s_subsets.p, (int)n, (float*)W.s_partial.p,
-                              (double*)W.s_loss_sq.p, direct ? direct : (float*)W.s_losses.p, F_ref, src, st));
+                              (const uint32_t*)W.s_subsets.p, batch.data(), (int)n, (float*)W.s_partial.p,
+                              (double*)W.s_loss_sq.p, direct ? direct : (float*)W.s_losses.p, F_ref, src,
+                              (const int*)W.status.p, direct ? L->h_words : nullptr, st));
     if (direct) mapped = n;
     else CUDA_TRY(cudaMemcpyAsync(losses + o, L->ws->s_losses.p, n * 4, cudaMemcpyDeviceToHost, st));
     // the host list is reused for the next pass: the copy above must have left it
@@ -1053,7 +1056,7 @@ static int search_impl(moe_layer_t* L, const void* x_calib, const float* F_ref, 
     i0 = i1;
   }
   mark(L);
-  if ((rc = check_status(L))) return rc;
+  if ((rc = check_status(L, mapped > 0))) return rc;
   if (mapped) memcpy(losses, L->h_words + kHostLosses, mapped * 4);
   o = 0;
   for (int i = 0; i < n_r; ++i) {

@@ -300,9 +300,12 @@ struct EnumSource {
   int k_stride;  // ranked experts recorded per token in topk_idx / pair_pos (>= E - r + 2)
 };
 int enumerate_num_blocks(int T, int nC);
+bool enumerate_takes_list(int nC);
+// host_subsets: the masks in host memory; the copy `subsets` in device memory is read only where
+// !enumerate_takes_list(nC).  status_out (or null): where *status goes with the losses.
 cudaError_t launch_enumerate(const float* logits, const bf16* Yall, int T, int E, int r, int h,
-                             const uint32_t* subsets, int nC, float* partial, double* loss_sq,
-                             float* losses, const float* Fref, const EnumSource& src,
-                             cudaStream_t st);
+                             const uint32_t* subsets, const uint32_t* host_subsets, int nC, float* partial,
+                             double* loss_sq, float* losses, const float* Fref, const EnumSource& src,
+                             const int* status, int* status_out, cudaStream_t st);
 
 }  // namespace moe

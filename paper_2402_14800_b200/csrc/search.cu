@@ -49,11 +49,10 @@ __device__ __forceinline__ void pair_weights(float l_first, float l_second, floa
 // all coefficients zero and an error of exactly 0.  `ref` (optional) is the target row f in fp32.
 // The rows of the next 8-element slice are fetched before the current one is used.
 template <int K, bool REF>
-__device__ __forceinline__ void pair_errors_fast(const bf16* __restrict__ Yt, int h,
+__device__ __forceinline__ void pair_errors_fast(const bf16* Yt, int h,
                                                  const int* order, const int* rowoff,
                                                  const float* l, int lane,
-                                                 float* s_err /* [16*16] */,
-                                                 const float* __restrict__ ref) {
+                                                 float* s_err /* [16*16] */, const float* ref) {
   constexpr int NV = K - 1 + (REF ? 1 : 0);
   constexpr int NG = NV * (NV + 1) / 2;
   float G[NG > 0 ? NG : 1];
@@ -67,19 +66,19 @@ __device__ __forceinline__ void pair_errors_fast(const bf16* __restrict__ Yt, in
   float4 cref0 = make_float4(0.f, 0.f, 0.f, 0.f), cref1 = cref0, nref0 = cref0, nref1 = cref0;
   if (lane < nvec) {
 #pragma unroll
-    for (int i = 0; i < K; ++i) cur[i] = __ldg(rows[i] + lane);
+    for (int i = 0; i < K; ++i) cur[i] = ld_l2(rows[i] + lane);
     if (REF) {
-      cref0 = __ldg(reinterpret_cast<const float4*>(ref) + 2 * lane);
-      cref1 = __ldg(reinterpret_cast<const float4*>(ref) + 2 * lane + 1);
+      cref0 = ld_l2(reinterpret_cast<const float4*>(ref) + 2 * lane);
+      cref1 = ld_l2(reinterpret_cast<const float4*>(ref) + 2 * lane + 1);
     }
   }
   for (int v = lane; v < nvec; v += 32) {
     if (v + 32 < nvec) {
 #pragma unroll
-      for (int i = 0; i < K; ++i) nxt[i] = __ldg(rows[i] + v + 32);
+      for (int i = 0; i < K; ++i) nxt[i] = ld_l2(rows[i] + v + 32);
       if (REF) {
-        nref0 = __ldg(reinterpret_cast<const float4*>(ref) + 2 * (v + 32));
-        nref1 = __ldg(reinterpret_cast<const float4*>(ref) + 2 * (v + 32) + 1);
+        nref0 = ld_l2(reinterpret_cast<const float4*>(ref) + 2 * (v + 32));
+        nref1 = ld_l2(reinterpret_cast<const float4*>(ref) + 2 * (v + 32) + 1);
       }
     }
     const float fr[8] = {cref0.x, cref0.y, cref0.z, cref0.w, cref1.x, cref1.y, cref1.z, cref1.w};
@@ -176,13 +175,23 @@ __device__ __forceinline__ void pair_errors_generic(const bf16* __restrict__ Yt,
     }
 }
 
+// The kept masks of a short list travel with the launch (a copy of their own to the device costs more than
+// the enumeration of a few hundred tokens).
+constexpr int kListMax = 1020;
+struct SubsetList {
+  uint16_t mask[kListMax];
+};
+
 // KT = K for the Gram form (K = 2 .. 6), 0 for any K through the generic form; REF = a target row
-// per token is given (progressive search).
+// per token is given (progressive search).  subsets == null: the masks are those of `list`.
+// The Gram form is a programmatic dependent of the last GEMM; the generic one, which re-reads its rows from
+// L1, is launched in plain stream order.
 template <int KT, bool REF>
 __global__ void __launch_bounds__(128)
-enumerate_kernel(const float* __restrict__ logits, const bf16* __restrict__ Yall, int T, int E,
-                 int r, int h, const uint32_t* __restrict__ subsets, int nC,
-                 float* __restrict__ partial, const float* __restrict__ Fref, EnumSource src) {
+enumerate_kernel(const float* logits, const bf16* Yall, int T, int E, int r, int h, const uint32_t* subsets, int nC,
+                 float* __restrict__ partial, const float* Fref, EnumSource src,
+                 const __grid_constant__ SubsetList list) {
+  pdl_launch_dependents();
   extern __shared__ float s_dyn[];
   const int nwarps = blockDim.x >> 5;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -194,7 +203,12 @@ enumerate_kernel(const float* __restrict__ logits, const bf16* __restrict__ Yall
   float* s_l = reinterpret_cast<float*>(base_order + nwarps * kMaxE) + warp * kMaxE;
   int* s_row = reinterpret_cast<int*>(base_order + 2 * nwarps * kMaxE) + warp * kMaxE;
 
+  uint16_t* s_mask = reinterpret_cast<uint16_t*>(base_order + 3 * nwarps * kMaxE);
+  if (!subsets)
+    for (int s = threadIdx.x; s < nC; s += blockDim.x) s_mask[s] = list.mask[s];
   for (int s = lane; s < nC; s += 32) acc[s] = 0.f;
+  __syncthreads();
+  pdl_wait();
   const int K = E - r + 2;
   const int gw = blockIdx.x * nwarps + warp;
   const int stride = gridDim.x * nwarps;
@@ -203,7 +217,7 @@ enumerate_kernel(const float* __restrict__ logits, const bf16* __restrict__ Yall
     // rank of every expert by (logit descending, index ascending)
     float mine = 0.f;
     if (lane < E) {
-      mine = logits[(size_t)t * E + lane];
+      mine = ld_l2(logits + (size_t)t * E + lane);
       s_l[lane] = mine;
     }
     __syncwarp();
@@ -211,8 +225,8 @@ enumerate_kernel(const float* __restrict__ logits, const bf16* __restrict__ Yall
       // only the K top-ranked experts were evaluated; they are listed in rank order, and their
       // outputs sit in the permuted row pair_pos[t][rank] of the token's chunk
       if (lane < K) {
-        s_order[lane] = src.topk_idx[(size_t)t * src.k_stride + lane];
-        s_row[lane] = (t / src.chunk_tokens) * src.chunk_rows + src.pair_pos[(size_t)t * src.k_stride + lane];
+        s_order[lane] = ld_l2(src.topk_idx + (size_t)t * src.k_stride + lane);
+        s_row[lane] = (t / src.chunk_tokens) * src.chunk_rows + ld_l2(src.pair_pos + (size_t)t * src.k_stride + lane);
       }
     } else if (lane < E) {
       int rank = 0;
@@ -226,11 +240,11 @@ enumerate_kernel(const float* __restrict__ logits, const bf16* __restrict__ Yall
     __syncwarp();
     const bf16* Yt = src.topk_idx ? Yall : Yall + (size_t)t * E * h;
     const float* ref = Fref ? Fref + (size_t)t * h : nullptr;
-if (KT > 0) pair_errors_fast<(KT > 0 ? KT : 2), REF>(Yt, h, s_order, s_row, s_l, lane, s_err, ref);
+    if (KT > 0) pair_errors_fast<(KT > 0 ? KT : 2), REF>(Yt, h, s_order, s_row, s_l, lane, s_err, ref);
     else pair_errors_generic(Yt, h, K, s_order, s_row, s_l, lane, s_err, ref);
     __syncwarp();
     for (int s = lane; s < nC; s += 32) {
-      const uint32_t mask = subsets[s];
+      const uint32_t mask = subsets ? ld_l2(reinterpret_cast<const int32_t*>(subsets) + s) : s_mask[s];
       int i = -1, j = -1;
       for (int q = 0; q < K; ++q) {  // the two best kept experts are always among the top K
         if ((mask >> s_order[q]) & 1u) {
@@ -251,25 +265,28 @@ if (KT > 0) pair_errors_fast<(KT > 0 ? KT : 2), REF>(Yt, h, s_order, s_row, s_l,
 
 // One warp per subset: lane i adds blocks i, i+32, ... in order, then a fixed shuffle tree;
 // the order depends only on the number of blocks, so the result is reproducible.
+// `losses` and `status_out` may be mapped host memory: the device's error word goes along with the losses.
 __global__ void __launch_bounds__(32)
-reduce_partials_kernel(const float* __restrict__ partial, int nblk, int nC,
-                       double* __restrict__ loss_sq, float* __restrict__ losses) {
+reduce_partials_kernel(const float* partial, int nblk, int nC, double* __restrict__ loss_sq,
+                       float* __restrict__ losses, const int* status, int* status_out) {
+  pdl_wait();
   const int s = blockIdx.x;
   const int lane = threadIdx.x;
   double v = 0.0;
-  for (int b = lane; b < nblk; b += 32) v += (double)partial[(size_t)b * nC + s];
+  for (int b = lane; b < nblk; b += 32) v += (double)ld_l2(partial + (size_t)b * nC + s);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if (lane == 0) {
     loss_sq[s] = v;
     losses[s] = (float)sqrt(v);
+    if (s == 0 && status_out) *status_out = ld_l2(status);
   }
 }
 
 int warps_for(int nC) { return nC <= 2048 ? 4 : 1; }
 size_t enumerate_smem(int nC) {
   const size_t nw = warps_for(nC);
-  return (nw * nC + nw * kMaxE * kMaxE + 3 * nw * kMaxE) * 4;
+  return (nw * nC + nw * kMaxE * kMaxE + 3 * nw * kMaxE) * 4 + (nC <= kListMax ? 2 * kListMax : 0);
 }
 
 }  // namespace
@@ -291,17 +308,23 @@ int enumerate_num_blocks(int T, int nC) {
   return cost(two) < cost(one) ? two : one;
 }
 
+bool enumerate_takes_list(int nC) { return nC <= kListMax; }
+
 cudaError_t launch_enumerate(const float* logits, const bf16* Yall, int T, int E, int r, int h,
-                             const uint32_t* subsets, int nC, float* partial, double* loss_sq,
-                             float* losses, const float* Fref, const EnumSource& src,
-                             cudaStream_t st) {
+                             const uint32_t* subsets, const uint32_t* host_subsets, int nC, float* partial,
+                             double* loss_sq, float* losses, const float* Fref, const EnumSource& src,
+                             const int* status, int* status_out, cudaStream_t st) {
   const int nw = warps_for(nC);
   const int nblk = enumerate_num_blocks(T, nC);
   const size_t smem = enumerate_smem(nC);
   if (smem > 96 * 1024) return cudaErrorInvalidValue;
   const int K = E - r + 2;
-  void (*kernel)(const float*, const bf16*, int, int, int, int, const uint32_t*, int, float*, const float*,
-                 EnumSource) = nullptr;
+  SubsetList list;
+  if (enumerate_takes_list(nC)) {
+    subsets = nullptr;
+    for (int i = 0; i < nC; ++i) list.mask[i] = (uint16_t)host_subsets[i];
+  }
+  auto kernel = enumerate_kernel<0, false>;
 #define MOE_ENUM_PICK(KK)                                                                   \
   case KK: kernel = Fref ? enumerate_kernel<KK, true> : enumerate_kernel<KK, false>; break
   switch (K) {
@@ -313,15 +336,16 @@ cudaError_t launch_enumerate(const float* logits, const bf16* Yall, int T, int E
     default: kernel = Fref ? enumerate_kernel<0, true> : enumerate_kernel<0, false>; break;
   }
 #undef MOE_ENUM_PICK
-  if (smem > 48 * 1024) {
-    cudaError_t ea = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-    if (ea != cudaSuccess) return ea;
-  }
-  kernel<<<nblk, nw * 32, smem, st>>>(logits, Yall, T, E, r, h, subsets, nC, partial, Fref, src);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (smem > 48 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   if (e != cudaSuccess) return e;
-  reduce_partials_kernel<<<nC, 32, 0, st>>>(partial, nblk, nC, loss_sq, losses);
-  return cudaGetLastError();
+  e = K <= 6 ? launch_pdl(kernel, dim3(nblk), dim3(nw * 32), smem, st, logits, Yall, T, E, r, h, subsets, nC, partial,
+                          Fref, src, list)
+             : launch_plain(kernel, dim3(nblk), dim3(nw * 32), smem, st, logits, Yall, T, E, r, h, subsets, nC, partial,
+                            Fref, src, list);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(reduce_partials_kernel, dim3(nC), dim3(32), 0, st, partial, nblk, nC, loss_sq, losses, status,
+                    status_out);
 }
 
 }  // namespace moe

@@ -712,3 +712,22 @@ def test_median_of_crowded_ratios(weights, T, scale):
     r = stats.ratio[:T].double().sort().values
     assert layer.calibrate_beta(x[:T].contiguous()) == float(((r[(T - 1) // 2] + r[T // 2]) / 2).float())
     layer.close()
+
+
+def test_subsets_that_travel_with_the_launch_and_subsets_in_memory():
+    # 1001 and 1015 subsets go along with the launch, 1092 through memory; six ranked experts a token each time
+    build.build()
+    W = synth.make_layer_weights(128, 64, 14, seed=76, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
+    x = synth.make_tokens(300, 128, seed=77, device=DEV)
+    alone = layer.prune_search(x, 10)
+    for sizes in ([10, 13], [10, 12], [13, 10]):
+        found = dict(zip(sizes, layer.prune_search_multi(x, sizes)))
+        assert found[10] == alone
+    # an expired wait is reported through the losses' way, once
+    lib = binding.load_library()
+    assert lib.moe_test_wait_expiry(layer._h, 1000, 0) == 0
+    with pytest.raises(binding.MoeError):
+        layer.prune_search(x, 10)
+    assert layer.prune_search(x, 10) == alone
+    layer.close()
