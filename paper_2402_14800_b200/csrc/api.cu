@@ -117,6 +117,8 @@ struct moe_layer {
   std::vector<cudaEvent_t> prof_ev;  // MOE_PROFILE_STAGES + 1 marks per recorded call
   size_t prof_used = 0;
   int* h_words = nullptr;  // pinned host words (host_words)
+  cudaStream_t out_stream = nullptr;  // copies of finished column slabs to the host (moe_forward_host)
+  cudaEvent_t out_ev[2] = {};         // slab finished, copies finished
   int large_kernel = 0, tile_cap = 0;  // moe_test_large_batch
 };
 
@@ -339,14 +341,16 @@ int permute_topk(moe_layer* L, const bf16* x, const int32_t* idx, const int32_t*
 }
 
 // The two grouped GEMMs of the experts over a batch described by `meta`, of at most `pairs`
-// token-expert pairs.
+// token-expert pairs.  A batch of the pair kernel can be taken in steps: `part` 1 = gate/up alone, 2 = rows
+// dn.w_row0 .. dn.n_w_rows of the down projection.
 int run_expert_gemms(moe_layer* L, const Meta* meta, bool weights_m, const GemmMaps& m_gu,
                      const GemmMaps& m_dn, GemmArgs gu, GemmArgs dn, GemmOut dn_kind,
-                     const bf16* gu_A, const bf16* dn_A, int simt_rows, long long pairs, int T = 0) {
+                     const bf16* gu_A, const bf16* dn_A, int simt_rows, long long pairs, int T = 0, int part = 0) {
   gu.meta = meta; dn.meta = meta;
   gu.r = L->r; dn.r = L->r;
   gu.K = L->h; gu.n_w_rows = 2 * L->f;
-  dn.K = L->f; dn.n_w_rows = L->h;
+  dn.K = L->f;
+  if (part != 2) dn.n_w_rows = L->h;
   gu.status = (int*)L->ws->status.p; dn.status = (int*)L->ws->status.p;
   gu.tile_cap = L->tile_cap; dn.tile_cap = L->tile_cap;
   if (L->debug_simt) {
@@ -362,9 +366,11 @@ int run_expert_gemms(moe_layer* L, const Meta* meta, bool weights_m, const GemmM
     mark(L);
     CUDA_TRY(launch_gemm_tokens_d(false, m_dn, dn, down_kb_per_item(T), L->stream));
   } else if (large_on_pairs(L, pairs)) {
-    CUDA_TRY(launch_gemm_pair_n(true, kOutActBf16, m_gu, gu, L->stream));
-    mark(L);
-    CUDA_TRY(launch_gemm_pair_n(false, dn_kind, m_dn, dn, L->stream));
+    if (part != 2) {
+      CUDA_TRY(launch_gemm_pair_n(true, kOutActBf16, m_gu, gu, L->stream));
+      mark(L);
+    }
+    if (part != 1) CUDA_TRY(launch_gemm_pair_n(false, dn_kind, m_dn, dn, L->stream));
   } else {
     CUDA_TRY(launch_gemm_tokens_m(true, kOutActBf16, m_gu, gu, L->stream));
     mark(L);
@@ -373,9 +379,26 @@ int run_expert_gemms(moe_layer* L, const Meta* meta, bool weights_m, const GemmM
   return MOE_OK;
 }
 
+// Column slabs in which a batch for the host leaves the device: the copy of one runs while the down projection
+// of the next is computed.  A slab is a whole number of the pair kernel's 512-row weight tiles.
+inline int host_slabs(const moe_layer* L, int T) {
+  if (decode_mode(T) || L->debug_simt || !large_on_pairs(L, 2ll * T)) return 1;
+  const int want = T < 2048 ? 2 : 4, tiles = L->h / 512;
+  if ((size_t)T * L->h < (size_t)1 << 22 || tiles < 2) return 1;
+  return want < tiles ? want : tiles;
+}
+
+int ensure_out_stream(moe_layer* L) {
+  if (!L->out_stream) CUDA_TRY(cudaStreamCreateWithFlags(&L->out_stream, cudaStreamNonBlocking));
+  for (cudaEvent_t& e : L->out_ev)
+    if (!e) CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  return MOE_OK;
+}
+
 // dist != nullptr: instead of combining, write || E_e0(x) - E_e1(x) ||_2 per token (y unused)
+// y_host != nullptr (pinned) and slabs > 1: y is also copied there, in column slabs
 int forward_impl(moe_layer* L, const void* x, int T, float beta, const void* residual, void* y,
-                 void* stats, float* dist = nullptr) {
+                 void* stats, float* dist = nullptr, void* y_host = nullptr, int slabs = 1) {
   if (!L) return fail(MOE_ERR_INVALID_ARG, "layer is NULL");
   if (T < 0 || T > kMaxTokens) return fail(MOE_ERR_INVALID_ARG, "T = %d outside 0..%d", T, kMaxTokens);
   if (T == 0) return MOE_OK;
@@ -466,6 +489,29 @@ int forward_impl(moe_layer* L, const void* x, int T, float beta, const void* res
   m_dn.w = (wm && decode_weights_m(L, T)) ? L->w2_128 : L->w2_256;
   memcpy(m_gu.t, L->ws->tok_x, sizeof(m_gu.t));
   memcpy(m_dn.t, L->ws->tok_act, sizeof(m_dn.t));
+  if (slabs > 1) {
+    const int tiles = (L->h + 511) / 512;
+    for (int s = 0; s < slabs; ++s) {
+      dn.w_row0 = 512 * (tiles * s / slabs);
+      dn.n_w_rows = s + 1 < slabs ? 512 * (tiles * (s + 1) / slabs) : L->h;
+      const int cols = dn.n_w_rows - dn.w_row0;
+      for (int part = s == 0 ? 1 : 2; part <= 2; ++part)
+        if ((rc = run_expert_gemms(L, meta, wm, m_gu, m_dn, gu, dn, kOutF32, (const bf16*)L->ws->xperm.p,
+                                   (const bf16*)L->ws->act.p, rows_cap, 2ll * T, T, part)))
+          return rc;
+      if (s == 0) mark(L);
+      CUDA_TRY(launch_combine((const float*)L->ws->O.p, ksplit, split_stride, (int32_t*)L->ws->pair_pos.p,
+                              (float*)L->ws->wn.p, (const bf16*)residual, T, L->h, (bf16*)y, st, dn.w_row0, cols));
+      CUDA_TRY(cudaEventRecord(L->out_ev[0], st));
+      CUDA_TRY(cudaStreamWaitEvent(L->out_stream, L->out_ev[0], 0));
+      CUDA_TRY(cudaMemcpy2DAsync((bf16*)y_host + dn.w_row0, (size_t)L->h * 2, (const bf16*)y + dn.w_row0,
+                                 (size_t)L->h * 2, (size_t)cols * 2, T, cudaMemcpyDeviceToHost, L->out_stream));
+    }
+    mark(L);
+    CUDA_TRY(cudaEventRecord(L->out_ev[1], L->out_stream));
+    CUDA_TRY(cudaStreamWaitEvent(st, L->out_ev[1], 0));
+    return MOE_OK;
+  }
   rc = run_expert_gemms(L, meta, wm, m_gu, m_dn, gu, dn, kOutF32, (const bf16*)L->ws->xperm.p,
                         (const bf16*)L->ws->act.p, rows_cap, 2ll * T, T);
   if (rc) return rc;
@@ -609,6 +655,9 @@ void moe_layer_destroy(moe_layer_t* L) {
                  &L->own.s_losses, &L->own.s_xpad, &L->own.s_meta, &L->own.s_xperm, &L->own.hx, &L->own.hy, &L->own.xn, &L->own.cosel, &L->own.k_idx, &L->own.k_wn, &L->own.k_pos, &L->own.k_nact};
   for (Buf* b : bufs) release(L, *b);
   for (cudaEvent_t e : L->prof_ev) cudaEventDestroy(e);
+  if (L->out_stream) cudaStreamDestroy(L->out_stream);
+  for (cudaEvent_t e : L->out_ev)
+    if (e) cudaEventDestroy(e);
   release_words(L);
   if (L->Wg) cudaFree(L->Wg);
   if (L->W13) cudaFree(L->W13);
@@ -760,9 +809,23 @@ int moe_forward_host(moe_layer_t* L, const void* x_host, int T, float beta, void
   int rc;
   if ((rc = grow(L, L->ws->hx, bytes))) return rc;
   if ((rc = grow(L, L->ws->hy, bytes))) return rc;
+  int slabs = host_slabs(L, T);
+  if (slabs > 1) {  // copies to pageable memory are staged by the runtime, row by row: leave those whole
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, y_host) != cudaSuccess || at.type != cudaMemoryTypeHost) {
+      cudaGetLastError();
+      slabs = 1;
+    } else if ((rc = ensure_out_stream(L))) {
+      return rc;
+    }
+  }
   CUDA_TRY(cudaMemcpyAsync(L->ws->hx.p, x_host, bytes, cudaMemcpyHostToDevice, L->stream));
-  if ((rc = forward_impl(L, L->ws->hx.p, T, beta, nullptr, L->ws->hy.p, nullptr))) return rc;
-  CUDA_TRY(cudaMemcpyAsync(y_host, L->ws->hy.p, bytes, cudaMemcpyDeviceToHost, L->stream));
+  rc = forward_impl(L, L->ws->hx.p, T, beta, nullptr, L->ws->hy.p, nullptr, nullptr, y_host, slabs);
+  if (rc) {  // nothing may still be on its way to the caller's buffer
+    if (slabs > 1) cudaStreamSynchronize(L->out_stream);
+    return rc;
+  }
+  if (slabs == 1) CUDA_TRY(cudaMemcpyAsync(y_host, L->ws->hy.p, bytes, cudaMemcpyDeviceToHost, L->stream));
   return check_status(L);
 }
 

@@ -191,7 +191,7 @@ cudaError_t launch_permute(const bf16* x, const int32_t* idx, const void* active
                            int E, cudaStream_t st);
 cudaError_t launch_combine(const float* O, int ksplit, size_t split_stride, const int32_t* pair_pos,
                            const float* wn, const bf16* residual, int T, int h, bf16* y,
-                           cudaStream_t st);
+                           cudaStream_t st, int col0 = 0, int cols = 0);  // columns col0 .. + cols (0: all)
 // general top-k path (k slots per token instead of two)
 cudaError_t launch_router_topk(const bf16* x, const bf16* Wg, int T, int h, int r, int k, float beta,
                                const KeptIds& kept, int32_t* idx, float* wn, int32_t* nact,
@@ -224,6 +224,7 @@ struct GemmArgs {
   int r;         // kept experts
   int K;         // contraction length (h for gate/up, f for down)
   int n_w_rows;  // weight rows per expert (2f interleaved for gate/up, h for down)
+  int w_row0;    // pair kernel: the launch computes rows w_row0 (a multiple of 512) .. n_w_rows
   // token-side operand rows: a_row = a_row_base + a_off_mul * off[c] + 128 * m
   int a_row_base, a_off_mul;
   // output rows: out_row = out_row_base + out_off_mul * off[c] + 128 * m; column offset c * out_col_mul

@@ -727,7 +727,7 @@ constexpr int PN_EPI_WARPS = 16;
 constexpr int PN_THREADS = 96 + 32 * PN_EPI_WARPS;
 
 struct ItemN {
-  int c, nt;          // expert, weight tile
+  int c, nt;          // expert, weight tile (of the whole matrix)
   int tok0;           // first token of the tile inside the expert's group
   int n, valid;       // columns of the MMA (a multiple of 32) and the tokens among them
 };
@@ -781,8 +781,9 @@ __device__ __forceinline__ void decode_item_n(const Meta& m, const GemmArgs& a, 
   const int rem = local - band * per_band * Nt;
   const int band_tiles = min(per_band, kt - band * per_band);
   t.c = c;
-  t.nt = rem / band_tiles;
-  const int i = band * per_band + rem - t.nt * band_tiles;
+  const int nt = rem / band_tiles;
+  t.nt = a.w_row0 / PN_W_ROWS + nt;
+  const int i = band * per_band + rem - nt * band_tiles;
   const int units = (m.count[c] + 31) >> 5;
   const int q = units / kt, extra = units - q * kt;
   t.tok0 = 32 * (i * q + min(i, extra));
@@ -861,7 +862,7 @@ gemm_pair_n_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args) {
     reinterpret_cast<int32_t*>(&s_meta)[i] = ld_l2(reinterpret_cast<const int32_t*>(args.meta) + i);
   __syncthreads();
   const int KB = (args.K + BK - 1) / BK;
-  const int Nt = (args.n_w_rows + PN_W_ROWS - 1) / PN_W_ROWS;
+  const int Nt = (args.n_w_rows - args.w_row0 + PN_W_ROWS - 1) / PN_W_ROWS;
   const int cap = args.tile_cap ? args.tile_cap : choose_tile_cap(s_meta, args, KB, Nt, n_pairs);
   if (threadIdx.x < kMaxE) s_tiles[threadIdx.x] = token_tiles(s_meta.count[threadIdx.x], cap);
   __syncwarp();

@@ -972,14 +972,13 @@ permute_kernel(const bf16* x, const int32_t* idx, const void* active, int T, int
 
 __global__ void __launch_bounds__(128)
 combine_kernel(const float* O, int ksplit, size_t split_stride, const int32_t* pair_pos,
-               const float* wn, const bf16* residual, int T, int h, bf16* y) {
+               const float* wn, const bf16* residual, int T, int h, int v0, int v1, bf16* y) {
   pdl_launch_dependents();
   pdl_wait();
   const int t = blockIdx.x;
   const int p0 = ld_l2(pair_pos + 2 * t), p1 = ld_l2(pair_pos + 2 * t + 1);
   const float w0 = ld_l2(wn + 2 * t), w1 = ld_l2(wn + 2 * t + 1);
-  const int nvec = h >> 3;
-  for (int v = blockIdx.y * blockDim.x + threadIdx.x; v < nvec; v += gridDim.y * blockDim.x) {
+  for (int v = v0 + blockIdx.y * blockDim.x + threadIdx.x; v < v1; v += gridDim.y * blockDim.x) {
     float a[8], b[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) { a[k] = 0.f; b[k] = 0.f; }
@@ -1567,11 +1566,12 @@ cudaError_t launch_permute(const bf16* x, const int32_t* idx, const void* active
 
 cudaError_t launch_combine(const float* O, int ksplit, size_t split_stride, const int32_t* pair_pos,
                            const float* wn, const bf16* residual, int T, int h, bf16* y,
-                           cudaStream_t st) {
-  int ychunks = ((h >> 3) + 127) / 128;
+                           cudaStream_t st, int col0, int cols) {
+  const int v0 = col0 >> 3, v1 = cols ? v0 + (cols >> 3) : h >> 3;
+  int ychunks = (v1 - v0 + 127) / 128;
   if (T > 4096) ychunks = 1;  // plenty of blocks already
   return launch_pdl(combine_kernel, dim3(T, ychunks), dim3(128), 0, st, O, ksplit, split_stride,
-                    pair_pos, wn, residual, T, h, y);
+                    pair_pos, wn, residual, T, h, v0, v1, y);
 }
 
 cudaError_t launch_router_topk(const bf16* x, const bf16* Wg, int T, int h, int r, int k, float beta,

@@ -731,3 +731,19 @@ def test_subsets_that_travel_with_the_launch_and_subsets_in_memory():
         layer.prune_search(x, 10)
     assert layer.prune_search(x, 10) == alone
     layer.close()
+
+
+@pytest.mark.parametrize("h,E,T", [(1024, 8, 4095), (1024, 8, 4096), (1600, 4, 2700), (2560, 8, 2047), (2560, 8, 2049), (4096, 8, 1025)])
+def test_host_calls_in_column_slabs_equal_the_device_call(h, E, T):
+    # below the line, two and four slabs, slabs of different widths, a last slab that ends inside a weight tile
+    build.build()
+    W = synth.make_layer_weights(h, 128, E, seed=78, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
+    x = synth.make_tokens(T, h, seed=79, device=DEV)
+    want = layer.forward(x, 0.3).cpu()
+    pinned, pageable = (torch.zeros_like(want).pin_memory(), torch.zeros_like(want))
+    for y in (pinned, pageable, pinned):
+        y.zero_()
+        assert torch.equal(layer.forward_host(x.cpu().pin_memory(), 0.3, y), want)
+    assert layer.device_status() == 0
+    layer.close()
