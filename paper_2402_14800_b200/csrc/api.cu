@@ -320,7 +320,8 @@ int check_status(moe_layer* L, bool sent = false) {
 // Which large-batch GEMM a batch of at most `pairs` token-expert pairs runs, and what its groups are
 // padded to.
 inline bool large_on_pairs(const moe_layer* L, long long pairs) {
-  return L->large_kernel == 1 || (L->large_kernel == 0 && pairs <= (long long)kPairMaxRows * L->r);
+  return L->large_kernel == 1 ||
+         (L->large_kernel == 0 && pairs <= (long long)(L->h < kPairWideH ? kPairMaxRows : kPairMaxRowsWide) * L->r);
 }
 inline int group_pad(const moe_layer* L, long long pairs) { return large_on_pairs(L, pairs) ? kPairPad : kTileRows; }
 

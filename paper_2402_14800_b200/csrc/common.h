@@ -20,13 +20,22 @@ constexpr int kInterleave = 16;           // W1/W3 rows are interleaved in group
 constexpr int kDecodeMaxT = 256;          // up to here the small-batch path (weights read once) is used
 constexpr int kTokensDPerExpert = 40;      // small batches with this many tokens per expert or more: token-major decode GEMM
 constexpr int kTokensDMaxKept = 6;         // ... on layers with at most this many kept experts
-// Large batches with at most this many pairs per kept expert (a forward call counts two per token, skipped
-// or not) run gemm_pair_n, the others gemm_tokens_m.  Alternating 1.5 s runs at the power cap, Mixtral
-// layer, 8 experts (gemm_tokens_m vs gemm_pair_n, whole step): 1500 tokens 1.30 vs 1.17 ms, 2500 1.85 vs
-// 1.70, 3500 2.40 vs 2.28, 5000 3.23 vs 3.16; at 8192 (2048 a group) -1.5 .. +1.8 % depending on the board,
-// and the search's 6144 a group was up to 6 % slower on the pairs: with little padding to save, both are
-// held by the board's power and the pairs draw 1-3 % more energy per call.
+// Large batches with at most so many pairs per kept expert (a forward call counts two per token, skipped or not)
+// run gemm_pair_n, the others gemm_tokens_m: kPairMaxRows on rows of fewer than kPairWideH columns, else
+// kPairMaxRowsWide.  Whole step, gemm_pair_n against gemm_tokens_m, alternating runs, pairs per expert
+// 1600 / 2048 / 4096 / 8192:
+//   (h, f, experts)    64, 64, 8        -1 % / +8 % / +16 % / +16 %
+//                      128, 448, 8      -4 / -4 / -3 / +9      256, 1024, 8     -6 / -7 / -1 / +8
+//                      512, 1024, 8    -22 / -19 / -10 / -5    1024, 2048, 8   -12 / -10 / -7 / -5
+//                      2048, 4096, 16   -8 / -7 / -7 / -5      4096, 1024, 8   -12 / -10 / -8 / -5
+// On narrow layers an item is a few k-blocks long and the two CTAs spend it on handing over to each other.  Mixtral
+// layer in 1.5 s loops at the power cap (ms): 8192 tokens (2048 a group) 4.77 vs 4.95, 16384 9.25 vs 9.45, 32768 (8192
+// a group) 18.56 vs 18.57, 65536 37.5-39.0 vs 36.2; search of 32768 tokens (6144 a group) 54.7 vs 56.0 on two boards,
+// 59.3 vs 58.0 on a third.  There the board's power is the limit, and the pairs draw less of it for a product while
+// there is padding to save (8192 tokens 4.62 vs 5.1 J); from 6144 a group on it depends on the board.
 constexpr int kPairMaxRows = 1536;
+constexpr int kPairMaxRowsWide = 4096;
+constexpr int kPairWideH = 512;
 // Top-k calls of more than kDecodeMaxT tokens with at most this many pairs per kept expert, half of the
 // weight-major kernel's token tile, run that kernel: it cuts the last round into K-slices, and hardly any
 // group needs a second tile.  Whole call in us, gemm_pair_n vs weight-major, layers of 16 experts (h, f):

@@ -747,3 +747,20 @@ def test_host_calls_in_column_slabs_equal_the_device_call(h, E, T):
         assert torch.equal(layer.forward_host(x.cpu().pin_memory(), 0.3, y), want)
     assert layer.device_status() == 0
     layer.close()
+
+
+@pytest.mark.parametrize("h", [448, 512])
+def test_large_groups_on_either_side_of_the_width_line(h):
+    # two kept experts, no skipping: groups of T tokens beyond the line of the narrow layers
+    build.build()
+    W = synth.make_layer_weights(h, 192, 3, seed=80, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2, 0b110)
+    line = 4096 if h >= 512 else 1536
+    assert layer.forward_kernel(line) == "gemm_pair_n_kernel" and layer.forward_kernel(line + 1) == "gemm_tokens_m_kernel"
+    for T in (1537, 2400, 4097):
+        x = synth.make_tokens(T, h, seed=81, device=DEV)
+        want = layer.forward(x)
+        for kernel in (1, 2, 0):
+            assert torch.equal(forced(layer, kernel).forward(x), want)
+    assert layer.device_status() == 0
+    layer.close()
