@@ -323,6 +323,9 @@ inline bool large_on_pairs(const moe_layer* L, long long pairs) {
   return L->large_kernel == 1 ||
          (L->large_kernel == 0 && pairs <= (long long)(L->h < kPairWideH ? kPairMaxRows : kPairMaxRowsWide) * L->r);
 }
+inline bool down_on_pairs(const moe_layer* L, long long pairs) {
+  return large_on_pairs(L, pairs) && (L->large_kernel == 1 || pairs <= (long long)kPairDownRows * L->r);
+}
 inline int group_pad(const moe_layer* L, long long pairs) { return large_on_pairs(L, pairs) ? kPairPad : kTileRows; }
 
 // Permutation of a top-k batch: idx [T][k], the first nact[t] slots of a token run.
@@ -371,7 +374,8 @@ int run_expert_gemms(moe_layer* L, const Meta* meta, bool weights_m, const GemmM
       CUDA_TRY(launch_gemm_pair_n(true, kOutActBf16, m_gu, gu, L->stream));
       mark(L);
     }
-    if (part != 1) CUDA_TRY(launch_gemm_pair_n(false, dn_kind, m_dn, dn, L->stream));
+    if (part != 1 && down_on_pairs(L, pairs)) CUDA_TRY(launch_gemm_pair_n(false, dn_kind, m_dn, dn, L->stream));
+    else if (part != 1) CUDA_TRY(launch_gemm_tokens_m(false, dn_kind, m_dn, dn, L->stream));
   } else {
     CUDA_TRY(launch_gemm_tokens_m(true, kOutActBf16, m_gu, gu, L->stream));
     mark(L);
@@ -383,7 +387,7 @@ int run_expert_gemms(moe_layer* L, const Meta* meta, bool weights_m, const GemmM
 // Column slabs in which a batch for the host leaves the device: the copy of one runs while the down projection
 // of the next is computed.  A slab is a whole number of the pair kernel's 512-row weight tiles.
 inline int host_slabs(const moe_layer* L, int T) {
-  if (decode_mode(T) || L->debug_simt || !large_on_pairs(L, 2ll * T)) return 1;
+  if (decode_mode(T) || L->debug_simt || !down_on_pairs(L, 2ll * T)) return 1;
   const int want = T < 2048 ? 2 : 4, tiles = L->h / 512;
   if ((size_t)T * L->h < (size_t)1 << 22 || tiles < 2) return 1;
   return want < tiles ? want : tiles;

@@ -30,11 +30,16 @@ constexpr int kTokensDMaxKept = 6;         // ... on layers with at most this ma
 //                      2048, 4096, 16   -8 / -7 / -7 / -5      4096, 1024, 8   -12 / -10 / -8 / -5
 // On narrow layers an item is a few k-blocks long and the two CTAs spend it on handing over to each other.  Mixtral
 // layer in 1.5 s loops at the power cap (ms): 8192 tokens (2048 a group) 4.77 vs 4.95, 16384 9.25 vs 9.45, 32768 (8192
-// a group) 18.56 vs 18.57, 65536 37.5-39.0 vs 36.2; search of 32768 tokens (6144 a group) 54.7 vs 56.0 on two boards,
-// 59.3 vs 58.0 on a third.  There the board's power is the limit, and the pairs draw less of it for a product while
-// there is padding to save (8192 tokens 4.62 vs 5.1 J); from 6144 a group on it depends on the board.
+// a group) 18.56 vs 18.57, 65536 37.5-39.0 vs 36.2.  There the board's power is the limit, and the pairs draw less of it
+// for a product while there is padding to save (8192 tokens 4.62 vs 5.1 J).
+// Beyond kPairDownRows pairs per expert only the gate/up launch is theirs: in the down launch, whose items run over
+// many k-blocks, pairs that started an item apart read weights and activations from HBM again (8192 tokens 4.0 GB
+// where gemm_tokens_m reads 2.1).  Search of 32768 tokens (6144 a group), three runs on one board: gemm_tokens_m
+// 55.5-55.7 ms (55.0 J), pairs 53.4-54.2 (53.5), pairs and gemm_tokens_m 53.5-53.6 (52.6); forward of 32768 tokens
+// 18.2-18.5, 18.1, 18.0-18.2.  At 3000 a group the pairs alone are the faster by 1 %, at 500 by 6 %.
 constexpr int kPairMaxRows = 1536;
-constexpr int kPairMaxRowsWide = 4096;
+constexpr int kPairMaxRowsWide = 8192;
+constexpr int kPairDownRows = 4096;
 constexpr int kPairWideH = 512;
 // Top-k calls of more than kDecodeMaxT tokens with at most this many pairs per kept expert, half of the
 // weight-major kernel's token tile, run that kernel: it cuts the last round into K-slices, and hardly any

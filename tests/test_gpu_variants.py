@@ -755,9 +755,9 @@ def test_large_groups_on_either_side_of_the_width_line(h):
     build.build()
     W = synth.make_layer_weights(h, 192, 3, seed=80, device=DEV)
     layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2, 0b110)
-    line = 4096 if h >= 512 else 1536
+    line = 8192 if h >= 512 else 1536
     assert layer.forward_kernel(line) == "gemm_pair_n_kernel" and layer.forward_kernel(line + 1) == "gemm_tokens_m_kernel"
-    for T in (1537, 2400, 4097):
+    for T in (1537, 2400, 4096, 4097, 8193):  # from 4097 to 8192 on the wide rows: gate/up on the pairs alone
         x = synth.make_tokens(T, h, seed=81, device=DEV)
         want = layer.forward(x)
         for kernel in (1, 2, 0):
