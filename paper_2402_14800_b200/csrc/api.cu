@@ -114,8 +114,9 @@ struct moe_layer {
   Workspace* ws = &own;
   // per-stage device timing (off unless moe_profile_enable)
   bool prof = false;
-  std::vector<cudaEvent_t> prof_ev;  // MOE_PROFILE_STAGES + 1 marks per recorded call
+  std::vector<cudaEvent_t> prof_ev;  // MOE_PROFILE_STAGES + 1 marks per recorded call or slab
   size_t prof_used = 0;
+  size_t prof_more = 0;  // sets of marks that continue the call before them (column slabs)
   int* h_words = nullptr;  // pinned host words (host_words)
   cudaStream_t out_stream = nullptr;  // copies of finished column slabs to the host (moe_forward_host)
   cudaEvent_t out_ev[2] = {};         // slab finished, copies finished
@@ -238,10 +239,11 @@ int ensure_gemm(moe_layer* L, int T, int k = 2) {
 }
 
 // Records a stage boundary on the handle's stream while profiling is on.
+constexpr size_t kMarks = MOE_PROFILE_STAGES + 1, kProfCalls = 8192;
+inline bool prof_room(const moe_layer* L) { return L->prof_used < kMarks * (kProfCalls + L->prof_more); }
 void mark(moe_layer* L) {
-  if (!L->prof) return;
+  if (!L->prof || !prof_room(L)) return;  // enough samples: stop recording
   if (L->prof_used == L->prof_ev.size()) {
-    if (L->prof_ev.size() >= 5 * 8192) return;  // enough samples; stop recording
     cudaEvent_t e;
     if (cudaEventCreate(&e) != cudaSuccess) return;
     L->prof_ev.push_back(e);
@@ -315,6 +317,13 @@ int check_status(moe_layer* L, bool sent = false) {
     return fail(MOE_ERR_DEVICE_TIMEOUT, "a bounded wait inside a GEMM kernel expired");
   }
   return MOE_OK;
+}
+
+// Drops what a call that failed half way has left of its marks, with the window before it.
+void prof_restart_if_torn(moe_layer* L) {
+  if (L->prof_used % kMarks == 0) return;
+  L->prof_used = 0;
+  L->prof_more = 0;
 }
 
 // Which large-batch GEMM a batch of at most `pairs` token-expert pairs runs, and what its groups are
@@ -436,7 +445,8 @@ int forward_impl(moe_layer* L, const void* x, int T, float beta, const void* res
     s_count = (int32_t*)(s + off[4]); s_nsk = (int32_t*)(s + off[5]); s_nt = (int32_t*)(s + off[6]);
   }
   Meta* meta = (Meta*)L->ws->meta.p;
-  if (L->prof && (L->prof_used % (MOE_PROFILE_STAGES + 1)) != 0) L->prof_used = 0;
+  if (L->prof) prof_restart_if_torn(L);
+  const bool recorded = L->prof && prof_room(L);
   mark(L);
   const bool single_gemv = T == 1 && L->single_gemv && !L->debug_simt && !dist;
   if (single_gemv) {
@@ -502,19 +512,23 @@ int forward_impl(moe_layer* L, const void* x, int T, float beta, const void* res
       dn.w_row0 = 512 * (tiles * s / slabs);
       dn.n_w_rows = s + 1 < slabs ? 512 * (tiles * (s + 1) / slabs) : L->h;
       const int cols = dn.n_w_rows - dn.w_row0;
+      if (s > 0 && recorded) {  // a set of marks for every slab: the later ones have two stages
+        ++L->prof_more;
+        for (int i = 0; i < 3; ++i) mark(L);
+      }
       for (int part = s == 0 ? 1 : 2; part <= 2; ++part)
         if ((rc = run_expert_gemms(L, meta, wm, m_gu, m_dn, gu, dn, kOutF32, (const bf16*)L->ws->xperm.p,
                                    (const bf16*)L->ws->act.p, rows_cap, 2ll * T, T, part)))
           return rc;
-      if (s == 0) mark(L);
+      mark(L);
       CUDA_TRY(launch_combine((const float*)L->ws->O.p, ksplit, split_stride, (int32_t*)L->ws->pair_pos.p,
                               (float*)L->ws->wn.p, (const bf16*)residual, T, L->h, (bf16*)y, st, dn.w_row0, cols));
+      mark(L);
       CUDA_TRY(cudaEventRecord(L->out_ev[0], st));
       CUDA_TRY(cudaStreamWaitEvent(L->out_stream, L->out_ev[0], 0));
       CUDA_TRY(cudaMemcpy2DAsync((bf16*)y_host + dn.w_row0, (size_t)L->h * 2, (const bf16*)y + dn.w_row0,
                                  (size_t)L->h * 2, (size_t)cols * 2, T, cudaMemcpyDeviceToHost, L->out_stream));
     }
-    mark(L);
     CUDA_TRY(cudaEventRecord(L->out_ev[1], L->out_stream));
     CUDA_TRY(cudaStreamWaitEvent(st, L->out_ev[1], 0));
     return MOE_OK;
@@ -827,9 +841,13 @@ int moe_forward_host(moe_layer_t* L, const void* x_host, int T, float beta, void
     }
   }
   CUDA_TRY(cudaMemcpyAsync(L->ws->hx.p, x_host, bytes, cudaMemcpyHostToDevice, L->stream));
+  if (L->prof) prof_restart_if_torn(L);
+  const size_t marks = L->prof_used, more = L->prof_more;
   rc = forward_impl(L, L->ws->hx.p, T, beta, nullptr, L->ws->hy.p, nullptr, nullptr, y_host, slabs);
   if (rc) {  // nothing may still be on its way to the caller's buffer
     if (slabs > 1) cudaStreamSynchronize(L->out_stream);
+    L->prof_used = marks;
+    L->prof_more = more;
     return rc;
   }
   if (slabs == 1) CUDA_TRY(cudaMemcpyAsync(y_host, L->ws->hy.p, bytes, cudaMemcpyDeviceToHost, L->stream));
@@ -990,7 +1008,7 @@ static int search_impl(moe_layer_t* L, const void* x_calib, const float* F_ref, 
   // While profiling, every chunk records one set of stage marks (permutation, gate/up, down, an
   // empty fourth stage) and the enumerations one more (three empty stages, then stage 3).
   const bool prof_saved = L->prof;
-  if (L->prof && (L->prof_used % (MOE_PROFILE_STAGES + 1)) != 0) L->prof_used = 0;
+  if (L->prof) prof_restart_if_torn(L);
   EnumSource src = {nullptr, nullptr, 0, 0, 0};
   GemmMaps m_gu, m_dn;
   m_gu.w = L->w13_256;
@@ -1216,23 +1234,24 @@ int moe_profile_enable(moe_layer_t* L, int on) {
   if (!L) return fail(MOE_ERR_INVALID_ARG, "layer is NULL");
   L->prof = on != 0;
   L->prof_used = 0;
+  L->prof_more = 0;
   return MOE_OK;
 }
 
 int moe_profile_read(moe_layer_t* L, float* stage_ms, int* calls) {
   if (!L || !stage_ms || !calls) return fail(MOE_ERR_INVALID_ARG, "NULL argument");
   CUDA_TRY(cudaStreamSynchronize(L->stream));
-  const size_t per = MOE_PROFILE_STAGES + 1;
-  const size_t n = L->prof_used / per;
+  const size_t n = L->prof_used / kMarks;
   for (int s = 0; s < MOE_PROFILE_STAGES; ++s) stage_ms[s] = 0.f;
   for (size_t c = 0; c < n; ++c)
     for (int s = 0; s < MOE_PROFILE_STAGES; ++s) {
       float ms = 0.f;
-      CUDA_TRY(cudaEventElapsedTime(&ms, L->prof_ev[c * per + s], L->prof_ev[c * per + s + 1]));
+      CUDA_TRY(cudaEventElapsedTime(&ms, L->prof_ev[c * kMarks + s], L->prof_ev[c * kMarks + s + 1]));
       stage_ms[s] += ms;
     }
-  *calls = (int)n;
+  *calls = (int)(n - L->prof_more);
   L->prof_used = 0;
+  L->prof_more = 0;
   return MOE_OK;
 }
 

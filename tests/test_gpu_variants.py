@@ -749,6 +749,29 @@ def test_host_calls_in_column_slabs_equal_the_device_call(h, E, T):
     layer.close()
 
 
+def test_stage_times_of_host_calls_in_column_slabs():
+    # every slab has a down GEMM and a combine of its own.  Four slabs of a layer whose down GEMM (0.25 TFLOP, 0.15 ms
+    # and more) takes several times what the combine (0.05 GB) does: with the GEMMs of three slabs in its stage, the
+    # combine would seem three times as long as the GEMM.
+    build.build()
+    W = synth.make_layer_weights(2048, 14336, 2, seed=82, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
+    x = synth.make_tokens(2100, 2048, seed=83, device=DEV)
+    xh, yh = x.cpu().pin_memory(), torch.empty(x.shape, dtype=x.dtype).pin_memory()
+    layer.forward(x)
+    layer.forward_host(xh, 0.0, yh)
+    for call in (lambda: layer.forward(x), lambda: layer.forward_host(xh, 0.0, yh)):
+        layer.profile_enable(True)
+        for _ in range(5):
+            call()
+        ms, calls = layer.profile_read()
+        assert calls == 5 and min(ms[:4]) > 0
+        assert ms[3] < 0.8 * ms[2], ms
+        assert layer.profile_read()[1] == 0   # a window of its own
+    layer.profile_enable(False)
+    layer.close()
+
+
 @pytest.mark.parametrize("h", [448, 512])
 def test_large_groups_on_either_side_of_the_width_line(h):
     # two kept experts, no skipping: groups of T tokens beyond the line of the narrow layers
