@@ -200,12 +200,12 @@ int moe_prune_search(moe_layer_t* layer, const void* x_calib, int T, int r, floa
  * loading the library holds until the process exits; T is therefore limited to
  * MOE_NOALLOC_MAX_TOKENS and larger T is rejected with MOE_ERR_INVALID_ARG.
  * The call makes no cudaMalloc/cudaFree and calls no allocating library
- * routine.  Its first call on a device is a warm-up: it looks up the array's
- * device address (cudaGetSymbolAddress), and under CUDA's lazy module loading
- * that look-up or the first launch may load this part of the library onto the
- * device, which takes device memory once (the code and the array).  Make that
- * first call at start-up, before any stream capture and before the device is
- * handed to the caller's own memory pool; the calls after it take nothing.
+ * routine.  Its first call on a device is a warm-up, whatever its T, h and r: it
+ * looks up the array's device address (cudaGetSymbolAddress) and, under CUDA's
+ * lazy module loading, loads every kernel that any later call may run, which
+ * takes device memory once (the code and the array).  Make that first call at
+ * start-up, before any stream capture and before the device is handed to the
+ * caller's own memory pool; the calls after it take nothing.
  * All calls share the one array, which keeps the previous call's contents:
  * every element that is read is rewritten first, so nothing needs clearing,
  * but two calls that overlap on the GPU (different streams or threads) race.

@@ -226,6 +226,8 @@ cudaError_t launch_set_dense_meta(Meta* meta, int E, int rows_per_expert, int of
 // k-th smallest (0-based) of ratio[T] for k = k0 and k1 (= k0 or k0 + 1), written to out[0], out[1]
 // (device memory or mapped host memory)
 cudaError_t launch_select2(const float* ratio, int T, int k0, int k1, float* out, cudaStream_t st);
+// brings every kernel of a calibration of up to MOE_NOALLOC_MAX_TOKENS tokens onto the device
+cudaError_t load_calibration_kernels();
 // W13[c][32q + s] = W1[id[c]][16q + s] (s < 16) | W3[id[c]][16q + s - 16] (s >= 16)
 cudaError_t launch_interleave(const bf16* W1, const bf16* W3, const KeptIds& kept, int r, int f,
                               int h, bf16* W13, cudaStream_t st);

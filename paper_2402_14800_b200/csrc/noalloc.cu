@@ -34,7 +34,8 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void* g_scratch_ptr[kMaxDevices] = {};
 
-// Device address of the scratch array on the current device, resolved once per device.
+// Device address of the scratch array on the current device, resolved once per device.  Which kernels a call runs
+// depends on T, h and r: the first call loads them all, so that the later ones take no device memory whatever they are.
 int scratch_address(StaticScratch** out) {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
@@ -46,6 +47,8 @@ int scratch_address(StaticScratch** out) {
     e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
     if (e != cudaSuccess || !p)
       return set_error(MOE_ERR_CUDA, "cudaGetSymbolAddress(static scratch): %s", cudaGetErrorString(e));
+    e = load_calibration_kernels();
+    if (e != cudaSuccess) return set_error(MOE_ERR_CUDA, "loading the kernels: %s", cudaGetErrorString(e));
     g_scratch_ptr[dev] = p;
   }
   *out = static_cast<StaticScratch*>(g_scratch_ptr[dev]);

@@ -1628,6 +1628,32 @@ cudaError_t launch_select2(const float* ratio, int T, int k0, int k1, float* out
   return launch_pdl(select2_kernel<0>, dim3(1), dim3(kSelThreads), 0, st, ratio, T, k0, k1, out);
 }
 
+// Under lazy module loading a kernel's code comes onto the device, and takes device memory, when it is first
+// launched or asked about: asks about every kernel that a calibration of up to 16384 tokens can run.
+template <int R> static cudaError_t load_routers(cudaError_t e) {
+  cudaFuncAttributes a;
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, router_kernel<R, true>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, router_kernel<R, false>);
+  return e;
+}
+template <int R> static cudaError_t load_ratios(cudaError_t e) {  // the forms of MOE_TILES_R
+  cudaFuncAttributes a;
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, ratio_kernel<R, 2, 4, true>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, ratio_kernel<R, 2, kRouteWarps, true>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, ratio_kernel<R, 2, kRouteWarps, false>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, ratio_kernel<R, 1, kRouteWarps, true>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, ratio_kernel<R, 1, kRouteWarps, false>);
+  return e;
+}
+cudaError_t load_calibration_kernels() {
+  cudaError_t e = load_ratios<kMaxE>(load_ratios<8>(cudaSuccess));
+  e = load_routers<2>(load_routers<4>(load_routers<6>(load_routers<8>(load_routers<kMaxE>(e)))));
+  cudaFuncAttributes a;
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, select2_kernel<8>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, select2_kernel<16>);
+  return e;
+}
+
 cudaError_t launch_interleave(const bf16* W1, const bf16* W3, const KeptIds& kept, int r, int f,
                               int h, bf16* W13, cudaStream_t st) {
   interleave_kernel<<<148 * 8, 256, 0, st>>>(W1, W3, kept, r, f, h, W13);
