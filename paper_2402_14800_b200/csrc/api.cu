@@ -866,7 +866,7 @@ int moe_calibrate_beta(moe_layer_t* L, const void* x, int T, float* beta_out) {
   memset(&ro, 0, sizeof(ro));
   ro.idx = (int32_t*)L->ws->idx.p; ro.wn = (float*)L->ws->wn.p; ro.ratio = (float*)L->ws->ratio.p;
   ro.skipped = (uint8_t*)L->ws->skipped.p;
-  if (L->h >= kRatioMinH) CUDA_TRY(launch_ratios((const bf16*)x, L->Wg, T, L->h, L->r, ro.ratio, L->stream));
+  if (calibrate_on_tiles(T, L->h, L->r)) CUDA_TRY(launch_ratios((const bf16*)x, L->Wg, T, L->h, L->r, ro.ratio, L->stream));
   else CUDA_TRY(launch_router((const bf16*)x, L->Wg, T, L->h, L->r, 0.f, L->kept, ro, L->stream));
   // the two values go straight to mapped host memory where the handle has some
   int* words = host_words(L, false);

@@ -67,10 +67,26 @@ constexpr int kRouterTcH = 2048;
 // Calibration on rows of at least so many columns has a router of its own (ratio_kernel); on narrower ones it runs the
 // forward router, whose ratios it then gives to the last bit.  The forward router's bits stay what they are: in a
 // stack a logit that moves in its last bit now and then flips a skip decision some layers on.  Calibration in us,
-// forward router / ratio_kernel, 8 experts, 300 and 8192 tokens: h 1024 19.2 / 17.4, 23.3 / 21.2; h 4096 23.3 / 19.1,
-// 35.9 / 28.0.  Error of the ratios against 64 bits (2-norm, 8192 tokens): h 1024 3.5e-7 / 2.6e-7, h 4096
-// (2000 tokens) 5.0e-7 / 2.6e-7.
+// forward router / ratio_kernel, 8 experts, 300, 8192 and 16384 tokens: h 1024 19.8 / 18.4, 24.1 / 21.5, 32.5 / 27.3;
+// h 4096 23.9 / 19.4, 37.1 / 27.7, 56.8 / 52.9.  Error of the ratios against 64 bits (2-norm, 8192 tokens): h 1024
+// 3.5e-7 / 2.6e-7, h 4096 (2000 tokens) 5.0e-7 / 2.6e-7.
+// Few experts: the forward router computes 2 or 4 columns where ratio_kernel computes 8, so on rows of kRatioFewH
+// columns and more it stays ahead where the rest is equal: with 3 and 4 experts on batches that L2 no longer holds
+// (h 2048, 4096, 6144, 8192, the same 67 MB: 32.3 / 30.0, 29.2 / 26.1, 29.6 / 28.1, 29.3 / 30.0; 88 MB: 41.9 / 41.5,
+// 37.0 / 43.8, 33.3 / 35.1, 33.7 / 41.6; 134 MB: 56.0 / 56.7, 47.4 / 51.9, 57.6 / 64.2, 43.4 / 47.4; the line is the
+// 4737th token of h 8192, with which its tiles go to four teams), with 2 experts from the second tile of a block on
+// (h 1536, 4096, 8192: 2400 tokens 20.7 / 22.1, 23.3 / 23.2, 26.7 / 27.9; 16384 tokens of h 4096 47.2 / 51.9).  With 5
+// and 6 experts either wins by turns (100 to 536 MB, h 1536 to 12288, ratio_kernel 0.82 to 1.17 of the forward router,
+// 0.96 on average: it stays).
 constexpr int kRatioMinH = 1024;
+constexpr int kRatioFewH = 1536;
+constexpr int kRatioTwoT = 148 * 16;
+constexpr size_t kRatioFewBytes = (size_t)74 << 20;
+inline bool calibrate_on_tiles(int T, int h, int r) {
+  if (h < kRatioFewH) return h >= kRatioMinH;
+  if (r == 2) return T <= kRatioTwoT;
+  return r > 4 || (size_t)T * h * 2 <= kRatioFewBytes;
+}
 constexpr int kDecodeKbPerItem = 112;      // k-blocks (of 64) per split-K item, decode down-proj
 
 // Device-resident description of one permuted batch, written by the permutation (beyond kPermuteOwnT
@@ -174,7 +190,7 @@ struct RouteOut {
 // w_const: Wg never changes (a handle's own rows) and may be read before the predecessor is done
 cudaError_t launch_router(const bf16* x, const bf16* Wg, int T, int h, int r, float beta,
                           const KeptIds& kept, const RouteOut& out, cudaStream_t st, bool w_const = true);
-// w_e1 / w_e0 of every token (calibration on rows of at least kRatioMinH columns)
+// w_e1 / w_e0 of every token (calibration, calibrate_on_tiles)
 cudaError_t launch_ratios(const bf16* x, const bf16* Wg, int T, int h, int r, float* ratio, cudaStream_t st,
                           bool w_const = true);
 // Large forward batches (kRouterTcT, kRouterTcH): the logits on the tensor cores (gemm_sm100.cu), the

@@ -88,7 +88,7 @@ extern "C" int moe_calibrate_beta_noalloc(const void* W_gate_kept, const void* x
   // Every element the selection reads (ratio[0..T)) is written by the router first, so stale
   // contents of an earlier call are never seen and nothing needs clearing.
   const bf16 *xb = static_cast<const bf16*>(x), *Wg = static_cast<const bf16*>(W_gate_kept);
-  cudaError_t e = h >= kRatioMinH ? launch_ratios(xb, Wg, T, h, r, ro.ratio, st, false)  // the rows are the caller's
+  cudaError_t e = calibrate_on_tiles(T, h, r) ? launch_ratios(xb, Wg, T, h, r, ro.ratio, st, false)  // the rows are the caller's
                                   : launch_router(xb, Wg, T, h, r, 0.f, ids, ro, st, false);
   if (e != cudaSuccess) return set_error(MOE_ERR_CUDA, "router launch: %s", cudaGetErrorString(e));
   e = launch_select2(s->ratio, T, (T - 1) / 2, T / 2, s->sel, st);

@@ -488,7 +488,7 @@ router_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part, floa
   if (!WHOLE) cp_async_wait<0>();  // the first part, fetched once more behind the last
 }
 
-// Calibration on rows of kRatioMinH columns and more, the top-k and the search router: a team of TW warps takes
+// Calibration (where calibrate_on_tiles says so), the top-k and the search router: a team of TW warps takes
 // tiles of 8 NT tokens in turn, its warps sharing the columns of a row (blocks of 64 columns); a block of
 // kRouteWarps warps is one team or several.  The products of 16 columns of up to 16 tokens with 8 router rows are
 // one mma.sync.m16n8k16: a [T x h] x [h x 16] contraction is bound by reading the token rows, which a handful of
@@ -496,8 +496,8 @@ router_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part, floa
 // passing through shared or tensor memory (the order of the columns inside a block is free, so the 16 bytes of a
 // row that a lane reads are its operands of two instructions).  Whole calibration call, before (router_kernel) ->
 // after, us: h 4096, 8 experts, 300 tokens 23.5 -> 19.5, 8192 36 -> 28.5, 16384 56.5 -> 50.5 (3.9 TB/s from DRAM);
-// h 2048, 16 experts, 16384 tokens 60 -> 39.  With 4 experts router_kernel, which then has half the arithmetic, stays
-// ahead on batches that L2 does not hold (16384 tokens of h 4096 46.5 -> 50.5).  What is slower: one warp that decides
+// h 2048, 16 experts, 16384 tokens 60 -> 39.  With 2 to 4
+// experts router_kernel, which then has half the arithmetic, stays ahead on long batches.  What is slower: one warp that decides
 // while the others wait (67 us at 16384 tokens), 8 tokens as the narrow operand (twice the instructions, 61), a column
 // phase of its own per block and deeper prefetch to L2 (no gain, and 58-60).
 //   - A logit: sums of 64 products by the tensor core, added up by each warp in column order and then over the

@@ -697,6 +697,35 @@ def test_allocation_free_calibration_of_ragged_rows_against_64_bits(h, r, T):
     assert abs(got - want) <= 2e-6 * want
 
 
+@pytest.mark.parametrize("h,kept,T,forward_bits", [
+    # on either side of the lines of few experts: 74 MiB of tokens with 3 and 4, 2368 tokens with 2, never with 5
+    (4096, 4, 9472, False), (4096, 4, 9473, True), (8192, 3, 4737, True), (1536, 2, 2368, False), (1536, 2, 2369, True),
+    (4096, 2, 16384, True), (4096, 5, 9473, False), (1024, 3, 40000, False)])
+def test_calibration_with_few_experts_takes_the_faster_router(h, kept, T, forward_bits):
+    # The forward router's ratios do not depend on the batch; calls of at most 4000 tokens record them.  Both routers
+    # give the median within the last bits, the forward router to the bit.
+    build.build()
+    W = synth.make_layer_weights(h, 64, 8, seed=84, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2, (1 << kept) - 1)
+    equal = 0
+    for seed in range(85, 90):
+        x = synth.make_tokens(T, h, seed=seed, device=DEV)
+        ratio = []
+        for part in x.tensor_split(-(-T // 4000)):
+            stats = binding.RoutingStats(part.shape[0], 8, DEV)
+            layer.forward(part.contiguous(), 0.0, stats=stats)
+            ratio.append(stats.ratio)
+        r = torch.cat(ratio).double().sort().values
+        want = float(((r[(T - 1) // 2] + r[T // 2]) / 2).float())
+        got = layer.calibrate_beta(x)
+        assert abs(got - want) <= 2e-6 * want
+        if T <= 16384:
+            assert binding.calibrate_beta_noalloc(W.W_gate[:kept].contiguous(), x) == got
+        equal += got == want
+    assert (equal == 5) if forward_bits else (equal < 5)
+    layer.close()
+
+
 @pytest.mark.parametrize("scale", [1.0, 2.0 ** -6, 2.0 ** -16, 0.0])
 @pytest.mark.parametrize("T", [2, 1000, 8193, 20000])
 def test_median_of_crowded_ratios(weights, T, scale):
