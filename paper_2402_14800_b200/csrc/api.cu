@@ -329,8 +329,8 @@ void prof_restart_if_torn(moe_layer* L) {
 // Which large-batch GEMM a batch of at most `pairs` token-expert pairs runs, and what its groups are
 // padded to.
 inline bool large_on_pairs(const moe_layer* L, long long pairs) {
-  return L->large_kernel == 1 ||
-         (L->large_kernel == 0 && pairs <= (long long)(L->h < kPairWideH ? kPairMaxRows : kPairMaxRowsWide) * L->r);
+  const long long rows = L->h < kPairWideH ? kPairMaxRows : (L->f < kPairDeepF ? kPairDownRows : kPairMaxRowsWide);
+  return L->large_kernel == 1 || (L->large_kernel == 0 && pairs <= rows * L->r);
 }
 inline bool down_on_pairs(const moe_layer* L, long long pairs) {
   return large_on_pairs(L, pairs) && (L->large_kernel == 1 || pairs <= (long long)kPairDownRows * L->r);

@@ -21,26 +21,31 @@ constexpr int kDecodeMaxT = 256;          // up to here the small-batch path (we
 constexpr int kTokensDPerExpert = 40;      // small batches with this many tokens per expert or more: token-major decode GEMM
 constexpr int kTokensDMaxKept = 6;         // ... on layers with at most this many kept experts
 // Large batches with at most so many pairs per kept expert (a forward call counts two per token, skipped or not)
-// run gemm_pair_n, the others gemm_tokens_m: kPairMaxRows on rows of fewer than kPairWideH columns, else
-// kPairMaxRowsWide.  Whole step, gemm_pair_n against gemm_tokens_m, alternating runs, pairs per expert
-// 1600 / 2048 / 4096 / 8192:
+// run gemm_pair_n, the others gemm_tokens_m: kPairMaxRows on rows of fewer than kPairWideH columns, kPairDownRows on
+// wider ones of experts with fewer than kPairDeepF features, else kPairMaxRowsWide.  Whole step, gemm_pair_n (in both
+// launches) against gemm_tokens_m, alternating runs, pairs per expert 1600 / 2048 / 4096 / 8192:
 //   (h, f, experts)    64, 64, 8        -1 % / +8 % / +16 % / +16 %
 //                      128, 448, 8      -4 / -4 / -3 / +9      256, 1024, 8     -6 / -7 / -1 / +8
 //                      512, 1024, 8    -22 / -19 / -10 / -5    1024, 2048, 8   -12 / -10 / -7 / -5
 //                      2048, 4096, 16   -8 / -7 / -7 / -5      4096, 1024, 8   -12 / -10 / -8 / -5
 // On narrow layers an item is a few k-blocks long and the two CTAs spend it on handing over to each other.  Mixtral
 // layer in 1.5 s loops at the power cap (ms): 8192 tokens (2048 a group) 4.77 vs 4.95, 16384 9.25 vs 9.45, 32768 (8192
-// a group) 18.56 vs 18.57, 65536 37.5-39.0 vs 36.2.  There the board's power is the limit, and the pairs draw less of it
-// for a product while there is padding to save (8192 tokens 4.62 vs 5.1 J).
+// a group) 18.56 vs 18.57, 65536 37.5-39.0 vs 36.2.  There the board's power is the limit.
 // Beyond kPairDownRows pairs per expert only the gate/up launch is theirs: in the down launch, whose items run over
-// many k-blocks, pairs that started an item apart read weights and activations from HBM again (8192 tokens 4.0 GB
-// where gemm_tokens_m reads 2.1).  Search of 32768 tokens (6144 a group), three runs on one board: gemm_tokens_m
-// 55.5-55.7 ms (55.0 J), pairs 53.4-54.2 (53.5), pairs and gemm_tokens_m 53.5-53.6 (52.6); forward of 32768 tokens
-// 18.2-18.5, 18.1, 18.0-18.2.  At 3000 a group the pairs alone are the faster by 1 %, at 500 by 6 %.
+// f / 64 k-blocks, pairs that started an item apart read weights and activations from HBM again (8192 tokens of the
+// Mixtral layer 4.0 GB where gemm_tokens_m reads 2.1).  Search of 32768 tokens (6144 a group), three runs on one
+// board: gemm_tokens_m 55.5-55.7 ms, pairs 53.4-54.2, pairs and gemm_tokens_m 53.5-53.6; forward of 32768 tokens
+// 18.2-18.5, 18.1, 18.0-18.2.  Below the line that mixture against the pairs in both launches, pairs per expert 500 /
+// 1024 / 1536 / 2048 / 3000 / 4096: Mixtral layer 1.01, 1.00, 1.02, 0.99, 1.00, 1.00 (a run differs by 2 %);
+// 1024 / 2048 / 4000: (2048, 4096, 16) 1.03, 1.05, 1.04, (4096, 1024, 8) 1.05, 1.09, 1.09, (1024, 256, 8) 1.07, 1.13,
+// 1.09.  Above it against gemm_tokens_m in both, 4500-5000 / 7000-8192: f 64 to 128 (h 512 to 4096) 1.02-1.05 /
+// 1.04-1.08, f 192 and 256 0.91-0.98 / 0.97-1.00, f 512 and more 0.92-0.98 / 0.98-1.00; hence kPairDeepF: with one or
+// two k-blocks in a down item a launch of either kind is its stores, and the pairs' half of the mixture wins too little.
 constexpr int kPairMaxRows = 1536;
 constexpr int kPairMaxRowsWide = 8192;
 constexpr int kPairDownRows = 4096;
 constexpr int kPairWideH = 512;
+constexpr int kPairDeepF = 192;
 // Top-k calls of more than kDecodeMaxT tokens with at most this many pairs per kept expert, half of the
 // weight-major kernel's token tile, run that kernel: it cuts the last round into K-slices, and hardly any
 // group needs a second tile.  Whole call in us, gemm_pair_n vs weight-major, layers of 16 experts (h, f):

@@ -816,3 +816,19 @@ def test_large_groups_on_either_side_of_the_width_line(h):
             assert torch.equal(forced(layer, kernel).forward(x), want)
     assert layer.device_status() == 0
     layer.close()
+
+
+@pytest.mark.parametrize("f,line", [(64, 4096), (128, 4096), (192, 8192)])
+def test_large_groups_of_experts_with_few_features(f, line):
+    # two kept experts, no skipping: groups of T tokens; beyond the line everything is the token-major kernel's
+    build.build()
+    W = synth.make_layer_weights(512, f, 3, seed=91, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2, 0b011)
+    assert layer.forward_kernel(line) == "gemm_pair_n_kernel" and layer.forward_kernel(line + 1) == "gemm_tokens_m_kernel"
+    for T in (4096, 4097, 4225):
+        x = synth.make_tokens(T, 512, seed=92, device=DEV)
+        want = layer.forward(x)
+        for kernel in (1, 2, 0):
+            assert torch.equal(forced(layer, kernel).forward(x), want)
+    assert layer.device_status() == 0
+    layer.close()
