@@ -49,6 +49,12 @@ int moe_test_wait_expiry_pair(moe_layer_t* layer, unsigned limit_us, int cta);
 int moe_test_large_batch(moe_layer_t* layer, int kernel, int tile_cap);
 
 /*
+ * Host side only.  Number of column slabs in which moe_forward_host would return a
+ * batch of T tokens to pinned memory (1 = in one piece; 0 for a bad argument).
+ */
+int moe_test_host_slabs(const moe_layer_t* layer, int T);
+
+/*
  * Host side only.  Make every later scratch or weight allocation of this process
  * see at most `bytes` of free device memory (the library compares its request
  * with cudaMemGetInfo before it calls cudaMalloc), so that MOE_ERR_OOM can be

@@ -83,6 +83,7 @@ def load_library(path: str | None = None):
     lib.moe_test_wait_expiry.argtypes = [vp, ctypes.c_uint, ci]
     lib.moe_test_wait_expiry_pair.argtypes = [vp, ctypes.c_uint, ci]
     lib.moe_test_large_batch.argtypes = [vp, ci, ci]
+    lib.moe_test_host_slabs.argtypes = [vp, ci]
     lib.moe_test_set_free_bytes_limit.restype = None
     lib.moe_test_set_free_bytes_limit.argtypes = [ctypes.c_longlong]
     lib.moe_last_error.restype = ctypes.c_char_p

@@ -394,13 +394,18 @@ int run_expert_gemms(moe_layer* L, const Meta* meta, bool weights_m, const GemmM
 }
 
 // Column slabs in which a batch for the host leaves the device: the copy of one runs while the down projection
-// of the next is computed.  A slab is a whole number of the pair kernel's 512-row weight tiles.  Mixtral layer, whole ->
-// slabs: 1500 tokens 1423 -> 1352 us, 5000 tokens 4150 -> 3750 (four slabs); 700 tokens 820 -> 865, the smaller launches
-// fill the machine worse than the copy is long, hence the line at 4 Mi values.
+// of the next is computed.  A slab is a whole number of the pair kernel's 512-row weight tiles.  Whole -> slabs in us:
+// Mixtral layer 700 tokens 820 -> 865, 1024 1092 -> 1033, 1500 1422 -> 1311, 5000 4150 -> 3750 (four slabs), 8192 6765 ->
+// 5781; pruned to 2 experts 1500 1258 -> 1153, 5000 4128 -> 4036, to 4 1272 -> 1172, 4211 -> 3609; (h, f, experts) =
+// (4096, 1024, 8) 1024 436 -> 425, 2047 793 -> 786, 8192 3003 -> 2851; (2048, 4096, 16) 2060 601 -> 563; (1024, 1024, 8),
+// whose slabs are copied in rows of 1 KB, 4200 448 -> 439, 5000 517 -> 520, 8100 830 -> 788.  Below 4 Mi values the
+// smaller launches fill the machine worse than the copy is long.  With few features there is little of a down projection
+// to copy beside, and the line is at 8 Mi: f 64 to 256, 1500 tokens of h 4096 559 -> 565 and 572 -> 579, 5000 of h 1024 471
+// -> 484; from 8 Mi on 2048 tokens of h 4096 733 -> 723, 8192 of h 1024 747 -> 735.
 inline int host_slabs(const moe_layer* L, int T) {
   if (decode_mode(T) || L->debug_simt || !down_on_pairs(L, 2ll * T)) return 1;
   const int want = T < 2048 ? 2 : 4, tiles = L->h / 512;
-  if ((size_t)T * L->h < (size_t)1 << 22 || tiles < 2) return 1;
+  if ((size_t)T * L->h < (size_t)(L->f < 1024 ? 8 : 4) << 20 || tiles < 2) return 1;
   return want < tiles ? want : tiles;
 }
 
@@ -728,6 +733,8 @@ int moe_test_wait_expiry_pair(moe_layer_t* L, unsigned limit_us, int cta) {
   CUDA_TRY(launch_wait_expiry_pair((int*)L->ws->status.p, (unsigned long long)limit_us * 1000ull, cta, L->stream));
   return MOE_OK;
 }
+
+int moe_test_host_slabs(const moe_layer_t* L, int T) { return L && T > 0 && T <= kMaxTokens ? host_slabs(L, T) : 0; }
 
 int moe_test_large_batch(moe_layer_t* L, int kernel, int tile_cap) {
   if (!L) return fail(MOE_ERR_INVALID_ARG, "layer is NULL");

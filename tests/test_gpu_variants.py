@@ -778,6 +778,25 @@ def test_host_calls_in_column_slabs_equal_the_device_call(h, E, T):
     layer.close()
 
 
+@pytest.mark.parametrize("h,f,E,sizes", [
+    # (tokens, slabs): 4 Mi values with many features, 8 Mi with few; two and four slabs, fewer tiles than four, a last
+    # slab that ends inside a weight tile, more pairs per expert than the pair kernel's down projection takes
+    (1024, 1024, 2, [(4095, 1), (4096, 2), (4097, 1)]), (1600, 1024, 4, [(2621, 1), (2622, 3)]),
+    (2560, 1024, 8, [(1638, 1), (1639, 2), (2047, 2), (2048, 4)]), (2560, 960, 8, [(2560, 1), (3277, 4)]),
+    (448, 1024, 8, [(9400, 1)])])
+def test_lines_of_the_column_slabs(h, f, E, sizes):
+    build.build()
+    W = synth.make_layer_weights(h, f, E, seed=93, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
+    for T, slabs in sizes:
+        assert binding.load_library().moe_test_host_slabs(layer._h, T) == slabs, T
+        x = synth.make_tokens(T, h, seed=94, device=DEV)
+        y = torch.zeros_like(x, device="cpu").pin_memory()
+        assert torch.equal(layer.forward_host(x.cpu().pin_memory(), 0.3, y), layer.forward(x, 0.3).cpu()), T
+    assert layer.device_status() == 0
+    layer.close()
+
+
 def test_stage_times_of_host_calls_in_column_slabs():
     # every slab has a down GEMM and a combine of its own.  Four slabs of a layer whose down GEMM (0.25 TFLOP, 0.15 ms
     # and more) takes several times what the combine (0.05 GB) does: with the GEMMs of three slabs in its stage, the
