@@ -176,16 +176,19 @@ __device__ __forceinline__ void pair_errors_generic(const bf16* __restrict__ Yt,
 }
 
 // The kept masks of a short list travel with the launch (a copy of their own to the device costs more than
-// the enumeration of a few hundred tokens).
+// the enumeration of a few hundred tokens).  A block moves them to shared memory eight at a time, every lane of a
+// warp reading the same 16 bytes: lanes that read different parameters are served one after the other.
 constexpr int kListMax = 1020;
 struct SubsetList {
-  uint16_t mask[kListMax];
+  uint4 eight[(kListMax + 7) / 8];  // uint16_t masks
 };
+constexpr size_t list_bytes(int nC) { return (size_t)(nC + 7) / 8 * 16; }
 
 // KT = K for the Gram form (K = 2 .. 6), 0 for any K through the generic form; REF = a target row
 // per token is given (progressive search).  subsets == null: the masks are those of `list`.
-// The Gram form is a programmatic dependent of the last GEMM; the generic one, which re-reads its rows from
-// L1, is launched in plain stream order.
+// The Gram form with a list is a programmatic dependent of the last GEMM.  The generic form, which re-reads its rows
+// from L1, and a longer list, whose masks every token reads from L1 again, are launched in plain stream order (the
+// masks read at L2: 8008 subsets, 1024 tokens 908 -> 1128 us, 2002 subsets, 4096 tokens 282 -> 401).
 template <int KT, bool REF>
 __global__ void __launch_bounds__(128)
 enumerate_kernel(const float* logits, const bf16* Yall, int T, int E, int r, int h, const uint32_t* subsets, int nC,
@@ -203,9 +206,12 @@ enumerate_kernel(const float* logits, const bf16* Yall, int T, int E, int r, int
   float* s_l = reinterpret_cast<float*>(base_order + nwarps * kMaxE) + warp * kMaxE;
   int* s_row = reinterpret_cast<int*>(base_order + 2 * nwarps * kMaxE) + warp * kMaxE;
 
-  uint16_t* s_mask = reinterpret_cast<uint16_t*>(base_order + 3 * nwarps * kMaxE);
+  const uint16_t* s_mask = reinterpret_cast<uint16_t*>(base_order + 3 * nwarps * kMaxE);
   if (!subsets)
-    for (int s = threadIdx.x; s < nC; s += blockDim.x) s_mask[s] = list.mask[s];
+    for (int i = warp; 8 * i < nC; i += nwarps) {
+      const uint4 eight = list.eight[i];
+      if (lane == 0) reinterpret_cast<uint4*>(base_order + 3 * nwarps * kMaxE)[i] = eight;
+    }
   for (int s = lane; s < nC; s += 32) acc[s] = 0.f;
   __syncthreads();
   pdl_wait();
@@ -244,7 +250,7 @@ enumerate_kernel(const float* logits, const bf16* Yall, int T, int E, int r, int
     else pair_errors_generic(Yt, h, K, s_order, s_row, s_l, lane, s_err, ref);
     __syncwarp();
     for (int s = lane; s < nC; s += 32) {
-      const uint32_t mask = subsets ? ld_l2(reinterpret_cast<const int32_t*>(subsets) + s) : s_mask[s];
+      const uint32_t mask = subsets ? __ldg(subsets + s) : s_mask[s];
       int i = -1, j = -1;
       for (int q = 0; q < K; ++q) {  // the two best kept experts are always among the top K
         if ((mask >> s_order[q]) & 1u) {
@@ -263,20 +269,27 @@ enumerate_kernel(const float* logits, const bf16* Yall, int T, int E, int r, int
   }
 }
 
-// One warp per subset: lane i adds blocks i, i+32, ... in order, then a fixed shuffle tree;
-// the order depends only on the number of blocks, so the result is reproducible.
+// Eight subsets per block: 32 threads of a subset add blocks i, i+32, ... in order, then one warp forms a fixed shuffle
+// tree of the 32 sums; the order depends only on the number of blocks, so the result is reproducible.  Eight subsets
+// are the 32 bytes that a read at L2 brings.
 // `losses` and `status_out` may be mapped host memory: the device's error word goes along with the losses.
-__global__ void __launch_bounds__(32)
+__global__ void __launch_bounds__(256)
 reduce_partials_kernel(const float* partial, int nblk, int nC, double* __restrict__ loss_sq,
                        float* __restrict__ losses, const int* status, int* status_out) {
+  __shared__ double s_sum[8][33];
   pdl_wait();
-  const int s = blockIdx.x;
-  const int lane = threadIdx.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int mine = blockIdx.x * 8 + (threadIdx.x & 7), first = threadIdx.x >> 3;
   double v = 0.0;
-  for (int b = lane; b < nblk; b += 32) v += (double)ld_l2(partial + (size_t)b * nC + s);
+  if (mine < nC)
+    for (int b = first; b < nblk; b += 32) v += (double)ld_l2(partial + (size_t)b * nC + mine);
+  s_sum[threadIdx.x & 7][first] = v;
+  __syncthreads();
+  v = s_sum[warp][lane];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if (lane == 0) {
+  const int s = blockIdx.x * 8 + warp;
+  if (lane == 0 && s < nC) {
     loss_sq[s] = v;
     losses[s] = (float)sqrt(v);
     if (s == 0 && status_out) *status_out = ld_l2(status);
@@ -286,7 +299,7 @@ reduce_partials_kernel(const float* partial, int nblk, int nC, double* __restric
 int warps_for(int nC) { return nC <= 2048 ? 4 : 1; }
 size_t enumerate_smem(int nC) {
   const size_t nw = warps_for(nC);
-  return (nw * nC + nw * kMaxE * kMaxE + 3 * nw * kMaxE) * 4 + (nC <= kListMax ? 2 * kListMax : 0);
+  return (nw * nC + nw * kMaxE * kMaxE + 3 * nw * kMaxE) * 4 + (nC <= kListMax ? list_bytes(nC) : 0);
 }
 
 }  // namespace
@@ -322,7 +335,7 @@ cudaError_t launch_enumerate(const float* logits, const bf16* Yall, int T, int E
   SubsetList list;
   if (enumerate_takes_list(nC)) {
     subsets = nullptr;
-    for (int i = 0; i < nC; ++i) list.mask[i] = (uint16_t)host_subsets[i];
+    for (int i = 0; i < nC; ++i) reinterpret_cast<uint16_t*>(list.eight)[i] = (uint16_t)host_subsets[i];
   }
   auto kernel = enumerate_kernel<0, false>;
 #define MOE_ENUM_PICK(KK)                                                                   \
@@ -339,12 +352,13 @@ cudaError_t launch_enumerate(const float* logits, const bf16* Yall, int T, int E
   cudaError_t e = cudaSuccess;
   if (smem > 48 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   if (e != cudaSuccess) return e;
-  e = K <= 6 ? launch_pdl(kernel, dim3(nblk), dim3(nw * 32), smem, st, logits, Yall, T, E, r, h, subsets, nC, partial,
+  e = K <= 6 && !subsets
+             ? launch_pdl(kernel, dim3(nblk), dim3(nw * 32), smem, st, logits, Yall, T, E, r, h, subsets, nC, partial,
                           Fref, src, list)
              : launch_plain(kernel, dim3(nblk), dim3(nw * 32), smem, st, logits, Yall, T, E, r, h, subsets, nC, partial,
                             Fref, src, list);
   if (e != cudaSuccess) return e;
-  return launch_pdl(reduce_partials_kernel, dim3(nC), dim3(32), 0, st, partial, nblk, nC, loss_sq, losses, status,
+  return launch_pdl(reduce_partials_kernel, dim3((nC + 7) / 8), dim3(256), 0, st, partial, nblk, nC, loss_sq, losses, status,
                     status_out);
 }
 

@@ -7,7 +7,9 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import moe_oracle as O
 from paper_2402_14800_b200 import binding, build, synth
+from tests import parity as P
 
 pytestmark = pytest.mark.gpu
 
@@ -759,6 +761,21 @@ def test_subsets_that_travel_with_the_launch_and_subsets_in_memory():
     with pytest.raises(binding.MoeError):
         layer.prune_search(x, 10)
     assert layer.prune_search(x, 10) == alone
+    layer.close()
+
+
+@pytest.mark.parametrize("E,r,T", [(4, 3, 1), (6, 4, 33), (13, 9, 130), (14, 10, 4100), (14, 9, 37), (16, 12, 129), (16, 8, 5)])
+def test_enumerations_of_every_list_length_against_the_oracle(E, r, T):
+    # 4 and 15 subsets (less than and not a multiple of the 8 that a block reduces), 715 and 1001 with the launch,
+    # 1820 through memory, 2002 and 12870 through memory and pair by pair; 1 to 1025 partial sums per subset
+    build.build()
+    W = synth.make_layer_weights(128, 64, E, seed=95)
+    layer = binding.MoeLayer(*(t.to(DEV) for t in (W.W_gate, W.W1, W.W3, W.W2)))
+    x = synth.make_tokens(T, 128, seed=96)
+    losses, best = layer.prune_search(x.to(DEV), r)
+    b = synth.bf16_bits
+    P.check_search(losses, best, O.prune_search_allexperts(b(x), b(W.W_gate), b(W.W1), b(W.W3), b(W.W2), r))
+    assert layer.prune_search(x.to(DEV), r) == (losses, best)
     layer.close()
 
 
