@@ -75,20 +75,23 @@ constexpr int kRouterTcH = 2048;
 // forward router / ratio_kernel, 8 experts, 300, 8192 and 16384 tokens: h 1024 19.8 / 18.4, 24.1 / 21.5, 32.5 / 27.3;
 // h 4096 23.9 / 19.4, 37.1 / 27.7, 56.8 / 52.9.  Error of the ratios against 64 bits (2-norm, 8192 tokens): h 1024
 // 3.5e-7 / 2.6e-7, h 4096 (2000 tokens) 5.0e-7 / 2.6e-7.
-// Few experts: the forward router computes 2 or 4 columns where ratio_kernel computes 8, so on rows of kRatioFewH
-// columns and more it stays ahead where the rest is equal: with 3 and 4 experts on batches that L2 no longer holds
+// Few experts: the forward router computes 2 or 4 columns where ratio_kernel computes 8, so on rows of kRatioFewMinH
+// to kRatioFewMaxH columns it stays ahead where the rest is equal: with 3 and 4 experts on batches that L2 no longer holds
 // (h 2048, 4096, 6144, 8192, the same 67 MB: 32.3 / 30.0, 29.2 / 26.1, 29.6 / 28.1, 29.3 / 30.0; 88 MB: 41.9 / 41.5,
 // 37.0 / 43.8, 33.3 / 35.1, 33.7 / 41.6; 134 MB: 56.0 / 56.7, 47.4 / 51.9, 57.6 / 64.2, 43.4 / 47.4; the line is the
 // 4737th token of h 8192, with which its tiles go to four teams), with 2 experts from the second tile of a block on
 // (h 1536, 4096, 8192: 2400 tokens 20.7 / 22.1, 23.3 / 23.2, 26.7 / 27.9; 16384 tokens of h 4096 47.2 / 51.9).  With 5
 // and 6 experts either wins by turns (100 to 536 MB, h 1536 to 12288, ratio_kernel 0.82 to 1.17 of the forward router,
-// 0.96 on average: it stays).
+// 0.96 on average: it stays).  Beyond kRatioFewMaxH, the widest rows measured, ratio_kernel stays too: a router that is
+// zero but for some columns then gives the ratios of the narrow one to the bit whatever the number of tokens, which
+// two routers with sums in different orders do not.
 constexpr int kRatioMinH = 1024;
-constexpr int kRatioFewH = 1536;
+constexpr int kRatioFewMinH = 1536;
+constexpr int kRatioFewMaxH = 12288;
 constexpr int kRatioTwoT = 148 * 16;
 constexpr size_t kRatioFewBytes = (size_t)74 << 20;
 inline bool calibrate_on_tiles(int T, int h, int r) {
-  if (h < kRatioFewH) return h >= kRatioMinH;
+  if (h < kRatioFewMinH || h > kRatioFewMaxH) return h >= kRatioMinH;
   if (r == 2) return T <= kRatioTwoT;
   return r > 4 || (size_t)T * h * 2 <= kRatioFewBytes;
 }
