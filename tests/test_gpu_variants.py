@@ -649,6 +649,18 @@ def test_forward_kernel_names_the_kernel_that_runs(weights):
     four.close()
 
 
+def overflow_one_logit(Wg, x):
+    """Makes the last expert's logit infinite in fp32, and no other one, on every 16th token (3e38 times 2; the column
+    is zero for everyone else).  Returns the mask of those tokens."""
+    mask = torch.arange(x.shape[0], device=DEV) % 16 == 7
+    Wg[:, 5], x[:, 5] = 0.0, 0.0
+    Wg[-1, 5], x[mask, 5] = 2.0, 3e38
+    logits = x.float() @ Wg.float().T
+    assert torch.isinf(logits[mask, -1]).all()
+    assert torch.isfinite(logits[:, :-1]).all() and torch.isfinite(logits[~mask]).all()
+    return mask
+
+
 @pytest.mark.parametrize("h,E,T", [
     # one team per block with tiles of 8 and of 16 tokens, four teams: the lines between them (1184 tokens, 4736, rows
     # of 2048 columns), tiles that end inside a warp's tokens; rows of one block of 64 columns, of fewer blocks than
@@ -661,21 +673,24 @@ def test_router_at_the_edges_of_its_tiles_against_64_bits(h, E, T):
     # products by the tensor core add little to it (0.7e-7 to 1.1e-7 seen, 2-norm over the batch).
     build.build()
     W = synth.make_layer_weights(h, 64, E, seed=70, device=DEV)
-    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
     x = synth.make_tokens(T, h, seed=71, device=DEV)
-    x[T // 2, 5] = 3e38  # an infinite logit leads alone
+    infinite = overflow_one_logit(W.W_gate, x)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
     ranked = (x.double() @ W.W_gate.double().T).sort(dim=1, descending=True)
     k = min(E, 4)
     _, idx, wn, n_active = layer.forward_topk(x, k, 0.0, record=True)
-    finite = torch.arange(T, device=DEV) != T // 2
-    same = (idx.long() == ranked.indices[:, :k]).all(1) & finite
+    same = (idx.long() == ranked.indices[:, :k]).all(1)
+    # the infinite logit leads, and the others rank behind it as ever (its weight is exp(inf - inf))
+    assert (idx[infinite, 0] == E - 1).all() and same[infinite].float().mean() > 0.98
+    finite = ~infinite
     assert same[finite].float().mean() > 0.99 and torch.isfinite(wn[finite]).all() and int(n_active.min()) >= 1
+    same &= finite
     want = torch.softmax(ranked.values[same, :k], 1)
     assert float((wn[same].double() - want).norm() / want.norm()) < 1.45e-7
-    # the median of the ratios: two logits of up to 8 in magnitude, whose last bit is 4.8e-7; the infinite one has
-    # a ratio of 0
+    # the median of the ratios: two logits of up to 8 in magnitude, whose last bit is 4.8e-7; the infinite ones have
+    # a ratio of 0 (one token in 16: with any other ratio there the median would lie some per cent off)
     ratio = torch.exp(ranked.values[:, 1] - ranked.values[:, 0])
-    ratio[T // 2] = 0.0
+    assert float(ratio[infinite].max()) == 0.0
     s = ratio.sort().values
     want = float((s[(T - 1) // 2] + s[T // 2]) / 2)
     assert abs(layer.calibrate_beta(x) - want) <= 2e-6 * want
@@ -688,10 +703,10 @@ def test_allocation_free_calibration_of_ragged_rows_against_64_bits(h, r, T):
     # rows that end inside a block of 64 columns; an infinite logit has a ratio of 0
     Wg = synth.make_layer_weights(max(64, -(-h // 64) * 64), 64, 16, seed=72, device=DEV).W_gate[:r, :h].contiguous()
     x = synth.make_tokens(T, h, seed=73, device=DEV)
-    x[7, 0] = 3e38
+    infinite = overflow_one_logit(Wg, x)
     top = (x.double() @ Wg.double().T).sort(dim=1, descending=True).values
     ratio = torch.exp(top[:, 1] - top[:, 0])
-    ratio[7] = 0.0
+    assert float(ratio[infinite].max()) == 0.0
     s = ratio.sort().values
     want = float((s[(T - 1) // 2] + s[T // 2]) / 2)
     got = binding.calibrate_beta_noalloc(Wg, x)
