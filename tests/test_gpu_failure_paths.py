@@ -127,3 +127,40 @@ def test_an_expired_wait_in_one_cta_of_a_pair_ends_both(tiny, cta):
         check_against_oracle(layer, host, 700, 0xFF, 0.3, seed=8)   # on the CTA pairs
     assert lib.moe_test_wait_expiry_pair(layer._h, 1000, 2) == -1 and lib.moe_test_wait_expiry_pair(layer._h, 0, 0) == -1
     layer.close()
+
+
+def test_error_paths_of_a_host_call_in_column_slabs():
+    # four slabs, whose copies run on a stream of the handle's own
+    build.build()
+    lib = binding.load_library()
+    W = synth.make_layer_weights(2048, 1024, 4, seed=9, device=DEV)
+    layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
+    x = synth.make_tokens(8000, 2048, seed=10, device=DEV)
+    xh = x.cpu().pin_memory()
+    yh = torch.zeros_like(xh).pin_memory()
+    assert lib.moe_test_host_slabs(layer._h, 2100) == 4 and lib.moe_test_host_slabs(layer._h, 8000) == 4
+    want = layer.forward(x[:2100].contiguous(), 0.3).cpu()
+    for expire in (lambda: lib.moe_test_wait_expiry(layer._h, 500, 0), lambda: lib.moe_test_wait_expiry_pair(layer._h, 500, 1)):
+        assert expire() == 0
+        with pytest.raises(binding.MoeError) as e:
+            layer.forward_host(xh[:2100], 0.3, yh[:2100])
+        assert e.value.code == MOE_ERR_DEVICE_TIMEOUT
+        assert layer.device_status() == 0                      # reported once
+        yh.zero_()
+        assert torch.equal(layer.forward_host(xh[:2100], 0.3, yh[:2100]), want)
+    # the staging buffers of the longer batch (33 MB) fit, its permuted rows (68 MB) do not: the call fails after the
+    # copy in, before the first slab
+    yh.zero_()
+    try:
+        lib.moe_test_set_free_bytes_limit(64 << 20)
+        with pytest.raises(binding.MoeError) as e:
+            layer.forward_host(xh, 0.3, yh)
+        assert e.value.code == MOE_ERR_OOM
+    finally:
+        lib.moe_test_set_free_bytes_limit(-1)
+    torch.cuda.synchronize()
+    assert not yh.any()
+    for T in (2100, 8000, 64):
+        assert torch.equal(layer.forward_host(xh[:T], 0.3, yh[:T]), layer.forward(x[:T].contiguous(), 0.3).cpu())
+    assert layer.device_status() == 0
+    layer.close()
