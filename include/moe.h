@@ -153,7 +153,7 @@ int moe_forward_host(moe_layer_t* layer, const void* x_host, int T, float beta, 
  * in this order, each starting at a multiple of 16 bytes:
  *   int32  idx[T][2]      original ids of e0, e1
  *   float  wn[T][2]       weights applied to E_e0, E_e1 (1, 0 after a skip)
- *   float  ratio[T]       w_e1 / w_e0
+ *   float  ratio[T]       w_e1 / w_e0 (the value the skip test took)
  *   uint8  skipped[T]
  *   int32  count[E][2]    token-expert pairs that ran, per expert and slot
  *   int32  n_skipped
@@ -168,7 +168,11 @@ size_t moe_routing_stats_bytes(int T, int E);
  * beta for dynamic skipping (Sec. 3.3): the median over the T calibration
  * tokens of w_e1 / w_e0 under this layer's router; for even T the mean of the
  * two middle values.  x [T][h] bf16 device, T >= 1; *beta_out is host memory.
- * Synchronises the handle's stream.
+ * Synchronises the handle's stream.  Routers for different sizes add up in
+ * different orders, so beta is the median of the ratios that a forward call on
+ * the same tokens records up to a few units in the last place (2e-6 relative):
+ * a token that lies that close to beta, such as the median token of an odd T, may
+ * fall on either side of the strict test.
  */
 int moe_calibrate_beta(moe_layer_t* layer, const void* x, int T, float* beta_out);
 
