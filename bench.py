@@ -493,7 +493,9 @@ def search_case(layer, x, steps, warmup, stream, dev, rank, local, world, peaks,
     en_bytes = T * H * 2 * K + T * E * 4
     ach = gu_flop / (gu_ms * 1e-3) / 1e12
     step_tf = (gu_flop + dn_flop) / (ms_step * 1e-3) / 1e12
-    roofline = {"bound": "tensor", "kernel": "gemm_tokens_m_kernel<gate_up> (expert evaluations of the search)",
+    # a chunk of the search is a batch of K pairs per token on the large-batch kernels
+    kernel = gate_up_kernel(layer, max(257, K * min(T, 8192) // 2))
+    roofline = {"bound": "tensor", "kernel": kernel + " (expert evaluations of the search)",
                 "achieved": ach, "peak": peaks["tf_sust"], "unit": "TFLOP/s", "frac": ach / peaks["tf_sust"],
                 "traffic": None, "frac_of_burst": ach / peaks["tf_burst"],
                 "frac_of_nominal_dense_bf16": ach / NOMINAL_BF16_TFLOPS,

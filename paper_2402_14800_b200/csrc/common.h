@@ -118,6 +118,12 @@ struct KeptIds {
 // predecessor wrote (or still reads).  Every kernel on the forward path calls
 // pdl_launch_dependents() and pdl_wait() first thing (the GEMMs after their set-up), so the
 // stream order of all memory accesses is unchanged and only launch latency and prologues overlap.
+// The one exception are the down launches of gemm_pair_n, gemm_weights_m and gemm_tokens_d: before they wait they
+// read the batch description (Meta) and fetch weights (handover_wait in gemm_sm100.cu), and their MMA warps never wait.
+// What that rests on: Meta is complete before the gate/up launch of the batch passes its own wait, and that launch
+// triggers only then.  So nothing from the gate/up launch to the last down launch of a batch (the combine kernels between
+// the column slabs of a host call among them) may write Meta or weights, nor may a kernel that does so trigger early
+// and be followed by a down launch directly.
 //
 // THE RULE for every kernel launched with launch_pdl: whatever an earlier kernel of the stream
 // may have written (token rows, routing records, permutation tables, the batch description,

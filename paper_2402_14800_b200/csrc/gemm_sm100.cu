@@ -575,7 +575,10 @@ gemm_tokens_m_kernel(const __grid_constant__ GemmMaps maps, const GemmArgs args)
 // shared memory of an SM, so they move in one by one as gate/up CTAs leave.  What they may touch before the last
 // of those has left: the batch description (written before the gate/up launch passed its wait) and the
 // weights, so they read the work list, set up and fetch the weights of their first stages; every role waits
-// before it touches anything else.  Before, launch latency, set-up and the first trip to HBM lay between the two.
+// before it touches anything else (the MMA warps touch what the producer fetched).  Before, launch latency, set-up and
+// the first trip to HBM lay between the two.  The down launches of a host call's later column slabs follow a combine
+// kernel, which triggers before its own wait: the batch description is that of the same batch, written before its
+// gate/up launch, and the combine writes neither it nor weights.
 template <bool GATE_UP> __device__ __forceinline__ void handover_wait() {
   if (GATE_UP) {
     pdl_wait();

@@ -495,18 +495,20 @@ router_kernel(const bf16* x, const bf16* Wg, int T, int h, int r, int part, floa
 // warp-level instructions keeps up with, and tokens go from global memory to the instruction's registers without
 // passing through shared or tensor memory (the order of the columns inside a block is free, so the 16 bytes of a
 // row that a lane reads are its operands of two instructions).  Whole calibration call, before (router_kernel) ->
-// after, us: h 4096, 8 experts, 300 tokens 23.5 -> 19.5, 8192 36 -> 28.5, 16384 56.5 -> 50.5 (3.9 TB/s from DRAM);
-// h 2048, 16 experts, 16384 tokens 60 -> 39.  With 2 to 4
-// experts router_kernel, which then has half the arithmetic, stays ahead on long batches.  What is slower: one warp that decides
-// while the others wait (67 us at 16384 tokens), 8 tokens as the narrow operand (twice the instructions, 61), a column
-// phase of its own per block and deeper prefetch to L2 (no gain, and 58-60).
+// after, us: h 4096, 8 experts, 300 tokens 23.9 -> 19.4, 8192 37.1 -> 27.7, 16384 56.8 -> 52.9, 32768 97.4 -> 85.8;
+// h 2048, 16 experts, 16384 tokens 60.3 -> 36.5.  With 2 to 4 experts router_kernel, which then has half the arithmetic,
+// stays ahead on long batches.  Forms that were slower (16384 tokens, when this one took 50): one warp that decides
+// while the others wait 67, 8 tokens as the narrow operand (twice the instructions) 61, prefetching deeper to L2 58-60;
+// a column phase of its own per block changed nothing.  Top-k calls in a row of layers with few columns or experts lose
+// 1-3 us to the router of chains of multiply-adds that ran before (E 4, h 512, f 64, 1000 tokens 33.4 -> 35.7 us a
+// call; alone the launch takes as long); tiles for teams of 4 warps or two blocks per SM did not change that.
 //   - A logit: sums of 64 products by the tensor core, added up by each warp in column order and then over the
 //     warps, both as compensated fp32 sums (the tensor core drops bits that an IEEE addition would round, which
 //     costs little over 64 products and too much over a row).
 //   - The router rows wait in shared memory in operand order, fetched before the wait for the predecessor where
 //     they never change; rows too long for it (h beyond 10880 with 8 experts, 4416 with 16) are read at L2.
-//   - Up to 8 NT loads of 16 bytes per lane are in flight; a slot is refilled, from the next tile if need be, as
-//     soon as it is used.
+//   - A lane has 8 NT slots of 16 bytes; a slot is refilled, from the next tile if need be, as soon as it is used, in
+//     order, so that fewer than that are in flight on average.
 //   - After a tile's one barrier every warp of the team adds up and decides its share of the tokens.
 
 // d += A (16 tokens x 16 columns) B (16 columns x 8 router rows)
