@@ -549,8 +549,8 @@ template <int R, int NT, int TW> struct TileCfg {
 
 // 16 bytes of a token row, read at L2 (the rule beside launch_pdl); their 256 bytes are fetched to L2 along with them.
 // `once`: a batch that L2 does not hold; the lines in flight are not allocated in L1 either, which holds few of
-// them beside the shared memory (16384 / 32768 tokens of h 4096 from DRAM 53.5 / 87 -> 50.1 / 82.6 us; 8192 tokens,
-// from L2, 27.9 -> 30.9).
+// them beside the shared memory (14000 / 16384 / 32768 tokens of h 4096 from DRAM 52.1 / 54.8 / 91.8 -> 49.6 / 51.3 /
+// 85.4 us; 8192 tokens, from L2, 27.9 -> 30.9).
 __device__ __forceinline__ uint4 ld_row(const uint4* p, bool once) {
   uint4 v;
   if (once)
@@ -1470,9 +1470,9 @@ cudaError_t launch_router(const bf16* x, const bf16* Wg, int T, int h, int r, fl
 // tile's end.  Then, up to two tiles of 16 per block, the whole block again; beyond, and for narrow rows that
 // leave 16 warps little to share, four teams, which run out of step and so keep more loads in flight.  Router
 // rows that do not fit shared memory are read once per tile and warp: the whole block shares them.  Calibration
-// in us, one team / four teams, 2000, 4096, 8192, 16384 tokens: h 4096 21.6 / 22.9, 25.1 / 25.6, 31.8 / 28.0,
-// 54.8 / 53.4; h 1024, 8192 tokens 26.0 / 21.2; h 128, 8192 tokens 23.7 / 19.6; h 8192, 16 experts (not in
-// shared memory), 4096 tokens 35 / 49.
+// in us, one team / four teams, 2000, 4096, 8192, 16384 tokens: h 4096, 8 experts 20.4 / 23.2, 24.6 / 24.8, 31.1 / 27.9,
+// 56.4 / 50.8, 16 experts 23.3 / 27.1, 28.0 / 29.0, 36.4 / 32.1; h 2048 19.4 / 20.7, 22.0 / 21.0, 27.0 / 23.7, 36.9 / 30.8;
+// h 1024 18.7 / 18.5, 21.2 / 19.0, 24.8 / 21.3; top-k call on h 128, 8192 tokens 79.2 / 72.5.
 constexpr int kRouteShort = 148 * 8;
 inline bool route_in_teams(int T, int h, bool whole) { return whole && (h < 2048 || T > 2 * 148 * 16); }
 template <typename... KArgs, typename... Args>
