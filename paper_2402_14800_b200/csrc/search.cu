@@ -282,13 +282,7 @@ reduce_partials_kernel(const float* partial, int nblk, int nC, double* __restric
   const int mine = blockIdx.x * 8 + (threadIdx.x & 7), first = threadIdx.x >> 3;
   double v = 0.0;
   if (mine < nC)
-    for (int b0 = first; b0 < nblk; b0 += 8 * 32) {  // eight reads in flight; adding 0 changes nothing
-      float part[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) part[u] = b0 + 32 * u < nblk ? ld_l2(partial + (size_t)(b0 + 32 * u) * nC + mine) : 0.f;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) v += (double)part[u];
-    }
+    for (int b = first; b < nblk; b += 32) v += (double)ld_l2(partial + (size_t)b * nC + mine);
   s_sum[threadIdx.x & 7][first] = v;
   __syncthreads();
   v = s_sum[warp][lane];
