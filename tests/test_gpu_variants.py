@@ -798,7 +798,7 @@ def test_enumerations_of_every_list_length_against_the_oracle(E, r, T):
 def test_host_calls_in_column_slabs_equal_the_device_call(h, E, T):
     # below the line, two and four slabs, slabs of different widths, a last slab that ends inside a weight tile
     build.build()
-    W = synth.make_layer_weights(h, 128, E, seed=78, device=DEV)
+    W = synth.make_layer_weights(h, 1024, E, seed=78, device=DEV)  # (with fewer features the line is at 8 Mi values)
     layer = binding.MoeLayer(W.W_gate, W.W1, W.W3, W.W2)
     x = synth.make_tokens(T, h, seed=79, device=DEV)
     want = layer.forward(x, 0.3).cpu()
